@@ -17,7 +17,7 @@ from paper_2205_10072_b200 import workloads
 def listed():
     return [
         # The paper's own use: a node asks for the rows of its own 32 ranks and owns no scratch memory.
-        {"name": "own rows, 32 of 1M", "kind": "range", "p": 2**20 + 2**14, "ranks": 32, "scratch": False},
+        {"name": "own rows 32 of 1M", "kind": "range", "p": 2**20 + 2**14, "ranks": 32, "scratch": False},
         # All ranks of the largest cluster of the paper's experiments (36 nodes x 32): the smallest tables.
         {"name": "table 1152", "kind": "table", "p": 1152},
         # The size up to which the paper's author verified: an ordinary large machine.
@@ -25,7 +25,7 @@ def listed():
         # A million ranks, just above a power of two (the benchmark's single p).
         {"name": "table 1M", "kind": "table", "p": 2**20 + 2**14},
         # One of 16 shards of the same job, built where it is needed.
-        {"name": "range, 64K of 1M", "kind": "range", "p": 2**20 + 2**14, "ranks": 65536 + 17, "scratch": True},
+        {"name": "range 64K of 1M", "kind": "range", "p": 2**20 + 2**14, "ranks": 65536 + 17, "scratch": True},
         # A broadcast from a root that is not rank 0, at a count that is no power of two's neighbour.
         {"name": "rooted 1.3M", "kind": "rooted", "p": 1300003},
         # Tables too large to want at once: eight chunks, receive rows as they are built, send rows after.
