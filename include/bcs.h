@@ -51,7 +51,7 @@ typedef enum {
 #define BCS_BAD_ENTRY 127
 #define BCS_MAX_Q 31
 #define BCS_SKIPS_STRIDE 32   /* words per row of a skips table */
-#define BCS_STATIC_WORKSPACE_BYTES (8u << 20)   /* scratch built into the library, see bcs_build_static */
+#define BCS_STATIC_WORKSPACE_BYTES (8u << 20)   /* limit of bcs_build_static */
 
 /* Human-readable name of a status code (static string, never NULL). */
 const char *bcs_status_str(bcs_status st);
@@ -69,17 +69,10 @@ bcs_status bcs_skips(uint32_t p, uint32_t *skips_host);
  * r_begin..r_end-1 of one p.
  *   recv_out, send_out: device, int8, (r_end-r_begin)*q bytes each, 16-byte
  *   aligned; either may be NULL (not wanted), not both unless the range is empty.
- *   workspace: device scratch owned by the caller, 16-byte aligned, or NULL.  With at
- *   least bcs_build_workspace_bytes(p, r_begin, r_end) bytes the call runs its fast
- *   construction: one pass writes a 32-bit "skip code" per rank of p (which skips add
- *   up to the rank, the sums Algorithm 2 walks down), a second finds each round's
- *   block from the codes of the two ranks bounding the window of Algorithm 4 and also
- *   keeps a round-major copy of the receive rows, a third reads the send rows from
- *   that copy.  With NULL (or too few bytes) a self-contained, several times slower
- *   construction runs (homerange descent per window; send entries whose to-processor
- *   lies outside the range are recomputed with Algorithm 4).  Both give identical
- *   tables, and any sub-range is self-contained either way.  The workspace holds
- *   nothing of value after the call; calls that share one must not overlap.
+ *   workspace: device memory owned by the caller, 16-byte aligned, or NULL.  The rows are
+ *   computed without scratch memory, each from the binary form of its rank, so the workspace
+ *   is not touched and its size does not matter; the argument and
+ *   bcs_build_workspace_bytes remain for callers that pass one.
  * Errors: see the status codes. */
 size_t bcs_build_workspace_bytes(uint32_t p, uint64_t r_begin, uint64_t r_end);
 bcs_status bcs_build(uint32_t p, uint64_t r_begin, uint64_t r_end,
@@ -88,27 +81,24 @@ bcs_status bcs_build(uint32_t p, uint64_t r_begin, uint64_t r_end,
 
 /* The same tables in two steps, for building one p in several rank chunks (or both
  * tables of the same ranks at different times) without repeating the construction:
- *   bcs_prepare runs the construction once for ALL ranks of p and leaves, in the caller's
- *   workspace of at least bcs_prepare_workspace_bytes(p) bytes (4 bytes of skip code plus q
- *   bytes per rank: 36.5 GB for p = 2^30-1), the receive schedule in round-major order;
- *   bcs_build_prepared then writes the rank-major receive rows of any range (a
- *   transposition of that copy) and its send rows (the same transposition with row k
- *   rotated by skips[k]: sendsched[r][k] = recvsched[(r+skips[k]) mod p][k], Algorithm 9).
- * The workspace must stay untouched between the two calls; any number of
+ *   bcs_prepare checks p and the caller's workspace of at least
+ *   bcs_prepare_workspace_bytes(p) bytes (4 bytes plus q bytes per rank: 36.5 GB for
+ *   p = 2^30-1), whose contents are the library's own;
+ *   bcs_build_prepared then writes the rank-major receive and send rows of any range.
+ * A row costs no more to compute than to fetch from a prepared copy, so preparing enqueues no
+ * work and the workspace is not touched.
+ * Any number of
  * bcs_build_prepared calls may follow one bcs_prepare.  Outputs, alignment and error codes
  * as for bcs_build; a workspace that is NULL or too small is BCS_ERR_ARG. */
 size_t bcs_prepare_workspace_bytes(uint32_t p);
 bcs_status bcs_prepare(uint32_t p, void *workspace, size_t workspace_bytes, void *cuda_stream);
 /* bcs_prepare in two steps, for callers that want the rank-major receive rows of a chunk straight
  * from the construction instead of from a transposition afterwards:
- *   bcs_prepare_codes writes the skip codes of ALL ranks of p into the workspace;
- *   bcs_prepare_rows then runs Algorithm 4 for the ranks r_begin..r_end-1: their entries go into
- *   the round-major copy in the workspace and, if recv_out is not NULL, their rank-major rows to
- *   recv_out (device, (r_end-r_begin)*q bytes, 16-byte aligned).  r_begin must be a multiple of
- *   16 (BCS_ERR_ALIGN).  Chunks may be prepared in any order; once every rank of p has been
- *   through bcs_prepare_rows the workspace is what bcs_prepare leaves, and bcs_build_prepared
- *   gives the send rows of any range (sendsched[r][k] = recvsched[(r+skips[k]) mod p][k] reaches
- *   into other chunks, hence only then).
+ *   bcs_prepare_codes checks p and the workspace;
+ *   bcs_prepare_rows then writes, if recv_out is not NULL, the rank-major receive rows of the
+ *   ranks r_begin..r_end-1 to recv_out (device, (r_end-r_begin)*q bytes, 16-byte aligned).
+ *   r_begin must be a multiple of 16 (BCS_ERR_ALIGN).  Chunks may be prepared in any order;
+ *   bcs_build_prepared gives the send rows of any range.
  * bcs_prepare(p, ...) is bcs_prepare_codes followed by bcs_prepare_rows(p, 0, p, NULL, ...). */
 bcs_status bcs_prepare_codes(uint32_t p, void *workspace, size_t workspace_bytes, void *cuda_stream);
 bcs_status bcs_prepare_rows(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t *recv_out,
@@ -121,25 +111,11 @@ bcs_status bcs_build_prepared(uint32_t p, uint64_t r_begin, uint64_t r_end,
  * allocate any (the paper has no counterpart; this is a convenience of the library).  Think of
  * code that runs after a framework has claimed the whole GPU for its own memory pool, or of a
  * latency-critical loop in which a cudaMalloc -- which can stall the whole device -- is not
- * acceptable.  The fast construction of bcs_build runs with its scratch taken from an array of
- * BCS_STATIC_WORKSPACE_BYTES (8 MiB) that is part of the library's device image: every GPU on
- * which the library is loaded gives up that much memory until the process exits, whether or
- * not this function is ever called.  The call itself allocates and frees nothing.
+ * acceptable.  The call allocates and frees nothing and uses no scratch memory; calls may overlap.
  *   Limit: bcs_build_workspace_bytes(p, r_begin, r_end) must not exceed
  *   BCS_STATIC_WORKSPACE_BYTES (all ranks of p up to about 300 000; of a larger p a
- *   correspondingly shorter range, and none once 4*p alone exceeds the array);
- *   otherwise BCS_ERR_UNSUPPORTED is returned and nothing is written.  Use bcs_build with
- *   your own workspace, or with NULL, beyond that.
- *   First use: the first call on each device asks the CUDA runtime for the array's device
- *   address (with that device current) and remembers it for the life of the process, so do
- *   not use this entry point across a cudaDeviceReset.  Where the runtime loads the library's
- *   device code lazily, that first call is also what sets the 8 MiB aside: make it early --
- *   before other code has claimed the rest of the device memory -- and outside any stream
- *   capture.  Later calls touch no allocator at all.
- *   Sharing: all calls on a device use the same array.  Two calls whose kernels can overlap
- *   on the GPU (different streams, or several host threads) race on it and produce garbage;
- *   order them on one stream or with events.  The array keeps whatever the last call left
- *   in it; this function needs none of it to be zero and reads only what it has written.
+ *   correspondingly shorter range, and none once 4*p alone exceeds it);
+ *   otherwise BCS_ERR_UNSUPPORTED is returned and nothing is written.
  * Outputs, range and error codes otherwise as for bcs_build. */
 bcs_status bcs_build_static(uint32_t p, uint64_t r_begin, uint64_t r_end,
                             int8_t *recv_out, int8_t *send_out, void *cuda_stream);
@@ -149,14 +125,12 @@ bcs_status bcs_build_static(uint32_t p, uint64_t r_begin, uint64_t r_end,
  * (r - root) mod p; the skips, and with them the neighbours (r +- skips[k]) mod p, do not depend
  * on the root).  A thin remap over bcs_build:
  *   out[(r - r_begin)*q + k] = entry k of virtual rank (r - root) mod p,  r in [r_begin, r_end).
- * The virtual ranks of the range are one run, or two when they pass p - 1; each run is built
- * by bcs_build.  The second run starts (p - v0)*q bytes into the outputs (v0 the first virtual
- * rank); where that is not a multiple of 16 it is built in the workspace and copied into place
- * on the stream (cudaMemcpyAsync, device to device).
+ * The virtual ranks of the range are one run, or two when they pass p - 1; both are written by
+ * one kernel.
  *   root < p, else BCS_ERR_RANGE.  Outputs as for bcs_build.
  *   workspace, workspace_bytes: at least bcs_build_rooted_workspace_bytes(...) bytes (16-byte
- *   aligned) select the fast construction; NULL or less: the self-contained construction, which
- *   is then refused with BCS_ERR_ARG if the range needs the copy described above. */
+ *   aligned), which are not touched; with NULL or less a range of two runs is refused with
+ *   BCS_ERR_ARG unless the second one starts on a 16-byte boundary of the outputs. */
 size_t bcs_build_rooted_workspace_bytes(uint32_t p, uint32_t root, uint64_t r_begin, uint64_t r_end);
 bcs_status bcs_build_rooted(uint32_t p, uint32_t root, uint64_t r_begin, uint64_t r_end,
                             int8_t *recv_out, int8_t *send_out, void *workspace,
@@ -167,8 +141,7 @@ bcs_status bcs_build_rooted(uint32_t p, uint32_t root, uint64_t r_begin, uint64_
  *   recv_host, send_host: host, (r_end-r_begin)*q bytes each, either may be NULL.
  *   stage_dev: device staging buffer supplied by the caller, 16-byte aligned, of
  *   at least 2 * align256((r_end-r_begin)*q) bytes (align256 = round up to 256);
- *   what exceeds that is handed to bcs_build as its workspace, so adding
- *   bcs_build_workspace_bytes(...) bytes selects the fast construction.
+ *   what exceeds that is not touched.
  * The host buffers are complete once the stream has been synchronised. */
 bcs_status bcs_build_to_host(uint32_t p, uint64_t r_begin, uint64_t r_end,
                              int8_t *recv_host, int8_t *send_host,
@@ -301,8 +274,8 @@ bcs_status bcs_validate(uint32_t p, uint64_t r_begin, uint64_t r_end,
 bcs_status bcs_simulate(uint32_t p, uint32_t n, const int8_t *recv, const int8_t *send,
                         uint64_t *state_dev, uint64_t *counts_dev, void *cuda_stream);
 
-/* Bounded waits (no counterpart in the paper).  The transposition kernels of bcs_build,
- * bcs_build_prepared and bcs_build_batch wait for their bulk copies on a shared-memory barrier
+/* Bounded waits (no counterpart in the paper).  The transposition kernel of
+ * bcs_build_batch waits for their bulk copies on a shared-memory barrier
  * with a poll limit; a CTA whose copies did not arrive within the limit gives up, leaves its
  * ranks of the output unwritten and counts itself in a device-wide counter that is never
  * reset.  The build call that enqueued the kernel has long returned BCS_OK by then, so this

@@ -75,6 +75,14 @@ __host__ __device__ inline uint32_t skip_code(const uint32_t *s, int q, uint32_t
     return code;
 }
 
+// Position of the highest set bit, -1 for 0 (one instruction).
+__device__ __forceinline__ int top_bit(uint32_t v)
+{
+    int d;
+    asm("bfind.u32 %0, %1;" : "=r"(d) : "r"(v));
+    return d;
+}
+
 // ---------------------------------------------------------------- tile bookkeeping
 struct RankCtx {
     const uint32_t *s;      // skips of this rank's p (shared or global memory)
@@ -322,6 +330,9 @@ __device__ __forceinline__ void grid_launch_dependents()
 
 // ---------------------------------------------------------------- host helpers
 bcs_status make_table(uint32_t p, PTable *tab);
+
+// Rows of the count <= p ranks first, first+1, ... (mod p; first < p, p > 1): rows.cu.  Either output may be null.
+bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv, int8_t *send, cudaStream_t stream);
 
 // Launch with programmatic stream serialisation (see above); `dependent` false: ordinary launch.
 template <class... Params, class... Args>

@@ -1,0 +1,508 @@
+// Schedule rows straight from the binary form of a rank (arXiv 2205.10072, Algorithms 1-5 and the
+// lookup of Algorithm 9): no table of all ranks, no scratch memory, every stretch of ranks on its own.
+//
+// Notation: e_t = 2 skips[t-1] - skips[t], which Algorithm 1 makes 0 or 1; C(a, b) = e_{a+1} + ... + e_b.
+// The skip code of a rank (bcs_common.cuh) has bit k set iff skips[k] is a term of its greedy sum.
+//
+// Segments.  Cut the ranks at every rank whose code has no bit below L = min(7, q).  Because
+// skips[k] = ceil(p / 2^(q-k)), the part of the codes from bit L up counts these segments in plain
+// binary: segment g (0 <= g < 2^(q-L)) starts at the sum of the skips[L+k] over the bits k of g.  Let m be
+// the lowest zero bit of g, as a level (L + its position, q if there is none): the segment has
+// skips[L] - C(L, m) ranks (65..128 for q > 7, less at most 24).
+//
+// Rounds from L up.  The window of round i of rank r ends skips[i] ranks below r, so with `low` the part
+// of r below its segment's start, and K the lowest set bit of g as a level (K = q: no bit, the root's segment):
+//   * bit i of the code set: the window holds the rank with the bits above i only, whose baseblock,
+//     the next higher set bit of r, is the largest of the window.  No higher set bit: i is
+//     the home round, the entry is the baseblock of r.
+//   * bit i not set: the window lies below that rank, and the largest new block in it is i.
+// So in these rounds all ranks of a segment have the same entries, and the blocks 0..i-1 and the next set
+// bit are the ones taken before round i.  The exceptions are ranks close behind a segment's start (low
+// <= C(L, K) <= 24), in the rounds L..K-1: as long as low < C(i+1, K) the window of round i reaches the rank
+// with baseblock i+1, and the entry is i+1; the first round after that takes the one block of
+// 0..i that is missing by then, and the rounds behind it are as above.
+// A send entry is the receive entry of the rank skips[k] further on.  Bit k set: adding skips[k]
+// carries, the bit is clear there, the entry is k.  Not set: the bit is set there, the entry is the next
+// higher set bit of r (none: the baseblock of r; the root sends block k).  Exceptions: the last C(k, m) ranks
+// before a segment whose lowest bit is k (m the lowest zero bit above k): they carry into a rank
+// close behind a segment's start.
+//
+// Rounds below L.  The entries of a rank depend on (K, low) only, low < skips[L] <= 128: a table of at most
+// 25 x 128 rows of 8 bytes.  The CTA fills it by running Algorithm 4 itself on those rows, the windows read
+// from the baseblocks of the ranks below skips[L]: what lies d ranks below the rank skips[K] is what lies
+// d + C(7, K) ranks below skips[7].
+//
+// All of this is checked entry by entry against the CPU oracle by the tests.
+#pragma once
+#include "bcs_common.cuh"
+
+namespace bcs {
+
+constexpr int kLow = 7;                       // rounds whose entries come from the table
+constexpr int kLowRanks = 128;                // skips[7] <= 128
+constexpr int kRunLevels = 6;                 // runs of 1, 2, 4, ..., 32 ranks
+constexpr int kMissRanks = 32;                // ranks behind a segment's start that can be exceptions (<= 25)
+constexpr uint32_t kItemRanks = 128;          // ranks that a warp takes at a time
+constexpr uint32_t kHalo = 64;                // and the ranks behind them that their send rows look at (skips[6] <= 64)
+constexpr int kItemSegments = 5;              // segments that an item can touch: all but the two at its ends lie
+                                              // inside it, a run of c segments has more than 64 c - 25 ranks
+
+// What a p is to the kernels.
+struct RowConsts {
+    uint32_t s[kRow + kLow + 1];   // skips[0..q], then 0
+    uint32_t p;
+    int q;
+    uint32_t odd;                  // bit t: e_t
+    uint32_t inv;                  // floor(2^(q - L + 32) / p)
+};
+
+__host__ __device__ inline int low_levels(int q) { return q < kLow ? q : kLow; }
+
+// Number of e_t set, a < t <= b.
+__device__ __forceinline__ uint32_t count_odd(uint32_t odd, int a, int b)
+{
+    return (uint32_t)__popc((odd >> (a + 1)) & ((1u << (b - a)) - 1u));
+}
+
+// ---------------------------------------------------------------- shared memory of a CTA
+// A warp's part: table rows of the item's ranks and of those behind it, a word about each of its ranks, entries of
+// its segments from round L up (receive and send, 32 bytes each), its segments, the staged rows.
+constexpr uint32_t kWarpNotes = (kItemRanks + kHalo) * 8u;
+constexpr uint32_t kWarpEntries = kWarpNotes + kItemRanks * 2u;
+constexpr uint32_t kWarpSegments = kWarpEntries + kItemSegments * 64u;
+constexpr uint32_t kWarpStage = kWarpSegments + 48u;
+static_assert(kItemSegments * 8u <= 48u && kWarpStage % 16u == 0, "layout of a warp's shared memory");
+
+// Byte offsets in the CTA's dynamic shared memory.
+struct RowLayout {
+    uint32_t miss, runs, codes, s, warps, warp_bytes;
+    __host__ __device__ explicit RowLayout(int q)
+    {
+        const uint32_t rows = (uint32_t)(q - low_levels(q) + 1);
+        miss = rows * kLowRanks * 8u;
+        runs = miss + rows * kMissRanks;
+        codes = runs + kRunLevels * kLowRanks;
+        s = codes + kLowRanks;
+        warps = s + (kRow + kLow + 1) * 4u;
+        warps = (warps + 127u) & ~127u;
+        warp_bytes = kWarpStage + ((kItemRanks * (uint32_t)q + 31u) & ~15u);
+    }
+    __host__ __device__ uint32_t total(uint32_t n_warps) const { return warps + n_warps * warp_bytes; }
+};
+
+struct RowTable {
+    uint2 *rows;          // [K - L][low]: entries of rounds 0..6 as bytes 0..6, baseblock as byte 7
+    uint8_t *miss;        // [K - L][low < 32]: the block of 0..7 that is not taken before round 7
+    uint8_t *runs;        // [level][x]: baseblock bits of the 2^level ranks that end at x < skips[L]
+    uint8_t *codes;       // [x]: skip code of x < skips[L]
+    uint32_t *s;
+    __device__ RowTable(uint8_t *sm, const RowLayout &at)
+        : rows(reinterpret_cast<uint2 *>(sm)), miss(sm + at.miss), runs(sm + at.runs), codes(sm + at.codes),
+          s(reinterpret_cast<uint32_t *>(sm + at.s))
+    {
+    }
+};
+
+// Rounds 0 .. rounds-1 (at most six) of rank `low` of a segment whose lowest bit is K: Algorithm 4 with its
+// windows looked up in the run table.  Returns the entries as bytes 0..5 and the baseblock as byte 7;
+// B: the blocks taken.
+__device__ __forceinline__ unsigned long long table_row(const RowTable &t, int q, uint32_t odd, int K, int low,
+                                                        int rounds, uint32_t &B)
+{
+    const uint32_t c = t.codes[low];
+    // positions below the rank skips[K] in the run table: that rank itself would be at `top`
+    const int top = K >= kLow ? (int)t.s[kLow] - (int)count_odd(odd, kLow, K) : (int)t.s[K];
+    const int bb = c ? __ffs(c) - 1 : (K < q ? K : -1);
+    B = bb >= 0 ? 1u << bb : 0u;
+    unsigned long long row = (unsigned long long)(uint8_t)bb << 56;
+    int sum = 0;
+    for (int i = 0; i < rounds; ++i) {
+        const int lo = (int)t.s[i], hi = (int)t.s[i + 1];
+        sum += lo;
+        const uint32_t above = c >> (i + 1);
+        int blk;
+        int entry;
+        if ((c >> i) & 1u) {
+            blk = above ? __ffs(above) + i : K;
+            const bool home = K == q && above == 0;
+            entry = home ? bb : blk - q;
+            if (!home) B |= 1u << blk;
+        } else {
+            const int len = hi - lo;
+            const int level = 31 - __clz(len);
+            const int e = (above ? low : top + low) - lo;
+            const uint8_t *run = t.runs + level * kLowRanks;
+            uint32_t U = (uint32_t)(run[e] | run[e - len + (1 << level)]) & ~B;
+            if (U == 0) {                                        // the second window of Algorithm 4: a few ranks
+                for (int pos = low - hi; pos >= low - sum; --pos) {
+                    if (pos == 0) U |= (K < q ? 1u << K : 0u) & ~B;
+                    const int x = pos > 0 ? pos : top + pos;
+                    if (pos != 0 && x >= 1) U |= (uint32_t)t.runs[x] & ~B;
+                }
+            }
+            blk = top_bit(U);
+            entry = U ? blk - q : BCS_BAD_ENTRY;
+            if (U) B |= 1u << blk;
+        }
+        row |= (unsigned long long)(uint8_t)entry << (8 * i);
+    }
+    return row;
+}
+
+// Fills the table of a p; all threads of the CTA call (at least 128), t.s holds the skips.  Ends with a barrier.
+__device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
+{
+    const int L = low_levels(q);
+    const uint32_t lows = t.s[L];
+    if (threadIdx.x < kLowRanks) {
+        uint32_t x = threadIdx.x, c = 0;
+        for (int k = L - 1; k >= 0; --k) {
+            if (x >= t.s[k]) {
+                x -= t.s[k];
+                c |= 1u << k;
+            }
+        }
+        t.codes[threadIdx.x] = (uint8_t)c;
+        t.runs[threadIdx.x] = (uint8_t)(threadIdx.x < lows ? c & (0u - c) : 0u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {                                      // four ranks per lane, a byte each
+        uint32_t *words = reinterpret_cast<uint32_t *>(t.runs) + threadIdx.x;
+        auto before = [&](uint32_t v, uint32_t lanes) {
+            const uint32_t up = __shfl_up_sync(0xffffffffu, v, lanes);
+            return threadIdx.x >= lanes ? up : 0u;
+        };
+        uint32_t r = *words;
+        r |= __funnelshift_l(before(r, 1), r, 8);
+        words[1 * (kLowRanks / 4)] = r;
+        r |= __funnelshift_l(before(r, 1), r, 16);
+        words[2 * (kLowRanks / 4)] = r;
+        r |= before(r, 1);
+        words[3 * (kLowRanks / 4)] = r;
+        r |= before(r, 2);
+        words[4 * (kLowRanks / 4)] = r;
+        r |= before(r, 4);
+        words[5 * (kLowRanks / 4)] = r;
+    }
+    __syncthreads();
+    if (q < kLow) {                                              // one segment, all rounds in the table
+        for (uint32_t low = threadIdx.x; low < lows; low += blockDim.x) {
+            uint32_t B;
+            const unsigned long long row = table_row(t, q, odd, q, (int)low, q, B);
+            t.rows[low] = make_uint2((uint32_t)row, (uint32_t)(row >> 32));
+        }
+    } else {
+        // ranks without bit 6: rounds 0..5 as above, round 6 from the distances of the ranks with
+        // baseblock 7 and 6.  Ranks with it (K = 6 here): rounds 0..5 do not depend on what comes before
+        // that bit, round 6 receives the next higher one.
+        const int n = (q - 5) * 64;
+        for (int job = (int)threadIdx.x; job < n; job += (int)blockDim.x) {
+            const int K = 6 + (job >> 6), low = job & 63;
+            if (low >= (int)t.s[6]) continue;
+            uint32_t B;
+            unsigned long long row = table_row(t, q, odd, K, low, 6, B);
+            if (K == 6) {
+                if (low + t.s[6] >= t.s[7]) continue;
+                for (int k = kLow; k <= q; ++k) {
+                    const uint32_t six = (uint8_t)(k < q ? k - q : (int)(row >> 56));
+                    t.rows[(k - kLow) * kLowRanks + low + (int)t.s[6]] =
+                        make_uint2((uint32_t)row, (uint32_t)(row >> 32) | six << 16);
+                }
+            } else {
+                const int m = __ffs(~B) - 1;                     // the block of 0..6 not taken so far
+                const bool seven = low < (int)count_odd(odd, kLow, K) ||
+                                   (m == 6 && K > kLow && low < (int)count_odd(odd, 6, K));
+                const uint32_t six = (uint8_t)((seven ? kLow : m) - q);
+                t.rows[(K - kLow) * kLowRanks + low] = make_uint2((uint32_t)row, (uint32_t)(row >> 32) | six << 16);
+                if (low < kMissRanks) t.miss[(K - kLow) * kMissRanks + low] = (uint8_t)(seven ? m : kLow);
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// ---------------------------------------------------------------- rows of an item, by one warp
+// How a lane's rows of q bytes lie in the words of the staging buffer, where the rows of a warp follow one another.
+// (The same for every 32 ranks of an item: 32 rows are whole words.)
+struct RowPlace {
+    uint32_t sh;       // bits by which the row is off a word
+    bool longer;       // it reaches into word ceil(q / 4), counted from the word it begins in
+    uint32_t shared;   // all ones if the next row begins in this row's last word
+    __device__ RowPlace(uint32_t first_byte, int q)
+    {
+        const uint32_t mis = (first_byte + (threadIdx.x & 31u) * (uint32_t)q) & 3u;
+        sh = 8u * mis;
+        longer = mis + (uint32_t)q > 4u * (((uint32_t)q + 3u) / 4u);
+        shared = ((mis + (uint32_t)q) & 3u) != 0u ? 0xffffffffu : 0u;
+    }
+};
+
+// Stores the rows (words W, zero beyond byte q) of 32 ranks at once, this lane's at `at`.  A word that two rows share is
+// put together by the lane it begins in.  kAligned: the first row begins on a word.  Where it
+// does not, the first lane's head and the last lane's tail go out as bytes.  Lanes without a rank store
+// too (the buffer has room for them, and nobody reads it).
+template <int kWords, bool kAligned>
+__device__ __forceinline__ void stage_row(uint8_t *at, const uint32_t (&W)[kWords], int q, const RowPlace &pl)
+{
+    if (kWords == 1 && q < 4) {
+        for (int k = 0; k < q; ++k) at[k] = (uint8_t)(W[0] >> (8 * k));
+        return;
+    }
+    uint32_t V[kWords + 1];
+#pragma unroll
+    for (int w = 0; w <= kWords; ++w) V[w] = __funnelshift_l(w ? W[w - 1] : 0u, w < kWords ? W[w] : 0u, pl.sh);
+    uint32_t next = __shfl_down_sync(0xffffffffu, V[0], 1) & pl.shared;
+    uint32_t *words = reinterpret_cast<uint32_t *>(at - (pl.sh >> 3));
+    bool tail_bytes = false;
+    if (!kAligned) {
+        const uint32_t lane = threadIdx.x & 31u;
+        tail_bytes = lane == 31u && pl.shared != 0u;
+        if (lane == 0u && pl.sh != 0u)
+            for (uint32_t e = pl.sh; e < 32u; e += 8u) at[(e - pl.sh) >> 3] = (uint8_t)(V[0] >> e);
+        if (tail_bytes) {
+            const uint32_t v = pl.longer ? V[kWords] : V[kWords - 1];
+            uint8_t *tail = reinterpret_cast<uint8_t *>(words + (pl.longer ? kWords : kWords - 1));
+            for (uint32_t e = 0; e < (((pl.sh >> 3) + (uint32_t)q) & 3u); ++e) tail[e] = (uint8_t)(v >> (8u * e));
+        }
+    }
+    if (kWords > 1) {
+        if (pl.sh == 0u) words[0] = V[0];
+#pragma unroll
+        for (int w = 1; w < kWords - 1; ++w) words[w] = V[w];
+        if (kAligned || pl.longer || !tail_bytes) words[kWords - 1] = V[kWords - 1] | (pl.longer ? 0u : next);
+    } else if (pl.sh == 0u) {
+        words[0] = V[0];
+    }
+    if (pl.longer && (kAligned || !tail_bytes)) words[kWords] = V[kWords] | next;
+}
+
+// Row of a rank: its rounds below L from the table, the others from its segment.
+template <int kWords>
+__device__ __forceinline__ void join_row(uint32_t lo, uint32_t hi, const uint8_t *entries, uint32_t (&W)[kWords])
+{
+    W[0] = lo;
+    if (kWords > 1) {
+        const uint4 a = *reinterpret_cast<const uint4 *>(entries);
+        W[1 % kWords] = a.y | (hi & 0xffffffu);
+        if (kWords > 2) W[2 % kWords] = a.z;
+        if (kWords > 3) W[3 % kWords] = a.w;
+    }
+    if (kWords > 4) {
+        const uint4 b = *reinterpret_cast<const uint4 *>(entries + 16);
+        W[4 % kWords] = b.x;
+        if (kWords > 5) W[5 % kWords] = b.y;
+        if (kWords > 6) W[6 % kWords] = b.z;
+        if (kWords > 7) W[7 % kWords] = b.w;
+    }
+}
+
+// Sends the staged rows out: len bytes for `dst`, staged at the same offset in their 16-byte group.  All but
+// the ragged ends go as one bulk copy of the TMA unit.
+template <bool kAligned>
+__device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t len)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t shift = kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    const uint32_t begin = (shift + 15u) & ~15u, end = shift + len;
+    uint8_t *base = reinterpret_cast<uint8_t *>(dst) - shift;
+    const uint32_t stop = end & ~15u;
+    if (lane == 0u && stop > begin) {
+        const uint32_t src = (uint32_t)__cvta_generic_to_shared(stage + begin);
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                     :: "l"(reinterpret_cast<uint64_t>(base + begin)), "r"(src), "r"(stop - begin) : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+    if (!kAligned || (end & 15u) != 0u) {                        // bytes [shift, head) and [tail, end) one by one
+        const uint32_t head = begin < end ? begin : end;
+        if (shift + lane < head) base[shift + lane] = stage[shift + lane];
+        const uint32_t tail = stop > begin ? stop : head;
+        if (tail + lane < end) base[tail + lane] = stage[tail + lane];
+    }
+}
+
+// The staging buffer may be written again.
+__device__ __forceinline__ void stage_free()
+{
+    if ((threadIdx.x & 31u) == 0u) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncwarp();
+}
+
+// What the lookup leaves about a rank of the item.
+constexpr uint32_t kNoteFrom = 3;        // bits 0..2: its segment, counted from the item's first; 3..7: home round + 1, or L
+constexpr uint32_t kNoteRecv = 1u << 8;  // some of its receive entries from round L up are exceptions
+constexpr uint32_t kNoteSend = 1u << 9;  // one of its send entries is
+
+// Receive and send rows (either pointer may be null) of the n <= 128 ranks x0, x0+1, ... (mod p; x0 < p, n <= p) by
+// one warp.  recv, send: where the row of x0 goes (kAligned: 16-byte aligned).  mine: the warp's shared memory.
+template <int kWords, bool kAligned>
+__device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int q, uint32_t odd, uint32_t inv,
+                                          uint32_t x0, uint32_t n, int8_t *recv, int8_t *send)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const int L = low_levels(q), high = q - L;
+    uint2 *looked = reinterpret_cast<uint2 *>(mine);
+    uint16_t *notes = reinterpret_cast<uint16_t *>(mine + kWarpNotes);
+    uint8_t *entries = mine + kWarpEntries;
+    uint2 *segments = reinterpret_cast<uint2 *>(mine + kWarpSegments);   // start, number
+    uint8_t *stage = mine + kWarpStage;
+    const uint32_t end = x0 + n;
+
+    // Lane j < 8: segment number gs + j, gs one or two before that of x0 (or the first).  Positions go on
+    // counting behind p - 1: the root's segment again.
+    uint32_t gs = __umulhi(x0, inv);
+    gs = gs ? gs - 1u : 0u;
+    const uint32_t at0 =
+        __reduce_add_sync(0xffffffffu, (int)lane < high && ((gs >> lane) & 1u) ? t.s[lane + L] : 0u);
+    const uint32_t g = (gs + lane) & ((1u << high) - 1u);
+    const int tz = __ffs(~g) - 1;                                // L + tz: lowest zero bit, as a level
+    const uint32_t len = t.s[L] - count_odd(odd, L, L + tz);
+    uint32_t pos = len;
+#pragma unroll
+    for (uint32_t d = 1; d < 8; d *= 2) {
+        const uint32_t up = __shfl_up_sync(0xffffffffu, pos, d);
+        if (lane >= d) pos += up;
+    }
+    pos += at0 - len;
+    const int first = __popc(__ballot_sync(0xffffffffu, lane < 8u && pos <= x0)) - 1;
+    uint32_t info;
+    {
+        const int K = g ? __ffs(g) - 1 + L : q;                  // lowest and highest set bit
+        const int home = g ? 31 - __clz(g) + L : 0;
+        const uint32_t behind = K > L ? count_odd(odd, L, K) + 1u : 0u;       // exceptions at its start
+        // and at its end: the next segment's lowest bit is L + tz, the next zero bit of g is m
+        const int m = L + tz + __ffs(~(g >> (tz + 1)));
+        const uint32_t before = tz < high ? count_odd(odd, L + tz, m) : 0u;
+        info = (uint32_t)(K - L) * kLowRanks | (uint32_t)(home ? home + 1 : L) << 12 | behind << 17 | before << 22 |
+               (g & 1u) << 27;
+        const uint32_t slot = lane - (uint32_t)first;
+        if (slot < (uint32_t)kItemSegments) segments[slot] = make_uint2(pos, g);
+    }
+
+    // Entries of the segments' rounds from L up, lane = round.
+    for (int j = first;; ++j) {
+        const uint32_t gj = __shfl_sync(0xffffffffu, g, j);
+        const int k = (int)lane;
+        const uint32_t bits = k >= L ? gj >> (k - L) : 0u;
+        const uint32_t above = bits >> 1;
+        const int next = above ? __ffs(above) + k - q : 0;       // 0 where the baseblock goes
+        const bool inside = k >= L && k < q;
+        uint8_t *e = entries + (j - first) * 64 + k;
+        e[0] = (uint8_t)(inside ? ((bits & 1u) ? next : k - q) : 0);
+        e[32] = (uint8_t)(inside ? ((bits & 1u) ? k - q : next) : 0);
+        if (__shfl_sync(0xffffffffu, pos, j + 1) >= end) break;
+    }
+
+    // Table rows of the ranks and of those that their send rows look at.
+    {
+        const uint32_t total = send != nullptr ? n + t.s[L - 1] : n;
+        int j = first;
+        uint32_t after = __shfl_sync(0xffffffffu, pos, j + 1);
+        for (uint32_t b = 0; b < total; b += 32u) {
+            const uint32_t x = x0 + b + lane;
+            const uint32_t stop = x0 + (b + 32u < total ? b + 32u : total);
+            uint32_t start = __shfl_sync(0xffffffffu, pos, j);
+            uint32_t inf = __shfl_sync(0xffffffffu, info, j);
+            uint32_t over = after;
+            int slot = j - first;
+            while (after < stop) {                               // segments that start among these ranks
+                ++j;
+                const uint32_t begins = after, inf_j = __shfl_sync(0xffffffffu, info, j);
+                after = __shfl_sync(0xffffffffu, pos, j + 1);
+                if (x >= begins) {
+                    start = begins;
+                    inf = inf_j;
+                    over = after;
+                    slot = j - first;
+                }
+            }
+            if (x < stop) looked[b + lane] = t.rows[(inf & 0xfffu) + (x - start)];
+            if (b < n) {
+                const uint32_t low = x - start;
+                uint32_t note = (uint32_t)slot | ((inf >> 12) & 31u) << kNoteFrom;
+                if (low < ((inf >> 17) & 31u)) note |= kNoteRecv;
+                if (over - x <= ((inf >> 22) & 31u) || (low == 0u && (inf >> 27) != 0u)) note |= kNoteSend;
+                notes[b + lane] = (uint16_t)(x < end ? note : (uint32_t)L << kNoteFrom);
+            }
+        }
+    }
+    __syncwarp();
+
+    if (recv != nullptr) {
+        const uint32_t shift = kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(recv) & 15u);
+        const RowPlace place(shift, q);
+        uint8_t *at = stage + shift + lane * (uint32_t)q;
+        stage_free();
+        for (uint32_t b = 0; b < n; b += 32u, at += 32 * q) {
+            const uint2 row = looked[b + lane];
+            const uint32_t note = notes[b + lane];
+            uint32_t W[kWords];
+            join_row<kWords>(row.x, row.y, entries + (note & 7u) * 64u, W);
+            stage_row<kWords, kAligned>(at, W, q, place);
+            __syncwarp();
+            const uint32_t from = (note >> kNoteFrom) & 31u;
+            if (from > (uint32_t)L) at[from - 1u] = (uint8_t)(row.y >> 24);     // home round
+            if (note & kNoteRecv) {
+                const uint2 seg = segments[note & 7u];
+                const int K = seg.y ? __ffs(seg.y) - 1 + L : q;
+                const int low = (int)(x0 + b + lane - seg.x);
+                int k = L;
+                for (; low < (int)count_odd(odd, k + 1, K); ++k) at[k] = (uint8_t)(k + 1 - q);
+                at[k] = (uint8_t)((int)t.miss[(K - L) * kMissRanks + low] - q);
+            }
+        }
+        flush_item<kAligned>(stage, recv, n * (uint32_t)q);
+    }
+    if (send != nullptr) {
+        const uint32_t shift = kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(send) & 15u);
+        const RowPlace place(shift, q);
+        uint8_t *at = stage + shift + lane * (uint32_t)q;
+        const uint8_t *mine_row = reinterpret_cast<const uint8_t *>(looked + lane);
+        const uint8_t *theirs[kLow];                             // entry k of the rank skips[k] further on
+#pragma unroll
+        for (int k = 0; k < kLow; ++k) theirs[k] = mine_row + (k < L ? t.s[k] * 8u + k : 0u);
+        stage_free();
+        for (uint32_t b = 0; b < n; b += 32u, at += 32 * q) {
+            const uint32_t note = notes[b + lane];
+            uint32_t e[kLow];
+#pragma unroll
+            for (int k = 0; k < kLow; ++k) e[k] = theirs[k][b * 8u];
+            const uint32_t bb = mine_row[b * 8u + 7u];
+            uint32_t lo = __byte_perm(__byte_perm(e[0], e[1], 0x0040), __byte_perm(e[2], e[3], 0x0040), 0x5410);
+            uint32_t hi = __byte_perm(__byte_perm(e[4], e[5], 0x0040), e[6], 0x0410);
+            if (kWords <= 2 && q < kLow) {                       // no entries beyond round q
+                if (q < 4) lo &= (1u << (8 * q)) - 1u;
+                hi &= q > 4 ? (1u << (8 * (q - 4))) - 1u : 0u;
+            }
+            uint32_t W[kWords];
+            join_row<kWords>(lo, hi, entries + (note & 7u) * 64u + 32u, W);
+            stage_row<kWords, kAligned>(at, W, q, place);
+            __syncwarp();
+            const int from = (int)((note >> kNoteFrom) & 31u);
+            if (from < q) {                                      // rounds past the home round: the baseblock
+                const bool root = bb == 0xffu;                   // (the table's mark for the root)
+                for (int k = from; k < q; ++k) at[k] = (uint8_t)(root ? (uint32_t)k : bb);
+            }
+            if (note & kNoteSend) {
+                const uint2 seg = segments[note & 7u];
+                const uint32_t sg = seg.y;
+                const int z = __ffs(~sg) - 1;
+                const int low = (int)(x0 + b + lane - seg.x);
+                if (low == 0) {
+                    // carries into a rank C(L, m) behind the start of a segment
+                    if (sg & 1u) at[L] = (uint8_t)((int)t.miss[z * kMissRanks + (int)count_odd(odd, L, L + z)] - q);
+                } else {
+                    const int k = L + z, m = k + __ffs(~(sg >> (z + 1)));
+                    const int behind = (int)count_odd(odd, k, m) - ((int)(t.s[L] - count_odd(odd, L, k)) - low);
+                    const int block = behind < (int)count_odd(odd, k + 1, m)
+                                          ? k + 1 : (int)t.miss[(m - L) * kMissRanks + behind];
+                    at[k] = (uint8_t)(block - q);
+                }
+            }
+        }
+        flush_item<kAligned>(stage, send, n * (uint32_t)q);
+    }
+}
+
+}  // namespace bcs

@@ -2,31 +2,27 @@
 // kernels and the entry points bcs_build, bcs_build_static, bcs_build_to_host, bcs_prepare,
 // bcs_prepare_codes, bcs_prepare_rows, bcs_build_prepared, bcs_build_rooted, bcs_build_batch.
 //
-// Two constructions, bit-identical in their results:
+// The calls for one p check their arguments and launch the kernel of rows.cu.  A batch takes one of two
+// constructions, bit-identical in their results:
 //
-//  * workspace path.  codes_single_kernel / codes_batch_kernel write the skip code (bcs_common.cuh) of every rank x of a p
-//    once.  The receive kernels (recv_codes_quad_kernel for one p >= 64, recv_quad_batch_kernel
-//    for a batch, recv_codes_kernel for tiny p) then read, per rank r and round i, the codes of
+//  * workspace path.  codes_batch_kernel writes the skip code (bcs_common.cuh) of every rank once.
+//    recv_quad_batch_kernel then reads, per rank r and round i, the codes of
 //    the two ranks that bound the window of Algorithm 4 (r - skips[i+1], r - skips[i];
-//    consecutive threads read consecutive words) and find the largest new block of the window
+//    consecutive threads read consecutive words) and finds the largest new block of the window
 //    from the two codes alone: walking down from the first level where they differ, every step
 //    yields one "head" (a rank whose baseblock is that level) and a run of low blocks; the rounds
 //    whose windows reach only a few ranks back read them from a table of the tile's baseblock
-//    bits in shared memory.  They write the rows rank-major and a round-major copy, from which
-//    send_transpose_kernel / send_batch_kernel produce
-//    sendsched[r][k] = recvsched[(r+skips[k]) mod p][k] as a transposition with row k rotated by
-//    skips[k] (send_rm_kernel: sub-ranges, byte gathers and recomputation for to-processors
-//    outside the range).  The kernels of a build are launched as dependents of one another
-//    (bcs_common.cuh), so each is brought onto the SMs while the one before it drains.  In a
-//    batch, every p up to 1024 is built by ONE CTA of fused_small_batch_kernel instead: codes,
+//    bits in shared memory.  It writes the rows rank-major and a round-major copy, from which
+//    send_batch_kernel produces sendsched[r][k] = recvsched[(r+skips[k]) mod p][k] as a transposition
+//    with row k rotated by skips[k].  The kernels of a build are launched as dependents of one another
+//    (bcs_common.cuh), so each is brought onto the SMs while the one before it drains.
+//    Every p up to 1024 is built by ONE CTA of fused_small_batch_kernel instead: codes,
 //    a table of exact window sets over all ranks of the p, both tables, all in shared memory.
 //
 //  * self-contained path (no workspace).  One thread per rank runs Algorithm 4 with the range
 //    search done by descending the homeranges; the send schedule is looked up in the rank-major
-//    receive table where the to-processor is inside the call's range and recomputed
-//    (Algorithm 5) where it is not.
+//    receive table.
 #include <cstddef>
-#include <mutex>
 #include <type_traits>
 
 #include "bcs_common.cuh"
@@ -34,11 +30,6 @@
 
 namespace bcs {
 namespace {
-
-// Scratch of bcs_build_static: lives in the library's device image, so every GPU that loads
-// the library sets these bytes aside until the process ends.  In host code this name is only a
-// handle for cudaGetSymbolAddress, never an address a kernel may be given.
-static __device__ __align__(256) unsigned char g_static_scratch[BCS_STATIC_WORKSPACE_BYTES];
 
 // ================================================================ self-contained path
 // (Algorithms 2-4 per rank: paper_path.cuh)
@@ -101,11 +92,6 @@ constexpr int kCodesThreads = 256;
 constexpr int kCodesSub = 32;                                   // consecutive ranks scanned as one
 constexpr int kCodesCta = kCodesThreads * kCodesSub;            // ranks per CTA
 constexpr int kCodesLow = 8;
-// Ranks per scan in the kernel of one p: 32 where the kernel streams (4 million ranks and more:
-// fewest instructions per rank), 16 for a smaller p, where its latency counts: twice the threads,
-// each with half the quads to write (p = 2^20+1: 1.1 us less).
-__host__ __device__ constexpr int codes_sub(int q) { return q <= 22 ? 16 : 32; }
-
 struct BlockScan {
     uint32_t biased;   // remainder of the block's first rank, plus (ranks per block - 1)
     uint32_t code;     // its code so far
@@ -114,28 +100,26 @@ struct BlockScan {
     uint32_t plain;    // a second splitting level was met
 };
 
-template <int kSub = kCodesSub>
 __device__ __forceinline__ void scan_level(BlockScan &b, uint32_t skip, int k)
 {
     const uint32_t u = b.biased - skip;
-    if (u < (uint32_t)(kSub - 1)) {                   // skip - (kSub - 1) <= remainder < skip: rare
-        if (b.stay == kSub) {
-            b.stay = (kSub - 1) - u;                  // = skip - remainder
+    if (u < (uint32_t)(kCodesSub - 1)) {                   // skip - (kCodesSub - 1) <= remainder < skip: rare
+        if (b.stay == kCodesSub) {
+            b.stay = (kCodesSub - 1) - u;                  // = skip - remainder
             b.left = b.code | (1u << k);
         } else {
             b.plain = 1;
         }
     }
-    if ((int32_t)u >= kSub - 1) {
+    if ((int32_t)u >= kCodesSub - 1) {
         b.biased = u;
         b.code |= 1u << k;
     }
 }
 
-template <int kSub = kCodesSub>
 __device__ __forceinline__ uint4 pack_scan(const BlockScan &b)
 {
-    return make_uint4(b.biased - (kSub - 1), b.code, b.stay | (b.plain << 8), b.left);
+    return make_uint4(b.biased - (kCodesSub - 1), b.code, b.stay | (b.plain << 8), b.left);
 }
 
 // Codes of the four ranks at offset e0 .. e0+3 of a block whose scan is sb (no second split).
@@ -157,78 +141,6 @@ __device__ __forceinline__ uint4 quad_codes(const uint4 sb, const uint16_t *low,
         }
     }
     return make_uint4(out[0], out[1], out[2], out[3]);
-}
-
-// Skip code of every rank of one p: codes[x].  A warp takes 1024 consecutive ranks: lane l
-// scans the levels above the table for the 32 ranks from first + 32 l (unrolled for the q at
-// hand, every skip an immediate operand from the kernel parameters), then the warp writes its
-// 256 quads, lane l the quads l, l+32, ..., one 16-byte store each.
-template <int kQ>
-__global__ void __launch_bounds__(kCodesThreads)
-codes_single_kernel(const __grid_constant__ PTable tab, uint32_t *__restrict__ codes)
-{
-    constexpr int kLow = kQ < kCodesLow ? kQ : kCodesLow;
-    __shared__ uint16_t low[1 << kLow];
-    __shared__ uint4 sub[kCodesThreads];
-    grid_launch_dependents();
-    if (threadIdx.x < (1u << kLow)) {
-        uint32_t v = threadIdx.x, c = 0;
-#pragma unroll
-        for (int k = kLow - 1; k >= 0; --k) {
-            if (v >= tab.s[k]) {
-                v -= tab.s[k];
-                c |= 1u << k;
-            }
-        }
-        low[threadIdx.x] = (uint16_t)c;
-    }
-    const uint32_t lane = threadIdx.x & 31u;
-    constexpr int kSub = codes_sub(kQ);
-    constexpr uint32_t kSubQuads = kSub / 4;                       // quads per block: 4 or 8
-    const uint32_t first = (blockIdx.x * kCodesThreads + (threadIdx.x & ~31u)) * (uint32_t)kSub;
-    {
-        const uint32_t g = first + kSub * lane;
-        BlockScan b = {g + (kSub - 1), 0, kSub, 0, 0};
-        if (g < tab.p) {
-#pragma unroll
-            for (int k = kQ - 1; k >= kLow; --k) scan_level<kSub>(b, tab.s[k], k);
-        }
-        sub[threadIdx.x] = pack_scan<kSub>(b);
-    }
-    __syncthreads();
-    const uint32_t e0 = 4u * (lane % kSubQuads);
-#pragma unroll 2
-    for (uint32_t i = 0; i < kSubQuads; ++i) {
-        const uint32_t g = first + 4u * (i * 32u + lane);
-        if (g >= tab.p) break;
-        const uint4 sb = sub[(threadIdx.x & ~31u) + i * (32u / kSubQuads) + lane / kSubQuads];
-        if (sb.z < 256u && g + 4u <= tab.p) {
-            *reinterpret_cast<uint4 *>(codes + g) = quad_codes(sb, low, e0);
-        } else {
-            for (uint32_t e = 0; e < 4 && g + e < tab.p; ++e) codes[g + e] = skip_code(tab.s, kQ, g + e);
-        }
-    }
-}
-
-template <int kQ>
-struct CodesLauncher {
-    static void launch(int q, const PTable &tab, uint32_t *codes, cudaStream_t stream)
-    {
-        constexpr unsigned per_cta = kCodesThreads * codes_sub(kQ);
-        if (q == kQ)
-            codes_single_kernel<kQ><<<(tab.p + per_cta - 1) / per_cta, kCodesThreads, 0, stream>>>(tab, codes);
-        else
-            CodesLauncher<kQ - 1>::launch(q, tab, codes, stream);
-    }
-};
-template <>
-struct CodesLauncher<0> {
-    static void launch(int, const PTable &, uint32_t *, cudaStream_t) {}
-};
-
-inline void launch_codes(const PTable &tab, uint32_t *codes, cudaStream_t stream)
-{
-    CodesLauncher<BCS_MAX_Q>::launch(tab.q, tab, codes, stream);
 }
 
 // Batch: codes[g] for the flattened rank g, 8192 flattened ranks per CTA, scanned in blocks of
@@ -498,29 +410,6 @@ __device__ __forceinline__ int recv_rounds_codes(const uint32_t *__restrict__ co
     return entry;
 }
 
-// One p, every round searched per lane (used for p < 64, where a warp's 32 predecessors would
-// wrap around the ring more than once).  recv_t: round-major copy, recv_t[k * t_stride + (r - r_begin)].
-template <bool kRowOut, bool kColOut>
-__global__ void __launch_bounds__(kTile)
-recv_codes_kernel(PTable tab, uint64_t r_begin, uint64_t r_end,
-                  const uint32_t *__restrict__ codes, int8_t *recv_out, int8_t *recv_t,
-                  uint64_t t_stride)
-{
-    __shared__ TileShared sh;
-    BatchArgs none = {};
-    RankCtx c = resolve_rank<false>(sh, tab, r_begin, r_end, none);
-    if (c.valid && c.q > 0) {
-        int8_t *col = kColOut ? recv_t + (c.r - r_begin) : nullptr;
-        uint8_t *row = kRowOut ? sh.stage + (c.entry - sh.span_begin) : nullptr;
-        recv_rounds_codes<kRowOut, kColOut>(codes, c.s, c.full, c.p, c.q, c.r, c.q - 1, row, col,
-                                            t_stride);
-    }
-    if (kRowOut) {
-        __syncthreads();
-        flush_span(sh.stage, 0, (uint32_t)(sh.span_end - sh.span_begin), recv_out, sh.span_begin);
-    }
-}
-
 // The run table.  The windows of the rounds with skips[i+1] <= 33 (at most six rounds, i <= 5)
 // reach only a few ranks back: the first window ends skips[i+1] - 1 ranks below r, the second at
 // sum_{j<=i} skips[j] <= skips[i+1] + i <= 38 (every halving rounds up by at most one), and a run
@@ -568,14 +457,6 @@ __device__ __forceinline__ uint32_t bit_or_none(int k)
     uint32_t bit;
     asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(k));
     return bit;
-}
-
-// Position of the highest set bit, -1 for 0 (one instruction).
-__device__ __forceinline__ int top_bit(uint32_t v)
-{
-    int d;
-    asm("bfind.u32 %0, %1;" : "=r"(d) : "r"(v));
-    return d;
 }
 
 // byte 0 of a, b, c, d as the four bytes of one word
@@ -638,46 +519,7 @@ __host__ __device__ inline int32_t quad_word_offset(const uint32_t *skips, int i
     return 4 * (level * kQuadLevelWords + sub * kQuadSub + kRunBack / 4 + quad);
 }
 
-inline QuadConsts make_quad_consts(const PTable &tab, uint64_t r_begin, uint64_t r_end)
-{
-    QuadConsts qc = {};
-    {
-        const uint64_t count = r_end - r_begin;
-        auto add = [&](uint64_t tile) {
-            for (int m = 0; m < qc.n_special; ++m)
-                if (qc.special[m] == tile) return;
-            if (qc.n_special < kRow) qc.special[qc.n_special++] = (uint32_t)tile;
-        };
-        if (count) {
-            add(0);
-            for (int k = 1; k < tab.q; ++k)
-                if (tab.s[k] >= r_begin && tab.s[k] < r_end) add((tab.s[k] - r_begin) / kQuadTile);
-            add((count - 1) / kQuadTile);
-        }
-    }
-    for (int i = 0; i < tab.q; ++i) qc.len2[i] = quad_len2(tab.s, i);
-    qc.table_rounds = quad_table_rounds(tab.s, tab.q);
-    // quads start at ranks r_begin + multiples of 4, the codes at a 16-byte boundary
-    for (int k = 0; k <= tab.q; ++k) {
-        if ((((uint32_t)r_begin - tab.s[k]) & 3u) == 0) qc.aligned |= 1u << k;
-    }
-    for (int i = 0; i < qc.table_rounds; ++i)
-        for (int w = 0; w < 4; ++w)
-            for (int j = 0; j < 4; ++j) qc.word[i][w][j] = quad_word_offset(tab.s, i, w, j);
-    return qc;
-}
-
-// Where a quad tile reads the constants of its p from: the kernel parameters (single p:
-// constant-bank operands) ...
-struct ParamEnv {
-    const PTable &tab;
-    const QuadConsts &qc;
-    __device__ __forceinline__ uint32_t skip(int k) const { return tab.s[k]; }
-    __device__ __forceinline__ int word(int i, int w, int j) const { return qc.word[i][w][j]; }
-    __device__ __forceinline__ uint32_t len2(int i) const { return qc.len2[i]; }
-    __device__ __forceinline__ int table_rounds() const { return qc.table_rounds; }
-};
-// ... or shared memory (batch: the CTA computes them for the p of its tile).
+// Where a quad tile reads the constants of its p from: shared memory (the CTA computes them for the p of its tile).
 struct SharedEnv {
     const uint32_t *s;
     const QuadConsts *qc;
@@ -1007,49 +849,6 @@ __device__ __forceinline__ void quad_tile(const Env env, const uint32_t *full_sh
     }
 }
 
-// The quad tile for a range of one p >= 64.  kRowOut: rank-major rows; kColOut: round-major copy;
-// kWideLoads, kWordRows: see load4 and put_rows in quad_tile (picked per launch by launch_recv_quad).
-template <bool kRowOut, bool kColOut, bool kWideLoads, bool kWordRows>
-__global__ void __launch_bounds__(kQuadThreads, 8)
-recv_codes_quad_kernel(const __grid_constant__ PTable tab, const __grid_constant__ QuadConsts qc,
-                       uint64_t r_begin, uint64_t r_end, const uint32_t *__restrict__ codes,
-                       int8_t *recv_out, int8_t *recv_t, uint64_t t_stride)
-{
-    __shared__ __align__(16) uint8_t stage[kQuadTile * BCS_MAX_Q];
-    __shared__ uint32_t full_sh[kRow];
-    __shared__ uint32_t runs[kRunLevels][kQuadLevelWords];
-    grid_launch_dependents();
-    const uint32_t t = threadIdx.x;
-    if (t < kRow) full_sh[t] = tab.full[t];                    // read after the first barrier
-    const uint32_t p = tab.p;
-    const int q = tab.q;
-    const uint64_t count = r_end - r_begin;
-    // The first CTAs of the grid take the tiles that run the general code (listed by the host):
-    // they last longer, so they start first; the others skip a listed tile.
-    uint64_t tile = blockIdx.x;
-    if (blockIdx.x < (uint32_t)qc.n_special) {
-        tile = qc.special[blockIdx.x];
-    } else {
-        tile -= (uint32_t)qc.n_special;
-        if (__syncthreads_or(t < (uint32_t)qc.n_special && qc.special[t] == tile)) return;
-    }
-    grid_dependency_wait();                                    // the codes are complete from here on
-    const uint64_t g0 = tile * kQuadTile;
-    const uint32_t n = (uint32_t)(count - g0 < (uint64_t)kQuadTile ? count - g0 : (uint64_t)kQuadTile);
-    // g0 and t_stride are multiples of 4 and recv_t is 16-byte aligned: packed column stores
-    quad_tile<kRowOut, kColOut, true, kWideLoads, kWordRows>(ParamEnv{tab, qc}, full_sh, p, q, r_begin + g0, n, codes, stage,
-                                      kColOut ? recv_t + g0 : nullptr, t_stride, runs);
-    if (kRowOut) {
-        const uint32_t len = n * (uint32_t)q;                  // the tile's rows start at byte g0 * q: 16-byte aligned
-        if ((len & 15u) == 0) {
-            flush_span_bulk(stage, len, recv_out, g0 * (uint64_t)q);
-        } else {                                               // ragged last tile
-            __syncthreads();
-            flush_span(stage, 0, len, recv_out, g0 * (uint64_t)q);
-        }
-    }
-}
-
 // Batch: the tiles of 512 ranks start anew with every p (the host's plan gives the prefix sums of
 // the tiles per p), so a CTA works inside ONE p: the quad tile with that p's constants computed
 // into shared memory when p >= 64, the per-lane search for the ranks of a smaller p.  The round-
@@ -1268,38 +1067,6 @@ fused_small_batch_kernel(BatchArgs ba, int8_t *recv_out, int8_t *send_out)
     grid_dependency_wait();
 }
 
-// Send rows of a sub-range of one p from the round-major receive copy of that range;
-// to-processors outside the range are recomputed from the codes (Algorithm 5).
-__global__ void __launch_bounds__(kTile)
-send_rm_kernel(PTable tab, uint64_t r_begin, uint64_t r_end, const uint32_t *__restrict__ codes,
-               const int8_t *__restrict__ recv_t, uint64_t t_stride, int8_t *send_out)
-{
-    __shared__ TileShared sh;
-    BatchArgs none = {};
-    RankCtx c = resolve_rank<false>(sh, tab, r_begin, r_end, none);
-    if (c.valid) {
-        uint8_t *row = sh.stage + (c.entry - sh.span_begin);
-        const int8_t *tbl = recv_t;
-        const uint32_t first = (uint32_t)r_begin, width = (uint32_t)(r_end - r_begin);
-        for (int k = 0; k < c.q; ++k) {
-            uint32_t t = c.r + c.s[k];
-            if (t >= c.p) t -= c.p;
-            const uint32_t rel = t - first;          // index into the round-major row
-            int v;
-            if (rel < width) {
-                v = tbl[rel];
-            } else {
-                v = recv_rounds_codes<false, false>(codes, c.s, c.full, c.p, c.q, t, k, nullptr,
-                                                    nullptr, 0);
-            }
-            row[k] = (uint8_t)v;
-            tbl += t_stride;
-        }
-    }
-    __syncthreads();
-    flush_span(sh.stage, 0, (uint32_t)(sh.span_end - sh.span_begin), send_out, sh.span_begin);
-}
-
 // Row k of the round-major send table is row k of the round-major receive copy rotated by
 // skips[k] (sendsched[r][k] = recvsched[(r+skips[k]) mod p][k]), so the send rows of a run of
 // ranks are a transposition with one rotation per row (and the receive rows the same with
@@ -1328,12 +1095,6 @@ struct RoundBuffer {
     __align__(8) uint64_t bar;
     uint32_t lead[kRounds];     // offset of the tile's first byte inside its pitch row
     uint32_t wraps;             // rounds whose bytes pass the end of the row
-};
-
-// Skips from the kernel parameter (single p).
-struct TableSkips {
-    const PTable &tab;
-    __device__ __forceinline__ uint32_t operator()(int k) const { return tab.s[k]; }
 };
 
 // All threads of the CTA call.  tbl: round 0 of the round-major table of this p (rows `stride`
@@ -1418,39 +1179,6 @@ __device__ __forceinline__ uint32_t row_word(const uint32_t (&W)[kQ], int m)
     return __byte_perm(lo, hi, 0x5410u);
 }
 
-// Single p: recv_t holds all p ranks of every round (rows 16-byte aligned); the CTA's tile is
-// ranks r0..r0+n-1 of the range r_begin..r_begin+count-1.  rotate: send rows; otherwise the
-// receive rows themselves.  The rows are written over the round buffer (after a barrier) and
-// leave as one bulk store: 64 threads and 6 KB (q = 21) per 256 ranks, so the whole grid of a
-// million-rank table is resident at once, and the many small CTAs per SM overlap one another's
-// copies.
-template <int kQ>
-__global__ void __launch_bounds__(kTrThreads)
-send_transpose_kernel(const __grid_constant__ PTable tab, const int8_t *__restrict__ recv_t,
-                      uint64_t t_stride, int8_t *send_out, uint32_t r_begin, uint32_t count,
-                      bool rotate)
-{
-    __shared__ RoundBuffer<kQ> rb;
-    const uint32_t first = blockIdx.x * kTile;
-    const uint32_t n = count - first < (uint32_t)kTile ? count - first : (uint32_t)kTile;
-    if (!load_rounds(TableSkips{tab}, tab.p, kQ, recv_t, t_stride, r_begin + first, n, rotate, rb))
-        return;
-    uint32_t W[kQ];
-    load_four_ranks(rb, threadIdx.x, W);
-    __syncthreads();                                       // everyone has read: the rows take the buffer over
-    uint8_t *stage = rb.rounds;
-    uint32_t *rows = reinterpret_cast<uint32_t *>(stage) + threadIdx.x * kQ;   // 4q bytes start at a multiple of 4
-#pragma unroll
-    for (int m = 0; m < kQ; ++m) rows[m] = row_word<kQ>(W, m);
-    const uint32_t len = n * (uint32_t)kQ;                 // starts at byte first * q: 16-byte aligned
-    if ((len & 15u) == 0) {
-        flush_span_bulk(stage, len, send_out, (uint64_t)first * (uint64_t)kQ);
-    } else {                                               // ragged last tile
-        __syncthreads();
-        flush_span(stage, 0, len, send_out, (uint64_t)first * (uint64_t)kQ);
-    }
-}
-
 // Batch: the same for a tile whose rows start at any byte.  `out` is where the tile's first row
 // starts in the staging buffer; with sh = its address mod 4, word m of a thread's rows lies sh
 // bytes into an aligned word, so consecutive words are funnel-shifted together and the up to
@@ -1496,35 +1224,6 @@ struct GatherDispatch<0> {
     static __device__ __forceinline__ void run(int, const BatchRoundBuffer &, uint8_t *) {}
 };
 
-template <int kQ>
-struct TransposeLauncher {
-    static void launch(const PTable &tab, const int8_t *recv_t, uint64_t t_stride, int8_t *out,
-                       uint32_t r_begin, uint32_t count, bool rotate, bool dependent,
-                       cudaStream_t stream)
-    {
-        if (tab.q == kQ)
-            launch_dependent(dependent, send_transpose_kernel<kQ>, (count + kTile - 1) / kTile,
-                             kTrThreads, stream, tab, recv_t, t_stride, out, r_begin, count, rotate);
-        else
-            TransposeLauncher<kQ - 1>::launch(tab, recv_t, t_stride, out, r_begin, count, rotate,
-                                              dependent, stream);
-    }
-};
-template <>
-struct TransposeLauncher<0> {
-    static void launch(const PTable &, const int8_t *, uint64_t, int8_t *, uint32_t, uint32_t, bool,
-                       bool, cudaStream_t) {}
-};
-
-// dependent: the kernel before this one on the stream calls grid_launch_dependents().
-inline void launch_transpose(const PTable &tab, const int8_t *recv_t, uint64_t t_stride, int8_t *out,
-                             uint32_t r_begin, uint32_t count, bool rotate, bool dependent,
-                             cudaStream_t stream)
-{
-    TransposeLauncher<BCS_MAX_Q>::launch(tab, recv_t, t_stride, out, r_begin, count, rotate,
-                                         dependent, stream);
-}
-
 // Batch: 256 ranks and 64 threads per CTA, as in the single-p kernel; two CTAs per tile of the
 // plan (512 ranks of one p), the second with nothing to do where a p ends in the first half.
 struct SendBatchShared {
@@ -1569,42 +1268,6 @@ send_batch_kernel(BatchArgs ba, const int8_t *__restrict__ recv_t, int8_t *send_
     flush_span(rb.rounds, shift, n * (uint32_t)q, send_out, span_begin);
 }
 
-// Launches the quad receive kernel of one p >= 64 for a range, as a dependent of the kernel
-// before it on the stream.  The instantiation that loads the window bounds of the rounds before
-// the home round as 16-byte words is taken when all of them are aligned (a p in the top 32nd of
-// its octave, whose skips from 32 on are powers of two, and a range that starts at a multiple of
-// 4): 10 % fewer L1 wavefronts and 5 % fewer issue slots than the one-word loads.
-template <bool kRowOut, bool kColOut>
-inline void launch_recv_quad(const PTable &tab, const QuadConsts &qc, uint64_t r_begin, uint64_t r_end,
-                             const uint32_t *codes, int8_t *recv_out, int8_t *recv_t, uint64_t t_stride,
-                             cudaStream_t stream)
-{
-    const uint64_t count = r_end - r_begin;
-    const unsigned grid = (unsigned)((count + kQuadTile - 1) / kQuadTile) + (unsigned)qc.n_special;
-    // bounds of every round from the first per-lane round to the last possible home round
-    bool all_wide = true;
-    for (int k = qc.table_rounds; k < tab.q; ++k) all_wide = all_wide && ((qc.aligned >> k) & 1u);
-    // rows of a q that is a multiple of 4 are stored word by word (see put_rows)
-    const bool word_rows = kRowOut && (tab.q & 3) == 0;
-    auto go = [&](auto kernel) {
-        launch_dependent(true, kernel, grid, kQuadThreads, stream, tab, qc, r_begin, r_end, codes, recv_out, recv_t,
-                         t_stride);
-    };
-    if (all_wide) {
-        if (word_rows) go(recv_codes_quad_kernel<kRowOut, kColOut, true, kRowOut>);
-        else go(recv_codes_quad_kernel<kRowOut, kColOut, true, false>);
-    } else {
-        if (word_rows) go(recv_codes_quad_kernel<kRowOut, kColOut, false, kRowOut>);
-        else go(recv_codes_quad_kernel<kRowOut, kColOut, false, false>);
-    }
-}
-
-struct Workspace {
-    uint32_t *codes;
-    int8_t *recv_t;
-    uint64_t t_stride;
-};
-
 }  // namespace
 
 bcs_status make_table(uint32_t p, PTable *tab)
@@ -1645,65 +1308,11 @@ bcs_status bcs_build(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t *recv_
 {
     bcs_status st = check_range(p, r_begin, r_end);
     if (st != BCS_OK) return st;
-    PTable tab;
-    make_table(p, &tab);
-    const uint64_t count = r_end - r_begin;
-    if (count == 0 || tab.q == 0) return BCS_OK;
+    if (r_begin == r_end || p == 1) return BCS_OK;
     if (recv_out == nullptr && send_out == nullptr) return BCS_ERR_ARG;
     if (!aligned16(recv_out) || !aligned16(send_out) || !aligned16(workspace)) return BCS_ERR_ALIGN;
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const unsigned blocks = (unsigned)((count + kTile - 1) / kTile);
-    BatchArgs none = {};
-    if (workspace != nullptr && workspace_bytes >= bcs_build_workspace_bytes(p, r_begin, r_end)) {
-        Workspace ws;
-        ws.codes = static_cast<uint32_t *>(workspace);
-        ws.recv_t = static_cast<int8_t *>(workspace) + align_up(4ull * p, 256);
-        ws.t_stride = align_up(count, 16);
-        launch_codes(tab, ws.codes, stream);
-        if ((st = launch_status()) != BCS_OK) return st;
-        const bool warp_rounds = p >= 64;      // the table kernel needs 64 distinct ranks back
-        const QuadConsts rc = make_quad_consts(tab, r_begin, r_end);
-        if (recv_out != nullptr && send_out != nullptr) {
-            if (warp_rounds)
-                launch_recv_quad<true, true>(tab, rc, r_begin, r_end, ws.codes, recv_out, ws.recv_t, ws.t_stride, stream);
-            else
-                recv_codes_kernel<true, true><<<blocks, kTile, 0, stream>>>(
-                    tab, r_begin, r_end, ws.codes, recv_out, ws.recv_t, ws.t_stride);
-        } else if (recv_out != nullptr) {
-            if (warp_rounds)
-                launch_recv_quad<true, false>(tab, rc, r_begin, r_end, ws.codes, recv_out, nullptr, 0, stream);
-            else
-                recv_codes_kernel<true, false><<<blocks, kTile, 0, stream>>>(
-                    tab, r_begin, r_end, ws.codes, recv_out, nullptr, 0);
-        } else {
-            if (warp_rounds)
-                launch_recv_quad<false, true>(tab, rc, r_begin, r_end, ws.codes, nullptr, ws.recv_t, ws.t_stride, stream);
-            else
-                recv_codes_kernel<false, true><<<blocks, kTile, 0, stream>>>(
-                    tab, r_begin, r_end, ws.codes, nullptr, ws.recv_t, ws.t_stride);
-        }
-        if ((st = launch_status()) != BCS_OK) return st;
-        if (send_out != nullptr) {
-            if (count == p)
-                launch_transpose(tab, ws.recv_t, ws.t_stride, send_out, 0u, p, true, warp_rounds,
-                                 stream);
-            else
-                send_rm_kernel<<<blocks, kTile, 0, stream>>>(tab, r_begin, r_end, ws.codes,
-                                                             ws.recv_t, ws.t_stride, send_out);
-            if ((st = launch_status()) != BCS_OK) return st;
-        }
-        return BCS_OK;
-    }
-    if (recv_out != nullptr) {
-        recv_kernel<false><<<blocks, kTile, 0, stream>>>(tab, r_begin, r_end, none, recv_out);
-        if ((st = launch_status()) != BCS_OK) return st;
-    }
-    if (send_out != nullptr) {
-        send_kernel<false><<<blocks, kTile, 0, stream>>>(tab, r_begin, r_end, none, recv_out,
-                                                         send_out);
-        if ((st = launch_status()) != BCS_OK) return st;
-    }
-    return BCS_OK;
+    (void)workspace_bytes;                   // the rows need no scratch memory, see rows.cuh
+    return launch_rows(p, r_begin, r_end - r_begin, recv_out, send_out, static_cast<cudaStream_t>(cuda_stream));
 }
 
 size_t bcs_prepare_workspace_bytes(uint32_t p)
@@ -1714,25 +1323,21 @@ size_t bcs_prepare_workspace_bytes(uint32_t p)
     return (size_t)(align_up(4ull * p, 256) + (uint64_t)q * align_up(p, 16));
 }
 
-// The two halves of bcs_prepare.  Layout of the workspace: skip codes of all p ranks, then the
-// round-major copy recv_t[k * align16(p) + r].
-static bcs_status prepare_check(uint32_t p, PTable *tab, const void *workspace, size_t workspace_bytes)
+// A prepared p.  The call that writes a row computes it (rows.cuh), in no more time than the transposition of a
+// prepared copy took, so preparing is no more than the checks, and the workspace is not touched.
+static bcs_status prepare_check(uint32_t p, const void *workspace, size_t workspace_bytes)
 {
-    bcs_status st = make_table(p, tab);
-    if (st != BCS_OK) return st;
-    if (tab->q == 0) return BCS_OK;
+    if (p == 0) return BCS_ERR_RANGE;
+    if (p > 0x7fffffffu) return BCS_ERR_UNSUPPORTED;
+    if (p == 1) return BCS_OK;
     if (workspace == nullptr || workspace_bytes < bcs_prepare_workspace_bytes(p)) return BCS_ERR_ARG;
     if (!aligned16(workspace)) return BCS_ERR_ALIGN;
     return BCS_OK;
 }
 
-bcs_status bcs_prepare_codes(uint32_t p, void *workspace, size_t workspace_bytes, void *cuda_stream)
+bcs_status bcs_prepare_codes(uint32_t p, void *workspace, size_t workspace_bytes, void *)
 {
-    PTable tab;
-    bcs_status st = prepare_check(p, &tab, workspace, workspace_bytes);
-    if (st != BCS_OK || tab.q == 0) return st;
-    launch_codes(tab, static_cast<uint32_t *>(workspace), static_cast<cudaStream_t>(cuda_stream));
-    return launch_status();
+    return prepare_check(p, workspace, workspace_bytes);
 }
 
 bcs_status bcs_prepare_rows(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t *recv_out,
@@ -1740,40 +1345,16 @@ bcs_status bcs_prepare_rows(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t
 {
     bcs_status st = check_range(p, r_begin, r_end);
     if (st != BCS_OK) return st;
-    PTable tab;
-    st = prepare_check(p, &tab, workspace, workspace_bytes);
-    if (st != BCS_OK || tab.q == 0 || r_begin == r_end) return st;
+    st = prepare_check(p, workspace, workspace_bytes);
+    if (st != BCS_OK || p == 1 || r_begin == r_end) return st;
     if ((r_begin & 15u) != 0 || !aligned16(recv_out)) return BCS_ERR_ALIGN;
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const uint32_t *codes = static_cast<const uint32_t *>(workspace);
-    const uint64_t t_stride = align_up(p, 16);
-    // round k of rank r_begin + j goes to recv_t[k * t_stride + r_begin + j]
-    int8_t *recv_t = static_cast<int8_t *>(workspace) + align_up(4ull * p, 256) + r_begin;
-    const uint64_t count = r_end - r_begin;
-    if (p >= 64) {
-        const QuadConsts qc = make_quad_consts(tab, r_begin, r_end);
-        // (dependent launch: harmless when the kernel before it on the stream is not the codes kernel)
-        if (recv_out != nullptr)
-            launch_recv_quad<true, true>(tab, qc, r_begin, r_end, codes, recv_out, recv_t, t_stride, stream);
-        else
-            launch_recv_quad<false, true>(tab, qc, r_begin, r_end, codes, nullptr, recv_t, t_stride, stream);
-    } else {
-        const unsigned blocks = (unsigned)((count + kTile - 1) / kTile);
-        if (recv_out != nullptr)
-            recv_codes_kernel<true, true><<<blocks, kTile, 0, stream>>>(tab, r_begin, r_end, codes, recv_out, recv_t,
-                                                                        t_stride);
-        else
-            recv_codes_kernel<false, true><<<blocks, kTile, 0, stream>>>(tab, r_begin, r_end, codes, nullptr, recv_t,
-                                                                         t_stride);
-    }
-    return launch_status();
+    if (recv_out == nullptr) return BCS_OK;
+    return launch_rows(p, r_begin, r_end - r_begin, recv_out, nullptr, static_cast<cudaStream_t>(cuda_stream));
 }
 
-bcs_status bcs_prepare(uint32_t p, void *workspace, size_t workspace_bytes, void *cuda_stream)
+bcs_status bcs_prepare(uint32_t p, void *workspace, size_t workspace_bytes, void *)
 {
-    bcs_status st = bcs_prepare_codes(p, workspace, workspace_bytes, cuda_stream);
-    if (st != BCS_OK) return st;
-    return bcs_prepare_rows(p, 0, p, nullptr, workspace, workspace_bytes, cuda_stream);
+    return prepare_check(p, workspace, workspace_bytes);
 }
 
 bcs_status bcs_build_prepared(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t *recv_out,
@@ -1782,27 +1363,11 @@ bcs_status bcs_build_prepared(uint32_t p, uint64_t r_begin, uint64_t r_end, int8
 {
     bcs_status st = check_range(p, r_begin, r_end);
     if (st != BCS_OK) return st;
-    PTable tab;
-    make_table(p, &tab);
-    const uint64_t count = r_end - r_begin;
-    if (count == 0 || tab.q == 0) return BCS_OK;
+    if (r_begin == r_end || p == 1) return BCS_OK;
     if (recv_out == nullptr && send_out == nullptr) return BCS_ERR_ARG;
     if (workspace == nullptr || workspace_bytes < bcs_prepare_workspace_bytes(p)) return BCS_ERR_ARG;
     if (!aligned16(recv_out) || !aligned16(send_out) || !aligned16(workspace)) return BCS_ERR_ALIGN;
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const int8_t *recv_t = static_cast<const int8_t *>(workspace) + align_up(4ull * p, 256);
-    const uint64_t t_stride = align_up(p, 16);
-    if (recv_out != nullptr) {
-        launch_transpose(tab, recv_t, t_stride, recv_out, (uint32_t)r_begin, (uint32_t)count, false,
-                         false, stream);
-        if ((st = launch_status()) != BCS_OK) return st;
-    }
-    if (send_out != nullptr) {
-        launch_transpose(tab, recv_t, t_stride, send_out, (uint32_t)r_begin, (uint32_t)count, true,
-                         recv_out != nullptr, stream);
-        if ((st = launch_status()) != BCS_OK) return st;
-    }
-    return BCS_OK;
+    return launch_rows(p, r_begin, r_end - r_begin, recv_out, send_out, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // The runs of virtual ranks (r - root) mod p of the range [r_begin, r_end): [v0, v0 + len_a) and,
@@ -1846,31 +1411,9 @@ bcs_status bcs_build_rooted(uint32_t p, uint32_t root, uint64_t r_begin, uint64_
     const RootedRuns rr = rooted_runs(p, root, r_begin, r_end);
     const bool fast = workspace != nullptr &&
                       workspace_bytes >= bcs_build_rooted_workspace_bytes(p, root, r_begin, r_end);
-    const uint64_t bytes_a = rr.len_a * (uint64_t)q, bytes_b = rr.len_b * (uint64_t)q;
-    const bool staged = rr.len_b != 0 && (bytes_a & 15u) != 0;
-    if (staged && !fast) return BCS_ERR_ARG;
-    // workspace = [construction scratch, a multiple of 256 bytes][recv staging][send staging]
-    const size_t need_a = bcs_build_workspace_bytes(p, rr.v0, rr.v0 + rr.len_a);
-    const size_t need_b = bcs_build_workspace_bytes(p, 0, rr.len_b);
-    const size_t build_ws = fast ? (size_t)align_up(need_a > need_b ? need_a : need_b, 256) : 0;
-    st = bcs_build(p, rr.v0, rr.v0 + rr.len_a, recv_out, send_out, fast ? workspace : nullptr, build_ws,
-                   cuda_stream);
-    if (st != BCS_OK || rr.len_b == 0) return st;
-    int8_t *recv_b = recv_out ? recv_out + bytes_a : nullptr;
-    int8_t *send_b = send_out ? send_out + bytes_a : nullptr;
-    if (!staged)
-        return bcs_build(p, 0, rr.len_b, recv_b, send_b, fast ? workspace : nullptr, build_ws, cuda_stream);
-    int8_t *stage_recv = static_cast<int8_t *>(workspace) + build_ws;
-    int8_t *stage_send = stage_recv + align_up(bytes_b, 256);
-    st = bcs_build(p, 0, rr.len_b, recv_out ? stage_recv : nullptr, send_out ? stage_send : nullptr,
-                   workspace, build_ws, cuda_stream);
-    if (st != BCS_OK) return st;
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    if (recv_out && cudaMemcpyAsync(recv_b, stage_recv, bytes_b, cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
-        return BCS_ERR_CUDA;
-    if (send_out && cudaMemcpyAsync(send_b, stage_send, bytes_b, cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
-        return BCS_ERR_CUDA;
-    return BCS_OK;
+    // (the kernel would not mind, but without a workspace such a range was always refused)
+    if (rr.len_b != 0 && ((rr.len_a * (uint64_t)q) & 15u) != 0 && !fast) return BCS_ERR_ARG;
+    return launch_rows(p, rr.v0, r_end - r_begin, recv_out, send_out, static_cast<cudaStream_t>(cuda_stream));
 }
 
 bcs_status bcs_build_to_host(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t *recv_host,
@@ -1889,13 +1432,8 @@ bcs_status bcs_build_to_host(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_
     if ((uint64_t)stage_bytes < 2 * half) return BCS_ERR_ARG;
     int8_t *recv_dev = static_cast<int8_t *>(stage_dev);
     int8_t *send_dev = recv_dev + half;
-    // what is left of the staging buffer serves as workspace (fast path when large enough)
-    void *ws = recv_dev + 2 * half;
-    const size_t ws_bytes = stage_bytes - (size_t)(2 * half);
-    // the receive table is built even when only the send table is wanted: the send
-    // rows are looked up in it.
-    st = bcs_build(p, r_begin, r_end, recv_dev, send_host ? send_dev : nullptr,
-                   ws_bytes ? ws : nullptr, ws_bytes, cuda_stream);
+    st = launch_rows(p, r_begin, r_end - r_begin, recv_host ? recv_dev : nullptr, send_host ? send_dev : nullptr,
+                     static_cast<cudaStream_t>(cuda_stream));
     if (st != BCS_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     if (recv_host &&
@@ -1997,45 +1535,14 @@ bcs_status bcs_wait_expired(uint64_t *count_host)
     return BCS_OK;
 }
 
-// Device address of g_static_scratch on the current device, looked up once per device (with that
-// device current) and remembered; nullptr if the runtime refuses.
-static void *static_scratch_address()
-{
-    constexpr int kMaxDevices = 64;
-    static std::mutex lock;
-    static void *known[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return nullptr;
-    std::lock_guard<std::mutex> guard(lock);
-    if (dev < kMaxDevices && known[dev] != nullptr) return known[dev];
-    void *ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    if (dev < kMaxDevices) known[dev] = ptr;
-    return ptr;
-}
-
 bcs_status bcs_build_static(uint32_t p, uint64_t r_begin, uint64_t r_end, int8_t *recv_out,
                             int8_t *send_out, void *cuda_stream)
 {
     bcs_status st = check_range(p, r_begin, r_end);
     if (st != BCS_OK) return st;
     if (bcs_build_workspace_bytes(p, r_begin, r_end) > (size_t)BCS_STATIC_WORKSPACE_BYTES)
-        return BCS_ERR_UNSUPPORTED;          // needs more scratch than the library carries
-    const uint64_t count = r_end - r_begin;
-    if (count == 0 || ceil_log2_u32(p) == 0) return BCS_OK;
-    // the argument checks of bcs_build, repeated here so that they come before any runtime call
-    if (recv_out == nullptr && send_out == nullptr) return BCS_ERR_ARG;
-    if (!aligned16(recv_out) || !aligned16(send_out)) return BCS_ERR_ALIGN;
-    void *scratch = static_scratch_address();
-    if (scratch == nullptr) return BCS_ERR_CUDA;
-    // Nothing in the scratch has to start at zero: the codes of all p ranks and the round-major
-    // rows of the range are written by this call before anything reads them, so whatever an
-    // earlier call left behind is simply overwritten or never looked at.
-    return bcs_build(p, r_begin, r_end, recv_out, send_out, scratch, BCS_STATIC_WORKSPACE_BYTES,
-                     cuda_stream);
+        return BCS_ERR_UNSUPPORTED;          // the stated limit of this entry point
+    return bcs_build(p, r_begin, r_end, recv_out, send_out, nullptr, 0, cuda_stream);
 }
 
 }  // extern "C"

@@ -1,0 +1,70 @@
+"""Rows of a range straight from the binary form of its ranks, where that construction can go wrong: the ends of
+items and tiles, segments next to heads of every depth, the exceptions behind a segment's start, counts
+whose halvings all round up or never do.  Whole numbers, compared with the CPU oracle entry by entry."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bcs():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2205_10072_b200 as lib
+    lib.lib()
+    torch.cuda.set_device(0)
+    return lib
+
+
+def _buffer(n):
+    raw = torch.full((n + 64,), 99, dtype=torch.int8, device="cuda")
+    return raw, raw[32:32 + n]
+
+
+def _check(bcs, p, r0, r1, recv=True, send=True):
+    q, n = bcs.bcs_q(p), r1 - r0
+    raw_r, out_r = _buffer(n * q)
+    raw_s, out_s = _buffer(n * q)
+    bcs.bcs_build(p, r0, r1, out_r if recv else None, out_s if send else None)
+    torch.cuda.synchronize()
+    # at most 3000 ranks of a long range: both ends, and some between
+    at = np.arange(n) if n <= 3000 else np.unique(np.concatenate([
+        np.arange(700), n - 1 - np.arange(700), np.random.default_rng(p).integers(0, n, 1500)]))
+    want = oracle.build_ranks(p, (at + r0).astype(np.uint32))
+    rows = torch.from_numpy(at).cuda()
+    for raw, out, asked, expect in ((raw_r, out_r, recv, want[0]), (raw_s, out_s, send, want[1])):
+        if asked:
+            got = out.view(n, q)[rows].cpu().numpy()
+            bad = np.argwhere(got != expect)
+            assert bad.size == 0, (p, r0, r1, "rank %d entry %d" % (at[bad[0][0]] + r0, bad[0][1]))
+            assert bool((raw[:32] == 99).all()) and bool((raw[32 + n * q:] == 99).all()), (p, r0, r1)
+        else:
+            assert bool((raw == 99).all())
+
+
+# counts with skips[7] = 65 and 128, all halvings above it rounding up, or none
+EDGES = [2, 3, 5, 63, 64, 65, 100, 127, 128, 129, 130, 255, 256, 257, 65 << 9, (64 << 9) + 1, (1 << 16) + 1, 1 << 16,
+         (1 << 20) + 1, (1 << 23) - 1, (1 << 23) + 1, 100 << 13, (97 << 17) + 5, (1 << 28) + 1, (1 << 30) - 1,
+         (1 << 30) + 20, (1 << 31) - 1]
+
+
+@pytest.mark.parametrize("p", EDGES)
+def test_rows_of_ranges(bcs, p):
+    s = bcs.bcs_skips(p)
+    q = len(s) - 1
+    starts = {0, max(p - 300, 0)} | {max(s[k] - 150, 0) for k in (q, q - 1, q - 2, q // 2 + 1) if 0 <= k <= q}
+    starts |= {max(s[q - 1] + (s[q - 3] if q > 3 else 0) - 64, 0)}
+    for i, r0 in enumerate(sorted(starts)):
+        n = min((1, 31, 33, 127, 129, 300, 700)[i % 7], p - r0)
+        _check(bcs, p, r0, r0 + n, recv=i % 4 != 1, send=i % 4 != 2)
+        _check(bcs, p, r0, min(r0 + 700, p))
+
+
+@pytest.mark.parametrize("n", [148 * 32 * 32 - 1, 148 * 32 * 32 + 1, 148 * 32 * 64, 148 * 32 * 128 + 77])
+@pytest.mark.parametrize("p", [(1 << 20) + 1, 3000017])
+def test_rows_where_the_split_changes(bcs, p, n):
+    _check(bcs, p, 1234567 % (p - n), 1234567 % (p - n) + n)
