@@ -100,8 +100,14 @@ def _ptr(t) -> int | None:
     return None if t is None else t.data_ptr()
 
 
+# Handle of the current stream without building a torch.cuda.Stream (3.2 us of a call's 8.8 us).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int | None:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device()) or None
         stream = torch.cuda.current_stream()
     return stream.cuda_stream or None
 
