@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "bcs.h"
+#include "ptx.cuh"
 
 namespace bcs {
 
@@ -73,14 +74,6 @@ __host__ __device__ inline uint32_t skip_code(const uint32_t *s, int q, uint32_t
         }
     }
     return code;
-}
-
-// Position of the highest set bit, -1 for 0 (one instruction).
-__device__ __forceinline__ int top_bit(uint32_t v)
-{
-    int d;
-    asm("bfind.u32 %0, %1;" : "=r"(d) : "r"(v));
-    return d;
 }
 
 // ---------------------------------------------------------------- tile bookkeeping
@@ -336,13 +329,13 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
 
 // Launch with programmatic stream serialisation (see above); `dependent` false: ordinary launch.
 template <class... Params, class... Args>
-inline void launch_dependent(bool dependent, void (*kernel)(Params...), unsigned grid, unsigned block,
+inline void launch_dependent(bool dependent, void (*kernel)(Params...), unsigned grid, unsigned block, size_t shared,
                              cudaStream_t stream, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = shared;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

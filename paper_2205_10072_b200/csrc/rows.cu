@@ -6,6 +6,11 @@
 // to-processor lies outside the range were searched for one by one), 32 ranks without a workspace 572 -> 8.2 us (a
 // descent of the homeranges per window), 8 chunks of about 2^28 ranks 9.35 -> 3.94 ms.  Small calls
 // last as long as launch, table and one item; large ones are bound by instruction issue (seven eighths of the slots).
+//
+// The start of a call (launch, CTAs onto the SMs, table) was most of a small call's time.  The kernel is launched as a
+// dependent of whatever runs before it on the stream and waits for that before its first store only, the
+// table holds what the CTA's segments need where these are few, and a CTA has no more warps than items: 32 ranks 8.2 ->
+// 4.4 us, all ranks of 1152: 8.6 -> 4.6, of 100 003: 10.2 -> 7.6, of about 2^20: 22.7 -> 18.4 us, back to back.
 #include <atomic>
 
 #include "rows.cuh"
@@ -16,28 +21,45 @@ namespace {
 constexpr unsigned kSms = 148;
 constexpr unsigned kRowThreads = 1024;
 
-// One CTA per SM at most; every warp takes items of `item` (32, 64 or 128) consecutive ranks, neighbouring warps
-// neighbouring items.  first: rank of the first row (< p); the count <= p ranks go on at 0 behind p - 1.
+// One CTA per SM at most; every warp takes items of `item` (32, 64 or 128) consecutive ranks, in turn over the CTAs.
+// first: rank of the first row (< p); the count <= p ranks go on at 0 behind p - 1.
 template <int kWords>
 __global__ void __launch_bounds__(kRowThreads, 1)
 rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, int8_t *recv,
             int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
+    grid_launch_dependents();
     const RowLayout at(rc.q);
     const RowTable t(sm, at);
-    if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
-    __syncthreads();
-    build_row_table(t, rc.q, rc.odd);
     const uint32_t n_warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
     const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
-    for (uint64_t b = ((uint64_t)blockIdx.x * n_warps + warp) * item; b < count; b += stride) {
+    const uint64_t begin = ((uint64_t)warp * gridDim.x + blockIdx.x) * item;
+    auto rank = [&](uint64_t b) {
+        const uint32_t x = first + (uint32_t)b;
+        return x >= rc.p ? x - rc.p : x;
+    };
+    if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
+    if (rc.q > kLow) {
+        // Where every warp has one item at most, the CTA's segments are few: rows for those only (all ranks of
+        // 1152 and 32 ranks of any p need two or three of up to 25 groups of rows).
+        const bool few = count <= stride;
+        if (threadIdx.x == 0) *t.wanted = few ? 0u : (2u << (rc.q - kLow)) - 1u;
+        if (few) {
+            __syncthreads();
+            if (begin < count) {
+                const uint32_t mask = wanted_rows(rc.q, rc.inv, rank(begin), item + kHalo);
+                if ((threadIdx.x & 31u) == 0u) atomicOr(t.wanted, mask);
+            }
+        }
+    }
+    build_row_table(t, rc.q, rc.odd);
+    grid_dependency_wait();                                      // nothing before this touches the outputs
+    uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
+    for (uint64_t b = begin; b < count; b += stride) {
         const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
-        uint32_t x0 = first + (uint32_t)b;
-        if (x0 >= rc.p) x0 -= rc.p;
         const uint64_t byte = b * (uint64_t)rc.q;
-        warp_rows<kWords, true>(t, mine, rc.q, rc.odd, rc.inv, x0, n, recv ? recv + byte : nullptr,
+        warp_rows<kWords, true>(t, mine, rc.q, rc.odd, rc.inv, rank(b), n, recv ? recv + byte : nullptr,
                                 send ? send + byte : nullptr);
     }
     stage_free();
@@ -72,8 +94,12 @@ bcs_status launch(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *r
     uint32_t item = kItemRanks;
     while (item > 32u && count < kSms * (kRowThreads / 32) * item) item /= 2;
     const unsigned items = (count + item - 1) / item;
-    rows_kernel<kWords><<<items < kSms ? items : kSms, kRowThreads, RowLayout(rc.q).total(kRowThreads / 32), stream>>>(
-        rc, first, count, item, recv, send);
+    const unsigned grid = items < kSms ? items : kSms;
+    // as many warps as there are items for, at least 8 (for the table): small CTAs let the next call's start beside them
+    unsigned warps = (items + grid - 1) / grid;
+    warps = warps < 8u ? 8u : (warps > kRowThreads / 32 ? kRowThreads / 32 : warps);
+    launch_dependent(true, rows_kernel<kWords>, grid, 32u * warps, RowLayout(rc.q).total(warps), stream, rc, first, count,
+                     item, recv, send);
     return launch_status();
 }
 

@@ -42,6 +42,7 @@ constexpr int kLow = 7;                       // rounds whose entries come from 
 constexpr int kLowRanks = 128;                // skips[7] <= 128
 constexpr int kRunLevels = 6;                 // runs of 1, 2, 4, ..., 32 ranks
 constexpr int kMissRanks = 32;                // ranks behind a segment's start that can be exceptions (<= 25)
+constexpr uint32_t kRootMark = 0x7f;          // in place of the root's baseblock in the table
 constexpr uint32_t kItemRanks = 128;          // ranks that a warp takes at a time
 constexpr uint32_t kHalo = 64;                // and the ranks behind them that their send rows look at (skips[6] <= 64)
 constexpr int kItemSegments = 5;              // segments that an item can touch: all but the two at its ends lie
@@ -75,15 +76,18 @@ static_assert(kItemSegments * 8u <= 48u && kWarpStage % 16u == 0, "layout of a w
 
 // Byte offsets in the CTA's dynamic shared memory.
 struct RowLayout {
-    uint32_t miss, runs, codes, s, warps, warp_bytes;
+    uint32_t miss, runs, codes, rounds, six, s, flags, warps, warp_bytes;
     __host__ __device__ explicit RowLayout(int q)
     {
         const uint32_t rows = (uint32_t)(q - low_levels(q) + 1);
         miss = rows * kLowRanks * 8u;
         runs = miss + rows * kMissRanks;
         codes = runs + kRunLevels * kLowRanks;
-        s = codes + kLowRanks;
-        warps = s + (kRow + kLow + 1) * 4u;
+        rounds = codes + kLowRanks;
+        six = rounds + 8u * 16u;
+        s = six + 64u * 8u;
+        flags = s + (kRow + kLow + 1) * 4u;
+        warps = flags + 16u + 32u;
         warps = (warps + 127u) & ~127u;
         warp_bytes = kWarpStage + ((kItemRanks * (uint32_t)q + 31u) & ~15u);
     }
@@ -95,75 +99,124 @@ struct RowTable {
     uint8_t *miss;        // [K - L][low < 32]: the block of 0..7 that is not taken before round 7
     uint8_t *runs;        // [level][x]: baseblock bits of the 2^level ranks that end at x < skips[L]
     uint8_t *codes;       // [x]: skip code of x < skips[L]
+    uint4 *rounds;        // [i]: what round i < 7 needs, see below
+    uint2 *six;           // rows of the ranks with bit 6 set, without round 6
     uint32_t *s;
+    uint32_t *wanted;     // bit K - L: the rows of K are wanted
+    uint8_t *list;        // the wanted K
     __device__ RowTable(uint8_t *sm, const RowLayout &at)
         : rows(reinterpret_cast<uint2 *>(sm)), miss(sm + at.miss), runs(sm + at.runs), codes(sm + at.codes),
-          s(reinterpret_cast<uint32_t *>(sm + at.s))
+          rounds(reinterpret_cast<uint4 *>(sm + at.rounds)), six(reinterpret_cast<uint2 *>(sm + at.six)),
+          s(reinterpret_cast<uint32_t *>(sm + at.s)), wanted(reinterpret_cast<uint32_t *>(sm + at.flags)),
+          list(sm + at.flags + 16)
     {
     }
 };
 
-// Rounds 0 .. rounds-1 (at most six) of rank `low` of a segment whose lowest bit is K: Algorithm 4 with its
+// Baseblock bits of the ranks from..to (1 <= from <= to < skips[L], at most 64 of them).
+__device__ __forceinline__ uint32_t run_bits(const RowTable &t, int from, int to)
+{
+    const int level = 31 - __clz(to - from + 1);
+    const uint8_t *run = t.runs + level * kLowRanks;
+    return run[to] | run[from + (1 << level) - 1];
+}
+
+// Rounds 0 .. kRounds-1 (at most six) of rank `low` of a segment whose lowest bit is K: Algorithm 4 with its
 // windows looked up in the run table.  Returns the entries as bytes 0..5 and the baseblock as byte 7;
-// B: the blocks taken.
-__device__ __forceinline__ unsigned long long table_row(const RowTable &t, int q, uint32_t odd, int K, int low,
-                                                        int rounds, uint32_t &B)
+// B: the blocks taken.  (The windows do not depend on one another, so all loads are under way at once; the chain from
+// round to round is a few operations on B.)
+template <int kRounds>
+__device__ __forceinline__ uint2 table_row(const RowTable &t, int q, uint32_t odd, int K, int low, uint32_t &B)
 {
     const uint32_t c = t.codes[low];
     // positions below the rank skips[K] in the run table: that rank itself would be at `top`
     const int top = K >= kLow ? (int)t.s[kLow] - (int)count_odd(odd, kLow, K) : (int)t.s[K];
+    uint32_t found[kRounds];
+#pragma unroll
+    for (int i = 0; i < kRounds; ++i) {
+        const uint4 r = t.rounds[i];                             // skips[i], run of that level, second run of the window
+        const int e = ((c >> (i + 1)) ? low : top + low) - (int)r.x;
+        found[i] = 0;
+        if (!((c >> i) & 1u)) found[i] = t.runs[r.y + (uint32_t)e] | t.runs[r.y + (uint32_t)e - r.z];
+    }
     const int bb = c ? __ffs(c) - 1 : (K < q ? K : -1);
     B = bb >= 0 ? 1u << bb : 0u;
-    unsigned long long row = (unsigned long long)(uint8_t)bb << 56;
-    int sum = 0;
-    for (int i = 0; i < rounds; ++i) {
-        const int lo = (int)t.s[i], hi = (int)t.s[i + 1];
-        sum += lo;
+    uint32_t entry[8] = {0, 0, 0, 0, 0, 0, 0, bb >= 0 ? (uint32_t)bb : kRootMark};
+#pragma unroll
+    for (int i = 0; i < kRounds; ++i) {
         const uint32_t above = c >> (i + 1);
-        int blk;
-        int entry;
+        uint32_t U = found[i] & ~B;
         if ((c >> i) & 1u) {
-            blk = above ? __ffs(above) + i : K;
-            const bool home = K == q && above == 0;
-            entry = home ? bb : blk - q;
-            if (!home) B |= 1u << blk;
-        } else {
-            const int len = hi - lo;
-            const int level = 31 - __clz(len);
-            const int e = (above ? low : top + low) - lo;
-            const uint8_t *run = t.runs + level * kLowRanks;
-            uint32_t U = (uint32_t)(run[e] | run[e - len + (1 << level)]) & ~B;
-            if (U == 0) {                                        // the second window of Algorithm 4: a few ranks
-                for (int pos = low - hi; pos >= low - sum; --pos) {
-                    if (pos == 0) U |= (K < q ? 1u << K : 0u) & ~B;
-                    const int x = pos > 0 ? pos : top + pos;
-                    if (pos != 0 && x >= 1) U |= (uint32_t)t.runs[x] & ~B;
-                }
+            const int blk = above ? __ffs(above) + i : K;
+            U = 1u << blk;
+            if (K == q && above == 0u) {                         // the home round
+                entry[i] = (uint32_t)bb;
+                continue;
             }
-            blk = top_bit(U);
-            entry = U ? blk - q : BCS_BAD_ENTRY;
-            if (U) B |= 1u << blk;
+        } else if (U == 0u) {
+            // The second window of Algorithm 4: at most i + 1 ranks that end skips[i+1] below, on both sides
+            // of the segment's start perhaps.
+            const int to = low - (int)t.s[i + 1], from = low - (int)t.rounds[i].w;
+            if (from <= to) {
+                if (to >= 1) U |= run_bits(t, from < 1 ? 1 : from, to);
+                if (from <= 0 && to >= 0 && K < q) U |= 1u << K;
+                if (from <= -1) {
+                    const int first = top + from < 1 ? 1 : top + from, last = top + (to < -1 ? to : -1);
+                    if (first <= last) U |= run_bits(t, first, last);
+                }
+                U &= ~B;
+            }
         }
-        row |= (unsigned long long)(uint8_t)entry << (8 * i);
+        const int blk = top_bit(U);
+        if (U) B |= 1u << blk;
+        entry[i] = (uint8_t)(U ? blk - q : BCS_BAD_ENTRY);
     }
-    return row;
+    return make_uint2(entry[0] | entry[1] << 8 | entry[2] << 16 | entry[3] << 24,
+                      entry[4] | entry[5] << 8 | entry[6] << 16 | entry[7] << 24);
 }
 
-// Fills the table of a p; all threads of the CTA call (at least 128), t.s holds the skips.  Ends with a barrier.
+template <int kRounds>
+__device__ __forceinline__ void build_whole_table(const RowTable &t, int q, uint32_t odd)
+{
+    if (q != kRounds) return;
+    for (uint32_t low = threadIdx.x; low < t.s[kRounds]; low += blockDim.x) {
+        uint32_t B;
+        t.rows[low] = table_row<kRounds>(t, q, odd, q, (int)low, B);
+    }
+}
+
+// Fills the table of a p, for the K whose bits in *t.wanted are set (q > 7); all threads of the CTA call (at least
+// 128).  t.s holds the skips and *t.wanted is set, by any thread.  Begins and ends with a barrier.
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {
+    __syncthreads();
     const int L = low_levels(q);
     const uint32_t lows = t.s[L];
     if (threadIdx.x < kLowRanks) {
         uint32_t x = threadIdx.x, c = 0;
-        for (int k = L - 1; k >= 0; --k) {
-            if (x >= t.s[k]) {
-                x -= t.s[k];
+#pragma unroll
+        for (int k = kLow - 1; k >= 0; --k) {
+            const uint32_t skip = t.s[k];
+            if (k < L && x >= skip) {
+                x -= skip;
                 c |= 1u << k;
             }
         }
         t.codes[threadIdx.x] = (uint8_t)c;
         t.runs[threadIdx.x] = (uint8_t)(threadIdx.x < lows ? c & (0u - c) : 0u);
+    } else if (threadIdx.x < kLowRanks + kLow) {
+        // window of round i, below the rank: skips[i+1] - skips[i] ranks that end skips[i] below it
+        const int i = (int)(threadIdx.x - kLowRanks);
+        const uint32_t lo = t.s[i], hi = t.s[i + 1];
+        const uint32_t len = hi > lo ? hi - lo : 1u;
+        const int level = 31 - __clz(len);
+        uint32_t sum = 0;
+        for (int k = 0; k <= i; ++k) sum += t.s[k];
+        t.rounds[i] = make_uint4(lo, (uint32_t)level * kLowRanks, len - (1u << level), sum);
+    }
+    if (threadIdx.x < 32u) {                                     // list of the K
+        const uint32_t wanted = q > kLow ? *t.wanted : 1u;
+        if ((wanted >> threadIdx.x) & 1u) t.list[__popc(wanted & ((1u << threadIdx.x) - 1u))] = (uint8_t)(kLow + threadIdx.x);
     }
     __syncthreads();
     if (threadIdx.x < 32) {                                      // four ranks per lane, a byte each
@@ -186,39 +239,64 @@ __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32
     }
     __syncthreads();
     if (q < kLow) {                                              // one segment, all rounds in the table
-        for (uint32_t low = threadIdx.x; low < lows; low += blockDim.x) {
-            uint32_t B;
-            const unsigned long long row = table_row(t, q, odd, q, (int)low, q, B);
-            t.rows[low] = make_uint2((uint32_t)row, (uint32_t)(row >> 32));
-        }
+        build_whole_table<1>(t, q, odd);
+        build_whole_table<2>(t, q, odd);
+        build_whole_table<3>(t, q, odd);
+        build_whole_table<4>(t, q, odd);
+        build_whole_table<5>(t, q, odd);
+        build_whole_table<6>(t, q, odd);
     } else {
         // ranks without bit 6: rounds 0..5 as above, round 6 from the distances of the ranks with
         // baseblock 7 and 6.  Ranks with it (K = 6 here): rounds 0..5 do not depend on what comes before
         // that bit, round 6 receives the next higher one.
-        const int n = (q - 5) * 64;
-        for (int job = (int)threadIdx.x; job < n; job += (int)blockDim.x) {
-            const int K = 6 + (job >> 6), low = job & 63;
+        const int n = (q > kLow ? __popc(*t.wanted) : 1) * 64;
+        for (int job = (int)threadIdx.x; job < n + 64; job += (int)blockDim.x) {
+            const int K = job < n ? t.list[job >> 6] : 6, low = job & 63;
             if (low >= (int)t.s[6]) continue;
             uint32_t B;
-            unsigned long long row = table_row(t, q, odd, K, low, 6, B);
+            uint2 row = table_row<6>(t, q, odd, K, low, B);
             if (K == 6) {
-                if (low + t.s[6] >= t.s[7]) continue;
-                for (int k = kLow; k <= q; ++k) {
-                    const uint32_t six = (uint8_t)(k < q ? k - q : (int)(row >> 56));
-                    t.rows[(k - kLow) * kLowRanks + low + (int)t.s[6]] =
-                        make_uint2((uint32_t)row, (uint32_t)(row >> 32) | six << 16);
-                }
+                t.six[low] = row;
             } else {
                 const int m = __ffs(~B) - 1;                     // the block of 0..6 not taken so far
                 const bool seven = low < (int)count_odd(odd, kLow, K) ||
                                    (m == 6 && K > kLow && low < (int)count_odd(odd, 6, K));
-                const uint32_t six = (uint8_t)((seven ? kLow : m) - q);
-                t.rows[(K - kLow) * kLowRanks + low] = make_uint2((uint32_t)row, (uint32_t)(row >> 32) | six << 16);
+                row.y |= (uint32_t)(uint8_t)((seven ? kLow : m) - q) << 16;
+                t.rows[(K - kLow) * kLowRanks + low] = row;
                 if (low < kMissRanks) t.miss[(K - kLow) * kMissRanks + low] = (uint8_t)(seven ? m : kLow);
             }
         }
+        __syncthreads();
+        for (int job = (int)threadIdx.x; job < n; job += (int)blockDim.x) {
+            const int K = t.list[job >> 6], low = job & 63;
+            const int at = low + (int)t.s[6];
+            uint2 row = make_uint2(0u, 0u);                      // (read, but not used, behind the last one)
+            if (at < (int)t.s[7]) {
+                row = t.six[low];
+                row.y |= (uint32_t)(uint8_t)(K < q ? K - q : (int)(row.y >> 24)) << 16;
+            }
+            if (at < kLowRanks) t.rows[(K - kLow) * kLowRanks + at] = row;
+        }
     }
     __syncthreads();
+}
+
+// Bits K - L of the rows that the ranks x0 .. x0+n-1 (mod p; x0 < p, n <= 1000) need: those of their segments, and where
+// the send exceptions of these carry to; by one warp, q > 7.
+__device__ __forceinline__ uint32_t wanted_rows(int q, uint32_t inv, uint32_t x0, uint32_t n)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const int high = q - kLow;
+    uint32_t from = __umulhi(x0, inv);                           // one before or behind, at most
+    from = from ? from - 1u : 0u;
+    uint32_t bits = 0;
+    if (lane <= n / 40u + 4u) {                                  // (a segment has more than 40 ranks)
+        const uint32_t g = (from + lane) & ((1u << high) - 1u);
+        const int z = __ffs(~g) - 1;                             // lowest zero bit, and the next one
+        bits = (g ? g & (0u - g) : 1u << high) | 1u << z;
+        if (z < high) bits |= 1u << (z + __ffs(~(g >> (z + 1))));
+    }
+    return __reduce_or_sync(0xffffffffu, bits);
 }
 
 // ---------------------------------------------------------------- rows of an item, by one warp
@@ -303,17 +381,12 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
 {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t shift = kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    fence_before_bulk();
     __syncwarp();
     const uint32_t begin = (shift + 15u) & ~15u, end = shift + len;
     uint8_t *base = reinterpret_cast<uint8_t *>(dst) - shift;
     const uint32_t stop = end & ~15u;
-    if (lane == 0u && stop > begin) {
-        const uint32_t src = (uint32_t)__cvta_generic_to_shared(stage + begin);
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                     :: "l"(reinterpret_cast<uint64_t>(base + begin)), "r"(src), "r"(stop - begin) : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    }
+    if (lane == 0u && stop > begin) bulk_store(base + begin, stage + begin, stop - begin);
     if (!kAligned || (end & 15u) != 0u) {                        // bytes [shift, head) and [tail, end) one by one
         const uint32_t head = begin < end ? begin : end;
         if (shift + lane < head) base[shift + lane] = stage[shift + lane];
@@ -325,7 +398,7 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
 // The staging buffer may be written again.
 __device__ __forceinline__ void stage_free()
 {
-    if ((threadIdx.x & 31u) == 0u) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    if ((threadIdx.x & 31u) == 0u) bulk_stores_read();
     __syncwarp();
 }
 
@@ -481,7 +554,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
             __syncwarp();
             const int from = (int)((note >> kNoteFrom) & 31u);
             if (from < q) {                                      // rounds past the home round: the baseblock
-                const bool root = bb == 0xffu;                   // (the table's mark for the root)
+                const bool root = bb == kRootMark;
                 for (int k = from; k < q; ++k) at[k] = (uint8_t)(root ? (uint32_t)k : bb);
             }
             if (note & kNoteSend) {

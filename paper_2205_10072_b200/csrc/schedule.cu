@@ -1491,14 +1491,14 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
                 codes_batch_flat_kernel<<<(unsigned)((total_ranks + kCodesTile - 1) / kCodesTile), kTile, 0, stream>>>(ba, codes);
             if ((st = launch_status()) != BCS_OK) return st;
             if (send_out != nullptr)
-                launch_dependent(true, recv_quad_batch_kernel<true>, (unsigned)total_tiles, kQuadThreads, stream, ba,
+                launch_dependent(true, recv_quad_batch_kernel<true>, (unsigned)total_tiles, kQuadThreads, 0, stream, ba,
                                  (const uint32_t *)codes, recv_out, recv_t);
             else
-                launch_dependent(true, recv_quad_batch_kernel<false>, (unsigned)total_tiles, kQuadThreads, stream, ba,
+                launch_dependent(true, recv_quad_batch_kernel<false>, (unsigned)total_tiles, kQuadThreads, 0, stream, ba,
                                  (const uint32_t *)codes, recv_out, (int8_t *)nullptr);
             if ((st = launch_status()) != BCS_OK) return st;
             if (send_out != nullptr) {
-                launch_dependent(true, send_batch_kernel, (unsigned)(2 * total_tiles), kTrThreads, stream, ba,
+                launch_dependent(true, send_batch_kernel, (unsigned)(2 * total_tiles), kTrThreads, 0, stream, ba,
                                  (const int8_t *)recv_t, send_out);
                 if ((st = launch_status()) != BCS_OK) return st;
             }
@@ -1507,10 +1507,10 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         // wait for them (the host cannot tell whether the list holds such p: their CTAs return at once
         // where it does not)
         if (send_out != nullptr)
-            launch_dependent(total_tiles != 0, fused_small_batch_kernel<true>, num_p, kFusedThreads, stream, ba,
+            launch_dependent(total_tiles != 0, fused_small_batch_kernel<true>, num_p, kFusedThreads, 0, stream, ba,
                              recv_out, send_out);
         else
-            launch_dependent(total_tiles != 0, fused_small_batch_kernel<false>, num_p, kFusedThreads, stream, ba,
+            launch_dependent(total_tiles != 0, fused_small_batch_kernel<false>, num_p, kFusedThreads, 0, stream, ba,
                              recv_out, (int8_t *)nullptr);
         return launch_status();
     }
