@@ -12,14 +12,17 @@
 // table holds what the CTA's segments need where these are few, and a CTA has no more warps than items: 32 ranks 8.2 ->
 // 4.4 us, all ranks of 1152: 8.6 -> 4.6, of 100 003: 10.2 -> 7.6, of about 2^20: 22.7 -> 18.4 us, back to back.
 #include <atomic>
+#include <type_traits>
 
 #include "rows.cuh"
+#include "wide.cuh"
 
 namespace bcs {
 namespace {
 
 constexpr unsigned kSms = 148;
 constexpr unsigned kRowThreads = 1024;
+constexpr unsigned wide_threads(int vectors) { return vectors == 2 ? 768 : 1024; }
 
 // One CTA per SM at most; every warp takes items of `item` (32, 64 or 128) consecutive ranks, in turn over the CTAs.
 // first: rank of the first row (< p); the count <= p ranks go on at 0 behind p - 1.
@@ -65,6 +68,38 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     stage_free();
 }
 
+// The same for large tables, q >= 16 (wide.cuh), all receive rows before the send rows; `item` is a multiple of 16.
+template <int kVec>
+__global__ void __launch_bounds__(wide_threads(kVec), 1)
+wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, int8_t *recv,
+            int8_t *send)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    grid_launch_dependents();
+    const WideLayout at(rc.q);
+    const RowTable t(sm, at.base);
+    if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
+    if (threadIdx.x == 0) *t.wanted = (2u << (rc.q - kLow)) - 1u;
+    build_row_table(t, rc.q, rc.odd);
+    if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
+    grid_dependency_wait();
+    const uint32_t n_warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
+    auto all = [&](auto is_send, int8_t *out) {
+        WideLane<kVec> mine;
+        mine.init(rc.q, 0u);
+        for (uint64_t b = ((uint64_t)warp * gridDim.x + blockIdx.x) * item; b < count; b += stride) {
+            const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
+            uint32_t x0 = first + (uint32_t)b;
+            if (x0 >= rc.p) x0 -= rc.p;
+            wide_rows<kVec, decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
+                                                      mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
+        }
+    };
+    if (recv != nullptr) all(std::false_type(), recv);
+    if (send != nullptr) all(std::true_type(), send);
+}
+
 // Opts a kernel in to large dynamic shared memory, once per device.
 template <auto kKernel>
 bool allow_shared()
@@ -78,6 +113,19 @@ bool allow_shared()
         return false;
     done.fetch_or(bit, std::memory_order_relaxed);
     return true;
+}
+
+bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send,
+                       cudaStream_t stream)
+{
+    if (!allow_shared<wide_kernel<wide_vectors(BCS_MAX_Q)>>()) return BCS_ERR_CUDA;
+    constexpr int kVec = wide_vectors(BCS_MAX_Q);                // (so many ranks: q > 21)
+    // (192 ranks an item 17 % more for its start; 1536: 5 % more for 2^27 ranks, the same for fewer)
+    constexpr uint32_t item = 384;
+    const unsigned items = (count + item - 1) / item;
+    launch_dependent(true, wide_kernel<kVec>, items < kSms ? items : kSms, wide_threads(kVec), WideLayout(rc.q).bytes,
+                     stream, rc, first, count, item, recv, send);
+    return launch_status();
 }
 
 template <int kWords>
@@ -117,6 +165,9 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     }
     for (int k = 1; k <= rc.q; ++k) rc.odd |= (2u * rc.s[k - 1] - rc.s[k]) << k;
     rc.inv = (uint32_t)((1ull << (rc.q - low_levels(rc.q) + 32)) / p);
+    // From 2^23 ranks on the wide kernel: 4 million ranks 51.6 us here, 59.5 there; 12.3 million 152 against 143, 2^25
+    // of q = 28 369 against 298, 2^27 of q = 30 1504 against 1211 us.  (Its tables take longer to build.)
+    if (count >= (1u << 23)) return launch_wide(rc, (uint32_t)first, (uint32_t)count, recv, send, stream);
     return launch<1>(rc, (uint32_t)first, (uint32_t)count, recv, send, stream);
 }
 

@@ -68,3 +68,33 @@ def test_rows_of_ranges(bcs, p):
 @pytest.mark.parametrize("p", [(1 << 20) + 1, 3000017])
 def test_rows_where_the_split_changes(bcs, p, n):
     _check(bcs, p, 1234567 % (p - n), 1234567 % (p - n) + n)
+
+
+# the kernel for 2^23 ranks and more: its lanes' places repeat every 16 ranks, 30 segments are located at a time
+@pytest.mark.parametrize("p,r0,n", [((1 << 23) + 1, 0, (1 << 23) + 1), (100 << 17, 4000003, (1 << 23) + 385),
+                                    ((1 << 24) - 1, 0, (1 << 24) - 1), ((1 << 30) + 20, (1 << 29) - 777777, (1 << 23) + 1),
+                                    ((1 << 31) - 1, (1 << 31) - 1 - (1 << 23) - 15, (1 << 23) + 15)])
+def test_rows_of_many_ranks(bcs, p, r0, n):
+    _check(bcs, p, r0, r0 + n, send=False)
+    _check(bcs, p, r0, r0 + n, recv=False)
+    q = bcs.bcs_q(p)
+    recv = torch.empty(n * q, dtype=torch.int8, device="cuda")
+    send = torch.empty(n * q, dtype=torch.int8, device="cuda")
+    bcs.bcs_build(p, r0, r0 + n, recv, send)
+    counts = torch.ones(3, dtype=torch.int64, device="cuda")
+    bcs.bcs_validate(p, r0, r0 + n, recv, send, counts)      # every row and every pair inside the range
+    assert counts.tolist() == [0, 0, 0]
+
+
+def test_many_ranks_rooted(bcs):
+    p, root = (1 << 23) + 12345, 5000001                       # the ranks pass p - 1 inside an item
+    q = bcs.bcs_q(p)
+    recv = torch.empty(p * q, dtype=torch.int8, device="cuda")
+    send = torch.empty(p * q, dtype=torch.int8, device="cuda")
+    ws = torch.empty(bcs.bcs_build_rooted_workspace_bytes(p, root, 0, p), dtype=torch.int8, device="cuda")
+    bcs.bcs_build_rooted(p, root, 0, p, recv, send, ws)
+    at = np.concatenate([np.arange(600), root - 600 + np.arange(1200), p - 1 - np.arange(600)])
+    want = oracle.build_ranks(p, ((at - root) % p).astype(np.uint32))
+    rows = torch.from_numpy(at).cuda()
+    for out, expect in ((recv, want[0]), (send, want[1])):
+        assert np.array_equal(out.view(p, q)[rows].cpu().numpy(), expect)
