@@ -22,7 +22,8 @@ namespace {
 
 constexpr unsigned kSms = 148;
 constexpr unsigned kRowThreads = 1024;
-constexpr unsigned wide_threads(int vectors) { return vectors == 2 ? 768 : 1024; }
+// 640 threads: at the speed of the memory (2^27 ranks) the write streams of 1024 cost 20 % and more.
+constexpr unsigned kWideThreads = 640;
 
 // One CTA per SM at most; every warp takes items of `item` (32, 64 or 128) consecutive ranks, in turn over the CTAs.
 // first: rank of the first row (< p); the count <= p ranks go on at 0 behind p - 1.
@@ -69,8 +70,7 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
 }
 
 // The same for large tables, q >= 16 (wide.cuh), all receive rows before the send rows; `item` is a multiple of 16.
-template <int kVec>
-__global__ void __launch_bounds__(wide_threads(kVec), 1)
+__global__ void __launch_bounds__(kWideThreads, 1)
 wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, int8_t *recv,
             int8_t *send)
 {
@@ -86,13 +86,13 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     const uint32_t n_warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
     auto all = [&](auto is_send, int8_t *out) {
-        WideLane<kVec> mine;
+        WideLane mine;
         mine.init(rc.q, 0u);
-        for (uint64_t b = ((uint64_t)warp * gridDim.x + blockIdx.x) * item; b < count; b += stride) {
+        for (uint64_t b = ((uint64_t)blockIdx.x * n_warps + warp) * item; b < count; b += stride) {
             const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
             uint32_t x0 = first + (uint32_t)b;
             if (x0 >= rc.p) x0 -= rc.p;
-            wide_rows<kVec, decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
+            wide_rows<decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
                                                       mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
         }
     };
@@ -118,12 +118,12 @@ bool allow_shared()
 bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send,
                        cudaStream_t stream)
 {
-    if (!allow_shared<wide_kernel<wide_vectors(BCS_MAX_Q)>>()) return BCS_ERR_CUDA;
-    constexpr int kVec = wide_vectors(BCS_MAX_Q);                // (so many ranks: q > 21)
-    // (192 ranks an item 17 % more for its start; 1536: 5 % more for 2^27 ranks, the same for fewer)
-    constexpr uint32_t item = 384;
+    if (!allow_shared<wide_kernel>()) return BCS_ERR_CUDA;
+    // An item's start costs as much as some 50 ranks: 12.3 million ranks 61 us a table with items of 768, 67 with 384;
+    // but from 2^25 ranks on the memory bounds it, and items close together are written faster (146 against 151 us).
+    const uint32_t item = count >= (1u << 25) ? 384u : 768u;
     const unsigned items = (count + item - 1) / item;
-    launch_dependent(true, wide_kernel<kVec>, items < kSms ? items : kSms, wide_threads(kVec), WideLayout(rc.q).bytes,
+    launch_dependent(true, wide_kernel, items < kSms ? items : kSms, kWideThreads, WideLayout(rc.q).bytes,
                      stream, rc, first, count, item, recv, send);
     return launch_status();
 }
@@ -165,8 +165,8 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     }
     for (int k = 1; k <= rc.q; ++k) rc.odd |= (2u * rc.s[k - 1] - rc.s[k]) << k;
     rc.inv = (uint32_t)((1ull << (rc.q - low_levels(rc.q) + 32)) / p);
-    // From 2^23 ranks on the wide kernel: 4 million ranks 51.6 us here, 59.5 there; 12.3 million 152 against 143, 2^25
-    // of q = 28 369 against 298, 2^27 of q = 30 1504 against 1211 us.  (Its tables take longer to build.)
+    // From 2^23 ranks on the wide kernel, whose tables take longer to build: 4 million ranks 51.5 us here, 59.5
+    // there; 12.3 million 152 against 120, 2^25 of q = 28 369 against 290, 2^27 of q = 30 1504 against 1230 us.
     if (count >= (1u << 23)) return launch_wide(rc, (uint32_t)first, (uint32_t)count, recv, send, stream);
     return launch<1>(rc, (uint32_t)first, (uint32_t)count, recv, send, stream);
 }

@@ -2,8 +2,8 @@
 //
 // The per-rank form (warp_rows) pays for every rank: shifting a row to its place among the words of its neighbours, an
 // exchange with the next lane, stores q bytes apart, a copy out of shared memory.  Here a lane makes aligned
-// 16-byte vectors of the output.  16 ranks are q vectors, so in steps of 16, 32 or 48 ranks a lane's vector
-// always begins with the same round k0 of a rank at the same place of the step.  It holds bytes of two rows at most
+// 16-byte vectors of the output.  16 ranks are q vectors, so in steps of 16 ranks a lane's vector always begins
+// with the same round k0 of a rank at the same place of the step (the lanes from q on repeat the first ones').  It holds bytes of two rows at most
 // (q >= 16), those of ranks A and A + 1:
 //     out = segment part | bytes of A's table row | bytes of (A+1)'s table row,
 // the first in registers for as long as the segment lasts, the others by byte permutations whose selectors
@@ -22,11 +22,7 @@ namespace bcs {
 
 constexpr int kWideMinQ = 16;
 
-// Vectors of a lane per step, and 16-rank groups of a step: q <= 21 has three groups on two vectors (80 to 98 % of
-// the lanes' vectors in use, q = 16: 75 %), a larger q one group on one (69 to 97 %).  Two segments never end in the
-// same step: for q <= 21 they have at least 65 - 14 ranks, for any q at least 65 - 24.
-__host__ __device__ constexpr int wide_vectors(int q) { return q <= 21 ? 2 : 1; }
-__host__ __device__ constexpr int wide_groups(int vectors) { return vectors == 2 ? 3 : 1; }
+constexpr uint32_t kStep = 16;        // ranks of a step (two segments never end in the same: they have 41 ranks or more)
 
 struct WideLayout {
     RowLayout base;                   // (its warps' part is not used)
@@ -133,25 +129,34 @@ struct Words {
     uint32_t w[4];
 };
 
-// The entries of segment g from round L up, in the lanes' vectors: rounds k0 .. k0+15 (mod q).
-template <int kVec, bool kSend>
-__device__ __forceinline__ void segment_part(uint32_t g, int q, const int (&k0)[kVec], Words (&part)[kVec])
+// The entries of a segment from round L up depend on its number g bit by bit: those from L + 3 up on the bits from 3 up
+// only, the same for eight segments in a row.
+constexpr int kNear = 3;
+
+// Entry of round k >= L in segment g; 0 where the baseblock goes.
+template <bool kSend>
+__device__ __forceinline__ uint32_t far_entry(uint32_t g, int k, int q)
+{
+    const uint32_t bits = g >> (k - kLow);
+    const uint32_t above = bits >> 1;
+    const uint32_t next = above ? (uint32_t)(__ffs(above) + k - q) & 0xffu : 0u;
+    return ((bits & 1u) != 0u) != kSend ? next : (uint32_t)(k - q) & 0xffu;
+}
+
+// Those of the rounds from L + 3 up, in the lane's vector: rounds k0 .. k0+15 (mod q).
+template <bool kSend>
+__device__ __forceinline__ Words far_part(uint32_t g, int q, int k0)
 {
     const int k = (int)(threadIdx.x & 31u);
-    const bool inside = k >= kLow && k < q;
-    const uint32_t bits = inside ? g >> (k - kLow) : 0u;
-    const uint32_t above = bits >> 1;
-    const uint32_t next = above ? (uint32_t)(__ffs(above) + k - q) & 0xffu : 0u;     // 0 where the baseblock goes
-    const uint32_t own = inside ? (uint32_t)(k - q) & 0xffu : 0u;
+    uint32_t e = k >= kLow + kNear && k < q ? far_entry<kSend>(g, k, q) : 0u;
     auto wrap = [&](int x) { return x >= q ? x - q : x; };
     // lane k: the entries of the rounds k .. k+3 (mod q)
-    uint32_t e = ((bits & 1u) != 0u) != kSend ? next : own;
-    e |= __shfl_sync(0xffffffffu, e, wrap(k + 1)) << 8;
-    e |= __shfl_sync(0xffffffffu, e, wrap(k + 2)) << 16;
+    e |= __shfl_sync(0xffffffffu, e, wrap(k < q ? k + 1 : 0)) << 8;
+    e |= __shfl_sync(0xffffffffu, e, wrap(k < q ? k + 2 : 0)) << 16;
+    Words part;
 #pragma unroll
-    for (int i = 0; i < kVec; ++i)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) part[i].w[w] = __shfl_sync(0xffffffffu, e, wrap(k0[i] + 4 * w));
+    for (int w = 0; w < 4; ++w) part.w[w] = __shfl_sync(0xffffffffu, e, wrap(k0 + 4 * w));
+    return part;
 }
 
 __device__ __forceinline__ uint4 wide_vector(const uint2 a, const uint2 b, const Words &c, const Pick &pick)
@@ -163,28 +168,46 @@ __device__ __forceinline__ uint4 wide_vector(const uint2 a, const uint2 b, const
     return make_uint4(x[0], x[1], x[2], x[3]);
 }
 
-// What a lane knows of its vectors, for all items of a table that begin at the same place of a 16-byte group: byte
+// What a lane knows of its vector, for all items of a table that begin at the same place of a 16-byte group: byte
 // 16 v - shift of a step is round k0 of its rank a (-1: the rank before it).
-template <int kVec>
 struct WideLane {
-    int a[kVec], k0[kVec];
-    uint32_t own[kVec][4];                                       // bytes of A's row
-    Pick pick[kVec];
-    int home;                                                    // home round that they are for, -1: none
+    uint32_t v;
+    int a, k0;
+    uint32_t own[4];                                             // bytes of A's row
+    uint32_t near[4];                                            // selectors of the rounds L .. L+2
+    Pick pick;
+    int home;                                                    // home round that it is for, -1: none
     __device__ __forceinline__ void init(int q, uint32_t shift)
     {
+        const uint32_t lane = threadIdx.x & 31u;
+        v = lane < (uint32_t)q ? lane : lane - (uint32_t)q;
+        const int byte = (int)(16u * v + (uint32_t)q - shift);   // shift < 16 <= q
+        a = byte / q - 1;
+        k0 = byte - byte / q * q;
         home = -1;
+        const int to_low = (k0 <= kLow ? kLow : kLow + q) - k0;  // where round L is, or would be
+        // nibbles 4 (a zero) but for 0, 1, 2 there
+        uint64_t n = 0x4444444444444444ull;
 #pragma unroll
-        for (int i = 0; i < kVec; ++i) {
-            const int byte = (int)(16u * ((threadIdx.x & 31u) + 32u * (uint32_t)i) + (uint32_t)q - shift);   // shift < 16 <= q
-            a[i] = byte / q - 1;
-            k0[i] = byte - byte / q * q;
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                const int n = q - k0[i] - 4 * w;
-                own[i][w] = n >= 4 ? 0xffffffffu : (n <= 0 ? 0u : (1u << (8 * n)) - 1u);
-            }
+        for (int i = 0; i < kNear; ++i) {
+            int b = to_low + i;                                  // k0 = L + 1 or L + 2: a round before L + 2 is q behind
+            b = b >= q ? b - q : b;
+            if (b < 16) n = (n & ~(15ull << (4 * b))) | (uint64_t)i << (4 * b);
         }
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const int n_own = q - k0 - 4 * w;
+            own[w] = n_own >= 4 ? 0xffffffffu : (n_own <= 0 ? 0u : (1u << (8 * n_own)) - 1u);
+            near[w] = (uint32_t)(n >> (16 * w)) & 0xffffu;
+        }
+    }
+    // The whole part of a segment: `far` and the entries of the rounds L .. L+2, bytes 0..2 of `three`.
+    __device__ __forceinline__ Words part(const Words &far, uint32_t three) const
+    {
+        Words c;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) c.w[w] = far.w[w] | pick_bytes(three, 0u, near[w]);
+        return c;
     }
 };
 
@@ -194,12 +217,11 @@ struct WideLane {
 // theirs too (else n is a multiple of 16).
 // sm: the CTA's shared memory, the row table at 0, the send table at send_at; ends: 32 bytes for the two vectors that are
 // not written as a whole.
-template <int kVec, bool kSend>
+template <bool kSend>
 __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, uint32_t send_at, uint8_t *ends, uint32_t p,
-                                          int q, uint32_t odd, uint32_t inv, WideLane<kVec> &mine, uint32_t x0, uint32_t n,
+                                          int q, uint32_t odd, uint32_t inv, WideLane &mine, uint32_t x0, uint32_t n,
                                           bool head, bool tail, int8_t *dst)
 {
-    constexpr uint32_t kGroups = (uint32_t)wide_groups(kVec), kStep = 16u * kGroups;     // ranks of a step
     constexpr uint32_t kRowStride = kLowRanks * 8u;
     const uint32_t lane = threadIdx.x & 31u;
     const int high = q - kLow;
@@ -218,21 +240,16 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
     gs = gs ? gs - 1u : 0u;                                      // the segment of y, or one or two before
     bool begun = false, head_left = skip != 0u;
     int start = 0, next = 0;                                     // first rank of the segment, of the next one
-    Words part[kVec];
-    uint32_t at[kVec];                                           // shared-memory offset of A's row
-    uint32_t to[kVec], until[kVec];                              // byte of the vector in the window; end of what the lane writes
-#pragma unroll
-    for (int i = 0; i < kVec; ++i) {
-        to[i] = 16u * (lane + 32u * (uint32_t)i);
-        until[i] = to[i] < step_bytes ? len : 0u;
-    }
+    Words far, part;
+    uint32_t at = 0;                                             // shared-memory offset of A's row
+    uint32_t to = 16u * mine.v;                                  // byte of the vector in the window
     int step = 0;                                                // its first rank
 
     auto store = [&](uint32_t b, const uint4 x) {
         if (!ragged || (b >= skip && b + 16u <= len)) *reinterpret_cast<uint4 *>(out + b) = x;
         else *reinterpret_cast<uint4 *>(ends + (b < skip ? 0 : 16)) = x;
     };
-    // bytes [from, until) of a vector that the window shows in part
+    // what a window shows of a vector that it does not hold as a whole
     auto store_end = [&](uint32_t vector, const uint8_t *bytes) {
         const uint32_t b = vector + lane;
         if (lane < 16u && b >= skip && b < len) out[b] = bytes[lane];
@@ -240,30 +257,34 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
     auto put = [&](int b, uint32_t value) {
         if (b >= (int)skip && b < (int)len) out[b] = (uint8_t)value;
     };
-    // Exceptions of the segment with ranks start .. next-1.  x: what its lane packed (below).
-    auto exceptions = [&](uint32_t x) {
-        const int row0 = (int)shift + start * q;
+    // Exceptions of this lane's segment g, whose first rank is `begin` and that of the next one `end`: a few bytes each, so all
+    // the segments of an item at once, one by lane (the whole warp on one segment after another took a fifth
+    // more instructions in all).
+    auto exceptions = [&](uint32_t g, int begin, int end) {
+        const int row0 = (int)shift + begin * q;
         if (!kSend) {
-            if (lane < (x & 31u)) {                              // its first ranks receive ahead
-                const int K = (int)(x >> 8);
-                const int row = row0 + (int)lane * q;
+            if (g & 1u) return;
+            const int K = g ? __ffs(g) - 1 + kLow : q;           // its first ranks receive ahead
+            const int last = (int)count_odd(odd, kLow, K);
+            for (int low = 0; low <= last; ++low) {
                 int k = kLow;
-                for (; (int)lane < (int)count_odd(odd, k + 1, K); ++k) put(row + k, (uint32_t)(k + 1 - q));
-                put(row + k, (uint32_t)((int)t.miss[(K - kLow) * kMissRanks + (int)lane] - q));
+                for (; low < (int)count_odd(odd, k + 1, K); ++k) put(row0 + low * q + k, (uint32_t)(k + 1 - q));
+                put(row0 + low * q + k, (uint32_t)((int)t.miss[(K - kLow) * kMissRanks + low] - q));
             }
         } else {
-            const uint32_t before = x & 31u;
-            if (lane - 1u < before) {                            // the last ranks carry into ones that do
-                const int k = (int)((x >> 5) & 31u), m = (int)((x >> 10) & 31u);
-                const uint32_t behind = before - lane;
-                const int block = behind < ((x >> 15) & 31u) ? k + 1 : (int)t.miss[(m - kLow) * kMissRanks + (int)behind];
-                put((int)shift + (next - (int)lane) * q + k, (uint32_t)(block - q));
+            const int z = __ffs(~g) - 1;
+            if (g & 1u) {                                        // the first rank carries into one that does
+                put(row0 + kLow, (uint32_t)((int)t.miss[z * kMissRanks + (int)count_odd(odd, kLow, kLow + z)] - q));
+            } else if (g == 0u) {                                // the root sends block k in round k
+                for (int k = kLow; k < q; ++k) put(row0 + k, (uint32_t)k);
             }
-            if ((x >> 30) != 0u) {
-                if ((x >> 31) != 0u) {                           // so does the first one, into the block kept in bits 20..27
-                    if (lane == 0u) put(row0 + kLow, (x >> 20) & 0xffu);
-                } else if ((int)lane >= kLow && (int)lane < q) { // the root sends block k in round k
-                    put(row0 + (int)lane, lane);
+            if (z < high) {                                      // so do the last ones
+                const int k = kLow + z, m = k + __ffs(~(g >> (z + 1)));
+                const int before = (int)count_odd(odd, k, m), deeper = (int)count_odd(odd, k + 1, m);
+                for (int d = 1; d <= before; ++d) {
+                    const int behind = before - d;
+                    const int block = behind < deeper ? k + 1 : (int)t.miss[(m - kLow) * kMissRanks + behind];
+                    put((int)shift + (end - d) * q + k, (uint32_t)(block - q));
                 }
             }
         }
@@ -288,20 +309,11 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
         // its rows, and the home round
         const uint32_t rows = kSend ? send_at + (((g & 1u) ? (uint32_t)(high + tz) : own) - 1u) * kRowStride : own * kRowStride;
         const uint32_t info = rows | (uint32_t)(g ? 31 - __clz(g) + kLow : kLow - 1) << 24;
-        uint32_t extra;                                          // its exceptions
-        if (!kSend) {
-            const int K = kLow + (int)own;
-            extra = (g & 1u) ? 0u : (count_odd(odd, kLow, K) + 1u) | (uint32_t)K << 8;
-        } else {
-            extra = g == 0u ? 1u << 30 : 0u;
-            if (g & 1u)
-                extra = 1u << 31 | ((uint32_t)t.miss[tz * kMissRanks + (int)count_odd(odd, kLow, kLow + tz)] - (uint32_t)q & 0xffu) << 20;
-            if (tz < high) {
-                const int k = kLow + tz, m = k + __ffs(~(g >> (tz + 1)));
-                extra |= count_odd(odd, k, m) | (uint32_t)k << 5 | (uint32_t)m << 10 | count_odd(odd, k + 1, m) << 15;
-            }
-        }
-        int j = 0;
+        // its entries in the rounds L .. L+2, and whether it begins eight segments
+        uint32_t three = (g & ((1u << kNear) - 1u)) == 0u ? 1u << 24 : 0u;
+#pragma unroll
+        for (int i = 0; i < kNear; ++i) three |= far_entry<kSend>(g, kLow + i, q) << (8 * i);
+        int j = 0, j0;                                           // segments j0 .. j have been gone through
         uint32_t base;                                           // position of rank x0
         if (!begun) {
             j = __popc(__ballot_sync(0xffffffffu, pos <= y)) - 1;
@@ -309,83 +321,88 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
             const uint32_t inf = __shfl_sync(0xffffffffu, info, j);
             start = (int)(__shfl_sync(0xffffffffu, pos, j) - base);
             next = (int)(__shfl_sync(0xffffffffu, pos, j + 1) - base);
-            segment_part<kVec, kSend>(__shfl_sync(0xffffffffu, g, j), q, mine.k0, part);
+            far = far_part<kSend>(__shfl_sync(0xffffffffu, g, j), q, mine.k0);
+            part = mine.part(far, __shfl_sync(0xffffffffu, three, j));
             const int home = (int)(inf >> 24);
-#pragma unroll
-            for (int i = 0; i < kVec; ++i) {
-                at[i] = (inf & 0xffffffu) + (uint32_t)((mine.a[i] - start) * 8);
-                if (home != mine.home) mine.pick[i] = make_pick<kSend>(mine.k0[i], q, home, home);
-            }
+            at = (inf & 0xffffffu) + (uint32_t)((mine.a - start) * 8);
+            if (home != mine.home) mine.pick = make_pick<kSend>(mine.k0, q, home, home);
             mine.home = home;
             begun = true;
         } else {
             base = __shfl_sync(0xffffffffu, pos, 0) - (uint32_t)start;
             next = (int)(__shfl_sync(0xffffffffu, pos, 1) - base);
         }
+        j0 = j;
+        bool done = false;
         for (;;) {
             // steps inside the segment
-            const int end = next < (int)n ? next : (int)n;
-            for (; step + (int)kStep <= end; step += (int)kStep) {
-#pragma unroll
-                for (int i = 0; i < kVec; ++i) {
-                    if (until[i] != 0u) {
-                        const uint2 ra = *reinterpret_cast<const uint2 *>(sm + at[i]);
-                        const uint2 rb = *reinterpret_cast<const uint2 *>(sm + at[i] + 8);
-                        store(to[i], wide_vector(ra, rb, part[i], mine.pick[i]));
-                    }
-                    at[i] += 8u * kStep;
-                    to[i] += step_bytes;
+            const int steps = ((next < (int)n ? next : (int)n) - step) / (int)kStep;
+            if (!ragged) {
+                uint8_t *o = out + to;
+#pragma unroll 2
+                for (int i = 0; i < steps; ++i) {
+                    const uint2 ra = *reinterpret_cast<const uint2 *>(sm + at);
+                    const uint2 rb = *reinterpret_cast<const uint2 *>(sm + at + 8);
+                    *reinterpret_cast<uint4 *>(o) = wide_vector(ra, rb, part, mine.pick);
+                    at += 8u * kStep;
+                    o += step_bytes;
+                }
+            } else {
+                for (int i = 0; i < steps; ++i) {
+                    const uint2 ra = *reinterpret_cast<const uint2 *>(sm + at);
+                    const uint2 rb = *reinterpret_cast<const uint2 *>(sm + at + 8);
+                    store(to + (uint32_t)i * step_bytes, wide_vector(ra, rb, part, mine.pick));
+                    at += 8u * kStep;
                 }
             }
+            to += (uint32_t)steps * step_bytes;
+            step += steps * (int)kStep;
             // the step in which it ends, or the last one of the item
-            const uint32_t inf2 = __shfl_sync(0xffffffffu, info, j + 1);
+            const uint32_t inf2 = __shfl_sync(0xffffffffu, info, j + 1), three2 = __shfl_sync(0xffffffffu, three, j + 1);
             const int home2 = (int)(inf2 >> 24);
-            Words coming[kVec];
-            segment_part<kVec, kSend>(__shfl_sync(0xffffffffu, g, j + 1), q, mine.k0, coming);
+            if ((three2 >> 24) != 0u) far = far_part<kSend>(__shfl_sync(0xffffffffu, g, j + 1), q, mine.k0);
+            const Words coming = mine.part(far, three2);
+            const int A = step + mine.a;
+            const uint32_t new_at = (inf2 & 0xffffffu) + (uint32_t)((A - next) * 8);
+            const bool behind = A >= next, behind_b = A + 1 >= next;
+            if (mine.home != home2)
+                mine.pick = make_pick<kSend>(mine.k0, q, behind ? home2 : mine.home, behind_b ? home2 : mine.home);
+            if (to < len) {
+                Words c;
 #pragma unroll
-            for (int i = 0; i < kVec; ++i) {
-                const int A = step + mine.a[i];
-                const uint32_t new_at = (inf2 & 0xffffffu) + (uint32_t)((A - next) * 8);
-                const bool behind = A >= next, behind_b = A + 1 >= next;
-                if (mine.home != home2)
-                    mine.pick[i] = make_pick<kSend>(mine.k0[i], q, behind ? home2 : mine.home, behind_b ? home2 : mine.home);
-                if (to[i] < until[i]) {
-                    Words c;
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        const uint32_t keep = behind_b ? (behind ? 0u : mine.own[i][w]) : 0xffffffffu;
-                        c.w[w] = (part[i].w[w] & keep) | (coming[i].w[w] & ~keep);
-                    }
-                    const uint2 ra = *reinterpret_cast<const uint2 *>(sm + (behind ? new_at : at[i]));
-                    const uint2 rb = *reinterpret_cast<const uint2 *>(sm + (uint32_t)((behind_b ? new_at : at[i]) + 8u));
-                    store(to[i], wide_vector(ra, rb, c, mine.pick[i]));
+                for (int w = 0; w < 4; ++w) {
+                    const uint32_t keep = behind_b ? (behind ? 0u : mine.own[w]) : 0xffffffffu;
+                    c.w[w] = (part.w[w] & keep) | (coming.w[w] & ~keep);
                 }
-                part[i] = coming[i];
-                if (mine.home != home2) mine.pick[i] = make_pick<kSend>(mine.k0[i], q, home2, home2);
-                at[i] = new_at + 8u * kStep;
-                to[i] += step_bytes;
+                const uint2 ra = *reinterpret_cast<const uint2 *>(sm + (behind ? new_at : at));
+                const uint2 rb = *reinterpret_cast<const uint2 *>(sm + (uint32_t)((behind_b ? new_at : at) + 8u));
+                store(to, wide_vector(ra, rb, c, mine.pick));
             }
+            part = coming;
+            if (mine.home != home2) mine.pick = make_pick<kSend>(mine.k0, q, home2, home2);
             mine.home = home2;
+            at = new_at + 8u * kStep;
+            to += step_bytes;
             step += (int)kStep;
-            const bool done = step * q >= (int)len;
-            __syncwarp();                                        // the vectors come first
-            if (ragged) {
-                if (head_left) store_end(0u, ends);
-                head_left = false;
-                if (done && (len & 15u) != 0u && (len >= 16u || skip == 0u)) store_end(len & ~15u, ends + 16);
-                __syncwarp();
-            }
-            exceptions(__shfl_sync(0xffffffffu, extra, j));
+            done = step * q >= (int)len;
             start = next;
             ++j;
-            if ((int)shift + start * q >= (int)len) return;
             next = (int)(__shfl_sync(0xffffffffu, pos, j + 1) - base);
-            if (done) {                                          // its first ranks were in that step
-                exceptions(__shfl_sync(0xffffffffu, extra, j));
-                return;
-            }
-            if (j == 30) break;                                  // (lane 31 is known as the next one only)
+            // (lane 31 is known as the next one only; the last step may hold the first ranks of segment j)
+            if (done || j == 30) break;
         }
+        __syncwarp();                                            // the vectors come first
+        if (ragged) {
+            if (head_left) store_end(0u, ends);
+            head_left = false;
+            if (done && (len & 15u) != 0u && (len >= 16u || skip == 0u)) store_end(len & ~15u, ends + 16);
+            __syncwarp();
+        }
+        {
+            const uint32_t after = __shfl_down_sync(0xffffffffu, pos, 1);
+            if ((int)lane >= j0 && (int)lane < j + (done ? 1 : 0)) exceptions(g, (int)(pos - base), (int)(after - base));
+        }
+        if (done) return;
         gs += 30u;
     }
 }
