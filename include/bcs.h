@@ -151,12 +151,9 @@ bcs_status bcs_build_to_host(uint32_t p, uint64_t r_begin, uint64_t r_end,
  *   rank_off_host[num_p+1]  prefix sums of p_j            (flattened rank index),
  *   entry_off_host[num_p+1] prefix sums of p_j * q_j      (byte offset of p_j's table),
  *   tile_off_host[num_p+1]  prefix sums of ceil(p_j / 512) over the p_j above 1024, 0 for the
- *                           others (the fast construction works on a larger p in tiles of 512
- *                           ranks that start anew with every p, and builds both tables of a
- *                           p_j <= 1024 in one thread block that keeps everything on chip),
- *   copy_off_host[num_p+1]  prefix sums of q_j * align16(p_j) over the p_j above 1024 (where
- *                           p_j's round-major scratch copy starts in the workspace; align16 =
- *                           round up to 16),
+ *                           others (a smaller p is built by one thread block),
+ *   copy_off_host[num_p+1]  prefix sums of q_j * align16(p_j) over the p_j above 1024 (align16 =
+ *                           round up to 16; not used by bcs_build_batch),
  *   skips_tab_host[num_p * BCS_SKIPS_STRIDE] row j = skips[0..q_j] of p_j (Algorithm 1),
  *                           the rest of the row 0,
  *   full_tab_host[num_p * BCS_SKIPS_STRIDE]  row j, word d = skip code of rank
@@ -173,11 +170,8 @@ bcs_status bcs_batch_plan(const uint32_t *p_list_host, uint32_t num_p,
  * total_tiles = tile_off[num_p], total_copy = copy_off[num_p] (the host knows all four).
  * Outputs: device int8, total_entries bytes each, 16-byte aligned; the table of p_j starts at
  * byte entry_off[j] and is rank-major with q_j bytes per rank, unpadded.  send_out may be NULL;
- * recv_out is required.  workspace as for bcs_build, of
- * bcs_build_batch_workspace_bytes(total_ranks, total_copy) bytes for the fast construction
- * (which also needs tile_off_dev and copy_off_dev; 256 bytes, never touched, when no p of the
- * list is above 1024: the pointer then only selects the construction), or NULL: then
- * tile_off_dev and copy_off_dev may be NULL too and the self-contained construction runs. */
+ * recv_out is required.  workspace: as for bcs_build, not touched; it, tile_off_dev and copy_off_dev
+ * may be NULL. */
 size_t bcs_build_batch_workspace_bytes(uint64_t total_ranks, uint64_t total_copy);
 bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_dev,
                            const uint64_t *entry_off_dev, const uint64_t *tile_off_dev,
@@ -274,16 +268,9 @@ bcs_status bcs_validate(uint32_t p, uint64_t r_begin, uint64_t r_end,
 bcs_status bcs_simulate(uint32_t p, uint32_t n, const int8_t *recv, const int8_t *send,
                         uint64_t *state_dev, uint64_t *counts_dev, void *cuda_stream);
 
-/* Bounded waits (no counterpart in the paper).  The transposition kernel of
- * bcs_build_batch waits for their bulk copies on a shared-memory barrier
- * with a poll limit; a CTA whose copies did not arrive within the limit gives up, leaves its
- * ranks of the output unwritten and counts itself in a device-wide counter that is never
- * reset.  The build call that enqueued the kernel has long returned BCS_OK by then, so this
- * poll is the only report.  The call waits for all work of the current device
- * (cudaDeviceSynchronize, whatever streams it was enqueued on) and then stores the counter in
- * *count_host (host).  0: every table written so far is complete.  Any increase since the last
- * reading: discard EVERY table built in between, not only the counted tiles -- a copy that
- * arrives after its CTA has gone may land in the shared memory of another CTA. */
+/* Waits for all work of the current device (cudaDeviceSynchronize) and stores in *count_host (host) how
+ * many waits of the library's kernels ran out: 0, since none of them waits with a limit.  (Kept for
+ * callers of earlier versions, whose transposition kernels did.) */
 bcs_status bcs_wait_expired(uint64_t *count_host);
 
 /* Position-weighted 64-bit checksum of a stretch of schedule entries, additive

@@ -1,0 +1,280 @@
+// All ranks of many p at once: bcs_build_batch.
+//
+// A CTA of 256 threads builds the row table of a p (rows.cuh) and computes rows from it; several CTAs share an SM, so
+// that one builds a table while the others compute.  Three kernels take a p by its size:
+//   * up to 1024 ranks: a CTA per p;
+//   * up to 2^21 ranks: CTAs take equal shares of the flattened ranks of the list, p by p;
+//   * more: all CTAs of a grid work on one p after another (launched only when the list is long enough to hold one).
+// Each is launched as a dependent of the kernel before it on the stream.
+//
+// Before: skip codes of all ranks, a search on them, a round-major copy and its transposition.  1024 p of 2^10..2^20:
+// 5456 -> 1423 us (9.1 ps a rank, both tables 4.1 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 22.7 us,
+// 16 p of 2^10..2^20: 94 -> 66 us.  Two CTAs of 256 threads per SM instead of three: 1505 us, four: more (spills).
+#include <type_traits>
+
+#include "rows.cuh"
+#include "wide.cuh"
+
+namespace bcs {
+namespace {
+
+constexpr unsigned kSms = 148;
+constexpr uint32_t kSmallP = 1024;
+constexpr int kSmallQ = 10;
+constexpr int kMiddleQ = 21;
+constexpr uint32_t kLargeThreads = 640, kBatchThreads = 256, kBatchWarps = kBatchThreads / 32;
+
+// What a CTA works on.
+struct BatchJob {
+    uint64_t rank0, rank1, entry0;   // flattened ranks and first byte of the p
+    uint32_t p, odd, inv;
+};
+
+// One warp: constants of p_j into t and job.
+__device__ __forceinline__ void load_job(const BatchArgs &ba, uint32_t j, const RowTable &t, BatchJob &job)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t p = ba.p_list[j];
+    const int q = ceil_log2_fast(p);
+    const uint32_t skip = ba.skips_tab[(size_t)j * kRow + lane];
+    const uint32_t before = __shfl_up_sync(0xffffffffu, skip, 1);
+    const uint32_t odd = __ballot_sync(0xffffffffu, lane >= 1u && (int)lane <= q && 2u * before != skip);
+    t.s[lane] = skip;
+    if (lane < kLow + 1) t.s[kRow + lane] = 0u;
+    if (lane == 0u) {
+        job.p = p;
+        job.odd = odd;
+        job.inv = p > 1u ? (uint32_t)((1ull << (q - low_levels(q) + 32)) / p) : 0u;
+        job.rank0 = ba.rank_off[j];
+        job.rank1 = ba.rank_off[j + 1];
+        job.entry0 = ba.entry_off[j];
+        *t.wanted = q > kLow ? (2u << (q - kLow)) - 1u : 1u;
+    }
+}
+
+// Ranks r0 .. r1-1 of a p by the warps of the CTA, the per-rank form, `item` (<= 128) ranks at a time.
+template <int kWords>
+__device__ __forceinline__ void narrow_piece(const RowTable &t, uint8_t *mine, const BatchJob &job, int q, uint32_t r0,
+                                             uint32_t r1, uint32_t item, int8_t *recv, int8_t *send)
+{
+    for (uint32_t r = r0 + (threadIdx.x >> 5) * item; r < r1; r += kBatchWarps * item) {
+        const uint32_t n = r1 - r < item ? r1 - r : item;
+        const uint64_t byte = job.entry0 + (uint64_t)r * (uint64_t)q;
+        warp_rows<kWords, false>(t, mine, q, job.odd, job.inv, r, n, recv + byte, send ? send + byte : nullptr);
+    }
+}
+
+// Ranks r0 .. r1-1 of a p (multiples of 16, or r1 = p), wide form: every warp takes one run, receive rows then send rows.
+__device__ __forceinline__ void wide_piece(const RowTable &t, const uint8_t *sm, const WideLayout &at, uint8_t *ends,
+                                           const BatchJob &job, int q, uint32_t r0, uint32_t r1, int8_t *recv, int8_t *send)
+{
+    const uint32_t item = ((r1 - r0 + kBatchWarps - 1u) / kBatchWarps + kStep - 1u) / kStep * kStep;
+    const uint32_t r = r0 + (threadIdx.x >> 5) * item;
+    if (r >= r1) return;
+    const uint32_t n = r1 - r < item ? r1 - r : item;
+    const bool head = r == 0u, tail = r + n == job.p;
+    const uint64_t byte = job.entry0 + (uint64_t)r * (uint64_t)q;
+    WideLane lane;
+    lane.init(q, (uint32_t)(byte & 15u));                        // (the outputs start on 16-byte boundaries)
+    wide_rows<false>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, recv + byte);
+    if (send != nullptr) {
+        lane.home = -1;
+        wide_rows<true>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, send + byte);
+    }
+}
+
+// p <= 1024: a CTA per p.
+__global__ void __launch_bounds__(kBatchThreads)
+batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *send)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ BatchJob job;
+    grid_launch_dependents();
+    const uint32_t j = ba.num_p - 1u - blockIdx.x;               // (lists often ascend: the longest first)
+    const uint32_t p = ba.p_list[j];
+    const int q = ceil_log2_fast(p);
+    if (p > kSmallP || q == 0) {
+        grid_dependency_wait();
+        return;
+    }
+    const RowLayout at(q);
+    const RowTable t(sm, at);
+    if (threadIdx.x < 32u) load_job(ba, j, t, job);
+    __syncthreads();
+    build_row_table(t, q, job.odd);
+    grid_dependency_wait();                                      // nothing before this touches the outputs
+    uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
+    const uint32_t item = p > 512u ? 128u : (p > 256u ? 64u : 32u);
+    if (q <= 4) narrow_piece<1>(t, mine, job, q, 0u, p, item, recv, send);
+    else if (q <= 8) narrow_piece<2>(t, mine, job, q, 0u, p, item, recv, send);
+    else narrow_piece<3>(t, mine, job, q, 0u, p, item, recv, send);
+    stage_free();
+}
+
+// 1024 < p <= 2^21: the CTA's share is `share` (a multiple of 16) flattened ranks.
+__global__ void __launch_bounds__(kBatchThreads, 3)
+batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t *recv, int8_t *send)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ BatchJob job;
+    __shared__ uint32_t found;
+    grid_launch_dependents();
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t g0 = (uint64_t)blockIdx.x * share;
+    const uint64_t g1 = g0 + share < ba.total_ranks ? g0 + share : ba.total_ranks;
+    bool waited = false;
+    uint32_t from = 0;                                           // (first warp only: where the search goes on)
+    if (threadIdx.x < 32u) from = find_segment_warp(ba.rank_off, ba.num_p, g0);
+    for (;;) {
+        __syncthreads();                                         // the p before is done with
+        if (threadIdx.x < 32u) {
+            uint32_t hits = 0;
+            for (;; from += 32u) {
+                const uint32_t j = from + lane;
+                const bool inside = j < ba.num_p && ba.rank_off[j] < g1;
+                const uint32_t p = inside ? ba.p_list[j] : 0u;
+                hits = __ballot_sync(0xffffffffu, p > kSmallP && p <= (1u << kMiddleQ));
+                if (hits != 0u || __any_sync(0xffffffffu, !inside)) break;
+            }
+            from += (uint32_t)__ffs(hits) - 1u;
+            if (lane == 0u) found = hits != 0u ? from : 0xffffffffu;
+        }
+        __syncthreads();
+        if (found == 0xffffffffu) break;
+        const int q = ceil_log2_fast(ba.p_list[found]);
+        const bool narrow = q < kWideMinQ;
+        const RowLayout at_narrow(q);
+        const RowTable t(sm, at_narrow);
+        if (threadIdx.x < 32u) load_job(ba, found, t, job);
+        ++from;
+        __syncthreads();
+        const uint32_t p = job.p;
+        const uint32_t r0 = g0 > job.rank0 ? ((uint32_t)(g0 - job.rank0) + 15u) & ~15u : 0u;
+        const uint32_t end = g1 < job.rank1 ? ((uint32_t)(g1 - job.rank0) + 15u) & ~15u : p;
+        const uint32_t r1 = end < p ? end : p;
+        if (r0 >= r1) continue;
+        build_row_table(t, q, job.odd);
+        const WideLayout at(q);
+        if (!narrow && send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
+        if (!waited) grid_dependency_wait();
+        waited = true;
+        if (narrow) {
+            uint8_t *mine = sm + at_narrow.warps + (threadIdx.x >> 5) * at_narrow.warp_bytes;
+            if (q <= 12) narrow_piece<3>(t, mine, job, q, r0, r1, kItemRanks, recv, send);
+            else narrow_piece<4>(t, mine, job, q, r0, r1, kItemRanks, recv, send);
+            stage_free();
+        } else {
+            wide_piece(t, sm, at, sm + at.ends + (threadIdx.x >> 5) * 32u, job, q, r0, r1, recv, send);
+        }
+    }
+    if (!waited) grid_dependency_wait();
+}
+
+// p > 2^21: all CTAs on every such p of the list.
+__global__ void __launch_bounds__(kLargeThreads, 1)
+batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *send)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ BatchJob job;
+    grid_launch_dependents();
+    grid_dependency_wait();
+    constexpr uint32_t item = 768;
+    uint32_t j = 0;
+    for (;;) {
+        for (; j < ba.num_p; ++j) {                              // the next one, kLargeThreads at a glance
+            if (j % kLargeThreads == 0u) {
+                const uint32_t k = j + threadIdx.x;
+                if (!__syncthreads_or(k < ba.num_p && ba.p_list[k] > (1u << kMiddleQ))) {
+                    j += kLargeThreads - 1u;
+                    continue;
+                }
+            }
+            if (ba.p_list[j] > (1u << kMiddleQ)) break;
+        }
+        if (j >= ba.num_p) break;
+        const uint32_t p = ba.p_list[j];
+        const int q = ceil_log2_fast(p);
+        const WideLayout at(q);
+        const RowTable t(sm, at.base);
+        __syncthreads();                                         // the p before is done with
+        if (threadIdx.x < 32u) load_job(ba, j, t, job);
+        __syncthreads();
+        build_row_table(t, q, job.odd);
+        if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
+        const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+        auto all = [&](auto is_send, int8_t *out) {
+            WideLane lane;
+            lane.init(q, (uint32_t)(job.entry0 & 15u));
+            for (uint64_t r = ((uint64_t)blockIdx.x * n_warps + warp) * item; r < p; r += (uint64_t)gridDim.x * n_warps * item) {
+                const uint32_t n = p - (uint32_t)r < item ? p - (uint32_t)r : item;
+                wide_rows<decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, p, q, job.odd, job.inv, lane,
+                                                    (uint32_t)r, n, r == 0, r + n == p, out + job.entry0 + r * (uint64_t)q);
+            }
+        };
+        all(std::false_type(), recv);
+        if (send != nullptr) all(std::true_type(), send);
+        ++j;
+    }
+}
+
+}  // namespace
+}  // namespace bcs
+
+using namespace bcs;
+
+extern "C" {
+
+size_t bcs_build_batch_workspace_bytes(uint64_t total_ranks, uint64_t total_copy)
+{
+    if (total_ranks == 0) return 0;
+    if (total_copy == 0) return 256;
+    return (size_t)(align_up(4ull * total_ranks, 256) + total_copy);
+}
+
+bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_dev,
+                           const uint64_t *entry_off_dev, const uint64_t *tile_off_dev,
+                           const uint64_t *copy_off_dev, const uint32_t *skips_tab_dev,
+                           const uint32_t *full_tab_dev, uint32_t num_p, uint64_t total_ranks,
+                           uint64_t total_entries, uint64_t total_tiles, uint64_t total_copy,
+                           int8_t *recv_out, int8_t *send_out, void *workspace, size_t workspace_bytes,
+                           void *cuda_stream)
+{
+    if (num_p == 0 || total_ranks == 0) return BCS_OK;
+    if (p_list_dev == nullptr || rank_off_dev == nullptr || entry_off_dev == nullptr ||
+        skips_tab_dev == nullptr || full_tab_dev == nullptr)
+        return BCS_ERR_ARG;
+    if (total_entries == 0) return BCS_OK;   // only p == 1 in the list
+    if (recv_out == nullptr) return BCS_ERR_ARG;
+    if (!aligned16(recv_out) || !aligned16(send_out) || !aligned16(workspace)) return BCS_ERR_ALIGN;
+    if ((total_ranks + kTile - 1) / kTile > 0x7fffffffull || total_tiles > 0x3fffffffull) return BCS_ERR_UNSUPPORTED;
+    (void)copy_off_dev;                      // the rows need no scratch memory, see rows.cuh
+    (void)total_copy;
+    (void)workspace_bytes;
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    const BatchArgs ba = {p_list_dev, rank_off_dev, entry_off_dev, skips_tab_dev, num_p, total_ranks};
+    static_assert(kSmallP == kFusedMaxP, "the plan counts tiles for the p above kSmallP");
+    // (without the plan's tiles the host cannot tell what sizes the list holds)
+    if (tile_off_dev == nullptr || total_tiles != 0) {
+        const WideLayout wide(kMiddleQ);
+        const RowLayout narrow(kWideMinQ - 1);
+        const uint32_t shared = wide.bytes > narrow.total(kBatchWarps) ? wide.bytes : narrow.total(kBatchWarps);
+        if (!allow_shared<batch_middle_kernel>()) return BCS_ERR_CUDA;
+        // Three shares per resident CTA where the list is long enough, so that none ends last by much; at most 32768
+        // ranks, at least 1024 (a table costs as much as some hundred ranks of each warp).
+        uint64_t share = align_up(total_ranks / (kSms * 3u * 3u), 512);
+        share = share < 1024 ? 1024 : (share > 32768 ? 32768 : share);
+        const uint64_t shares = (total_ranks + share - 1) / share;
+        launch_dependent(true, batch_middle_kernel, (unsigned)shares, kBatchThreads, shared, stream, ba, (uint32_t)share,
+                         recv_out, send_out);
+        if (total_ranks > (1u << kMiddleQ)) {
+            if (!allow_shared<batch_large_kernel>()) return BCS_ERR_CUDA;
+            launch_dependent(true, batch_large_kernel, kSms, kLargeThreads, WideLayout(BCS_MAX_Q).bytes, stream, ba, recv_out,
+                             send_out);
+        }
+    }
+    launch_dependent(true, batch_small_kernel, num_p, kBatchThreads, RowLayout(kSmallQ).total(kBatchWarps), stream, ba,
+                     recv_out, send_out);
+    return launch_status();
+}
+
+}  // extern "C"

@@ -1,9 +1,10 @@
 // Shared pieces of the schedule, round-table and checksum translation units: per-p tables,
-// the Section 2 primitives of arXiv 2205.10072 as device functions, and the tile bookkeeping
-// that turns per-rank rows into contiguous, 16-byte vectorised output spans.
+// the Section 2 primitives of arXiv 2205.10072 as device functions, lists of p, launches.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <atomic>
 
 #include "bcs.h"
 #include "ptx.cuh"
@@ -11,10 +12,7 @@
 namespace bcs {
 
 constexpr int kTile = 256;                    // ranks (= threads) per CTA of the schedule kernels
-constexpr int kStageBytes = kTile * 32 + 16;  // kTile rows of <= 31 bytes + alignment shift
-constexpr uint32_t kFusedMaxP = 1024;         // batch: a p up to here is built by one CTA of the fused kernel
-constexpr int kFusedMaxQ = 10;                //        (q <= 10)
-constexpr int kCachedRows = 4;                // per-p table rows a batch CTA keeps in shared memory
+constexpr uint32_t kFusedMaxP = 1024;         // batch: a p up to here is built by one CTA
 constexpr int kRow = BCS_SKIPS_STRIDE;        // words per table row
 
 // Per-p constants (kernel parameter of the single-p kernels).
@@ -32,13 +30,8 @@ struct BatchArgs {
     const uint64_t *rank_off;
     const uint64_t *entry_off;
     const uint32_t *skips_tab;   // [num_p][kRow]
-    const uint32_t *full_tab;    // [num_p][kRow]
     uint32_t num_p;
     uint64_t total_ranks;
-    // workspace construction only: tiles of 512 ranks that start anew with every p, and where
-    // the round-major copy of each p starts (every round padded to a multiple of 16 bytes)
-    const uint64_t *tile_off;    // [num_p + 1] prefix sums of ceil(p_j / 512)
-    const uint64_t *copy_off;    // [num_p + 1] prefix sums of q_j * align16(p_j)
 };
 
 __host__ __device__ inline int ceil_log2_u32(uint32_t p)
@@ -76,100 +69,9 @@ __host__ __device__ inline uint32_t skip_code(const uint32_t *s, int q, uint32_t
     return code;
 }
 
-// ---------------------------------------------------------------- tile bookkeeping
-struct RankCtx {
-    const uint32_t *s;      // skips of this rank's p (shared or global memory)
-    const uint32_t *full;   // full[] of this rank's p
-    uint32_t p;
-    int q;
-    uint32_t r;
-    uint32_t pj;            // index of p in the batch (0 for the single-p kernels)
-    uint64_t rank0;         // flattened index of rank 0 of this p (0 for single p)
-    uint64_t entry;         // byte offset of the rank's row in the output
-    bool valid;
-};
-
-struct TileShared {
-    uint32_t skips[kCachedRows][kRow];
-    uint32_t full[kCachedRows][kRow];
-    uint64_t span_begin, span_end;
-    uint64_t rank0_first, entry0_first;   // batch: rank and entry offset of the CTA's first p
-    uint32_t j_first, j_last;
-    uint32_t p_first;
-    __align__(16) uint8_t stage[kStageBytes];
-};
-
-// Copies stage[shift, shift+len) to out[byte0, byte0+len); (byte0 & 15) == shift and `out`
-// is 16-byte aligned, so all but the ragged ends go out as 16-byte vectors.
-__device__ __forceinline__ void flush_span(const uint8_t *stage, uint32_t shift, uint32_t len,
-                                           int8_t *out, uint64_t byte0)
-{
-    uint8_t *dst = reinterpret_cast<uint8_t *>(out) + (byte0 - shift);
-    const uint32_t end = shift + len;
-    const uint32_t nvec = (end + 15u) >> 4;
-    for (uint32_t v = threadIdx.x; v < nvec; v += blockDim.x) {
-        uint32_t lo = v << 4, hi = lo + 16u;
-        if (lo >= shift && hi <= end) {
-            *reinterpret_cast<uint4 *>(dst + lo) = *reinterpret_cast<const uint4 *>(stage + lo);
-        } else {
-            uint32_t from = lo < shift ? shift : lo, to = hi > end ? end : hi;
-            for (uint32_t e = from; e < to; ++e) dst[e] = stage[e];
-        }
-    }
-}
-
-// The same for a staging buffer whose span starts `lag` = 1..3 bytes EARLIER in its 16-byte group
-// than the span does in global memory: stage[shift - lag, shift - lag + len) goes to
-// out[byte0, byte0 + len) with (byte0 & 15) == shift, shift >= lag.  (Rows that must start on a word
-// in shared memory while the table starts at any byte of the output.)  Every 16-byte vector of the
-// output is put together from five aligned words of the staging buffer, funnel-shifted by `lag`
-// bytes; the ragged ends go out as bytes.  The four bytes before `stage` must be readable.
-__device__ __forceinline__ void flush_span_lagging(const uint8_t *stage, uint32_t shift, uint32_t lag, uint32_t len,
-                                                   int8_t *out, uint64_t byte0)
-{
-    uint8_t *dst = reinterpret_cast<uint8_t *>(out) + (byte0 - shift);
-    const uint32_t end = shift + len;
-    const uint32_t nvec = (end + 15u) >> 4;
-    const uint32_t bits = 8u * (4u - lag);
-    for (uint32_t v = threadIdx.x; v < nvec; v += blockDim.x) {
-        const uint32_t lo = v << 4, hi = lo + 16u;
-        if (lo >= shift && hi <= end) {
-            // output bytes lo .. lo+15 are staging bytes lo-lag .. lo+15-lag: words at lo-4, lo, ..., lo+12
-            const uint32_t *w = reinterpret_cast<const uint32_t *>(stage + lo) - 1;
-            const uint32_t w0 = w[0], w1 = w[1], w2 = w[2], w3 = w[3], w4 = w[4];
-            *reinterpret_cast<uint4 *>(dst + lo) =
-                make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits),
-                           __funnelshift_r(w2, w3, bits), __funnelshift_r(w3, w4, bits));
-        } else {
-            const uint32_t from = lo < shift ? shift : lo, to = hi > end ? end : hi;
-            for (uint32_t e = from; e < to; ++e) dst[e] = stage[e - lag];
-        }
-    }
-}
-
-// The same for a span that starts 16-byte aligned in shared and global memory and is a multiple
-// of 16 bytes long, as one bulk copy of the TMA unit (cp.async.bulk, shared -> global) issued by
-// one thread.  Call with all threads of the CTA, after the rows have been written and INSTEAD of
-// the barrier that precedes flush_span: every thread makes its shared-memory writes visible to
-// the asynchronous proxy, the CTA synchronises, thread 0 issues the copy and waits until the
-// unit has read the staging buffer (the global writes complete on their own).
-__device__ __forceinline__ void flush_span_bulk(const uint8_t *stage, uint32_t len, int8_t *out,
-                                                uint64_t byte0)
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x == 0 && len != 0) {
-        const uint32_t src = (uint32_t)__cvta_generic_to_shared(stage);
-        const uint64_t dst = reinterpret_cast<uint64_t>(out) + byte0;
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                     :: "l"(dst), "r"(src), "r"(len) : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-    }
-}
-
+// ---------------------------------------------------------------- spans of rows, lists of p
 // Copies in[byte0, byte0+len) to stage[shift, shift+len), (byte0 & 15) == shift, `in` 16-byte
-// aligned: the mirror image of flush_span.
+// aligned: 16-byte loads but for the ragged ends.
 __device__ __forceinline__ void load_span(uint8_t *stage, uint32_t shift, uint32_t len,
                                           const int8_t *in, uint64_t byte0)
 {
@@ -187,19 +89,8 @@ __device__ __forceinline__ void load_span(uint8_t *stage, uint32_t shift, uint32
     }
 }
 
-// Largest j with off[j] <= g, searched in [lo, hi].
-__device__ __forceinline__ uint32_t find_segment(const uint64_t *off, uint32_t lo, uint32_t hi,
-                                                 uint64_t g)
-{
-    while (lo < hi) {
-        uint32_t mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= g) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// The same search by a whole warp: 32 probes per step instead of one, so a table of a few
-// thousand offsets takes three dependent loads instead of twelve.  All 32 lanes must call.
+// Largest j with off[j] <= g, by a whole warp: 32 probes per step, so a table of a few thousand offsets takes
+// three dependent loads.  All 32 lanes must call.
 __device__ __forceinline__ uint32_t find_segment_warp(const uint64_t *off, uint32_t num, uint64_t g)
 {
     const uint32_t lane = threadIdx.x & 31u;
@@ -213,95 +104,6 @@ __device__ __forceinline__ uint32_t find_segment_warp(const uint64_t *off, uint3
         hi = lo + step < hi ? lo + step : hi;
     }
     return lo;
-}
-
-// Resolves the rank this thread works on.  Single p: consecutive ranks from r_begin.
-// Batch: flattened index g over all (p_j, r); the CTA looks up the first and last p it
-// touches once, keeps the first few table rows in shared memory, and each thread finds
-// its own p between the two.
-template <bool kBatch>
-__device__ __forceinline__ RankCtx resolve_rank(TileShared &sh, const PTable &tab,
-                                                uint64_t r_begin, uint64_t r_end,
-                                                const BatchArgs &ba)
-{
-    RankCtx c;
-    const uint64_t g0 = (uint64_t)blockIdx.x * kTile;
-    if (!kBatch) {
-        if (threadIdx.x < kRow) {
-            sh.skips[0][threadIdx.x] = tab.s[threadIdx.x];
-            sh.full[0][threadIdx.x] = tab.full[threadIdx.x];
-        }
-        const uint64_t count = r_end - r_begin;
-        const uint64_t g1 = g0 + kTile < count ? g0 + kTile : count;
-        if (threadIdx.x == 0) {
-            sh.span_begin = g0 * (uint64_t)tab.q;
-            sh.span_end = g1 * (uint64_t)tab.q;
-        }
-        __syncthreads();
-        const uint64_t g = g0 + threadIdx.x;
-        c.s = sh.skips[0];
-        c.full = sh.full[0];
-        c.p = tab.p;
-        c.q = tab.q;
-        c.pj = 0;
-        c.rank0 = 0;
-        c.valid = g < count;
-        c.r = (uint32_t)(r_begin + g);
-        c.entry = g * (uint64_t)tab.q;
-        return c;
-    }
-    const uint64_t g1 = g0 + kTile < ba.total_ranks ? g0 + kTile : ba.total_ranks;
-    if (threadIdx.x < 32) {
-        const uint32_t jf = find_segment_warp(ba.rank_off, ba.num_p, g0);
-        const uint32_t jl = ba.rank_off[jf + 1] >= g1 ? jf : find_segment_warp(ba.rank_off, ba.num_p, g1 - 1);
-        if (threadIdx.x == 0) {
-            sh.j_first = jf;
-            sh.j_last = jl;
-            sh.p_first = ba.p_list[jf];
-            sh.rank0_first = ba.rank_off[jf];
-            sh.entry0_first = ba.entry_off[jf];
-            const int qf = ceil_log2_fast(sh.p_first);
-            const int ql = ceil_log2_fast(ba.p_list[jl]);
-            sh.span_begin = sh.entry0_first + (g0 - sh.rank0_first) * (uint64_t)qf;
-            sh.span_end = ba.entry_off[jl] + (g1 - ba.rank_off[jl]) * (uint64_t)ql;
-        }
-    }
-    __syncthreads();
-    const uint32_t jf = sh.j_first, jl = sh.j_last;
-    {
-        const uint32_t row = threadIdx.x / (2 * kRow), col = threadIdx.x % (2 * kRow);
-        if (row < kCachedRows && jf + row <= jl) {
-            if (col < kRow)
-                sh.skips[row][col] = ba.skips_tab[(size_t)(jf + row) * kRow + col];
-            else
-                sh.full[row][col - kRow] = ba.full_tab[(size_t)(jf + row) * kRow + col - kRow];
-        }
-    }
-    __syncthreads();
-    const uint64_t g = g0 + threadIdx.x;
-    c.valid = g < g1;
-    if (jf == jl) {                                  // the whole CTA inside one p: no per-thread lookups
-        c.s = sh.skips[0];
-        c.full = sh.full[0];
-        c.pj = jf;
-        c.p = sh.p_first;
-        c.q = ceil_log2_fast(c.p);
-        c.rank0 = sh.rank0_first;
-        c.r = (uint32_t)(g - c.rank0);
-        c.entry = sh.entry0_first + (uint64_t)c.r * (uint64_t)c.q;
-        return c;
-    }
-    const uint32_t j = c.valid ? find_segment(ba.rank_off, jf, jl, g) : jf;
-    const bool cached = j - jf < (uint32_t)kCachedRows;
-    c.s = cached ? sh.skips[j - jf] : ba.skips_tab + (size_t)j * kRow;
-    c.full = cached ? sh.full[j - jf] : ba.full_tab + (size_t)j * kRow;
-    c.pj = j;
-    c.p = ba.p_list[j];
-    c.q = ceil_log2_fast(c.p);
-    c.rank0 = ba.rank_off[j];
-    c.r = (uint32_t)(g - c.rank0);
-    c.entry = ba.entry_off[j] + (uint64_t)c.r * (uint64_t)c.q;
-    return c;
 }
 
 // ---------------------------------------------------------------- dependent launches
@@ -343,6 +145,21 @@ inline void launch_dependent(bool dependent, void (*kernel)(Params...), unsigned
     cfg.attrs = attr;
     cfg.numAttrs = dependent ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+// Opts a kernel in to large dynamic shared memory (what a little static use leaves of 227 KB), once per device.
+template <auto kKernel>
+bool allow_shared()
+{
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return true;
+    if (cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess)
+        return false;
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return true;
 }
 
 inline bool aligned16(const void *ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }

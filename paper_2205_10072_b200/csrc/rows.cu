@@ -11,7 +11,6 @@
 // dependent of whatever runs before it on the stream and waits for that before its first store only, the
 // table holds what the CTA's segments need where these are few, and a CTA has no more warps than items: 32 ranks 8.2 ->
 // 4.4 us, all ranks of 1152: 8.6 -> 4.6, of 100 003: 10.2 -> 7.6, of about 2^20: 22.7 -> 18.4 us, back to back.
-#include <atomic>
 #include <type_traits>
 
 #include "rows.cuh"
@@ -57,6 +56,7 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
             }
         }
     }
+    __syncthreads();
     build_row_table(t, rc.q, rc.odd);
     grid_dependency_wait();                                      // nothing before this touches the outputs
     uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
@@ -80,6 +80,7 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     const RowTable t(sm, at.base);
     if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
     if (threadIdx.x == 0) *t.wanted = (2u << (rc.q - kLow)) - 1u;
+    __syncthreads();
     build_row_table(t, rc.q, rc.odd);
     if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
     grid_dependency_wait();
@@ -98,21 +99,6 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     };
     if (recv != nullptr) all(std::false_type(), recv);
     if (send != nullptr) all(std::true_type(), send);
-}
-
-// Opts a kernel in to large dynamic shared memory, once per device.
-template <auto kKernel>
-bool allow_shared()
-{
-    static std::atomic<uint64_t> done{0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
-    if (done.load(std::memory_order_relaxed) & bit) return true;
-    if (cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
-        return false;
-    done.fetch_or(bit, std::memory_order_relaxed);
-    return true;
 }
 
 bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send,

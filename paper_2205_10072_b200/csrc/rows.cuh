@@ -186,10 +186,9 @@ __device__ __forceinline__ void build_whole_table(const RowTable &t, int q, uint
 }
 
 // Fills the table of a p, for the K whose bits in *t.wanted are set (q > 7); all threads of the CTA call (at least
-// 128).  t.s holds the skips and *t.wanted is set, by any thread.  Begins and ends with a barrier.
+// 128), after a barrier behind the writes of t.s (the skips, then zeros) and *t.wanted.  Ends with a barrier.
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {
-    __syncthreads();
     const int L = low_levels(q);
     const uint32_t lows = t.s[L];
     if (threadIdx.x < kLowRanks) {

@@ -98,3 +98,33 @@ def test_many_ranks_rooted(bcs):
     rows = torch.from_numpy(at).cuda()
     for out, expect in ((recv, want[0]), (send, want[1])):
         assert np.array_equal(out.view(p, q)[rows].cpu().numpy(), expect)
+
+
+def _batch(bcs, plist, send=True):
+    plan = bcs.bcs_batch_plan(plist)
+    raw_r, recv = _buffer(plan.total_entries)
+    raw_s, out_s = _buffer(plan.total_entries)
+    bcs.bcs_build_batch(plan.to("cuda"), recv, out_s if send else None)
+    torch.cuda.synchronize()
+    assert bool((raw_r[:32] == 99).all()) and bool((raw_r[32 + plan.total_entries:] == 99).all())
+    assert bool((raw_s[:32] == 99).all()) and bool((raw_s[32 + plan.total_entries:] == 99).all())
+    assert send or bool((raw_s == 99).all())
+    for p, lo, hi in zip(plist, plan.entry_off[:-1].tolist(), plan.entry_off[1:].tolist()):
+        if p == 1:
+            continue
+        one_r = torch.empty(hi - lo, dtype=torch.int8, device="cuda")
+        one_s = torch.empty(hi - lo, dtype=torch.int8, device="cuda")
+        bcs.bcs_build(p, 0, p, one_r, one_s)                 # (compared with the oracle above)
+        assert torch.equal(recv[lo:hi], one_r), p
+        assert not send or torch.equal(out_s[lo:hi], one_s), p
+
+
+# the sizes at which a batch changes kernels and row forms (1024, 2^15, 2^21), tables that start at any byte, shares that
+# end inside a p, lists of one p
+@pytest.mark.parametrize("plist", [[1024, 1025, 3, 32768, 1, 32769, 65537, 1023, 40001, 2, 65535],
+                                   [(1 << 21) + 1, 5, (1 << 21), 1, (1 << 21) - 1, 77, (1 << 22) + 5],
+                                   [33333], [1], [2, 1], [(1 << 20) + 1] * 3, [1025] * 40, [127, 128, 129, 130] * 30])
+@pytest.mark.parametrize("send", [True, False])
+def test_batches(bcs, plist, send):
+    if bcs.bcs_batch_plan(plist).total_entries:
+        _batch(bcs, plist, send)
