@@ -161,6 +161,7 @@ allgather_kernel(PTable tab, uint32_t n, uint32_t r, uint32_t rounds_per_cta,
     __shared__ __align__(16) int8_t recv_k[kUnpack ? BCS_MAX_Q + 1 : 1][kAgCols];
     __shared__ __align__(16) uint8_t send_rows[kPack ? kAgRowBytes : 16];
     __shared__ __align__(16) uint8_t recv_rows[kUnpack ? kAgRowBytes : 16];
+    grid_launch_dependents();
     const uint32_t p = tab.p;
     const int q = tab.q;
     const uint32_t rounds = n - 1u + (uint32_t)q;
@@ -170,6 +171,7 @@ allgather_kernel(PTable tab, uint32_t n, uint32_t r, uint32_t rounds_per_cta,
     const uint32_t cols = avail < (uint32_t)kAgCols ? avail : (uint32_t)kAgCols;   // buffers staged
     uint32_t hi = r + p - j0;                                      // (r - j0) mod p: virtual rank of column 0
     if (hi >= p) hi -= p;
+    grid_dependency_wait();                                        // (the rows may be the work of the kernel before this one)
     StagedRows sr = {};
     if (kPack) sr = load_rows_descending(send, p, q, hi, cols, send_rows);
     if (kUnpack) sr = load_rows_descending(recv, p, q, hi, cols, recv_rows);   // same offsets for both tables
@@ -260,11 +262,14 @@ bcs_status bcs_allgather_tables(uint32_t p, uint32_t n, uint32_t r, const int8_t
     dim3 grid(col_blocks, chunks);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     if (pack_out && unpack_out)
-        allgather_kernel<true, true><<<grid, kAgThreads, 0, stream>>>(tab, n, r, per_cta, recv, send, pack_out, unpack_out);
+        launch_dependent(true, allgather_kernel<true, true>, grid, kAgThreads, 0, stream, tab, n, r, per_cta, recv, send,
+                         pack_out, unpack_out);
     else if (pack_out)
-        allgather_kernel<true, false><<<grid, kAgThreads, 0, stream>>>(tab, n, r, per_cta, recv, send, pack_out, nullptr);
+        launch_dependent(true, allgather_kernel<true, false>, grid, kAgThreads, 0, stream, tab, n, r, per_cta, recv, send,
+                         pack_out, unpack_out);
     else
-        allgather_kernel<false, true><<<grid, kAgThreads, 0, stream>>>(tab, n, r, per_cta, recv, send, nullptr, unpack_out);
+        launch_dependent(true, allgather_kernel<false, true>, grid, kAgThreads, 0, stream, tab, n, r, per_cta, recv, send,
+                         pack_out, unpack_out);
     return launch_status();
 }
 

@@ -16,11 +16,9 @@ constexpr uint32_t kFusedMaxP = 1024;         // batch: a p up to here is built 
 constexpr int kRow = BCS_SKIPS_STRIDE;        // words per table row
 
 // Per-p constants (kernel parameter of the single-p kernels).
-//   s[k]    = skips[k] of Algorithm 1, k = 0..q (q <= 31)
-//   full[d] = skip code of rank skips[d]-1, d = 0..q (see skip_code below)
+//   s[k] = skips[k] of Algorithm 1, k = 0..q (q <= 31), then 0
 struct PTable {
     uint32_t s[kRow];
-    uint32_t full[kRow];
     uint32_t p;
     int q;
 };
@@ -131,11 +129,11 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
 
 // Launch with programmatic stream serialisation (see above); `dependent` false: ordinary launch.
 template <class... Params, class... Args>
-inline void launch_dependent(bool dependent, void (*kernel)(Params...), unsigned grid, unsigned block, size_t shared,
+inline void launch_dependent(bool dependent, void (*kernel)(Params...), dim3 grid, unsigned block, size_t shared,
                              cudaStream_t stream, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = shared;
     cfg.stream = stream;

@@ -8,7 +8,9 @@ namespace {
 
 // ---------------------------------------------------------------- Algorithm 6: round tables
 constexpr int kExpandThreads = 256;
-constexpr uint32_t kExpandRecords = 8192;      // records (128 KB of output) that a CTA aims for
+constexpr uint32_t kExpandRecords = 8192;      // records (128 KB of output) that a CTA aims for where there are many,
+constexpr uint32_t kExpandFewest = 512;        // and where they would not give every SM four CTAs (p = 1152, n = 64: 10 CTAs
+constexpr uint32_t kExpandCtas = 148 * 4;      // of 8192 records took 10.2 us)
 constexpr uint32_t kExpandSharedBytes = 48 * 1024;
 
 // A CTA takes `ranks_per_cta` consecutive ranks.  Their records are one contiguous stretch of
@@ -30,12 +32,14 @@ expand_kernel(PTable tab, uint32_t n, uint64_t r_begin, uint64_t r_end, uint32_t
     // per rank of the CTA and per round k of a phase: {send entry - x, recv entry - x, to, from}.
     // Algorithm 6 adds q to an entry after each use and starts entries k < x at +q because
     // their first use is in the second phase; both are covered by adding q * floor(i / q).
+    grid_launch_dependents();
     extern __shared__ int4 base[];             // [ranks_per_cta][q], then (kBuildRows) the skips
     uint32_t *skips_sh = reinterpret_cast<uint32_t *>(base + (size_t)ranks_per_cta * tab.q);
     if (kBuildRows) {
         if (threadIdx.x < kRow) skips_sh[threadIdx.x] = tab.s[threadIdx.x];
         __syncthreads();
     }
+    grid_dependency_wait();                    // (the rows may be the work of the kernel before this one)
     const uint32_t q = (uint32_t)tab.q;
     const uint32_t p = tab.p;
     const uint32_t rounds = n - 1u + q;
@@ -153,20 +157,23 @@ bcs_status bcs_expand(uint32_t p, uint32_t n, uint64_t r_begin, uint64_t r_end,
     if (!aligned16(table_out)) return BCS_ERR_ALIGN;
     // ranks per CTA: about kExpandRecords records, as far as the per-rank constants fit in shared memory
     const uint32_t rounds = n - 1u + (uint32_t)tab.q;
-    uint32_t per_cta = (kExpandRecords + rounds - 1) / rounds;
+    const uint64_t share = count * rounds / kExpandCtas;
+    const uint32_t aim = share > kExpandRecords ? kExpandRecords : (share < kExpandFewest ? kExpandFewest : (uint32_t)share);
+    uint32_t per_cta = (aim + rounds - 1) / rounds;
     const uint32_t extra = recv == nullptr ? kRow * 4u : 0u;     // room for the skips when the rows are built here
     const uint32_t fit = (kExpandSharedBytes - extra) / (16u * (uint32_t)tab.q);
     if (per_cta > fit) per_cta = fit;
     const uint64_t blocks = (count + per_cta - 1) / per_cta;
     if (blocks > 0x7fffffffull) return BCS_ERR_UNSUPPORTED;
+    const size_t shared = (size_t)per_cta * tab.q * 16u + extra;
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    int4 *out = reinterpret_cast<int4 *>(table_out);
     if (recv == nullptr)                               // no tables: the kernel builds the rows it needs
-        expand_kernel<true><<<(unsigned)blocks, kExpandThreads, (size_t)per_cta * tab.q * 16u + kRow * 4u,
-                              static_cast<cudaStream_t>(cuda_stream)>>>(
-            tab, n, r_begin, r_end, per_cta, nullptr, nullptr, reinterpret_cast<int4 *>(table_out));
+        launch_dependent(true, expand_kernel<true>, (unsigned)blocks, kExpandThreads, shared, stream, tab, n, r_begin, r_end,
+                         per_cta, recv, send, out);
     else
-        expand_kernel<false><<<(unsigned)blocks, kExpandThreads, (size_t)per_cta * tab.q * 16u,
-                               static_cast<cudaStream_t>(cuda_stream)>>>(
-            tab, n, r_begin, r_end, per_cta, recv, send, reinterpret_cast<int4 *>(table_out));
+        launch_dependent(true, expand_kernel<false>, (unsigned)blocks, kExpandThreads, shared, stream, tab, n, r_begin, r_end,
+                         per_cta, recv, send, out);
     return launch_status();
 }
 

@@ -49,7 +49,7 @@ bcs_status bcs_batch_plan(const uint32_t *p_list_host, uint32_t num_p, uint64_t 
         copy_off_host[j] = copy;
         for (int k = 0; k < kRow; ++k) {
             skips_tab_host[(size_t)j * kRow + k] = tab.s[k];
-            full_tab_host[(size_t)j * kRow + k] = tab.full[k];
+            full_tab_host[(size_t)j * kRow + k] = k <= tab.q ? skip_code(tab.s, tab.q, tab.s[k] - 1u) : 0u;
         }
         ranks += tab.p;
         entries += (uint64_t)tab.p * (uint64_t)tab.q;

@@ -9,13 +9,12 @@ bcs_status make_table(uint32_t p, PTable *tab)
     if (p == 0) return BCS_ERR_RANGE;
     if (p > 0x7fffffffu) return BCS_ERR_UNSUPPORTED;
     const int q = ceil_log2_u32(p);
-    for (int k = 0; k < kRow; ++k) tab->s[k] = tab->full[k] = 0;
+    for (int k = 0; k < kRow; ++k) tab->s[k] = 0;
     uint32_t v = p;
     for (int k = q; k >= 0; --k) {   // Algorithm 1: successive ceil-halving
         tab->s[k] = v;
         v = (v + 1u) / 2u;
     }
-    for (int d = 0; d <= q; ++d) tab->full[d] = skip_code(tab->s, q, tab->s[d] - 1u);
     tab->p = p;
     tab->q = q;
     return BCS_OK;
