@@ -1,4 +1,8 @@
-"""ctypes binding of libbcs.so: argument marshalling only (include/bcs.h has the contracts)."""
+"""Binding of libbcs.so: argument marshalling only (include/bcs.h has the contracts).
+
+The calls that enqueue work go through an extension module linked to the library (csrc/calls.c) where it has been
+built, the others through ctypes.
+"""
 from __future__ import annotations
 
 import ctypes
@@ -102,14 +106,40 @@ def _ptr(t) -> int | None:
 
 # Handle of the current stream without building a torch.cuda.Stream (3.2 us of a call's 8.8 us).
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream) -> int | None:
     if stream is None:
-        if _raw_stream is not None:
-            return _raw_stream(torch.cuda.current_device()) or None
+        if _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device()) or None
         stream = torch.cuda.current_stream()
     return stream.cuda_stream or None
+
+
+class _Calls:
+    """The calls that enqueue work, by name without "bcs_"; the first use of one loads the library."""
+
+    def __getattr__(self, name):
+        library = lib()
+        call = getattr(_extension(), name, None) or getattr(library, "bcs_" + name)
+        setattr(self, name, call)
+        return call
+
+
+def _extension():
+    """The extension module linked to the library that lib() has loaded, or None."""
+    if build_ext.LIB_PATH != os.path.join(os.path.dirname(build_ext.CALLS_PATH), "libbcs.so") or \
+            not os.path.exists(build_ext.CALLS_PATH):
+        return None
+    try:
+        from . import _calls
+    except ImportError:
+        return None
+    return _calls
+
+
+_call = _Calls()
 
 
 def bcs_status_str(status: int) -> str:
@@ -127,7 +157,7 @@ def bcs_skips(p: int) -> list[int]:
 
 
 def _nbytes(t) -> int:
-    return 0 if t is None else t.numel() * t.element_size()
+    return 0 if t is None else t.nbytes
 
 
 def bcs_build_workspace_bytes(p: int, r_begin: int, r_end: int) -> int:
@@ -138,7 +168,7 @@ def bcs_build(p: int, r_begin: int, r_end: int, recv_out, send_out, workspace=No
               stream=None) -> None:
     """recv_out / send_out: CUDA int8 tensors of (r_end-r_begin)*q elements, or None;
     workspace: CUDA tensor of bcs_build_workspace_bytes(...) bytes (fast path) or None."""
-    _check(lib().bcs_build(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out), _ptr(workspace),
+    _check(_call.build(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out), _ptr(workspace),
                            _nbytes(workspace), _stream(stream)), "bcs_build")
 
 
@@ -150,7 +180,7 @@ def bcs_build_rooted(p: int, root: int, r_begin: int, r_end: int, recv_out, send
                      workspace=None, stream=None) -> None:
     """As bcs_build for a broadcast rooted at `root`: row r is the rank-0-rooted row of virtual
     rank (r - root) mod p."""
-    _check(lib().bcs_build_rooted(p, root, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
+    _check(_call.build_rooted(p, root, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
                                   _ptr(workspace), _nbytes(workspace), _stream(stream)),
            "bcs_build_rooted")
 
@@ -162,26 +192,26 @@ def bcs_prepare_workspace_bytes(p: int) -> int:
 def bcs_prepare(p: int, workspace, stream=None) -> None:
     """Runs the construction once for all ranks of p into `workspace` (CUDA tensor of
     bcs_prepare_workspace_bytes(p) bytes) for later bcs_build_prepared calls."""
-    _check(lib().bcs_prepare(p, _ptr(workspace), _nbytes(workspace), _stream(stream)), "bcs_prepare")
+    _check(_call.prepare(p, _ptr(workspace), _nbytes(workspace), _stream(stream)), "bcs_prepare")
 
 
 def bcs_prepare_codes(p: int, workspace, stream=None) -> None:
     """First half of bcs_prepare: the skip codes of all ranks of p into `workspace`."""
-    _check(lib().bcs_prepare_codes(p, _ptr(workspace), _nbytes(workspace), _stream(stream)),
+    _check(_call.prepare_codes(p, _ptr(workspace), _nbytes(workspace), _stream(stream)),
            "bcs_prepare_codes")
 
 
 def bcs_prepare_rows(p: int, r_begin: int, r_end: int, recv_out, workspace, stream=None) -> None:
     """Second half, for one range (r_begin a multiple of 16): its entries into the round-major copy
     in `workspace` and, if recv_out is not None, its rank-major receive rows into recv_out."""
-    _check(lib().bcs_prepare_rows(p, r_begin, r_end, _ptr(recv_out), _ptr(workspace),
+    _check(_call.prepare_rows(p, r_begin, r_end, _ptr(recv_out), _ptr(workspace),
                                   _nbytes(workspace), _stream(stream)), "bcs_prepare_rows")
 
 
 def bcs_build_prepared(p: int, r_begin: int, r_end: int, recv_out, send_out, workspace,
                        stream=None) -> None:
     """Rank-major receive / send rows of a range from a workspace filled by bcs_prepare."""
-    _check(lib().bcs_build_prepared(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
+    _check(_call.build_prepared(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
                                     _ptr(workspace), _nbytes(workspace), _stream(stream)),
            "bcs_build_prepared")
 
@@ -189,7 +219,7 @@ def bcs_build_prepared(p: int, r_begin: int, r_end: int, recv_out, send_out, wor
 def bcs_build_static(p: int, r_begin: int, r_end: int, recv_out, send_out, stream=None) -> None:
     """bcs_build with the library's built-in 8 MiB scratch: for callers that cannot allocate or
     pass a workspace.  Raises BcsError (BCS_ERR_UNSUPPORTED) when the range needs more."""
-    _check(lib().bcs_build_static(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
+    _check(_call.build_static(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
                                   _stream(stream)), "bcs_build_static")
 
 
@@ -272,7 +302,7 @@ def bcs_build_batch_workspace_bytes(total_ranks: int, total_copy: int) -> int:
 def bcs_build_batch(plan_dev: BatchPlan, recv_out, send_out, workspace=None, stream=None) -> None:
     """plan_dev: a BatchPlan whose tensors live on the CUDA device; workspace: CUDA tensor of
     plan.workspace_bytes() bytes (fast construction) or None."""
-    _check(lib().bcs_build_batch(plan_dev.p_list.data_ptr(), plan_dev.rank_off.data_ptr(),
+    _check(_call.build_batch(plan_dev.p_list.data_ptr(), plan_dev.rank_off.data_ptr(),
                                  plan_dev.entry_off.data_ptr(), plan_dev.tile_off.data_ptr(),
                                  plan_dev.copy_off.data_ptr(), plan_dev.skips_tab.data_ptr(),
                                  plan_dev.full_tab.data_ptr(), plan_dev.num_p, plan_dev.total_ranks,
@@ -284,7 +314,7 @@ def bcs_build_batch(plan_dev: BatchPlan, recv_out, send_out, workspace=None, str
 def bcs_expand(p: int, n: int, r_begin: int, r_end: int, recv, send, table_out, stream=None) -> None:
     """recv/send: CUDA int8 rows of ranks r_begin..r_end-1; table_out: CUDA int32
     [(r_end-r_begin), n-1+q, 4]."""
-    _check(lib().bcs_expand(p, n, r_begin, r_end, _ptr(recv), _ptr(send), _ptr(table_out),
+    _check(_call.expand(p, n, r_begin, r_end, _ptr(recv), _ptr(send), _ptr(table_out),
                             _stream(stream)), "bcs_expand")
 
 
@@ -307,7 +337,7 @@ def bcs_allgather_tables(p: int, n: int, r: int, recv, send, pack_out, unpack_ou
                          stream=None) -> None:
     """recv/send: full [p][q] CUDA int8 tables; pack_out/unpack_out: CUDA int32 [n-1+q, p]
     (or None): blocks of buffer[j] processor r packs / unpacks per round (Algorithm 9)."""
-    _check(lib().bcs_allgather_tables(p, n, r, _ptr(recv), _ptr(send), _ptr(pack_out),
+    _check(_call.allgather_tables(p, n, r, _ptr(recv), _ptr(send), _ptr(pack_out),
                                       _ptr(unpack_out), _stream(stream)), "bcs_allgather_tables")
 
 

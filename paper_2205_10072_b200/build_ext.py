@@ -4,6 +4,7 @@ from __future__ import annotations
 import glob
 import os
 import subprocess
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
@@ -11,6 +12,9 @@ LIB_PATH = os.path.join(_PKG, "libbcs.so")
 SOURCES = sorted(glob.glob(os.path.join(_PKG, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(_ROOT, "include", "*.h")) +
                  glob.glob(os.path.join(_PKG, "csrc", "*.cuh")))
+# The calls of the library for Python (csrc/calls.c), linked to it.
+CALLS_PATH = os.path.join(_PKG, "_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+CALLS_SOURCE = os.path.join(_PKG, "csrc", "calls.c")
 # The benchmark's integer-rate probe is a library of its own: it is not part of the product and
 # only bench.py loads it.
 PROBE_LIB_PATH = os.path.join(_PKG, "libbcs_probe.so")
@@ -39,7 +43,7 @@ def stale() -> bool:
 def _nvcc(lib: str, sources: list, verbose: bool, extra: list = ()) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = lib + ".%d.tmp" % os.getpid()
-    cmd = [nvcc] + NVCC_FLAGS + list(extra) + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources
+    cmd = [nvcc] + NVCC_FLAGS + ["-Xlinker", "-soname=" + os.path.basename(lib)] + list(extra) + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources
     subprocess.check_call(cmd)
     os.replace(tmp, lib)
 
@@ -48,7 +52,22 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Runs nvcc (cross-compiles without a GPU).  Returns the path of the shared library."""
     if force or stale():
         _nvcc(LIB_PATH, SOURCES, verbose)
+    build_calls(force)
     return LIB_PATH
+
+
+def build_calls(force: bool = False) -> str:
+    """The extension module with the library's calls (without Python's headers: none, ctypes serves)."""
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        return ""
+    if force or _stale(CALLS_PATH, [CALLS_SOURCE, LIB_PATH] + HEADERS):
+        tmp = CALLS_PATH + ".%d.tmp" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC",
+                               "-I", include, "-I", os.path.join(_ROOT, "include"),
+                               "-o", tmp, CALLS_SOURCE, LIB_PATH, "-Wl,-rpath,$ORIGIN"])
+        os.replace(tmp, CALLS_PATH)
+    return CALLS_PATH
 
 
 def build_probe(force: bool = False, verbose: bool = False) -> str:
