@@ -21,8 +21,6 @@ namespace {
 
 constexpr unsigned kSms = 148;
 constexpr unsigned kRowThreads = 1024;
-// 640 threads: at the speed of the memory (2^27 ranks) the write streams of 1024 cost 20 % and more.
-constexpr unsigned kWideThreads = 640;
 
 // One CTA per SM at most; every warp takes items of `item` (32, 64 or 128) consecutive ranks, in turn over the CTAs.
 // first: rank of the first row (< p); the count <= p ranks go on at 0 behind p - 1.
@@ -69,10 +67,13 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     stage_free();
 }
 
-// The same for large tables, q >= 16 (wide.cuh), all receive rows before the send rows; `item` is a multiple of 16.
-__global__ void __launch_bounds__(kWideThreads, 1)
-wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, int8_t *recv,
-            int8_t *send)
+// The same for larger tables, q >= 16 (wide.cuh), one CTA per SM; `item` is a multiple of 16.  halves: half of the warps
+// write the receive rows and half the send rows; otherwise all warps the ones before the others.
+// (No more than 640 threads: at the speed of the memory the write streams of 1024 cost 20 % and more.)
+template <unsigned kThreads, int kCtas>
+__global__ void __launch_bounds__(kThreads, kCtas)
+wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, bool halves,
+            int8_t *recv, int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
     grid_launch_dependents();
@@ -84,33 +85,39 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     build_row_table(t, rc.q, rc.odd);
     if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
     grid_dependency_wait();
-    const uint32_t n_warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
+    const uint32_t warp = threadIdx.x >> 5;
+    uint32_t n_warps = blockDim.x >> 5, index = warp;
     auto all = [&](auto is_send, int8_t *out) {
         WideLane mine;
         mine.init(rc.q, 0u);
-        for (uint64_t b = ((uint64_t)blockIdx.x * n_warps + warp) * item; b < count; b += stride) {
+        const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
+        for (uint64_t b = ((uint64_t)blockIdx.x * n_warps + index) * item; b < count; b += stride) {
             const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
             uint32_t x0 = first + (uint32_t)b;
             if (x0 >= rc.p) x0 -= rc.p;
             wide_rows<decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
-                                                      mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
+                                                mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
         }
     };
-    if (recv != nullptr) all(std::false_type(), recv);
-    if (send != nullptr) all(std::true_type(), send);
+    bool receives = recv != nullptr, sends = send != nullptr;
+    if (halves && receives && sends) {
+        n_warps /= 2;
+        sends = warp >= n_warps;
+        receives = !sends;
+        if (sends) index -= n_warps;
+    }
+    if (receives) all(std::false_type(), recv);
+    if (sends) all(std::true_type(), send);
 }
 
-bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send,
+template <unsigned kThreads, int kCtas>
+bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, uint32_t item, bool halves, int8_t *recv, int8_t *send,
                        cudaStream_t stream)
 {
-    if (!allow_shared<wide_kernel>()) return BCS_ERR_CUDA;
-    // An item's start costs as much as some 50 ranks: 12.3 million ranks 61 us a table with items of 768, 67 with 384;
-    // but from 2^25 ranks on the memory bounds it, and items close together are written faster (146 against 151 us).
-    const uint32_t item = count >= (1u << 25) ? 384u : 768u;
+    if (!allow_shared<wide_kernel<kThreads, kCtas>>()) return BCS_ERR_CUDA;
     const unsigned items = (count + item - 1) / item;
-    launch_dependent(true, wide_kernel, items < kSms ? items : kSms, kWideThreads, WideLayout(rc.q).bytes,
-                     stream, rc, first, count, item, recv, send);
+    launch_dependent(true, wide_kernel<kThreads, kCtas>, items < kSms ? items : kSms, kThreads,
+                     WideLayout(rc.q).bytes, stream, rc, first, count, item, halves, recv, send);
     return launch_status();
 }
 
@@ -151,10 +158,24 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     }
     for (int k = 1; k <= rc.q; ++k) rc.odd |= (2u * rc.s[k - 1] - rc.s[k]) << k;
     rc.inv = (uint32_t)((1ull << (rc.q - low_levels(rc.q) + 32)) / p);
-    // From 2^23 ranks on the wide kernel, whose tables take longer to build: 4 million ranks 51.5 us here, 59.5
-    // there; 12.3 million 152 against 120, 2^25 of q = 28 369 against 290, 2^27 of q = 30 1504 against 1230 us.
-    if (count >= (1u << 23)) return launch_wide(rc, (uint32_t)first, (uint32_t)count, recv, send, stream);
-    return launch<1>(rc, (uint32_t)first, (uint32_t)count, recv, send, stream);
+    const uint32_t ranks = (uint32_t)count, x0 = (uint32_t)first;
+    // The wide kernel from 96 Ki ranks on (its tables take longer to build: 65 000 ranks 5.8 against 4.1 us here).  Up to
+    // 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
+    // are built beside it (700 001 ranks 12.3 us, 13.7 with 640 threads, 14.9 per rank; 1.3 million 18.2, 18.0, 23.4; 2.1
+    // million 21.4, 20.6, 29.3).  Beyond, all receive rows before the send rows, item by item: an item's start costs as
+    // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
+    // faster (12.3 million ranks 61 us a table with items of 768, 67 with 384; 2^25: 151 and 146 us).
+    if (rc.q >= kWideMinQ && count >= 98304) {
+        const bool halves = count < (1u << 23);
+        auto run = [&](uint32_t warps) {
+            if (recv != nullptr && send != nullptr) warps /= 2;
+            return (ranks + kSms * warps * kStep - 1u) / (kSms * warps * kStep) * kStep;
+        };
+        if (count <= (1u << 20)) return launch_wide<384, 2>(rc, x0, ranks, run(12), halves, recv, send, stream);
+        if (halves) return launch_wide<640, 1>(rc, x0, ranks, run(20), halves, recv, send, stream);
+        return launch_wide<640, 1>(rc, x0, ranks, count >= (1u << 25) ? 384u : 768u, halves, recv, send, stream);
+    }
+    return launch<1>(rc, x0, ranks, recv, send, stream);
 }
 
 }  // namespace bcs

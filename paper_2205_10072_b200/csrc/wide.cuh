@@ -257,21 +257,44 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
     auto put = [&](int b, uint32_t value) {
         if (b >= (int)skip && b < (int)len) out[b] = (uint8_t)value;
     };
-    // Exceptions of this lane's segment g, whose first rank is `begin` and that of the next one `end`: a few bytes each, so all
-    // the segments of an item at once, one by lane (the whole warp on one segment after another took a fifth
-    // more instructions in all).
-    auto exceptions = [&](uint32_t g, int begin, int end) {
-        const int row0 = (int)shift + begin * q;
+    // Receive exceptions of the segment with lowest bit K whose first row starts at byte row0.  With t(0) > t(1) > ... the levels
+    // t = 8 .. K of which e_t is set, rank `low` receives block k + 1 in the rounds k = L .. t(low) - 2, then the missing one;
+    // the rank behind the last such level has the missing one in round L.
+    auto receive_ahead = [&](int K, int row0) {
+        uint32_t levels = odd & ((2u << K) - 1u) & ~((2u << kLow) - 1u);
+        for (int low = 0;; ++low) {
+            const int top = top_bit(levels);                     // -1 behind the last one
+            const int row = row0 + low * q;
+            int k = kLow;
+            for (; k <= top - 2; ++k) put(row + k, (uint32_t)(k + 1 - q));
+            put(row + k, (uint32_t)((int)t.miss[(K - kLow) * kMissRanks + low] - q));
+            if (levels == 0u) break;
+            levels &= ~(1u << top);
+        }
+    };
+    // Exceptions of the lanes' segments: g, its first row's byte, that of the next one's first row, whether it counts.  A few
+    // bytes each, so all the segments of an item at once, one by lane (the whole warp on one segment after another took a
+    // fifth more instructions in all); but those with hundreds, near multiples of large skips, by the warp.
+    constexpr int kAlone = kLow + 4;
+    auto exceptions = [&](uint32_t g, int row0, int row1, bool counts) {
         if (!kSend) {
-            if (g & 1u) return;
             const int K = g ? __ffs(g) - 1 + kLow : q;           // its first ranks receive ahead
-            const int last = (int)count_odd(odd, kLow, K);
-            for (int low = 0; low <= last; ++low) {
-                int k = kLow;
-                for (; low < (int)count_odd(odd, k + 1, K); ++k) put(row0 + low * q + k, (uint32_t)(k + 1 - q));
-                put(row0 + low * q + k, (uint32_t)((int)t.miss[(K - kLow) * kMissRanks + low] - q));
+            if (counts && !(g & 1u) && K <= kAlone) receive_ahead(K, row0);
+            uint32_t heavy = __ballot_sync(0xffffffffu, counts && K > kAlone);
+            for (; heavy != 0u; heavy &= heavy - 1u) {
+                const int j = __ffs(heavy) - 1;
+                const int heavy_k = __shfl_sync(0xffffffffu, K, j);
+                const int row = __shfl_sync(0xffffffffu, row0, j) + (int)lane * q;
+                int missing = kLow;                              // round of the lane's missing block
+                for (int k = kLow; k <= heavy_k - 2; ++k) {
+                    if ((int)lane >= (int)count_odd(odd, k + 1, heavy_k)) continue;
+                    put(row + k, (uint32_t)(k + 1 - q));
+                    missing = k + 1;
+                }
+                if ((int)lane <= (int)count_odd(odd, kLow, heavy_k))
+                    put(row + missing, (uint32_t)((int)t.miss[(heavy_k - kLow) * kMissRanks + (int)lane] - q));
             }
-        } else {
+        } else if (counts) {
             const int z = __ffs(~g) - 1;
             if (g & 1u) {                                        // the first rank carries into one that does
                 put(row0 + kLow, (uint32_t)((int)t.miss[z * kMissRanks + (int)count_odd(odd, kLow, kLow + z)] - q));
@@ -284,7 +307,7 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
                 for (int d = 1; d <= before; ++d) {
                     const int behind = before - d;
                     const int block = behind < deeper ? k + 1 : (int)t.miss[(m - kLow) * kMissRanks + behind];
-                    put((int)shift + (end - d) * q + k, (uint32_t)(block - q));
+                    put(row1 - d * q + k, (uint32_t)(block - q));
                 }
             }
         }
@@ -400,7 +423,8 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
         }
         {
             const uint32_t after = __shfl_down_sync(0xffffffffu, pos, 1);
-            if ((int)lane >= j0 && (int)lane < j + (done ? 1 : 0)) exceptions(g, (int)(pos - base), (int)(after - base));
+            exceptions(g, (int)shift + (int)(pos - base) * q, (int)shift + (int)(after - base) * q,
+                       (int)lane >= j0 && (int)lane < j + (done ? 1 : 0));
         }
         if (done) return;
         gs += 30u;

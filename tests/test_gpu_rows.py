@@ -64,10 +64,11 @@ def test_rows_of_ranges(bcs, p):
         _check(bcs, p, r0, min(r0 + 700, p))
 
 
-@pytest.mark.parametrize("n", [148 * 32 * 32 - 1, 148 * 32 * 32 + 1, 148 * 32 * 64, 148 * 32 * 128 + 77])
+@pytest.mark.parametrize("n", [98303, 98304, 1 << 20, (1 << 20) + 1, 148 * 32 * 32 - 1, 148 * 32 * 32 + 1, 148 * 32 * 64, 148 * 32 * 128 + 77])
 @pytest.mark.parametrize("p", [(1 << 20) + 1, 3000017])
 def test_rows_where_the_split_changes(bcs, p, n):
-    _check(bcs, p, 1234567 % (p - n), 1234567 % (p - n) + n)
+    r0 = 1234567 % (p - n + 1)
+    _check(bcs, p, r0, r0 + n)
 
 
 # the kernel for 2^23 ranks and more: its lanes' places repeat every 16 ranks, 30 segments are located at a time
