@@ -8,8 +8,9 @@
 // Each is launched as a dependent of the kernel before it on the stream.
 //
 // Before: skip codes of all ranks, a search on them, a round-major copy and its transposition.  1024 p of 2^10..2^20:
-// 5456 -> 1423 us (9.1 ps a rank, both tables 4.1 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 22.7 us,
-// 16 p of 2^10..2^20: 94 -> 66 us.  Two CTAs of 256 threads per SM instead of three: 1505 us, four: more (spills).
+// 5456 -> 1437 us (9.2 ps a rank, both tables 4.1 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 18.2 us,
+// 16 p of 2^10..2^20: 94 -> 45 us.  Middle kernel with two CTAs of 256 threads per SM instead of three: 1505 us, four: more
+// (spills).
 #include <type_traits>
 
 #include "rows.cuh"
@@ -57,7 +58,7 @@ template <int kWords>
 __device__ __forceinline__ void narrow_piece(const RowTable &t, uint8_t *mine, const BatchJob &job, int q, uint32_t r0,
                                              uint32_t r1, uint32_t item, int8_t *recv, int8_t *send)
 {
-    for (uint32_t r = r0 + (threadIdx.x >> 5) * item; r < r1; r += kBatchWarps * item) {
+    for (uint32_t r = r0 + (threadIdx.x >> 5) * item; r < r1; r += (blockDim.x >> 5) * item) {
         const uint32_t n = r1 - r < item ? r1 - r : item;
         const uint64_t byte = job.entry0 + (uint64_t)r * (uint64_t)q;
         warp_rows<kWords, false>(t, mine, q, job.odd, job.inv, r, n, recv + byte, send ? send + byte : nullptr);
@@ -84,7 +85,8 @@ __device__ __forceinline__ void wide_piece(const RowTable &t, const uint8_t *sm,
 }
 
 // p <= 1024: a CTA per p.
-__global__ void __launch_bounds__(kBatchThreads)
+template <unsigned kThreads, int kCtas>
+__global__ void __launch_bounds__(kThreads, kCtas)
 batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
@@ -104,7 +106,9 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
     build_row_table(t, q, job.odd);
     grid_dependency_wait();                                      // nothing before this touches the outputs
     uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
-    const uint32_t item = p > 512u ? 128u : (p > 256u ? 64u : 32u);
+    constexpr uint32_t warps = kThreads / 32;
+    const uint32_t turns = (p + warps * kItemRanks - 1u) / (warps * kItemRanks) * warps;
+    const uint32_t item = ((p + turns - 1u) / turns + 31u) & ~31u;
     if (q <= 4) narrow_piece<1>(t, mine, job, q, 0u, p, item, recv, send);
     else if (q <= 8) narrow_piece<2>(t, mine, job, q, 0u, p, item, recv, send);
     else narrow_piece<3>(t, mine, job, q, 0u, p, item, recv, send);
@@ -217,6 +221,23 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
     }
 }
 
+// A CTA per p of the list, up to kCtas of them per SM.  alone: no larger p, nothing runs beside them.  Where the list is then
+// too short to fill the card, they ask for so much shared memory that they spread over all SMs (else some held five and
+// others one: 300 p of 3..1024 11.7 -> 8.9 us).
+template <unsigned kThreads, int kCtas>
+bcs_status launch_small(const BatchArgs &ba, bool alone, int8_t *recv, int8_t *send, cudaStream_t stream)
+{
+    uint32_t shared = RowLayout(kSmallQ).total(kThreads / 32);
+    const uint32_t per_sm = (ba.num_p + kSms - 1) / kSms;
+    if (alone && per_sm < (uint32_t)kCtas) {
+        const uint32_t spread = (226u * 1024u / per_sm - 1280u) & ~127u;     // (1 KB of each CTA is the system's)
+        if (shared < spread) shared = spread;
+    }
+    if (!allow_shared<batch_small_kernel<kThreads, kCtas>>()) return BCS_ERR_CUDA;
+    launch_dependent(true, batch_small_kernel<kThreads, kCtas>, ba.num_p, kThreads, shared, stream, ba, recv, send);
+    return launch_status();
+}
+
 }  // namespace
 }  // namespace bcs
 
@@ -254,14 +275,18 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
     const BatchArgs ba = {p_list_dev, rank_off_dev, entry_off_dev, skips_tab_dev, num_p, total_ranks};
     static_assert(kSmallP == kFusedMaxP, "the plan counts tiles for the p above kSmallP");
     // (without the plan's tiles the host cannot tell what sizes the list holds)
-    if (tile_off_dev == nullptr || total_tiles != 0) {
+    const bool small_only = tile_off_dev != nullptr && total_tiles == 0;
+    if (!small_only) {
         const WideLayout wide(kMiddleQ);
         const RowLayout narrow(kWideMinQ - 1);
         const uint32_t shared = wide.bytes > narrow.total(kBatchWarps) ? wide.bytes : narrow.total(kBatchWarps);
         if (!allow_shared<batch_middle_kernel>()) return BCS_ERR_CUDA;
-        // Three shares per resident CTA where the list is long enough, so that none ends last by much; at most 32768
-        // ranks, at least 1024 (a table costs as much as some hundred ranks of each warp).
-        uint64_t share = align_up(total_ranks / (kSms * 3u * 3u), 512);
+        // Up to 2^23 ranks a share per resident CTA: every share costs a search and a table or two, some 10 us (16 p
+        // of 2^10..2^20 66.8 us with three, 44.7 with one; 64 p of about 2^17 143 and 122 us).  Beyond, three, so that none
+        // ends last by much (150 p of 2^12..2^18, 10 million ranks, 182 us, with one 200).  At most 32768 ranks, at
+        // least 1024 (a table costs as much as some hundred ranks of each warp).
+        const uint64_t ctas = kSms * 3u * (total_ranks <= (1u << 23) ? 1u : 3u);
+        uint64_t share = align_up(total_ranks / ctas, 128);
         share = share < 1024 ? 1024 : (share > 32768 ? 32768 : share);
         const uint64_t shares = (total_ranks + share - 1) / share;
         launch_dependent(true, batch_middle_kernel, (unsigned)shares, kBatchThreads, shared, stream, ba, (uint32_t)share,
@@ -272,9 +297,10 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
                              send_out);
         }
     }
-    launch_dependent(true, batch_small_kernel, num_p, kBatchThreads, RowLayout(kSmallQ).total(kBatchWarps), stream, ba,
-                     recv_out, send_out);
-    return launch_status();
+    // CTAs of 256 threads while all are resident at once (the shorter chain counts), else of 128 (less waiting at
+    // barriers, longer items): 700 p of 3..1024 13.7 against 16.5 us, 1000 p 21.9 against 18.0.
+    if (num_p <= kSms * 5u) return launch_small<256, 5>(ba, small_only, recv_out, send_out, stream);
+    return launch_small<128, 8>(ba, small_only, recv_out, send_out, stream);
 }
 
 }  // extern "C"

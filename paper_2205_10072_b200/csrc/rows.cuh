@@ -219,11 +219,13 @@ __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32
         }
         t.codes[threadIdx.x] = (uint8_t)c;
         t.bits[threadIdx.x] = (uint8_t)(threadIdx.x < lows ? c & (0u - c) : 0u);
-    } else if (threadIdx.x < kLowRanks + kLow - 1) {
+    }
+    const uint32_t round = blockDim.x > kLowRanks ? threadIdx.x - kLowRanks : threadIdx.x;
+    if (round < kLow - 1u) {
         // Windows of round i, as ends of runs counted from the rank (`len` ranks are two runs of 2^floor(log2 len)): the
         // first skips[i+1] - skips[i] ranks that end skips[i] below it, the second those from there to the sum of
         // the skips 0..i below it.
-        const int i = (int)(threadIdx.x - kLowRanks);
+        const int i = (int)round;
         const int lo = (int)t.s[i], hi = (int)t.s[i + 1];
         int sum = 0;
         for (int k = 0; k <= i; ++k) sum += (int)t.s[k];

@@ -129,3 +129,10 @@ def _batch(bcs, plist, send=True):
 def test_batches(bcs, plist, send):
     if bcs.bcs_batch_plan(plist).total_entries:
         _batch(bcs, plist, send)
+
+
+# lists of small p that are spread over the SMs or not, with CTAs of 256 and of 128 threads; a share per CTA or several
+@pytest.mark.parametrize("plist", [range(500, 560), range(3, 593), range(200, 940), range(200, 941), range(1, 1025), [777] * 1200,
+                                   [1 << 20] * 8, [1 << 20] * 8 + [1025, 9]])
+def test_batch_splits(bcs, plist):
+    _batch(bcs, list(plist))
