@@ -8,8 +8,8 @@
 // Each is launched as a dependent of the kernel before it on the stream.
 //
 // Before: skip codes of all ranks, a search on them, a round-major copy and its transposition.  1024 p of 2^10..2^20:
-// 5456 -> 1437 us (9.2 ps a rank, both tables 4.1 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 18.2 us,
-// 16 p of 2^10..2^20: 94 -> 45 us.  Middle kernel with two CTAs of 256 threads per SM instead of three: 1505 us, four: more
+// 5456 -> 1298 us (8.3 ps a rank, both tables 4.5 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 18.1 us,
+// 16 p of 2^10..2^20: 94 -> 44 us.  Middle kernel with two CTAs of 256 threads per SM instead of three: 1505 us, four: more
 // (spills).
 #include <type_traits>
 
@@ -76,11 +76,11 @@ __device__ __forceinline__ void wide_piece(const RowTable &t, const uint8_t *sm,
     const bool head = r == 0u, tail = r + n == job.p;
     const uint64_t byte = job.entry0 + (uint64_t)r * (uint64_t)q;
     WideLane lane;
-    lane.init(q, (uint32_t)(byte & 15u));                        // (the outputs start on 16-byte boundaries)
-    wide_rows<false>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, recv + byte);
+    lane.init<true>(q, (uint32_t)(byte & 15u));                        // (the outputs start on 16-byte boundaries)
+    wide_rows<false, true>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, recv + byte);
     if (send != nullptr) {
         lane.home = -1;
-        wide_rows<true>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, send + byte);
+        wide_rows<true, true>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, send + byte);
     }
 }
 
@@ -208,10 +208,10 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
         auto all = [&](auto is_send, int8_t *out) {
             WideLane lane;
-            lane.init(q, (uint32_t)(job.entry0 & 15u));
+            lane.init<true>(q, (uint32_t)(job.entry0 & 15u));
             for (uint64_t r = ((uint64_t)blockIdx.x * n_warps + warp) * item; r < p; r += (uint64_t)gridDim.x * n_warps * item) {
                 const uint32_t n = p - (uint32_t)r < item ? p - (uint32_t)r : item;
-                wide_rows<decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, p, q, job.odd, job.inv, lane,
+                wide_rows<decltype(is_send)::value, true>(t, sm, at.send, sm + at.ends + warp * 32u, p, q, job.odd, job.inv, lane,
                                                     (uint32_t)r, n, r == 0, r + n == p, out + job.entry0 + r * (uint64_t)q);
             }
         };

@@ -70,7 +70,7 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
 // The same for larger tables, q >= 16 (wide.cuh), one CTA per SM; `item` is a multiple of 16.  halves: half of the warps
 // write the receive rows and half the send rows; otherwise all warps the ones before the others.
 // (No more than 640 threads: at the speed of the memory the write streams of 1024 cost 20 % and more.)
-template <unsigned kThreads, int kCtas>
+template <unsigned kThreads, int kCtas, bool kAnyStep>
 __global__ void __launch_bounds__(kThreads, kCtas)
 wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, bool halves,
             int8_t *recv, int8_t *send)
@@ -89,13 +89,13 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     uint32_t n_warps = blockDim.x >> 5, index = warp;
     auto all = [&](auto is_send, int8_t *out) {
         WideLane mine;
-        mine.init(rc.q, 0u);
+        mine.template init<kAnyStep>(rc.q, 0u);
         const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
         for (uint64_t b = ((uint64_t)blockIdx.x * n_warps + index) * item; b < count; b += stride) {
             const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
             uint32_t x0 = first + (uint32_t)b;
             if (x0 >= rc.p) x0 -= rc.p;
-            wide_rows<decltype(is_send)::value>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
+            wide_rows<decltype(is_send)::value, kAnyStep>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
                                                 mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
         }
     };
@@ -110,13 +110,16 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     if (sends) all(std::true_type(), send);
 }
 
-template <unsigned kThreads, int kCtas>
+template <unsigned kThreads, int kCtas, bool kAnyStep = false>
 bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, uint32_t item, bool halves, int8_t *recv, int8_t *send,
                        cudaStream_t stream)
 {
-    if (!allow_shared<wide_kernel<kThreads, kCtas>>()) return BCS_ERR_CUDA;
+    if constexpr (!kAnyStep) {
+        if (step_ranks(rc.q) != 16u) return launch_wide<kThreads, kCtas, true>(rc, first, count, item, halves, recv, send, stream);
+    }
+    if (!allow_shared<wide_kernel<kThreads, kCtas, kAnyStep>>()) return BCS_ERR_CUDA;
     const unsigned items = (count + item - 1) / item;
-    launch_dependent(true, wide_kernel<kThreads, kCtas>, items < kSms ? items : kSms, kThreads,
+    launch_dependent(true, wide_kernel<kThreads, kCtas, kAnyStep>, items < kSms ? items : kSms, kThreads,
                      WideLayout(rc.q).bytes, stream, rc, first, count, item, halves, recv, send);
     return launch_status();
 }
@@ -161,10 +164,10 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     const uint32_t ranks = (uint32_t)count, x0 = (uint32_t)first;
     // The wide kernel from 96 Ki ranks on (its tables take longer to build: 65 000 ranks 5.8 against 4.1 us here).  Up to
     // 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
-    // are built beside it (700 001 ranks 12.3 us, 13.7 with 640 threads, 14.9 per rank; 1.3 million 18.2, 18.0, 23.4; 2.1
+    // are built beside it (with steps of 16 ranks: 700 001 ranks 12.3 us, 13.7 with 640 threads, 14.9 per rank; 1.3 million 18.2, 18.0, 23.4; 2.1
     // million 21.4, 20.6, 29.3).  Beyond, all receive rows before the send rows, item by item: an item's start costs as
     // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
-    // faster (12.3 million ranks 61 us a table with items of 768, 67 with 384; 2^25: 151 and 146 us).
+    // faster (12.3 million ranks 54 us a table with items of 800, 61 with 400; 2^25: 151 and 146 us).
     if (rc.q >= kWideMinQ && count >= 98304) {
         const bool halves = count < (1u << 23);
         auto run = [&](uint32_t warps) {
@@ -173,7 +176,8 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
         };
         if (count <= (1u << 20)) return launch_wide<384, 2>(rc, x0, ranks, run(12), halves, recv, send, stream);
         if (halves) return launch_wide<640, 1>(rc, x0, ranks, run(20), halves, recv, send, stream);
-        return launch_wide<640, 1>(rc, x0, ranks, count >= (1u << 25) ? 384u : 768u, halves, recv, send, stream);
+        const uint32_t item = count >= (1u << 25) ? 384u : 768u;            // (whole steps: 400 and 800 where these have 20 ranks)
+        return launch_wide<640, 1>(rc, x0, ranks, step_ranks(rc.q) == 20u ? item / 24u * 25u : item, halves, recv, send, stream);
     }
     return launch<1>(rc, x0, ranks, recv, send, stream);
 }

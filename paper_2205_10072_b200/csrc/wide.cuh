@@ -3,7 +3,8 @@
 // The per-rank form (warp_rows) pays for every rank: shifting a row to its place among the words of its neighbours, an
 // exchange with the next lane, stores q bytes apart, a copy out of shared memory.  Here a lane makes aligned
 // 16-byte vectors of the output.  16 ranks are q vectors, so in steps of 16 ranks a lane's vector always begins
-// with the same round k0 of a rank at the same place of the step (the lanes from q on repeat the first ones').  It holds bytes of two rows at most
+// with the same round k0 of a rank at the same place of the step (the lanes from q on repeat the first ones').  Where fewer
+// ranks are whole vectors already, a step takes as many as 32 lanes hold.  A vector holds bytes of two rows at most
 // (q >= 16), those of ranks A and A + 1:
 //     out = segment part | bytes of A's table row | bytes of (A+1)'s table row,
 // the first in registers for as long as the segment lasts, the others by byte permutations whose selectors
@@ -22,7 +23,19 @@ namespace bcs {
 
 constexpr int kWideMinQ = 16;
 
-constexpr uint32_t kStep = 16;        // ranks of a step (two segments never end in the same: they have 41 ranks or more)
+constexpr uint32_t kStep = 16;        // items are multiples of this many ranks
+
+// Ranks of a step: as many as are whole vectors and 32 of these at most, 512 / q rounded down to a multiple of
+// 16 / gcd(16, q); and 2^32 divided by it, rounded up.  Two segments never end in the same step: they have 41 ranks or more.
+// (16 ranks for all q left 12 of 32 lanes idle for q = 20: 200 p of 2^19..2^20 1341 -> 1224 us, 3000 of 2^15..2^16 1316 -> 1086.)
+__host__ __device__ constexpr uint32_t step_ranks(int q)
+{
+    return q == 16 ? 32u : (q == 18 || q == 20 ? 24u : (q == 24 ? 20u : 16u));
+}
+__host__ __device__ constexpr uint32_t step_inverse(int q)
+{
+    return q == 16 ? 1u << 27 : (q == 18 || q == 20 ? 0xffffffffu / 24u + 1u : (q == 24 ? 0xffffffffu / 20u + 1u : 1u << 28));
+}
 
 struct WideLayout {
     RowLayout base;                   // (its warps' part is not used)
@@ -177,10 +190,12 @@ struct WideLane {
     uint32_t near[4];                                            // selectors of the rounds L .. L+2
     Pick pick;
     int home;                                                    // home round that it is for, -1: none
+    template <bool kAnyStep>
     __device__ __forceinline__ void init(int q, uint32_t shift)
     {
         const uint32_t lane = threadIdx.x & 31u;
-        v = lane < (uint32_t)q ? lane : lane - (uint32_t)q;
+        const uint32_t vectors = kAnyStep ? step_ranks(q) * (uint32_t)q / 16u : (uint32_t)q;
+        v = lane < vectors ? lane : lane - vectors;
         const int byte = (int)(16u * v + (uint32_t)q - shift);   // shift < 16 <= q
         a = byte / q - 1;
         k0 = byte - byte / q * q;
@@ -217,7 +232,8 @@ struct WideLane {
 // theirs too (else n is a multiple of 16).
 // sm: the CTA's shared memory, the row table at 0, the send table at send_at; ends: 32 bytes for the two vectors that are
 // not written as a whole.
-template <bool kSend>
+// kAnyStep: false where step_ranks(q) is known to be 16 (a constant: 0.2-0.3 us less for tables of up to 2 million ranks).
+template <bool kSend, bool kAnyStep>
 __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, uint32_t send_at, uint8_t *ends, uint32_t p,
                                           int q, uint32_t odd, uint32_t inv, WideLane &mine, uint32_t x0, uint32_t n,
                                           bool head, bool tail, int8_t *dst)
@@ -231,7 +247,8 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
     const uint32_t len = n * (uint32_t)q + (tail ? shift : 0u);
     const uint32_t skip = head ? shift : 0u;
     const bool ragged = skip != 0u || (len & 15u) != 0u;
-    const uint32_t step_bytes = kStep * (uint32_t)q;
+    const uint32_t ranks = kAnyStep ? step_ranks(q) : 16u, step_bytes = ranks * (uint32_t)q;     // of a step
+    const uint32_t by_ranks = step_inverse(q);
 
     // Ranks are counted from x0 on; y: the first one that the window shows.
     const uint32_t lead = shift != 0u ? 1u : 0u;
@@ -359,15 +376,16 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
         bool done = false;
         for (;;) {
             // steps inside the segment
-            const int steps = ((next < (int)n ? next : (int)n) - step) / (int)kStep;
+            const int room = (next < (int)n ? next : (int)n) - step;
+            const int steps = kAnyStep ? (int)__umulhi(room > 0 ? (uint32_t)room : 0u, by_ranks) : room / 16;
             if (!ragged) {
                 uint8_t *o = out + to;
-#pragma unroll 2
+#pragma unroll 1                                                 // (a handful: 1024 p of 2^10..2^20 1330 us unrolled, 1295 not)
                 for (int i = 0; i < steps; ++i) {
                     const uint2 ra = *reinterpret_cast<const uint2 *>(sm + at);
                     const uint2 rb = *reinterpret_cast<const uint2 *>(sm + at + 8);
                     *reinterpret_cast<uint4 *>(o) = wide_vector(ra, rb, part, mine.pick);
-                    at += 8u * kStep;
+                    at += 8u * ranks;
                     o += step_bytes;
                 }
             } else {
@@ -375,11 +393,11 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
                     const uint2 ra = *reinterpret_cast<const uint2 *>(sm + at);
                     const uint2 rb = *reinterpret_cast<const uint2 *>(sm + at + 8);
                     store(to + (uint32_t)i * step_bytes, wide_vector(ra, rb, part, mine.pick));
-                    at += 8u * kStep;
+                    at += 8u * ranks;
                 }
             }
             to += (uint32_t)steps * step_bytes;
-            step += steps * (int)kStep;
+            step += steps * (int)ranks;
             // the step in which it ends, or the last one of the item
             const uint32_t inf2 = __shfl_sync(0xffffffffu, info, j + 1), three2 = __shfl_sync(0xffffffffu, three, j + 1);
             const int home2 = (int)(inf2 >> 24);
@@ -404,9 +422,9 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
             part = coming;
             if (mine.home != home2) mine.pick = make_pick<kSend>(mine.k0, q, home2, home2);
             mine.home = home2;
-            at = new_at + 8u * kStep;
+            at = new_at + 8u * ranks;
             to += step_bytes;
-            step += (int)kStep;
+            step += (int)ranks;
             done = step * q >= (int)len;
             start = next;
             ++j;

@@ -71,6 +71,13 @@ def test_rows_where_the_split_changes(bcs, p, n):
     _check(bcs, p, r0, r0 + n)
 
 
+# steps of 24, 16 and 20 ranks (32 for q = 16: the batches below), runs and items that end inside one
+@pytest.mark.parametrize("p,r0,n", [(140001, 0, 140001), (262144, 100000, 98311), (600011, 0, 600011), (1 << 20, 777, 98304 + 24),
+                                    ((1 << 23) + 1, (1 << 22) + 12345, 100001), (1 << 24, (1 << 23) - 200000, 400009)])
+def test_rows_of_other_steps(bcs, p, r0, n):
+    _check(bcs, p, r0, r0 + n)
+
+
 # the kernel for 2^23 ranks and more: its lanes' places repeat every 16 ranks, 30 segments are located at a time
 @pytest.mark.parametrize("p,r0,n", [((1 << 23) + 1, 0, (1 << 23) + 1), (100 << 17, 4000003, (1 << 23) + 385),
                                     ((1 << 24) - 1, 0, (1 << 24) - 1), ((1 << 30) + 20, (1 << 29) - 777777, (1 << 23) + 1),
@@ -124,7 +131,7 @@ def _batch(bcs, plist, send=True):
 # end inside a p, lists of one p
 @pytest.mark.parametrize("plist", [[1024, 1025, 3, 32768, 1, 32769, 65537, 1023, 40001, 2, 65535],
                                    [(1 << 21) + 1, 5, (1 << 21), 1, (1 << 21) - 1, 77, (1 << 22) + 5],
-                                   [33333], [1], [2, 1], [(1 << 20) + 1] * 3, [1025] * 40, [127, 128, 129, 130] * 30])
+                                   [33333], [65536, 140001, 600011, 1 << 20], [1], [2, 1], [(1 << 20) + 1] * 3, [1025] * 40, [127, 128, 129, 130] * 30])
 @pytest.mark.parametrize("send", [True, False])
 def test_batches(bcs, plist, send):
     if bcs.bcs_batch_plan(plist).total_entries:
