@@ -31,7 +31,6 @@ METRIC = "schedule ranks built/sec (int8 recv+send, q entries)"
 UNIT = "ranks/s"
 SM_COUNT = 148
 ISSUE_PER_SM = 4 * 32          # thread instructions per clock: 4 schedulers x 32 lanes
-ALU_LANES_PER_SM = 64          # INT32 lanes per SM per clock (one pipe)
 
 
 # ------------------------------------------------------------------------------------ inputs
@@ -57,13 +56,6 @@ def _executed_counts():
                               "dram_bytes": None if ln[2] == "-" else float(ln[2]),
                               "ranks_captured": float(ln[3])}
     return out
-
-
-def _model_ops():
-    """tests/skipcode_model_ops.json, written by `python -m tests.skipcode_mirror --write`: integer
-    operations per rank that the counted CPU restatement of the construction needs."""
-    with open(os.path.join(ROOT, "tests", "skipcode_model_ops.json")) as f:
-        return json.load(f)
 
 
 class ClockSampler:
@@ -206,12 +198,10 @@ def _no_flush():
     pass
 
 
-def _alu_roofline(kernels, ranks, ms, out_bytes, hbm_gbs, sm_max_mhz, counts, model, measured):
-    """Roofline block of a construction step (integer-issue bound).
-    kernels: keys of profiles/executed_instructions.txt whose kernels ran in the `ms` that were timed;
-    model: integer operations per rank of the counted CPU restatement, or None."""
+def _alu_roofline(kernels, ranks, ms, out_bytes, hbm_gbs, sm_max_mhz, counts, measured):
+    """Roofline block of a construction step bound by instruction issue.
+    kernels: keys of profiles/executed_instructions.txt whose kernels ran in the `ms` that were timed."""
     issue_peak = SM_COUNT * ISSUE_PER_SM * sm_max_mhz * 1e6 / 1e12           # T thread-inst/s
-    one_pipe = SM_COUNT * ALU_LANES_PER_SM * sm_max_mhz * 1e6 / 1e12
     per_rank = sum(counts[k]["thread_inst_per_rank"] for k in kernels)
     achieved = per_rank * ranks / (ms * 1e-3) / 1e12
     t_int_ms = per_rank * ranks / (issue_peak * 1e12) * 1e3
@@ -223,20 +213,11 @@ def _alu_roofline(kernels, ranks, ms, out_bytes, hbm_gbs, sm_max_mhz, counts, mo
             "peak_source": "issue limit: 148 SMs x 4 schedulers x 32 lanes x %.0f MHz (max SM clock)" % sm_max_mhz,
             "t_int_ms": t_int_ms, "t_hbm_ms": t_hbm_ms, "roofline_ms": max(t_int_ms, t_hbm_ms),
             "frac_of_max_t_int_t_hbm": max(t_int_ms, t_hbm_ms) / ms,
-            "hbm_peak_gbs": hbm_gbs}
+            "frac_of_hbm": t_hbm_ms / ms, "hbm_peak_gbs": hbm_gbs}
     if measured:
         two_pipe = max(measured["logic_imad_mix"], measured["logic_add_mix"])
         roof["peak_measured"] = measured
         roof["frac_of_measured_two_pipe_mix"] = achieved / two_pipe
-    if model is not None:
-        m_ach = model * ranks / (ms * 1e-3) / 1e12
-        roof["model"] = {"int_ops_per_rank": model, "achieved": m_ach, "unit": "Tint-op/s",
-                         "source": "tests/skipcode_model_ops.json (tests/skipcode_mirror.py --write)",
-                         "frac_of_issue_limit": m_ach / issue_peak,
-                         "frac_of_one_pipe_%.1fT" % one_pipe: m_ach / one_pipe}
-        if measured:
-            roof["model"]["frac_of_measured_two_pipe_mix"] = m_ach / max(measured["logic_imad_mix"],
-                                                                         measured["logic_add_mix"])
     return roof
 
 
@@ -256,33 +237,31 @@ class LargeP:
         self.recv = torch.empty(cap * self.q, dtype=torch.int8, device="cuda")
         self.send = torch.empty(cap * self.q, dtype=torch.int8, device="cuda")
         self.ws = torch.empty(bcs.bcs_prepare_workspace_bytes(self.p), dtype=torch.int8, device="cuda")
-        self.launches_per_step = 1 + 2 * len(self.chunks)
+        self.launches_per_step = 2 * len(self.chunks)    # bcs_prepare_codes launches nothing
 
     def step(self):
         bcs, p, ws = self.bcs, self.p, self.ws
         bcs.bcs_prepare_codes(p, ws)
-        for r0, r1 in self.chunks:                   # receive rows of the chunk, round-major copy
+        for r0, r1 in self.chunks:                   # receive rows of the chunk
             bcs.bcs_prepare_rows(p, r0, r1, self.recv, ws)
-        for r0, r1 in self.chunks:                   # send rows of the chunk (Algorithm 9's lookup)
+        for r0, r1 in self.chunks:                   # send rows of the chunk
             bcs.bcs_build_prepared(p, r0, r1, None, self.send, ws)
 
     def parts_ms(self, reps=3):
-        """codes / receive rows / send rows of a step, by CUDA events."""
+        """receive rows / send rows of a step, by CUDA events."""
         torch, bcs, p, ws = self.torch, self.bcs, self.p, self.ws
-        acc = [0.0, 0.0, 0.0]
+        acc = [0.0, 0.0]
         for _ in range(reps):
-            ev = [torch.cuda.Event(enable_timing=True) for _ in range(4)]
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
             ev[0].record()
-            bcs.bcs_prepare_codes(p, ws)
-            ev[1].record()
             for r0, r1 in self.chunks:
                 bcs.bcs_prepare_rows(p, r0, r1, self.recv, ws)
-            ev[2].record()
+            ev[1].record()
             for r0, r1 in self.chunks:
                 bcs.bcs_build_prepared(p, r0, r1, None, self.send, ws)
-            ev[3].record()
+            ev[2].record()
             torch.cuda.synchronize()
-            for i in range(3):
+            for i in range(2):
                 acc[i] += ev[i].elapsed_time(ev[i + 1]) / reps
         return acc
 
@@ -352,7 +331,7 @@ class LargeP:
                        "built (two chunk buffers per table; inputs are scalars: no H2D)"}
 
 
-def _bench_single(torch, bcs, workloads, flush, steps, hbm_gbs, sm_max_mhz, counts, model, measured):
+def _bench_single(torch, bcs, workloads, flush, steps, hbm_gbs, sm_max_mhz, counts, measured):
     """Single p = 2^20+1: one bcs_build per step, L2 flushed before every step."""
     p = workloads.P_SINGLE
     q = bcs.bcs_q(p)
@@ -362,14 +341,7 @@ def _bench_single(torch, bcs, workloads, flush, steps, hbm_gbs, sm_max_mhz, coun
     ws = torch.empty(bcs.bcs_build_workspace_bytes(p, 0, p), dtype=torch.int8, device="cuda")
     ms = _event_ms(torch, lambda: bcs.bcs_build(p, 0, p, recv, send, ws), flush, steps, 5)
     step_ms = statistics.mean(ms)
-    # codes + receive kernel as the step runs them (rows and round-major copy), by bcs_prepare_rows
-    pws = torch.empty(bcs.bcs_prepare_workspace_bytes(p), dtype=torch.int8, device="cuda")
-
-    def recv_part():
-        bcs.bcs_prepare_codes(p, pws)
-        bcs.bcs_prepare_rows(p, 0, p, recv, pws)
-    recv_ms = statistics.mean(_event_ms(torch, recv_part, flush, max(20, steps // 4), 3))
-    slow_ms = statistics.mean(_event_ms(torch, lambda: bcs.bcs_build(p, 0, p, recv, send, None), flush, 10, 2))
+    recv_ms = statistics.mean(_event_ms(torch, lambda: bcs.bcs_build(p, 0, p, recv, None, ws), flush, max(20, steps // 4), 3))
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record()
     for _ in range(2000):
@@ -381,18 +353,9 @@ def _bench_single(torch, bcs, workloads, flush, steps, hbm_gbs, sm_max_mhz, coun
            "ranks_per_s": p / step_ms * 1e3, "out_gbs": 2 * nb / step_ms / 1e6,
            "l2": "flushed before every timed step (256 MiB write)",
            "back_to_back_ms": e0.elapsed_time(e1) / 2000,
-           "kernel_ms": {"codes+recv (bcs_prepare_codes + bcs_prepare_rows)": recv_ms,
-                         "send transposition (difference)": max(step_ms - recv_ms, 0.0),
-                         "self_contained_construction_step": slow_ms},
-           "roofline": _alu_roofline(["codes_single_kernel@q21", "recv_codes_quad_kernel<true,true>@q21"], p,
-                                     recv_ms, nb + nb, hbm_gbs, sm_max_mhz, counts,
-                                     model["q21_p1048577"]["recv_int_ops_per_rank"], measured),
-           "step_roofline": _alu_roofline(["codes_single_kernel@q21", "recv_codes_quad_kernel<true,true>@q21",
-                                           "send_transpose_kernel@q21"], p, step_ms, 2 * nb, hbm_gbs,
-                                          sm_max_mhz, counts,
-                                          model["q21_p1048577"]["recv_int_ops_per_rank"]
-                                          + model["q21_p1048577"]["send_int_ops_per_rank"], measured)}
-    res["roofline"]["traffic"] = counts["recv_codes_quad_kernel<true,true>@q21"]["dram_bytes"]
+           "kernel_ms": {"receive rows alone": recv_ms},
+           "roofline": _alu_roofline(["wide_kernel@q21"], p, step_ms, 2 * nb, hbm_gbs, sm_max_mhz, counts, measured)}
+    res["roofline"]["traffic"] = counts["wide_kernel@q21"]["dram_bytes"]
     # property check and brute-force broadcast of the tables just built
     viol = torch.zeros(3, dtype=torch.int64, device="cuda")
     v_ms = statistics.mean(_event_ms(torch, lambda: bcs.bcs_validate(p, 0, p, recv, send, viol), flush, 10, 2))
@@ -468,7 +431,7 @@ def _bench_checksum(torch, bcs, flush, hbm_gbs, peak_src, table, steps, counts):
                          "peak_source": peak_src}}
 
 
-def _bench_batch(torch, bcs, workloads, flush, full, hbm_gbs, sm_max_mhz, counts, model, measured):
+def _bench_batch(torch, bcs, workloads, flush, full, hbm_gbs, sm_max_mhz, counts, measured):
     out = {}
     plan = bcs.bcs_batch_plan(workloads.small_sweep())
     dplan = plan.to("cuda")
@@ -479,17 +442,13 @@ def _bench_batch(torch, bcs, workloads, flush, full, hbm_gbs, sm_max_mhz, counts
     ms = statistics.mean(_event_ms(
         torch, lambda: bcs.bcs_build_batch(dplan, br, bs, bw),
         flush, 20, 3))
-    batch_kernels = ["codes_batch_kernel", "recv_quad_batch_kernel<true>", "send_batch_kernel"]
-    small_kernels = ["fused_small_batch_kernel<true>"]
     out["batch_small_sweep"] = {
         "workload": "every p in 2..1024, all ranks, one bcs_build_batch (one launch: a CTA per p)",
         "ranks": plan.total_ranks, "ms": ms, "ranks_per_s": plan.total_ranks / ms * 1e3,
         "out_gbs": 2 * plan.total_entries / ms / 1e6,
         "l2": "flushed before every timed step",
-        "roofline": _alu_roofline([k + "@small_sweep" for k in small_kernels], plan.total_ranks, ms,
-                                  2 * plan.total_entries, hbm_gbs, sm_max_mhz, counts,
-                                  model["small_sweep_2_1024"]["recv_int_ops_per_rank"]
-                                  + model["small_sweep_2_1024"]["send_int_ops_per_rank"], measured)}
+        "roofline": _alu_roofline(["batch_small_kernel@small_sweep"], plan.total_ranks, ms,
+                                  2 * plan.total_entries, hbm_gbs, sm_max_mhz, counts, measured)}
     plist = workloads.batch_p_list() if full else workloads.batch_p_list(count=256)
     plan = bcs.bcs_batch_plan(plist)
     dplan = plan.to("cuda")
@@ -507,10 +466,8 @@ def _bench_batch(torch, bcs, workloads, flush, full, hbm_gbs, sm_max_mhz, counts
         "ranks": plan.total_ranks, "ms": ms, "ranks_per_s": plan.total_ranks / ms * 1e3,
         "out_gbs": 2 * plan.total_entries / ms / 1e6,
         "l2": "outputs (%.1f GB) exceed L2" % (2 * plan.total_entries / 1e9),
-        "roofline": _alu_roofline([k + "@256p_sample" for k in batch_kernels], plan.total_ranks, ms,
-                                  2 * plan.total_entries, hbm_gbs, sm_max_mhz, counts,
-                                  model["batch_4096p"]["recv_int_ops_per_rank"]
-                                  + model["batch_4096p"]["send_int_ops_per_rank"], measured)}
+        "roofline": _alu_roofline(["batch_middle_kernel@256p_sample"], plan.total_ranks, ms,
+                                  2 * plan.total_entries, hbm_gbs, sm_max_mhz, counts, measured)}
     return out
 
 
@@ -590,7 +547,6 @@ def run_ours(args) -> None:
 
     hbm_gbs, sm_max_mhz, peak_src = _peaks()
     counts = _executed_counts()
-    model = _model_ops()
     flush_buf = torch.empty(256 << 20, dtype=torch.int8, device="cuda")   # > 126 MB L2
 
     def flush():
@@ -600,7 +556,7 @@ def run_ours(args) -> None:
         if rank == 0:
             print(json.dumps({"only": args.only, "steps": args.steps,
                               "aux": _run_part(args, torch, bcs, workloads, flush, hbm_gbs, sm_max_mhz,
-                                               peak_src, counts, model)}))
+                                               peak_src, counts)}))
         return
 
     large = LargeP(torch, bcs, workloads)
@@ -633,28 +589,21 @@ def run_ours(args) -> None:
     out = None
     if rank == 0:
         measured = Probe(torch).all()
-        codes_ms, rows_ms, send_ms = large.parts_ms()
-        m30 = model["q30_p1073741823"]
-        roof = _alu_roofline(["recv_codes_quad_kernel<true,true>@q30"], p, rows_ms, 2 * p * q, hbm_gbs,
-                             sm_max_mhz, counts, m30["recv_int_ops_per_rank"] - m30["code_ops_per_rank"],
-                             measured)
-        roof["kernel"] = "recv_codes_quad_kernel<true,true> (8 launches of bcs_prepare_rows: %.1f%% of the step)" \
-                         % (100 * rows_ms / (codes_ms + rows_ms + send_ms))
-        roof["traffic"] = None
-        roof["traffic_note"] = ("not captured at this size (8 GB per launch); the DRAM bytes of a 2^22-rank "
-                                "range of the same p are in profiles/, they do not scale in proportion "
-                                "(re-reads of the skip codes depend on what the L2 still holds)")
-        step_roof = _alu_roofline(["codes_single_kernel@q30", "recv_codes_quad_kernel<true,true>@q30",
-                                   "send_transpose_kernel@q30"], p, ms_per_step, 2 * p * q, hbm_gbs,
-                                  sm_max_mhz, counts,
-                                  m30["recv_int_ops_per_rank"] + m30["send_int_ops_per_rank"], measured)
+        rows_ms, send_ms = large.parts_ms()
+        gbs = 2 * p * q / ms_per_step / 1e6
+        roof = {"bound": "hbm", "kernel": "wide_kernel (8 launches for the receive rows, 8 for the send rows: the whole step)",
+                "achieved": gbs, "peak": hbm_gbs, "unit": "GB/s", "frac": gbs / hbm_gbs, "peak_source": peak_src,
+                "traffic": None,
+                "traffic_note": "not captured at this size (4 GB per launch); the DRAM bytes of a 2^24-rank range of the "
+                                "same p are in profiles/"}
+        step_roof = _alu_roofline(["wide_kernel@q30"], p, ms_per_step, 2 * p * q, hbm_gbs, sm_max_mhz, counts, measured)
         checked_ms, violations = large.checked_step()
         out = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "u32", "data": "synthetic",
             "config": {"workload": WORKLOAD_LARGE, "p": p, "q": q, "chunks": len(large.chunks),
-                       "send_variant": "lookup (rotated transposition of the round-major receive copy)",
+                       "send_variant": "computed from the binary form of the rank, as the receive rows",
                        "l2": "no flush: every step streams 64 GB of outputs through 8 GB chunk buffers, "
                              "far beyond the 126 MB L2",
                        "workspace_bytes": large.ws.numel(),
@@ -662,7 +611,7 @@ def run_ours(args) -> None:
                        "timed_wall_s": t_wall},
             "out_gbs": 2 * p * q / ms_per_step / 1e6,
             "timing": {"median_ms": statistics.median(ms), "min_ms": min(ms), "max_ms": max(ms)},
-            "kernel_ms": {"codes (bcs_prepare_codes)": codes_ms, "receive rows (8 x bcs_prepare_rows)": rows_ms,
+            "kernel_ms": {"receive rows (8 x bcs_prepare_rows)": rows_ms,
                           "send rows (8 x bcs_build_prepared)": send_ms},
             "roofline": roof, "step_roofline": step_roof,
             "gpu_launches": large.launches_per_step * args.steps, "clocks": clk.summary(),
@@ -676,9 +625,8 @@ def run_ours(args) -> None:
         # ---- the other workloads (each with its own roofline block)
         cfg = {}
         cfg["single_p"] = _bench_single(torch, bcs, workloads, flush, 300, hbm_gbs, sm_max_mhz, counts,
-                                        model, measured)
-        cfg.update(_bench_batch(torch, bcs, workloads, flush, True, hbm_gbs, sm_max_mhz, counts, model,
-                                measured))
+                                        measured)
+        cfg.update(_bench_batch(torch, bcs, workloads, flush, True, hbm_gbs, sm_max_mhz, counts, measured))
         cfg["expand"], table = _bench_expand(torch, bcs, workloads, flush, hbm_gbs, peak_src, 20, counts)
         cfg["checksum"] = _bench_checksum(torch, bcs, flush, hbm_gbs, peak_src, table, 20, counts)
         del table
@@ -699,7 +647,7 @@ def run_ours(args) -> None:
         print(json.dumps(out))
 
 
-def _run_part(args, torch, bcs, workloads, flush, hbm_gbs, sm_max_mhz, peak_src, counts, model):
+def _run_part(args, torch, bcs, workloads, flush, hbm_gbs, sm_max_mhz, peak_src, counts):
     """One part alone, small enough for a profiler (see profiles/ for the commands)."""
     res = {}
     if args.only == "probe":
@@ -709,29 +657,16 @@ def _run_part(args, torch, bcs, workloads, flush, hbm_gbs, sm_max_mhz, peak_src,
         res["int_rate_probe"]["unit"] = "Tint-op/s"
     elif args.only == "build":
         res["single_p"] = _bench_single(torch, bcs, workloads, flush, args.steps, hbm_gbs, sm_max_mhz, counts,
-                                        model, None)
+                                        None)
     elif args.only == "large-sample":
-        # 2^22 ranks in the middle of p = 2^30-1 through bcs_build with its workspace: the same codes and
-        # receive kernels as the headline's step on 4.4 GB of device memory (the send rows of a
-        # sub-range come from the gather kernel, which the headline does not use)
+        # 2^24 ranks in the middle of p = 2^30-1: the headline's kernel on 1 GB of outputs
         p = workloads.P_LARGE
         q = bcs.bcs_q(p)
-        r0, r1 = 1 << 29, (1 << 29) + (1 << 22)
+        r0, r1 = 1 << 29, (1 << 29) + (1 << 24)
         recv = torch.empty((r1 - r0) * q, dtype=torch.int8, device="cuda")
         send = torch.empty((r1 - r0) * q, dtype=torch.int8, device="cuda")
-        ws = torch.empty(bcs.bcs_build_workspace_bytes(p, r0, r1), dtype=torch.int8, device="cuda")
-        ms = _event_ms(torch, lambda: bcs.bcs_build(p, r0, r1, recv, send, ws), _no_flush, args.steps, 1)
+        ms = _event_ms(torch, lambda: bcs.bcs_build(p, r0, r1, recv, send, None), _no_flush, args.steps, 1)
         res["large_sample"] = {"p": p, "ranks": r1 - r0, "ms": statistics.mean(ms)}
-    elif args.only == "large-transpose":
-        # the send transposition of the headline on a p with the same q = 30 that fits in 20 GB
-        p = (1 << 29) + 1
-        q = bcs.bcs_q(p)
-        ws = torch.empty(bcs.bcs_prepare_workspace_bytes(p), dtype=torch.int8, device="cuda")
-        bcs.bcs_prepare(p, ws)
-        r0, r1 = 1 << 28, (1 << 28) + (1 << 24)
-        send = torch.empty((r1 - r0) * q, dtype=torch.int8, device="cuda")
-        ms = _event_ms(torch, lambda: bcs.bcs_build_prepared(p, r0, r1, None, send, ws), _no_flush, args.steps, 1)
-        res["large_transpose"] = {"p": p, "ranks": r1 - r0, "ms": statistics.mean(ms)}
     elif args.only == "allgather":
         res["allgather_tables"] = _bench_allgather(torch, bcs, workloads, flush, hbm_gbs, peak_src, args.steps,
                                                    counts)
@@ -741,7 +676,7 @@ def _run_part(args, torch, bcs, workloads, flush, hbm_gbs, sm_max_mhz, peak_src,
         if args.only == "checksum":
             res["checksum"] = _bench_checksum(torch, bcs, flush, hbm_gbs, peak_src, table, args.steps, counts)
     elif args.only == "batch":
-        res = _bench_batch(torch, bcs, workloads, flush, False, hbm_gbs, sm_max_mhz, counts, model, None)
+        res = _bench_batch(torch, bcs, workloads, flush, False, hbm_gbs, sm_max_mhz, counts, None)
     return res
 
 
@@ -752,7 +687,7 @@ def main() -> None:
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--only", default="all",
-                    choices=["all", "build", "large-sample", "large-transpose", "expand", "checksum", "batch",
+                    choices=["all", "build", "large-sample", "expand", "checksum", "batch",
                              "allgather", "probe"],
                     help="run one part only (small, profiler-friendly runs); 'all' is the benchmark")
     args = ap.parse_args()
