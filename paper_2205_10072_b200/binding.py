@@ -167,7 +167,7 @@ def bcs_build_workspace_bytes(p: int, r_begin: int, r_end: int) -> int:
 def bcs_build(p: int, r_begin: int, r_end: int, recv_out, send_out, workspace=None,
               stream=None) -> None:
     """recv_out / send_out: CUDA int8 tensors of (r_end-r_begin)*q elements, or None;
-    workspace: CUDA tensor of bcs_build_workspace_bytes(...) bytes (fast path) or None."""
+    workspace: CUDA tensor of bcs_build_workspace_bytes(...) bytes or None (not touched)."""
     _check(_call.build(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out), _ptr(workspace),
                            _nbytes(workspace), _stream(stream)), "bcs_build")
 
@@ -190,35 +190,35 @@ def bcs_prepare_workspace_bytes(p: int) -> int:
 
 
 def bcs_prepare(p: int, workspace, stream=None) -> None:
-    """Runs the construction once for all ranks of p into `workspace` (CUDA tensor of
-    bcs_prepare_workspace_bytes(p) bytes) for later bcs_build_prepared calls."""
+    """Checks p and `workspace` (CUDA tensor of bcs_prepare_workspace_bytes(p) bytes) for later
+    bcs_build_prepared calls; these compute the rows, nothing is prepared."""
     _check(_call.prepare(p, _ptr(workspace), _nbytes(workspace), _stream(stream)), "bcs_prepare")
 
 
 def bcs_prepare_codes(p: int, workspace, stream=None) -> None:
-    """First half of bcs_prepare: the skip codes of all ranks of p into `workspace`."""
+    """First half of bcs_prepare: the same checks."""
     _check(_call.prepare_codes(p, _ptr(workspace), _nbytes(workspace), _stream(stream)),
            "bcs_prepare_codes")
 
 
 def bcs_prepare_rows(p: int, r_begin: int, r_end: int, recv_out, workspace, stream=None) -> None:
-    """Second half, for one range (r_begin a multiple of 16): its entries into the round-major copy
-    in `workspace` and, if recv_out is not None, its rank-major receive rows into recv_out."""
+    """Second half, for one range (r_begin a multiple of 16): its receive rows into recv_out, if
+    that is not None."""
     _check(_call.prepare_rows(p, r_begin, r_end, _ptr(recv_out), _ptr(workspace),
                                   _nbytes(workspace), _stream(stream)), "bcs_prepare_rows")
 
 
 def bcs_build_prepared(p: int, r_begin: int, r_end: int, recv_out, send_out, workspace,
                        stream=None) -> None:
-    """Rank-major receive / send rows of a range from a workspace filled by bcs_prepare."""
+    """Rank-major receive / send rows of a range of a p that bcs_prepare was called for."""
     _check(_call.build_prepared(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
                                     _ptr(workspace), _nbytes(workspace), _stream(stream)),
            "bcs_build_prepared")
 
 
 def bcs_build_static(p: int, r_begin: int, r_end: int, recv_out, send_out, stream=None) -> None:
-    """bcs_build with the library's built-in 8 MiB scratch: for callers that cannot allocate or
-    pass a workspace.  Raises BcsError (BCS_ERR_UNSUPPORTED) when the range needs more."""
+    """bcs_build for callers that cannot allocate or pass a workspace.  Raises BcsError
+    (BCS_ERR_UNSUPPORTED) when bcs_build_workspace_bytes of the range is above 8 MiB."""
     _check(_call.build_static(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
                                   _stream(stream)), "bcs_build_static")
 
@@ -349,7 +349,7 @@ def bcs_simulate(p: int, n: int, recv, send, state, counts_out, stream=None) -> 
 
 
 def bcs_wait_expired() -> int:
-    """CTAs of the transposition kernel that gave up waiting for their copies (0 = none)."""
+    """Waits that ran out, 0: no kernel waits with a limit.  Synchronises the device."""
     v = _c.c_uint64(0)
     _check(lib().bcs_wait_expired(_c.byref(v)), "bcs_wait_expired")
     return v.value
