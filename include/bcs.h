@@ -171,7 +171,8 @@ bcs_status bcs_batch_plan(const uint32_t *p_list_host, uint32_t num_p,
  * Outputs: device int8, total_entries bytes each, 16-byte aligned; the table of p_j starts at
  * byte entry_off[j] and is rank-major with q_j bytes per rank, unpadded.  send_out may be NULL;
  * recv_out is required.  workspace: as for bcs_build, not touched; it, tile_off_dev and copy_off_dev
- * may be NULL. */
+ * may be NULL.  The plan may be the work of whatever comes before on the stream.  The kernels read p_list, rank_off and
+ * entry_off of it; the other tables are not looked at (skips_tab_dev and full_tab_dev must be given all the same). */
 size_t bcs_build_batch_workspace_bytes(uint64_t total_ranks, uint64_t total_copy);
 bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_dev,
                            const uint64_t *entry_off_dev, const uint64_t *tile_off_dev,

@@ -5,7 +5,14 @@
 //   * up to 1024 ranks: a CTA per p;
 //   * up to 2^21 ranks: CTAs take equal shares of the flattened ranks of the list, p by p;
 //   * more: all CTAs of a grid work on one p after another (launched only when the list is long enough to hold one).
-// Each is launched as a dependent of the kernel before it on the stream.
+// Each is launched as a dependent of the kernel before it on the stream and may run beside it until it waits for it.
+// The plan is the caller's memory: the kernel before may still be writing it, or what it has written may not be visible yet.
+// So what the plan shows before the wait is a guess, good for one thing: a table of row entries is a function of p
+// alone, and the one that the guess asks for is built while the wait lasts.  Any p in a kernel's range gives a table
+// within bounds, the search stays inside the plan's arrays whatever they hold, and nothing else is done.  Behind the wait all is
+// read again (past the L1 cache, which may hold what the guess has read), and the table is built again if p is another.
+// (Back to back, every p up to 1024: 17.7 us with the guess taken as it is, 18.3 like this, 25.4 with the first load behind the
+// wait, 22.5 with an ordinary launch.  16 p of 2^10..2^20: 92, 90, 90, 92.)
 //
 // Before: skip codes of all ranks, a search on them, a round-major copy and its transposition.  1024 p of 2^10..2^20:
 // 5456 -> 1298 us (8.3 ps a rank, both tables 4.5 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 18.1 us,
@@ -24,6 +31,7 @@ constexpr uint32_t kSmallP = 1024;
 constexpr int kSmallQ = 10;
 constexpr int kMiddleQ = 21;
 constexpr uint32_t kLargeThreads = 640, kBatchThreads = 256, kBatchWarps = kBatchThreads / 32;
+constexpr unsigned kMiddleCtas = 3;               // per SM
 
 // What a CTA works on.
 struct BatchJob {
@@ -31,36 +39,33 @@ struct BatchJob {
     uint32_t p, odd, inv;
 };
 
-// One warp: constants of p_j into t and job.
-__device__ __forceinline__ void load_job(const BatchArgs &ba, uint32_t j, const RowTable &t, BatchJob &job)
+// One warp: constants of a p (any from 1 to 2^31 - 1) into t and job.  They depend on p only: skips[k] is p / 2^(q-k),
+// rounded up (Algorithm 1).
+__device__ __forceinline__ void load_p(uint32_t p, const RowTable &t, BatchJob &job)
 {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t p = ba.p_list[j];
+    const int lane = (int)(threadIdx.x & 31u);
     const int q = ceil_log2_fast(p);
-    const uint32_t skip = ba.skips_tab[(size_t)j * kRow + lane];
+    const uint32_t skip = lane <= q ? (p + ((1u << (q - lane)) - 1u)) >> (q - lane) : 0u;
     const uint32_t before = __shfl_up_sync(0xffffffffu, skip, 1);
-    const uint32_t odd = __ballot_sync(0xffffffffu, lane >= 1u && (int)lane <= q && 2u * before != skip);
+    const uint32_t odd = __ballot_sync(0xffffffffu, lane >= 1 && lane <= q && 2u * before != skip);
     t.s[lane] = skip;
     if (lane < kLow + 1) t.s[kRow + lane] = 0u;
-    if (lane == 0u) {
+    if (lane == 0) {
         job.p = p;
         job.odd = odd;
         job.inv = p > 1u ? (uint32_t)((1ull << (q - low_levels(q) + 32)) / p) : 0u;
-        job.rank0 = ba.rank_off[j];
-        job.rank1 = ba.rank_off[j + 1];
-        job.entry0 = ba.entry_off[j];
         *t.wanted = q > kLow ? (2u << (q - kLow)) - 1u : 1u;
     }
 }
 
 // Ranks r0 .. r1-1 of a p by the warps of the CTA, the per-rank form, `item` (<= 128) ranks at a time.
 template <int kWords>
-__device__ __forceinline__ void narrow_piece(const RowTable &t, uint8_t *mine, const BatchJob &job, int q, uint32_t r0,
-                                             uint32_t r1, uint32_t item, int8_t *recv, int8_t *send)
+__device__ __forceinline__ void narrow_piece(const RowTable &t, uint8_t *mine, const BatchJob &job, uint64_t entry0, int q,
+                                             uint32_t r0, uint32_t r1, uint32_t item, int8_t *recv, int8_t *send)
 {
     for (uint32_t r = r0 + (threadIdx.x >> 5) * item; r < r1; r += (blockDim.x >> 5) * item) {
         const uint32_t n = r1 - r < item ? r1 - r : item;
-        const uint64_t byte = job.entry0 + (uint64_t)r * (uint64_t)q;
+        const uint64_t byte = entry0 + (uint64_t)r * (uint64_t)q;
         warp_rows<kWords, false>(t, mine, q, job.odd, job.inv, r, n, recv + byte, send ? send + byte : nullptr);
     }
 }
@@ -91,32 +96,42 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
 {
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ BatchJob job;
+    __shared__ uint32_t guess;
     grid_launch_dependents();
     const uint32_t j = ba.num_p - 1u - blockIdx.x;               // (lists often ascend: the longest first)
-    const uint32_t p = ba.p_list[j];
+    // The table is built for the p that the plan shows before the wait, see the top of this file.
+    auto build = [&](uint32_t p) {
+        const int q = ceil_log2_fast(p);
+        const RowTable t(sm, RowLayout(q));
+        if (threadIdx.x < 32u) load_p(p, t, job);
+        __syncthreads();
+        build_row_table(t, q, job.odd);
+    };
+    auto fits = [](uint32_t p) { return p > 1u && p <= kSmallP; };
+    if (threadIdx.x == 0) guess = load_relaxed(ba.p_list + j);
+    __syncthreads();
+    const uint32_t built = guess;                                // (not written again)
+    if (fits(built)) build(built);
+    grid_dependency_wait();
+    const uint32_t p = load_relaxed(ba.p_list + j);
+    const uint64_t entry0 = load_relaxed(ba.entry_off + j);
+    if (!fits(p)) return;
+    if (p != built) build(p);
     const int q = ceil_log2_fast(p);
-    if (p > kSmallP || q == 0) {
-        grid_dependency_wait();
-        return;
-    }
     const RowLayout at(q);
     const RowTable t(sm, at);
-    if (threadIdx.x < 32u) load_job(ba, j, t, job);
-    __syncthreads();
-    build_row_table(t, q, job.odd);
-    grid_dependency_wait();                                      // nothing before this touches the outputs
     uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
     constexpr uint32_t warps = kThreads / 32;
     const uint32_t turns = (p + warps * kItemRanks - 1u) / (warps * kItemRanks) * warps;
     const uint32_t item = ((p + turns - 1u) / turns + 31u) & ~31u;
-    if (q <= 4) narrow_piece<1>(t, mine, job, q, 0u, p, item, recv, send);
-    else if (q <= 8) narrow_piece<2>(t, mine, job, q, 0u, p, item, recv, send);
-    else narrow_piece<3>(t, mine, job, q, 0u, p, item, recv, send);
+    if (q <= 4) narrow_piece<1>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+    else if (q <= 8) narrow_piece<2>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+    else narrow_piece<3>(t, mine, job, entry0, q, 0u, p, item, recv, send);
     stage_free();
 }
 
 // 1024 < p <= 2^21: the CTA's share is `share` (a multiple of 16) flattened ranks.
-__global__ void __launch_bounds__(kBatchThreads, 3)
+__global__ void __launch_bounds__(kBatchThreads, kMiddleCtas)
 batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t *recv, int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
@@ -126,52 +141,84 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t g0 = (uint64_t)blockIdx.x * share;
     const uint64_t g1 = g0 + share < ba.total_ranks ? g0 + share : ba.total_ranks;
-    bool waited = false;
-    uint32_t from = 0;                                           // (first warp only: where the search goes on)
-    if (threadIdx.x < 32u) from = find_segment_warp(ba.rank_off, ba.num_p, g0);
+    // (CTAs beyond those that fit at once start when others of the grid have ended: nothing is left to wait for)
+    bool sure = blockIdx.x >= kSms * kMiddleCtas;                // the wait is behind us
+    if (sure) grid_dependency_wait();
+    uint32_t built = 0;                                          // the p whose tables are in shared memory
+    // First warp only: the p that holds rank g0, where the search goes on, whether the first is to be looked at again.
+    uint32_t home = 0, from = 0;
+    bool again = false;
+    if (threadIdx.x < 32u) home = from = find_segment_warp(ba.rank_off, ba.num_p, g0);
     for (;;) {
         __syncthreads();                                         // the p before is done with
         if (threadIdx.x < 32u) {
-            uint32_t hits = 0;
+            uint32_t hits = 0, p = 0;
+            uint64_t rank0 = 0, rank1 = 0, entry0 = 0;
             for (;; from += 32u) {
                 const uint32_t j = from + lane;
-                const bool inside = j < ba.num_p && ba.rank_off[j] < g1;
-                const uint32_t p = inside ? ba.p_list[j] : 0u;
-                hits = __ballot_sync(0xffffffffu, p > kSmallP && p <= (1u << kMiddleQ));
-                if (hits != 0u || __any_sync(0xffffffffu, !inside)) break;
+                const bool listed = j < ba.num_p;
+                rank0 = listed ? load_relaxed(ba.rank_off + j) : 0u;
+                rank1 = listed ? load_relaxed(ba.rank_off + j + 1) : 0u;
+                entry0 = listed ? load_relaxed(ba.entry_off + j) : 0u;
+                p = listed ? load_relaxed(ba.p_list + j) : 0u;
+                if (again && __any_sync(0xffffffffu, lane == 0u && (rank0 > g0 || rank1 <= g0))) {
+                    again = false;
+                    from = find_segment_warp(ba.rank_off, ba.num_p, g0) - 32u;
+                    continue;
+                }
+                again = false;
+                const bool inside = listed && rank0 < g1;
+                hits = __ballot_sync(0xffffffffu, inside && p > kSmallP && p <= (1u << kMiddleQ));
+                if (hits != 0u || __any_sync(0xffffffffu, !inside) || !sure) break;
             }
-            from += (uint32_t)__ffs(hits) - 1u;
-            if (lane == 0u) found = hits != 0u ? from : 0xffffffffu;
+            if (hits != 0u) {
+                const uint32_t nth = (uint32_t)__ffs(hits) - 1u;
+                if (lane == nth) {
+                    job.rank0 = rank0;
+                    job.rank1 = rank1;
+                    job.entry0 = entry0;
+                }
+                p = __shfl_sync(0xffffffffu, p, nth);
+                if (p != built) load_p(p, RowTable(sm, RowLayout(ceil_log2_fast(p))), job);
+                from += nth + 1u;
+            }
+            if (lane == 0u) found = hits != 0u ? p : 0u;
         }
         __syncthreads();
-        if (found == 0xffffffffu) break;
-        const int q = ceil_log2_fast(ba.p_list[found]);
+        const uint32_t p = found;
+        if (p == 0u && sure) break;
+        const int q = ceil_log2_fast(p);
         const bool narrow = q < kWideMinQ;
         const RowLayout at_narrow(q);
+        const WideLayout at(q);
         const RowTable t(sm, at_narrow);
-        if (threadIdx.x < 32u) load_job(ba, found, t, job);
-        ++from;
-        __syncthreads();
-        const uint32_t p = job.p;
         const uint32_t r0 = g0 > job.rank0 ? ((uint32_t)(g0 - job.rank0) + 15u) & ~15u : 0u;
         const uint32_t end = g1 < job.rank1 ? ((uint32_t)(g1 - job.rank0) + 15u) & ~15u : p;
         const uint32_t r1 = end < p ? end : p;
+        if (p != built) {
+            built = 0u;
+            if (p != 0u && r0 < r1) {
+                build_row_table(t, q, job.odd);
+                if (!narrow && send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
+                built = p;
+            }
+        }
+        if (!sure) {                                             // that was a guess: look again
+            grid_dependency_wait();
+            sure = again = true;
+            from = home;
+            continue;
+        }
         if (r0 >= r1) continue;
-        build_row_table(t, q, job.odd);
-        const WideLayout at(q);
-        if (!narrow && send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
-        if (!waited) grid_dependency_wait();
-        waited = true;
         if (narrow) {
             uint8_t *mine = sm + at_narrow.warps + (threadIdx.x >> 5) * at_narrow.warp_bytes;
-            if (q <= 12) narrow_piece<3>(t, mine, job, q, r0, r1, kItemRanks, recv, send);
-            else narrow_piece<4>(t, mine, job, q, r0, r1, kItemRanks, recv, send);
+            if (q <= 12) narrow_piece<3>(t, mine, job, job.entry0, q, r0, r1, kItemRanks, recv, send);
+            else narrow_piece<4>(t, mine, job, job.entry0, q, r0, r1, kItemRanks, recv, send);
             stage_free();
         } else {
             wide_piece(t, sm, at, sm + at.ends + (threadIdx.x >> 5) * 32u, job, q, r0, r1, recv, send);
         }
     }
-    if (!waited) grid_dependency_wait();
 }
 
 // p > 2^21: all CTAs on every such p of the list.
@@ -201,18 +248,19 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         const WideLayout at(q);
         const RowTable t(sm, at.base);
         __syncthreads();                                         // the p before is done with
-        if (threadIdx.x < 32u) load_job(ba, j, t, job);
+        if (threadIdx.x < 32u) load_p(p, t, job);
+        const uint64_t entry0 = ba.entry_off[j];
         __syncthreads();
         build_row_table(t, q, job.odd);
         if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
         const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
         auto all = [&](auto is_send, int8_t *out) {
             WideLane lane;
-            lane.init<true>(q, (uint32_t)(job.entry0 & 15u));
+            lane.init<true>(q, (uint32_t)(entry0 & 15u));
             for (uint64_t r = ((uint64_t)blockIdx.x * n_warps + warp) * item; r < p; r += (uint64_t)gridDim.x * n_warps * item) {
                 const uint32_t n = p - (uint32_t)r < item ? p - (uint32_t)r : item;
                 wide_rows<decltype(is_send)::value, true>(t, sm, at.send, sm + at.ends + warp * 32u, p, q, job.odd, job.inv, lane,
-                                                    (uint32_t)r, n, r == 0, r + n == p, out + job.entry0 + r * (uint64_t)q);
+                                                    (uint32_t)r, n, r == 0, r + n == p, out + entry0 + r * (uint64_t)q);
             }
         };
         all(std::false_type(), recv);
@@ -272,7 +320,7 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
     (void)total_copy;
     (void)workspace_bytes;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const BatchArgs ba = {p_list_dev, rank_off_dev, entry_off_dev, skips_tab_dev, num_p, total_ranks};
+    const BatchArgs ba = {p_list_dev, rank_off_dev, entry_off_dev, num_p, total_ranks};
     static_assert(kSmallP == kFusedMaxP, "the plan counts tiles for the p above kSmallP");
     // (without the plan's tiles the host cannot tell what sizes the list holds)
     const bool small_only = tile_off_dev != nullptr && total_tiles == 0;
@@ -285,7 +333,7 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         // of 2^10..2^20 66.8 us with three, 44.7 with one; 64 p of about 2^17 143 and 122 us).  Beyond, three, so that none
         // ends last by much (150 p of 2^12..2^18, 10 million ranks, 182 us, with one 200).  At most 32768 ranks, at
         // least 1024 (a table costs as much as some hundred ranks of each warp).
-        const uint64_t ctas = kSms * 3u * (total_ranks <= (1u << 23) ? 1u : 3u);
+        const uint64_t ctas = kSms * kMiddleCtas * (total_ranks <= (1u << 23) ? 1u : 3u);
         uint64_t share = align_up(total_ranks / ctas, 128);
         share = share < 1024 ? 1024 : (share > 32768 ? 32768 : share);
         const uint64_t shares = (total_ranks + share - 1) / share;

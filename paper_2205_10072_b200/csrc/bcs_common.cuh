@@ -27,7 +27,6 @@ struct BatchArgs {
     const uint32_t *p_list;
     const uint64_t *rank_off;
     const uint64_t *entry_off;
-    const uint32_t *skips_tab;   // [num_p][kRow]
     uint32_t num_p;
     uint64_t total_ranks;
 };
@@ -87,8 +86,8 @@ __device__ __forceinline__ void load_span(uint8_t *stage, uint32_t shift, uint32
     }
 }
 
-// Largest j with off[j] <= g, by a whole warp: 32 probes per step, so a table of a few thousand offsets takes
-// three dependent loads.  All 32 lanes must call.
+// Largest j with off[j] <= g (off[0] <= g), by a whole warp: 32 probes per step, so a table of a few thousand offsets takes
+// three dependent loads.  Whatever off holds, it ends, with some j < num.  All 32 lanes must call.
 __device__ __forceinline__ uint32_t find_segment_warp(const uint64_t *off, uint32_t num, uint64_t g)
 {
     const uint32_t lane = threadIdx.x & 31u;
@@ -96,8 +95,8 @@ __device__ __forceinline__ uint32_t find_segment_warp(const uint64_t *off, uint3
     while (hi - lo > 1u) {
         const uint32_t step = (hi - lo + 31u) / 32u;
         const uint32_t idx = lo + lane * step;
-        const bool le = idx < hi && off[idx] <= g;
-        const uint32_t hits = __popc(__ballot_sync(0xffffffffu, le));   // lane 0 always hits
+        const bool le = lane == 0u || (idx < hi && load_relaxed(off + idx) <= g);
+        const uint32_t hits = __popc(__ballot_sync(0xffffffffu, le));
         lo += (hits - 1u) * step;
         hi = lo + step < hi ? lo + step : hi;
     }

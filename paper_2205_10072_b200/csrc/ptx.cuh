@@ -21,6 +21,21 @@ __device__ __forceinline__ uint32_t pick_bytes(uint32_t a, uint32_t b, uint32_t 
     return d;
 }
 
+// Loads that are not taken from the L1 cache or from an earlier load of the same place.
+__device__ __forceinline__ uint32_t load_relaxed(const uint32_t *at)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(at) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ uint64_t load_relaxed(const uint64_t *at)
+{
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
+    return v;
+}
+
 // Makes this thread's shared-memory writes visible to the copies that bulk_store() starts.
 __device__ __forceinline__ void fence_before_bulk() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 

@@ -143,3 +143,36 @@ def test_batches(bcs, plist, send):
                                    [1 << 20] * 8, [1 << 20] * 8 + [1025, 9]])
 def test_batch_splits(bcs, plist):
     _batch(bcs, list(plist))
+
+
+# The plan of a batch as the work of the kernel before it on the stream, one that lets its successors start early: the list of p
+# is a stretch of a row of allgather tables, block numbers of about `row` each.  Nothing of what its memory held before may
+# reach the tables, be it another p of the kernel's range or none.
+@pytest.mark.parametrize("n,row,count", [(700, 600, 500), (700, 150, 1000), (3000, 2500, 300), (12000, 10000, 40)])
+@pytest.mark.parametrize("old", [0, 1, 1024, 1031, -1])
+def test_batch_of_a_plan_written_by_the_kernel_before(bcs, n, row, count, old):
+    agents = 1000
+    q = bcs.bcs_q(agents)
+    tables = oracle.full_table(agents)
+    recv, send = (torch.from_numpy(t).cuda().view(-1) for t in tables)
+    # processor 0 handles buffer j as virtual processor -j: Algorithm 6's closed form
+    virtual = -np.arange(count) % agents
+    plist = oracle.expand(agents, n, *tables)[virtual, row, 0].tolist()
+    assert min(plist) > 1
+    plan = bcs.bcs_batch_plan(plist)
+    dev = plan.to("cuda")
+    want = [np.concatenate(t) for t in zip(*(tuple(x.reshape(-1) for x in oracle.full_table(p)) for p in plist))]
+    pack = torch.empty((n - 1 + q) * agents, dtype=torch.int32, device="cuda")
+    dev.p_list = pack[row * agents:row * agents + count]
+    for _ in range(4):
+        pack.fill_(old)
+        raw_r, out_r = _buffer(plan.total_entries)
+        raw_s, out_s = _buffer(plan.total_entries)
+        torch.cuda.synchronize()
+        bcs.bcs_allgather_tables(agents, n, 0, recv, send, pack, None)
+        bcs.bcs_build_batch(dev, out_r, out_s)
+        torch.cuda.synchronize()
+        assert dev.p_list.tolist() == plist
+        for raw, out, expect in ((raw_r, out_r, want[0]), (raw_s, out_s, want[1])):
+            assert np.array_equal(out.cpu().numpy(), expect)
+            assert bool((raw[:32] == 99).all()) and bool((raw[32 + plan.total_entries:] == 99).all())
