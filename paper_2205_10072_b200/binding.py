@@ -122,13 +122,14 @@ class _Calls:
 
     def __getattr__(self, name):
         library = lib()
-        call = getattr(_extension(), name, None) or getattr(library, "bcs_" + name)
+        call = getattr(_extension(library), name, None) or getattr(library, "bcs_" + name)
         setattr(self, name, call)
         return call
 
 
-def _extension():
-    """The extension module linked to the library that lib() has loaded, or None."""
+def _extension(library):
+    """The extension module linked to the library that lib() has loaded, or None.  Arguments that are not plain integers
+    (or None for an address) it hands on to `library`."""
     if build_ext.LIB_PATH != os.path.join(os.path.dirname(build_ext.CALLS_PATH), "libbcs.so") or \
             not os.path.exists(build_ext.CALLS_PATH):
         return None
@@ -136,6 +137,7 @@ def _extension():
         from . import _calls
     except ImportError:
         return None
+    _calls.set_library(library)
     return _calls
 
 

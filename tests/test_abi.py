@@ -116,3 +116,34 @@ def test_argument_errors_need_no_gpu(lib):
     assert L.bcs_expand(10, 4, 0, 10, None, None, None, None) == 1             # no table to write to
     assert L.bcs_build_to_host(10, 0, 10, None, None, 16, 1024, None) == 1
     assert L.bcs_build_to_host(10, 0, 10, 16, None, 16, 16, None) == 1   # staging too small
+
+
+def test_arguments_that_the_fast_calls_take_are_those_of_ctypes(lib):
+    """The calls through the extension module refuse what ctypes refuses (None or a fraction as a number) and take what it
+    takes (its own integers and pointers); empty ranges, so that nothing is enqueued."""
+    import ctypes
+    from types import SimpleNamespace
+    from paper_2205_10072_b200 import binding
+    stream = SimpleNamespace(cuda_stream=0)
+    at = SimpleNamespace(data_ptr=lambda: ctypes.c_void_p(0), nbytes=0)
+    for p in (10, True, ctypes.c_uint32(10)):
+        lib.bcs_build(p, 0, 0, None, None, stream=stream)
+    lib.bcs_build(10, ctypes.c_uint64(3), 3, at, at, at, stream=stream)
+    lib.bcs_expand(10, 4, 3, 3, at, None, None, stream=stream)
+    lib.bcs_build_rooted(10, 3, 3, 3, None, at, stream=stream)
+    for number in (None, 3.0, "3"):
+        for call in (lambda: lib.bcs_build(10, number, 3, None, None, stream=stream),
+                     lambda: lib.bcs_build(number, 0, 0, None, None, stream=stream),
+                     lambda: lib.bcs_build_rooted(10, number, 3, 3, None, None, stream=stream),
+                     lambda: lib.bcs_build_static(10, 0, number, None, None, stream=stream),
+                     lambda: lib.bcs_prepare(number, None, stream=stream),
+                     lambda: lib.bcs_prepare_codes(number, None, stream=stream),
+                     lambda: lib.bcs_prepare_rows(10, number, 0, None, at, stream=stream),
+                     lambda: lib.bcs_build_prepared(10, number, 0, None, None, at, stream=stream),
+                     lambda: lib.bcs_expand(10, 4, number, 0, None, None, None, stream=stream),
+                     lambda: lib.bcs_allgather_tables(1, 4, number, None, None, None, None, stream=stream),
+                     lambda: binding._call.build_batch(0, 0, 0, 0, 0, 0, 0, number, 0, 0, 0, 0, None, None, None, 0, None)):
+            with pytest.raises(ctypes.ArgumentError):
+                call()
+    with pytest.raises(TypeError):                               # too few
+        binding._call.build(10, 0, 0)
