@@ -165,13 +165,23 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     for (int k = 1; k <= rc.q; ++k) rc.odd |= (2u * rc.s[k - 1] - rc.s[k]) << k;
     rc.inv = (uint32_t)((1ull << (rc.q - low_levels(rc.q) + 32)) / p);
     const uint32_t ranks = (uint32_t)count, x0 = (uint32_t)first;
-    // The wide kernel from 96 Ki ranks on (its tables take longer to build: 65 000 ranks 5.8 against 4.1 us here).  Up to
+    // The wide kernel where the per-rank form is the slower one back to back.  That gets slower in steps: above 148 x 16 x 32 ranks
+    // (75 776) a CTA has more than 16 warps and the next call's does not fit beside it, above 148 x 32 x 32 (151 552) items have
+    // more than 32 ranks.  The wide kernel's tables cost more the larger q is.  Both tables, us, per rank / wide:
+    //     ranks      q = 17    q = 19    q = 21    q = 22    q = 24    q = 26    q = 30
+    //     65 536    4.2/5.8   4.3/6.2   4.4/6.7   4.4/6.8   4.4/7.5   4.3/7.8   4.1/8.2
+    //     81 920    4.8/6.0   4.7/6.3   4.8/7.0   4.8/7.1   4.8/7.9   7.2/7.9   6.8/8.4
+    //     90 112    6.9/6.0   6.9/6.3   7.2/6.9   7.2/7.1   7.2/7.8   7.2/8.0   6.7/8.3
+    //     98 304    7.5/6.1   7.5/6.4   7.4/7.0   7.4/7.2   7.4/8.0   7.5/8.1   7.1/8.5
+    //    131 072              7.4/6.7   7.5/7.4   7.5/7.5   7.6/8.2   7.5/8.3   7.2/8.7
+    //    163 840              9.4/6.9   9.7/7.6  10.5/7.8  10.8/8.5  11.0/8.6  10.7/8.9
+    // (One call and a wait for it: the per-rank form 18 us, the wide one 20 at q = 17, 22 at 21, 24 from 24 on.)  Up to
     // 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
     // are built beside it (with steps of 16 ranks: 700 001 ranks 12.3 us, 13.7 with 640 threads, 14.9 per rank; 1.3 million 18.2, 18.0, 23.4; 2.1
     // million 21.4, 20.6, 29.3).  Beyond, all receive rows before the send rows, item by item: an item's start costs as
     // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
     // faster (12.3 million ranks 54 us a table with items of 800, 61 with 400; 2^25: 151 and 146 us).
-    if (rc.q >= kWideMinQ && count >= 98304) {
+    if (rc.q >= kWideMinQ && count >= (rc.q <= 22 ? 98304u : kSms * 32u * 32u + 1u)) {
         const bool halves = count < (1u << 23);
         auto run = [&](uint32_t warps) {
             if (recv != nullptr && send != nullptr) warps /= 2;

@@ -65,7 +65,7 @@ def test_rows_of_ranges(bcs, p):
 
 
 @pytest.mark.parametrize("n", [98303, 98304, 1 << 20, (1 << 20) + 1, 148 * 32 * 32 - 1, 148 * 32 * 32 + 1, 148 * 32 * 64, 148 * 32 * 128 + 77])
-@pytest.mark.parametrize("p", [(1 << 20) + 1, 3000017])
+@pytest.mark.parametrize("p", [(1 << 20) + 1, 3000017, (1 << 22) + 1, 40000003])
 def test_rows_where_the_split_changes(bcs, p, n):
     r0 = 1234567 % (p - n + 1)
     _check(bcs, p, r0, r0 + n)
@@ -76,6 +76,16 @@ def test_rows_where_the_split_changes(bcs, p, n):
                                     ((1 << 23) + 1, (1 << 22) + 12345, 100001), (1 << 24, (1 << 23) - 200000, 400009)])
 def test_rows_of_other_steps(bcs, p, r0, n):
     _check(bcs, p, r0, r0 + n)
+
+
+# the wide form places bytes by q: each q that the tests above leave out, skips that are all odd but the first ones or all even
+# or neither, from an odd rank on, in the launches of up to 2^20 ranks (the per-rank form ends at 151 552) and above it
+@pytest.mark.parametrize("p", [(1 << q - 1) + 1 for q in (23, 24, 25, 26, 27, 28, 29)] + [(1 << q) - 1 for q in (23, 25, 26, 27, 28, 29)] +
+                              [(3 << q - 2) + 12345 for q in (23, 24, 25, 26, 27, 28, 29)])
+def test_wide_rows_of_every_q(bcs, p):
+    for n in (151553, (1 << 20) + 77):
+        for r0 in ((p - n) // 2 | 1, p - n):
+            _check(bcs, p, r0, r0 + n)
 
 
 # the kernel for 2^23 ranks and more: its lanes' places repeat every 16 ranks, 30 segments are located at a time
