@@ -175,13 +175,14 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     //     98 304    7.5/6.1   7.5/6.4   7.4/7.0   7.4/7.2   7.4/8.0   7.5/8.1   7.1/8.5
     //    131 072              7.4/6.7   7.5/7.4   7.5/7.5   7.6/8.2   7.5/8.3   7.2/8.7
     //    163 840              9.4/6.9   9.7/7.6  10.5/7.8  10.8/8.5  11.0/8.6  10.7/8.9
-    // (One call and a wait for it: the per-rank form 18 us, the wide one 20 at q = 17, 22 at 21, 24 from 24 on.)  Up to
+    // Without send rows there is no send table: 98 304 ranks of q = 26 then take 6.5 and 5.9 us.  (One call with both and a wait for
+    // it: the per-rank form 18 us, the wide one 20 at q = 17, 22 at 21, 24 from 24 on.)  Up to
     // 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
     // are built beside it (with steps of 16 ranks: 700 001 ranks 12.3 us, 13.7 with 640 threads, 14.9 per rank; 1.3 million 18.2, 18.0, 23.4; 2.1
     // million 21.4, 20.6, 29.3).  Beyond, all receive rows before the send rows, item by item: an item's start costs as
     // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
     // faster (12.3 million ranks 54 us a table with items of 800, 61 with 400; 2^25: 151 and 146 us).
-    if (rc.q >= kWideMinQ && count >= (rc.q <= 22 ? 98304u : kSms * 32u * 32u + 1u)) {
+    if (rc.q >= kWideMinQ && count >= (rc.q <= 22 || send == nullptr ? 98304u : kSms * 32u * 32u + 1u)) {
         const bool halves = count < (1u << 23);
         auto run = [&](uint32_t warps) {
             if (recv != nullptr && send != nullptr) warps /= 2;
