@@ -12,7 +12,7 @@
 // within bounds, the search stays inside the plan's arrays whatever they hold, and nothing else is done.  Behind the wait all is
 // read again (past the L1 cache, which may hold what the guess has read), and the table is built again if p is another.
 // (Back to back, every p up to 1024: 17.7 us with the guess taken as it is, 18.3 like this, 25.4 with the first load behind the
-// wait, 22.5 with an ordinary launch.  16 p of 2^10..2^20: 92, 90, 90, 92.)
+// wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8, 18.7.)
 //
 // Before: skip codes of all ranks, a search on them, a round-major copy and its transposition.  1024 p of 2^10..2^20:
 // 5456 -> 1298 us (8.3 ps a rank, both tables 4.5 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 18.1 us,
@@ -137,6 +137,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ BatchJob job;
     __shared__ uint32_t found;
+    __shared__ uint32_t home, from;                              // first warp only: what a guess has found to hold rank g0, where to look on
     grid_launch_dependents();
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t g0 = (uint64_t)blockIdx.x * share;
@@ -145,17 +146,19 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
     bool sure = blockIdx.x >= kSms * kMiddleCtas;                // the wait is behind us
     if (sure) grid_dependency_wait();
     uint32_t built = 0;                                          // the p whose tables are in shared memory
-    // First warp only: the p that holds rank g0, where the search goes on, whether the first is to be looked at again.
-    uint32_t home = 0, from = 0;
-    bool again = false;
-    if (threadIdx.x < 32u) home = from = find_segment_warp(ba.rank_off, ba.num_p, g0);
+    if (threadIdx.x < 32u) {
+        const uint32_t j = find_segment_warp(ba.rank_off, ba.num_p, g0);
+        if (lane == 0u) home = from = j;
+    }
     for (;;) {
         __syncthreads();                                         // the p before is done with
         if (threadIdx.x < 32u) {
             uint32_t hits = 0, p = 0;
             uint64_t rank0 = 0, rank1 = 0, entry0 = 0;
-            for (;; from += 32u) {
-                const uint32_t j = from + lane;
+            uint32_t base = from;
+            bool again = base == home;
+            for (;; base += 32u) {
+                const uint32_t j = base + lane;
                 const bool listed = j < ba.num_p;
                 rank0 = listed ? load_relaxed(ba.rank_off + j) : 0u;
                 rank1 = listed ? load_relaxed(ba.rank_off + j + 1) : 0u;
@@ -163,7 +166,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
                 p = listed ? load_relaxed(ba.p_list + j) : 0u;
                 if (again && __any_sync(0xffffffffu, lane == 0u && (rank0 > g0 || rank1 <= g0))) {
                     again = false;
-                    from = find_segment_warp(ba.rank_off, ba.num_p, g0) - 32u;
+                    base = find_segment_warp(ba.rank_off, ba.num_p, g0) - 32u;
                     continue;
                 }
                 again = false;
@@ -180,9 +183,15 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
                 }
                 p = __shfl_sync(0xffffffffu, p, nth);
                 if (p != built) load_p(p, RowTable(sm, RowLayout(ceil_log2_fast(p))), job);
-                from += nth + 1u;
+                base += nth + 1u;
             }
-            if (lane == 0u) found = hits != 0u ? p : 0u;
+            if (lane == 0u) {
+                found = hits != 0u ? p : 0u;
+                if (sure) {                                      // (a guess is looked at again)
+                    from = base;
+                    home = 0xffffffffu;
+                }
+            }
         }
         __syncthreads();
         const uint32_t p = found;
@@ -205,8 +214,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
         }
         if (!sure) {                                             // that was a guess: look again
             grid_dependency_wait();
-            sure = again = true;
-            from = home;
+            sure = true;
             continue;
         }
         if (r0 >= r1) continue;
