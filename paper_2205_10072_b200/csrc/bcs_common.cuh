@@ -144,17 +144,20 @@ inline void launch_dependent(bool dependent, void (*kernel)(Params...), dim3 gri
     cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
 }
 
-// Opts a kernel in to large dynamic shared memory (what a little static use leaves of 227 KB), once per device.
+// Opts a kernel in to large dynamic shared memory (what a little static use leaves of 227 KB), once per device.  If the
+// runtime refuses, its error is not left for launch_status() of a later call.
 template <auto kKernel>
 bool allow_shared()
 {
     static std::atomic<uint64_t> done{0};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess;
     const uint64_t bit = dev < 64 ? 1ull << dev : 0;
-    if (done.load(std::memory_order_relaxed) & bit) return true;
-    if (cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess)
+    if (known && (done.load(std::memory_order_relaxed) & bit)) return true;
+    if (!known || cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess) {
+        (void)cudaGetLastError();
         return false;
+    }
     done.fetch_or(bit, std::memory_order_relaxed);
     return true;
 }

@@ -147,3 +147,19 @@ def test_arguments_that_the_fast_calls_take_are_those_of_ctypes(lib):
                 call()
     with pytest.raises(TypeError):                               # too few
         binding._call.build(10, 0, 0)
+
+
+def test_a_refused_call_leaves_no_error_behind(tmp_path):
+    """The opt-in to large shared memory, refused by the runtime (here, because there is no device), takes its error with it: the
+    next call asks the runtime for the last one."""
+    import subprocess
+    from paper_2205_10072_b200 import build_ext
+    source = tmp_path / "refused.cu"
+    source.write_text('#include "bcs_common.cuh"\n#include <stdio.h>\n__global__ void kernel() {}\nint main() {\n'
+                      '    const bool allowed = bcs::allow_shared<kernel>();\n'
+                      '    printf("%d %d", (int)allowed, (int)cudaPeekAtLastError());\n}\n')
+    flags = [f for f in build_ext.NVCC_FLAGS if f != "--shared"]
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + flags +
+                          ["-I", os.path.join(os.path.dirname(build_ext.LIB_PATH), "csrc"), "-o", str(tmp_path / "refused"), str(source)])
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")
+    assert subprocess.check_output([str(tmp_path / "refused")], env=env, text=True) == "0 0"
