@@ -149,17 +149,39 @@ def test_arguments_that_the_fast_calls_take_are_those_of_ctypes(lib):
         binding._call.build(10, 0, 0)
 
 
+FAKE_RUNTIME = r"""
+#include <cuda_runtime.h>
+#include <stdio.h>
+static cudaError_t last = cudaSuccess;
+static bool device = false;
+static cudaError_t fail(cudaError_t e) { return last = e; }
+static cudaError_t fake_device(int *dev) { *dev = 0; return device ? cudaSuccess : fail(cudaErrorNoDevice); }
+template <class T> static cudaError_t fake_attribute(T, cudaFuncAttribute, int) { return fail(cudaErrorInvalidValue); }
+static cudaError_t fake_last() { const cudaError_t e = last; last = cudaSuccess; return e; }
+#define cudaGetDevice fake_device
+#define cudaFuncSetAttribute fake_attribute
+#define cudaGetLastError fake_last
+#include "bcs_common.cuh"
+__global__ void kernel() {}
+int main()
+{
+    for (int i = 0; i < 2; ++i) {
+        device = i == 1;
+        const bool allowed = bcs::allow_shared<kernel>();
+        printf("%d %d ", (int)allowed, (int)bcs::launch_status());
+    }
+}
+"""
+
+
 def test_a_refused_call_leaves_no_error_behind(tmp_path):
-    """The opt-in to large shared memory, refused by the runtime (here, because there is no device), takes its error with it: the
-    next call asks the runtime for the last one."""
+    """The opt-in to large shared memory, refused by the runtime (a fake here), takes its error with it: the next call asks for the
+    last one after its launch."""
     import subprocess
     from paper_2205_10072_b200 import build_ext
     source = tmp_path / "refused.cu"
-    source.write_text('#include "bcs_common.cuh"\n#include <stdio.h>\n__global__ void kernel() {}\nint main() {\n'
-                      '    const bool allowed = bcs::allow_shared<kernel>();\n'
-                      '    printf("%d %d", (int)allowed, (int)cudaPeekAtLastError());\n}\n')
+    source.write_text(FAKE_RUNTIME)
     flags = [f for f in build_ext.NVCC_FLAGS if f != "--shared"]
     subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + flags +
                           ["-I", os.path.join(os.path.dirname(build_ext.LIB_PATH), "csrc"), "-o", str(tmp_path / "refused"), str(source)])
-    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")
-    assert subprocess.check_output([str(tmp_path / "refused")], env=env, text=True) == "0 0"
+    assert subprocess.check_output([str(tmp_path / "refused")], text=True) == "0 0 0 0 "
