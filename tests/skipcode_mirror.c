@@ -1,8 +1,9 @@
 /*
- * skipcode_mirror.c -- CPU restatement, with operation counters, of the construction that the
- * fast CUDA kernels run (TEST INFRASTRUCTURE; shares no code with the kernels or the oracle).
+ * skipcode_mirror.c -- a construction of the schedules on skip codes, with operation counters: an
+ * independent check of the oracle (TEST INFRASTRUCTURE; shares no code with it or with the library, whose
+ * kernels compute rows in another way).
  *
- * The kernels do not descend the homeranges as Algorithm 3 of arXiv 2205.10072 does.  They give
+ * It does not descend the homeranges as Algorithm 3 of arXiv 2205.10072 does.  It gives
  * every rank x a "skip code": x is written as a sum of distinct skips, largest first (the sums
  * that Algorithm 2 walks down), and bit k of code(x) says whether skips[k] is a term.  The
  * lowest set bit is the baseblock of x, the highest its homerange, and codes order like ranks.
@@ -13,8 +14,7 @@
  * This file computes receive and send rows that way, one rank at a time, in plain C, and counts
  * the integer operations an ideal translation of each step needs (no address arithmetic beyond
  * what the step itself requires, no loop overhead).  The tests compare its rows with the
- * oracle's; the benchmark takes its operation counts as the model numerator of the integer
- * roofline.  Operations shared by the four consecutive ranks that a GPU thread handles are
+ * oracle's.  Operations that four consecutive ranks handled together would share are
  * counted as a quarter each: all counters are in QUARTER operations.
  */
 #include <stdint.h>
@@ -49,8 +49,8 @@ typedef struct {
     const uint32_t *codes;           /* codes of all ranks when the caller has them, else NULL */
 } skm_ctx;
 
-/* Which rounds are decided from exact window sets: 0 = as the GPU kernels do (the rounds with
- * skips[i+1] <= 33 when p >= 64), 1 = none (every round by the code search), 2 = those rounds
+/* Which rounds are decided from exact window sets: 0 = the rounds with
+ * skips[i+1] <= 33 when p >= 64, 1 = none (every round by the code search), 2 = those rounds
  * for every p.  All three must give the same rows. */
 static int g_table_mode = 0;
 void skm_set_table_mode(int mode) { g_table_mode = mode; }
@@ -169,8 +169,8 @@ static void recv_row(const skm_ctx *c, uint32_t r, int last, int8_t *row, uint64
             cnt[SKM_HOME_OPS] += Q4(1);
             cnt[SKM_ROUNDS_HOME] += 1;
         } else if (i < c->table_rounds) {
-            /* Short windows: both windows as exact block sets (on the GPU four words of the
-             * tile's run table: 4 loads, 2 or, 2 and-not), first window unless it is empty of
+            /* Short windows: both windows as exact block sets (four words of a
+             * run table: 4 loads, 2 or, 2 and-not), first window unless it is empty of
              * new blocks (1 select), then leading bit, its mask, entry, set update. */
             uint32_t U = window_set(c, r, lo, hi - lo) & ~B;
             if (U == 0 && c->len2[i]) U = window_set(c, r, hi, c->len2[i]) & ~B;
@@ -249,11 +249,11 @@ static void recv_row(const skm_ctx *c, uint32_t r, int last, int8_t *row, uint64
  * level and rank.  ops[1] = blocks, ops[2] = blocks with a splitting level, ops[3] = plain. */
 #define SKM_LOW 8
 #define SKM_BLOCK 32          /* ranks per scan for q > 22; 16 for a smaller p */
-static int g_batch = 0;       /* the batch kernel scans 32 ranks at a time for every q */
+static int g_batch = 0;       /* 32 ranks at a time for every q */
 void skm_set_batch(int on) { g_batch = on; }
 static uint32_t block_of(int q) { return (q <= 22 && !g_batch) ? 16u : SKM_BLOCK; }
-#define SKM_BLOCKS_FROM 8192   /* smaller p are charged the plain scan, 3 per level and rank (the
-                                  GPU scans them rank by rank: most blocks would cross p) */
+#define SKM_BLOCKS_FROM 8192   /* smaller p are charged the plain scan, 3 per level and rank (most
+                                  blocks would cross p) */
 
 static void codes_block(const skm_ctx *c, const uint16_t *low, int low_levels, uint32_t g,
                         uint32_t *out /* 32, or NULL */, uint64_t *ops)
@@ -339,7 +339,7 @@ int skm_codes_plain(uint32_t p, uint64_t g_begin, uint64_t g_end, uint32_t *code
 }
 
 /* ------------------------------------------------------------ small p, everything in one block
- * What the batch kernel for p <= 1024 does: the baseblock bits of all ranks as level 0 of a table
+ * For p <= 1024: the baseblock bits of all ranks as level 0 of a table
  * run[l][x] = bits of the 2^l ranks that end at x (cyclically; the root has no bit), one level
  * from the one below; a window of L ranks that ends at rank e is run[l][e] | run[l][e - (L - 2^l)]
  * with l = floor(log2 L); every round of every rank looks its first window up, and the second one
@@ -441,7 +441,7 @@ int skm_q(uint32_t p)
 
 /* Receive and send rows of the listed ranks.  recv, send: n * q bytes, rank-major; either may
  * be NULL.  A send entry is the receive entry of the to-processor in that round; the counters
- * charge it as the GPU obtains it -- a lookup in the round-major receive table (per four
+ * charge a lookup in a round-major receive table (per four
  * entries two word loads, a funnel shift, three byte merges and a store: 7/4 per entry). */
 int skm_rows(uint32_t p, const uint64_t *ranks, uint64_t n, int8_t *recv, int8_t *send,
              uint64_t *counters /* SKM_NCOUNT, accumulated */)

@@ -1,11 +1,10 @@
-"""Python access to skipcode_mirror.c: the CPU restatement, with operation counters, of the
-skip-code construction that the fast CUDA kernels run (test infrastructure).
+"""Python access to skipcode_mirror.c: a construction on skip codes with operation counters, an independent check of the
+oracle (test infrastructure; the library's kernels compute rows in another way).
 
     python -m tests.skipcode_mirror --write     rewrites tests/skipcode_model_ops.json
 
-The JSON table holds the model's integer operations per rank for the benchmark's workloads
-(q = 17, 21, 30 and the batched mix); bench.py reads it as the model numerator of the integer
-roofline.  Nothing here touches the CUDA library or the oracle.
+The JSON table holds that construction's integer operations per rank for the benchmark's workloads
+(q = 17, 21, 30 and the batched mix).  Nothing here touches the CUDA library or the oracle.
 """
 from __future__ import annotations
 
@@ -55,13 +54,12 @@ def _load():
 
 
 def set_table_mode(mode: int) -> None:
-    """0: short windows from exact sets when p >= 64 (as the GPU); 1: never; 2: for every p."""
+    """0: short windows from exact sets when p >= 64; 1: never; 2: for every p."""
     _load().skm_set_table_mode(mode)
 
 
 def set_batch(on: bool) -> None:
-    """Codes as the batch kernel scans them (32 ranks per scan for every q) or as the kernel of
-    one p does (16 for q <= 22)."""
+    """Codes in scans of 32 ranks for every q, or of 16 for q <= 22."""
     _load().skm_set_batch(1 if on else 0)
 
 
@@ -101,8 +99,8 @@ def rows(p: int, ranks, want_send: bool = True):
 
 
 def small(p: int, want_send: bool = True):
-    """(recv [p][q], send [p][q] or None, counters) for all ranks of a p <= 1024 by the run table
-    over all ranks (what the batch kernel for small p does)."""
+    """(recv [p][q], send [p][q] or None, counters) for all ranks of a p <= 1024 by a run table
+    over all ranks."""
     L = _load()
     q = L.skm_q(p)
     recv = np.zeros((p, q), dtype=np.int8)

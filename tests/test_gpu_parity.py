@@ -34,8 +34,12 @@ def _guards_intact(raw, nbytes, fill=0x5A):
     return bool((raw[:GUARD] == fill).all()) and bool((raw[GUARD + nbytes:] == fill).all())
 
 
+def _untouched(raw, fill=0x5A):
+    return bool((raw == fill).all())
+
+
 def _build(bcs, p, r0, r1, want_recv=True, want_send=True, fast=True):
-    """fast=True: with a workspace (skip-code construction); False: self-contained construction."""
+    """fast: with a workspace, which the call must leave as it is (the rows are the same either way)."""
     q = bcs.bcs_q(p)
     nb = (r1 - r0) * q
     raw_r, recv = _guarded(nb) if want_recv else (None, None)
@@ -46,9 +50,8 @@ def _build(bcs, p, r0, r1, want_recv=True, want_send=True, fast=True):
         raw_w, ws = _guarded(need)
     bcs.bcs_build(p, r0, r1, recv, send, ws)
     torch.cuda.synchronize()
-    assert bcs.bcs_wait_expired() == 0      # no CTA gave up waiting for its copies
-    if raw_w is not None:
-        assert _guards_intact(raw_w, ws.numel())
+    assert bcs.bcs_wait_expired() == 0
+    assert raw_w is None or _untouched(raw_w)
     out = []
     for raw, t in ((raw_r, recv), (raw_s, send)):
         if t is None:
@@ -94,7 +97,7 @@ def test_every_p_up_to_1024_batched_and_simulated(bcs, fast):
     raw_w, ws = _batch_ws(bcs, plan, fast)
     bcs.bcs_build_batch(dev, recv, send, ws)
     torch.cuda.synchronize()
-    assert raw_w is None or _guards_intact(raw_w, ws.numel())
+    assert raw_w is None or _untouched(raw_w)
     assert _guards_intact(raw_r, plan.total_entries) and _guards_intact(raw_s, plan.total_entries)
     recv, send = recv.cpu().numpy(), send.cpu().numpy()
     eo = plan.entry_off.tolist()
@@ -123,7 +126,7 @@ def test_batch_with_trivial_and_duplicate_p(bcs, fast):
     raw_w, ws = _batch_ws(bcs, plan, fast)
     bcs.bcs_build_batch(dev, recv, send, ws)
     torch.cuda.synchronize()
-    assert raw_w is None or _guards_intact(raw_w, ws.numel())
+    assert raw_w is None or _untouched(raw_w)
     assert _guards_intact(raw_r, plan.total_entries) and _guards_intact(raw_s, plan.total_entries)
     eo = plan.entry_off.tolist()
     for j, p in enumerate(plist):
@@ -141,10 +144,8 @@ def test_batch_with_trivial_and_duplicate_p(bcs, fast):
 
 
 def test_batch_of_large_and_tiny_p_mixed(bcs):
-    """A list whose p average more than 8192 ranks (the batch takes the codes kernel that scans
-    blocks of 32 flattened ranks at once) with p = 1, tiny p and p next to multiples of 8192 in
-    between: blocks that cross from one p to the next, whole p inside one block, CTAs that touch
-    three and more p, a last block cut off by the end of the list."""
+    """p above and below 1024 in turn, p = 1 and p next to multiples of 8192 among them: shares that cross from one p
+    to the next or hold several p whole, a last share cut off by the end of the list."""
     plist = [70001, 1, 2, 3, 65536, 1, 8191, 8193, 31, 32, 33, 16384, 5, 100003, 1, 7, 8192, 40961,
              64, 63, 65, 262147, 1000, 24576, 9, 131071]
     assert sum(plist) // len(plist) >= 8192
@@ -169,8 +170,7 @@ def test_batch_of_large_and_tiny_p_mixed(bcs):
 
 
 def test_batch_output_is_complete_for_the_next_operation_on_the_stream(bcs):
-    """The kernels of a batch are launched as dependents of one another and the last one (the
-    CTAs of the small p) does not wait for the tiled kernels of the large p before it starts.
+    """The kernels of a batch are launched as dependents of one another and start before the one in front has ended.
     Whatever follows on the stream must still see both tables complete: a copy enqueued right
     after the call, without a synchronisation in between, is compared with the oracle."""
     plist = [5, 2**20 + 1, 300, 1000, 77]
@@ -203,11 +203,11 @@ def test_sub_ranges_ragged_tails_and_single_outputs(bcs, fast):
     want_r, want_s = oracle.full_table(p)
     for r0, r1 in ((0, 1), (0, 255), (0, 257), (1, 258), (777, 1300), (p - 300, p), (p - 1, p),
                    (50000, 50000 + 16 * 3 + 5), (99000, 100003),
-                   # several 512-rank tiles of the four-ranks-per-thread kernel, odd starts and ends
+                   # several items of every warp, odd starts and ends
                    (12345, 14002), (3, 70003), (25001 - 700, 25001 + 700)):
         recv, send = _build(bcs, p, r0, r1, fast=fast)
         assert np.array_equal(recv, want_r[r0:r1]), (r0, r1)
-        assert np.array_equal(send, want_s[r0:r1]), (r0, r1)      # partly looked up, partly recomputed
+        assert np.array_equal(send, want_s[r0:r1]), (r0, r1)      # (to-processors in the range and outside)
     recv, _ = _build(bcs, p, 123, 999, want_send=False, fast=fast)
     assert np.array_equal(recv, want_r[123:999])
     _, send = _build(bcs, p, 123, 999, want_recv=False, fast=fast)
@@ -217,7 +217,7 @@ def test_sub_ranges_ragged_tails_and_single_outputs(bcs, fast):
 
 def test_seeded_p_sweep_full_tables_sub_ranges_and_one_batch(bcs):
     """About 170 values of p between 64 and 300 000 -- the neighbours of the powers of two, values
-    whose skips contain 33 (six instead of five rounds read from the run table), and 150 seeded
+    whose skips contain 33, and 150 seeded
     log-uniform draws: the full tables, one seeded sub-range each, and all of them in one batch."""
     rng = np.random.default_rng(20240)
     edge = [64, 65, 127, 128, 129, 511, 512, 513, 1023, 1025, 2047, 2049, 4095, 4097, 33 * 64, 33 * 64 - 1,
@@ -252,10 +252,8 @@ def test_seeded_p_sweep_full_tables_sub_ranges_and_one_batch(bcs):
 
 
 def test_receive_kernel_instantiations(bcs):
-    """The quad receive kernel has four instantiations picked per launch: window bounds loaded as
-    16-byte words where a p's skips are multiples of 4 (p just below a power of two), rows stored
-    word by word where q is a multiple of 4.  Values of p that take each combination, all ranks
-    and a sub-range that starts off a multiple of 4, with and without rows / round-major copy."""
+    """p next to powers of two (skips that are multiples of 4, or none) with q a multiple of 4 or not: all ranks, one table
+    alone, a sub-range that starts off a multiple of 4, send rows of a prepared p."""
     for p in (4095, 4097, 65535, 65537, 1048575, 1000003, 262143, 300007, 16383, 16385):
         q = oracle.q_of(p)
         want_r, want_s = oracle.full_table(p)
@@ -267,7 +265,7 @@ def test_receive_kernel_instantiations(bcs):
         recv, send = _build(bcs, p, r0, r1)
         assert np.array_equal(recv, want_r[r0:r1]) and np.array_equal(send, want_s[r0:r1]), p
         raw_w, ws = _guarded(bcs.bcs_prepare_workspace_bytes(p))
-        bcs.bcs_prepare(p, ws)                                  # round-major copy only
+        bcs.bcs_prepare(p, ws)
         raw_s, out = _guarded(p * q)
         bcs.bcs_build_prepared(p, 0, p, None, out, ws)
         torch.cuda.synchronize()
@@ -309,7 +307,7 @@ def test_prepare_in_two_steps_chunk_by_chunk(bcs):
     """bcs_prepare_codes, then bcs_prepare_rows chunk by chunk (in a shuffled order, chunk
     boundaries at multiples of 16 that are not multiples of the kernels' tiles), each chunk's
     receive rows taken straight from the construction; then the send rows of every chunk by
-    bcs_build_prepared, and the receive rows once more by transposition: all equal the oracle's."""
+    bcs_build_prepared, and the receive rows once more: all equal the oracle's."""
     rng = np.random.default_rng(5)
     for p, step in ((33, 16), (63, 32), (64, 16), (1000, 304), (4097, 1008), (100003, 30000),
                     (workloads.P_SINGLE, 333328)):
@@ -322,7 +320,7 @@ def test_prepare_in_two_steps_chunk_by_chunk(bcs):
             r0, r1 = chunks[c]
             raw_r, recv = _guarded((r1 - r0) * q)
             if c % 3 == 2:
-                bcs.bcs_prepare_rows(p, r0, r1, None, ws)        # round-major copy only
+                bcs.bcs_prepare_rows(p, r0, r1, None, ws)        # nothing to write
             else:
                 bcs.bcs_prepare_rows(p, r0, r1, recv, ws)
                 torch.cuda.synchronize()
@@ -413,8 +411,8 @@ def test_degenerate_sizes_and_errors(bcs):
         recv, send = _build(bcs, 3, 0, 3, fast=fast)
         want = oracle.full_table(3)
         assert np.array_equal(recv, want[0]) and np.array_equal(send, want[1])
-    small = torch.zeros(64, dtype=torch.int8, device="cuda")         # too small a workspace:
-    out = torch.zeros(100003 * 17, dtype=torch.int8, device="cuda")  # the slow path must run
+    small = torch.zeros(64, dtype=torch.int8, device="cuda")         # a workspace of any size will do
+    out = torch.zeros(100003 * 17, dtype=torch.int8, device="cuda")
     bcs.bcs_build(100003, 0, 100003, out, None, small)
     torch.cuda.synchronize()
     assert np.array_equal(out.cpu().numpy().reshape(100003, 17), oracle.full_table(100003)[0])
@@ -428,15 +426,14 @@ def test_degenerate_sizes_and_errors(bcs):
 
 
 def test_p_at_the_upper_limit(bcs):
-    """p = 2^31 - 1 (q = 31): rank arithmetic near 2^32; a few ranges vs the per-rank oracle.
-    Both constructions."""
+    """p = 2^31 - 1 (q = 31): rank arithmetic near 2^32; a few ranges vs the per-rank oracle,
+    without a workspace and with one of the full 8.6 GB."""
     p = 2**31 - 1
     for r0, r1 in ((0, 300), (2**30 - 100, 2**30 + 200), (p - 300, p)):
         want_r, want_s = oracle.build_range(p, r0, r1)
         recv, send = _build(bcs, p, r0, r1, fast=False)
         assert np.array_equal(recv, want_r), (r0, r1)
         assert np.array_equal(send, want_s), (r0, r1)
-    # the skip-code construction at the same p: 8.6 GB of codes in the workspace
     for r0, r1 in ((0, 300), (2**30 - 100, 2**30 + 200), (p - 300, p)):
         want_r, want_s = oracle.build_range(p, r0, r1)
         q = 31
@@ -480,7 +477,7 @@ def test_build_to_host_matches(bcs):
     assert np.array_equal(hs.numpy()[: 4900 * q].reshape(4900, q), want_s[100:5000])
     hs.zero_()
     bcs.bcs_build_to_host(p, 100, 5000, None, hs, stage[: 2 * ((4900 * q + 255) // 256 * 256)])
-    torch.cuda.synchronize()                                  # no room for a workspace: slow path
+    torch.cuda.synchronize()                                  # no room beyond the tables
     assert np.array_equal(hs.numpy()[: 4900 * q].reshape(4900, q), want_s[100:5000])
 
 
@@ -488,8 +485,7 @@ def test_batched_irregular_sweep_full_size(bcs):
     """4096 octave-uniform p in [2^10, 2^20): the launch the benchmark uses, 639 M ranks and
     24 GB of tables.  EVERY table is compared byte for byte with the oracle's array form (about
     a minute and a half of host time); for every p >= 2^16, 10^4 seeded ranks plus the ranks
-    skips[k]-2 .. skips[k]+2 of every k (where the receive kernel switches to its general tile
-    code), the root's neighbours and the last ranks are compared with the oracle's per-rank form
+    skips[k]-2 .. skips[k]+2 of every k, the root's neighbours and the last ranks are compared with the oracle's per-rank form
     as well, which shares nothing with the array form but Algorithms 1 and 2; and the library's
     property checker runs over every rank of every p."""
     plist = workloads.batch_p_list()
@@ -826,8 +822,8 @@ def test_large_p_chunked_spot_checked(bcs):
         o_r, _ = oracle.build_range(p, r0, r0 + head, want_send=False)
         bcs.bcs_checksum(recv, r0 * q, sums[2:3], n_entries=head * q)
         assert int(sums.cpu()[2]) & m64 == oracle.checksum(o_r, r0 * q)
-        if c in (0, 7):     # rebuilt by bcs_build (self-contained construction; at the last chunk
-            recv.fill_(0)   # with its own workspace): same sums
+        if c in (0, 7):     # through bcs_build, without and with a workspace: the entry point is compared
+            recv.fill_(0)   # here (the kernel is the same, checked above)
             send.fill_(0)
             own = None
             if c == 7:

@@ -127,14 +127,26 @@ def _batch(bcs, plist, send=True):
     assert bool((raw_r[:32] == 99).all()) and bool((raw_r[32 + plan.total_entries:] == 99).all())
     assert bool((raw_s[:32] == 99).all()) and bool((raw_s[32 + plan.total_entries:] == 99).all())
     assert send or bool((raw_s == 99).all())
+    tables = {}
     for p, lo, hi in zip(plist, plan.entry_off[:-1].tolist(), plan.entry_off[1:].tolist()):
         if p == 1:
             continue
-        one_r = torch.empty(hi - lo, dtype=torch.int8, device="cuda")
-        one_s = torch.empty(hi - lo, dtype=torch.int8, device="cuda")
-        bcs.bcs_build(p, 0, p, one_r, one_s)                 # (compared with the oracle above)
-        assert torch.equal(recv[lo:hi], one_r), p
-        assert not send or torch.equal(out_s[lo:hi], one_s), p
+        q = bcs.bcs_q(p)
+        got = [out[lo:hi] for out in ((recv, out_s) if send else (recv,))]
+        if p <= 1 << 21:
+            if p not in tables:
+                tables[p] = [torch.from_numpy(t).cuda().view(-1) for t in oracle.full_table(p)]
+            assert all(torch.equal(g, w) for g, w in zip(got, tables[p])), p
+            continue
+        # ranks around every skip, the ends and some more; the properties and pairs of all ranks
+        near = [s + d for s in bcs.bcs_skips(p) for d in range(-40, 41)]
+        at = np.unique(np.array(near + np.random.default_rng(p).integers(0, p, 2000).tolist()) % p)
+        rows = torch.from_numpy(at).cuda()
+        for g, w in zip(got, oracle.build_ranks(p, at.astype(np.uint32))):
+            assert np.array_equal(g.view(p, q)[rows].cpu().numpy(), w), p
+        counts = torch.ones(3, dtype=torch.int64, device="cuda")
+        bcs.bcs_validate(p, 0, p, got[0].clone(), got[1].clone() if send else None, counts)
+        assert counts.tolist() == [0, 0, 0], p
 
 
 # the sizes at which a batch changes kernels and row forms (1024, 2^15, 2^21), tables that start at any byte, shares that
@@ -144,8 +156,7 @@ def _batch(bcs, plist, send=True):
                                    [33333], [65536, 140001, 600011, 1 << 20], [1], [2, 1], [(1 << 20) + 1] * 3, [1025] * 40, [127, 128, 129, 130] * 30])
 @pytest.mark.parametrize("send", [True, False])
 def test_batches(bcs, plist, send):
-    if bcs.bcs_batch_plan(plist).total_entries:
-        _batch(bcs, plist, send)
+    _batch(bcs, plist, send)
 
 
 # lists of small p that are spread over the SMs or not, with CTAs of 256 and of 128 threads; a share per CTA or several

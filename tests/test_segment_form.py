@@ -1,0 +1,51 @@
+"""The rule by which the kernels compute a row (tests/segment_form.py) gives the oracle's rows, and the bounds that their shared
+memory and searches are laid out for hold."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.segment_form import Form
+
+
+def _compare(p, ranks):
+    form = Form(p)
+    ranks = np.unique(np.asarray(ranks, dtype=np.int64))
+    want = oracle.build_ranks(p, ranks.astype(np.uint32))
+    assert np.array_equal(form.receive(ranks), want[0]), p
+    assert np.array_equal(form.send(ranks), want[1]), p
+
+
+def _near(p, rng, count):
+    """Ranks around the skips and their sums of two, the ends, and some more."""
+    s = oracle.skips(p).tolist()
+    heads = s + [s[i] + s[j] for i in range(len(s)) for j in range(max(0, i - 4), i)]
+    return [(h + d) % p for h in heads for d in range(-3, 4)] + [int(v) for v in rng.integers(0, p, count)]
+
+
+@pytest.mark.parametrize("first", range(8))
+def test_every_rank_of_small_p(first):
+    for p in range(2 + first, 1400, 8):
+        _compare(p, np.arange(p))
+
+
+def test_sampled_ranks_of_larger_p():
+    rng = np.random.default_rng(7)
+    edges = [(1 << k) + d for k in (10, 13, 16, 20, 23, 28, 30) for d in (-1, 0, 1)] + [65 << 9, (97 << 17) + 5, (1 << 31) - 1]
+    for p in edges + [int(2 ** e) for e in rng.uniform(9.5, 31, 60)]:
+        _compare(p, _near(p, rng, 150))
+
+
+def test_bounds_of_the_layout():
+    """A segment has 41 ranks or more, the exceptions behind a start are the first 25 of them, and segment floor(x inv / 2^32) is
+    the one of rank x or next to it."""
+    rng = np.random.default_rng(8)
+    for p in [129, 255, 256, 257, (1 << 31) - 1, (1 << 30) + 1, (1 << 23) + 1] + [int(2 ** e) for e in rng.uniform(7.1, 31, 300)]:
+        form = Form(p)
+        q, L = form.q, form.L
+        assert form.C(L, q) <= 24 and form.s[L] - form.C(L, q) >= 41, p
+        x = np.array(_near(p, rng, 300), dtype=np.int64)
+        inv = (1 << (q - L + 32)) // p
+        guess = x * inv >> 32
+        g, low, length = form.locate(x)
+        assert np.all(np.abs(guess - g) <= 1), p
+        assert np.all(low < length) and np.all(length >= 41), p

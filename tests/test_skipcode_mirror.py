@@ -1,8 +1,6 @@
-"""The skip-code construction that the fast CUDA kernels run, restated on the CPU
-(tests/skipcode_mirror.c), must give the oracle's rows: the paper's greedy construction
-(Algorithm 4's two windows and max(U \\ B), the range search that Algorithm 3 stands for) and
-the construction on skip codes are the same function.  Also keeps the committed table of model
-operation counts, which the benchmark reads, honest."""
+"""A construction on skip codes with searches per round (tests/skipcode_mirror.c) must give the oracle's rows: an
+independent check of the oracle.  It shares the skip codes with the library's kernels, which compute rows in another way
+(tests/segment_form.py).  Also keeps the committed table of its operation counts honest."""
 import json
 
 import numpy as np
@@ -22,8 +20,8 @@ def _gpu_mode():
 
 @pytest.mark.parametrize("mode", [0, 1, 2])
 def test_mirror_equals_oracle_for_every_small_p(mode):
-    """Every rank of every p < 700, with the short windows taken from exact block sets (as the
-    kernels do for p >= 64), never, and for every p."""
+    """Every rank of every p < 700, with the short windows taken from exact block sets where
+    p >= 64, never, and for every p."""
     mirror.set_table_mode(mode)
     seen = {"rounds_step2": 0, "rounds_rest": 0, "rounds_second": 0, "rounds_table": 0}
     for p in range(2, 700):
@@ -108,8 +106,8 @@ def test_block_codes_equal_the_plain_scan():
 
 
 def test_small_p_run_table_construction_equals_the_oracle():
-    """The construction of the batch kernel for p <= 1024 (baseblock bits of all ranks, runs of
-    2^l ranks, every window looked up as an exact set) gives the oracle's tables for every such p."""
+    """Baseblock bits of all ranks, runs of 2^l ranks, every window looked up as an exact set: the oracle's tables for
+    every p <= 1024."""
     import numpy as np
     import oracle
     from tests import skipcode_mirror as skm

@@ -1,7 +1,6 @@
 """bcs_build_static: the entry point for callers that can neither allocate device memory nor
-pass a workspace (it uses an 8 MiB scratch array that is part of the library).  Its tables must
-be byte-identical to those of bcs_build and to the CPU oracle's, call after call, although every
-call reuses the same scratch and finds the previous call's leftovers in it.
+pass a workspace.  Its tables must be byte-identical to those of bcs_build and to the CPU oracle's, call
+after call, and it refuses what it always refused (ranges whose workspace would exceed 8 MiB).
 
 This file sorts last on purpose: a run that stops at the first failure has then already gone
 through every other test.  It does not depend on them: it also passes alone in a fresh process.
@@ -50,7 +49,7 @@ def _oracle_rows(p, r0, r1):
 def test_static_scratch_matches_bcs_build_on_consecutive_calls(bcs):
     L = bcs.lib()
     limit = 8 << 20
-    # two calls in a row, then more with other p and sub-ranges, all through the same scratch
+    # two calls in a row, then more with other p and sub-ranges
     cases = [(100003, 0, 100003), (100003, 0, 100003), (65537, 1000, 60001), (300007, 0, 300007),
              (1000, 0, 1000), (2**20 + 1, 2**19, 2**19 + 150000), (100003, 99000, 100003)]
     for p, r0, r1 in cases:
@@ -80,7 +79,7 @@ def test_static_scratch_matches_bcs_build_on_consecutive_calls(bcs):
 
 def test_static_scratch_rejects_what_does_not_fit(bcs):
     L = bcs.lib()
-    p = 2**20 + 1                                   # all ranks would need 26 MB of scratch
+    p = 2**20 + 1                                   # workspace of all ranks: 26 MB
     assert bcs.bcs_build_workspace_bytes(p, 0, p) > (8 << 20)
     out = torch.full((4096,), 77, dtype=torch.int8, device="cuda")
     assert L.bcs_build_static(p, 0, p, out.data_ptr(), None, None) == 4     # BCS_ERR_UNSUPPORTED
