@@ -303,7 +303,7 @@ def bcs_build_batch_workspace_bytes(total_ranks: int, total_copy: int) -> int:
 
 def bcs_build_batch(plan_dev: BatchPlan, recv_out, send_out, workspace=None, stream=None) -> None:
     """plan_dev: a BatchPlan whose tensors live on the CUDA device; workspace: CUDA tensor of
-    plan.workspace_bytes() bytes (fast construction) or None."""
+    plan.workspace_bytes() bytes or None (not touched)."""
     _check(_call.build_batch(plan_dev.p_list.data_ptr(), plan_dev.rank_off.data_ptr(),
                                  plan_dev.entry_off.data_ptr(), plan_dev.tile_off.data_ptr(),
                                  plan_dev.copy_off.data_ptr(), plan_dev.skips_tab.data_ptr(),

@@ -1,10 +1,10 @@
 // All ranks of many p at once: bcs_build_batch.
 //
-// A CTA of 256 threads builds the row table of a p (rows.cuh) and computes rows from it; several CTAs share an SM, so
-// that one builds a table while the others compute.  Three kernels take a p by its size:
-//   * up to 1024 ranks: a CTA per p;
-//   * up to 2^21 ranks: CTAs take equal shares of the flattened ranks of the list, p by p;
-//   * more: all CTAs of a grid work on one p after another (launched only when the list is long enough to hold one).
+// A CTA builds the row table of a p (rows.cuh) and computes rows from it; where several CTAs share an SM, one builds a
+// table while the others compute.  Three kernels take a p by its size:
+//   * up to 1024 ranks: a CTA of 128 or 256 threads per p;
+//   * up to 2^21 ranks: CTAs of 256 threads take equal shares of the flattened ranks of the list, p by p;
+//   * more: CTAs of 640 threads, one per SM, work on one p after another (launched only when the list is long enough to hold one).
 // Each is launched as a dependent of the kernel before it on the stream and may run beside it until it waits for it.
 // The plan is the caller's memory: the kernel before may still be writing it, or what it has written may not be visible yet.
 // So what the plan shows before the wait is a guess, good for one thing: a table of row entries is a function of p
@@ -14,10 +14,9 @@
 // (Back to back, every p up to 1024: 17.7 us with the guess taken as it is, 18.3 like this, 25.4 with the first load behind the
 // wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8, 18.7.)
 //
-// Before: skip codes of all ranks, a search on them, a round-major copy and its transposition.  1024 p of 2^10..2^20:
-// 5456 -> 1298 us (8.3 ps a rank, both tables 4.5 TB/s; bound by instruction issue), every p up to 1024: 31.3 -> 18.1 us,
-// 16 p of 2^10..2^20: 94 -> 44 us.  Middle kernel with two CTAs of 256 threads per SM instead of three: 1505 us, four: more
-// (spills).
+// Up to 1024 ranks the tables are most of the work: every p up to 1024 18.4 us, 57 % of the issue slots.  Above, instruction issue
+// and the integer pipe bound it: 1024 p of 2^10..2^20 1288 us (both tables 4.6 TB/s).  That kernel holds two narrow and two wide
+// forms in 80 registers and spills a few bytes at its three CTAs per SM; two per SM take 1368 us, four 1490.
 #include <type_traits>
 
 #include "rows.cuh"
@@ -279,7 +278,7 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
 
 // A CTA per p of the list, up to kCtas of them per SM.  alone: no larger p, nothing runs beside them.  Where the list is then
 // too short to fill the card, they ask for so much shared memory that they spread over all SMs (else some held five and
-// others one: 300 p of 3..1024 11.7 -> 8.9 us).
+// others one: 300 p of 3..900 11.9 -> 8.4 us).
 template <unsigned kThreads, int kCtas>
 bcs_status launch_small(const BatchArgs &ba, bool alone, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
@@ -338,9 +337,10 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         const uint32_t shared = wide.bytes > narrow.total(kBatchWarps) ? wide.bytes : narrow.total(kBatchWarps);
         if (!allow_shared<batch_middle_kernel>()) return BCS_ERR_CUDA;
         // Up to 2^23 ranks a share per resident CTA: every share costs a search and a table or two, some 10 us (16 p
-        // of 2^10..2^20 66.8 us with three, 44.7 with one; 64 p of about 2^17 143 and 122 us).  Beyond, three, so that none
-        // ends last by much (150 p of 2^12..2^18, 10 million ranks, 182 us, with one 200).  At most 32768 ranks, at
-        // least 1024 (a table costs as much as some hundred ranks of each warp).
+        // of 2^10..2^20 79 us with three, 75 with one; 3000 of 2^10..2^11 167, 154).  Beyond, three, so that none
+        // ends last by much (150 p of 2^12..2^18 164 us, with one 168; 300 of 2^14..2^18 326, 348; 3000 of 2^12..2^13 383, 485;
+        // but 64 of 2^17..2^18, few tables, 165, 143).  At most 32768 ranks, at least 1024 (a table costs as much as some
+        // hundred ranks of each warp).
         const uint64_t ctas = kSms * kMiddleCtas * (total_ranks <= (1u << 23) ? 1u : 3u);
         uint64_t share = align_up(total_ranks / ctas, 128);
         share = share < 1024 ? 1024 : (share > 32768 ? 32768 : share);
@@ -354,7 +354,8 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         }
     }
     // CTAs of 256 threads while all are resident at once (the shorter chain counts), else of 128 (less waiting at
-    // barriers, longer items): 700 p of 3..1024 13.7 against 16.5 us, 1000 p 21.9 against 18.0.
+    // barriers, longer items): us with 256 / 128, 300 p of 3..900 8.4/11.7, 700 of 3..702 11.5/12.1, 740 of 280..1019 13.4/14.6;
+    // 800 of 1000 17.3/16.0, 1000 of 33 8.6/5.3, 1000 of 3..1002 16.2/18.2, 2000 of 2..1024 36.8/36.4, 5000 of 777 96/93.
     if (num_p <= kSms * 5u) return launch_small<256, 5>(ba, small_only, recv_out, send_out, stream);
     return launch_small<128, 8>(ba, small_only, recv_out, send_out, stream);
 }

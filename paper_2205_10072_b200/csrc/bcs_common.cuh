@@ -11,7 +11,7 @@
 
 namespace bcs {
 
-constexpr int kTile = 256;                    // ranks (= threads) per CTA of the schedule kernels
+constexpr int kTile = 256;                    // ranks (= threads) per CTA of the checks (validate.cu)
 constexpr uint32_t kFusedMaxP = 1024;         // batch: a p up to here is built by one CTA
 constexpr int kRow = BCS_SKIPS_STRIDE;        // words per table row
 
@@ -104,12 +104,11 @@ __device__ __forceinline__ uint32_t find_segment_warp(const uint64_t *off, uint3
 }
 
 // ---------------------------------------------------------------- dependent launches
-// The kernels of one construction run back to back on one stream, each a few tens of
-// microseconds long, so the time in which one grid drains and the next is brought onto the SMs
-// counts.  A kernel launched with launch_dependent() may be made resident as soon as every CTA
+// Calls follow one another on a stream, many of them a few microseconds long, so the time in which one grid drains and
+// the next is brought onto the SMs counts.  A kernel launched with launch_dependent() may be made resident as soon as every CTA
 // of the kernel before it on the stream has called grid_launch_dependents() (or has exited); it
-// runs its set-up and then blocks in grid_dependency_wait() until that kernel has completed and
-// its writes are visible.  Both calls do nothing in a kernel that was launched the ordinary way.
+// runs its set-up, which relies on nothing that another kernel may have written, and then blocks in grid_dependency_wait() until
+// that kernel has completed and its writes are visible.  Both calls do nothing in a kernel that was launched the ordinary way.
 __device__ __forceinline__ void grid_dependency_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -1,7 +1,6 @@
 // The paper's own per-rank construction (arXiv 2205.10072, Algorithms 2-4) as device functions:
 // one thread runs Algorithm 4 for one rank with the range search done by descending the
-// homeranges.  Used by the self-contained kernels of the schedule translation unit and by the
-// round-table kernel when it has to build the rows of its ranks itself.
+// homeranges.  Used by the round-table kernel when it has to build the rows of its ranks itself.
 #pragma once
 #include "bcs_common.cuh"
 

@@ -1,19 +1,15 @@
-// Receive and send rows of a stretch of ranks of one p: the kernel behind bcs_build and its relatives.
+// Receive and send rows of a stretch of ranks of one p: the kernels behind bcs_build and its relatives.
 //
-// One launch, nothing read from memory, no table of all ranks (rows.cuh).  Before it: skip codes of all ranks, a
-// search on them per round, a round-major copy and its transposition, three launches.  All ranks of
-// 100 003: 23.2 -> 10.2 us, of about 2^20: 38.4 -> 22.7 us, 65 553 ranks of it 104 -> 10.3 us (send rows whose
-// to-processor lies outside the range were searched for one by one), 32 ranks without a workspace 572 -> 8.2 us (a
-// descent of the homeranges per window), 8 chunks of about 2^28 ranks 9.35 -> 3.94 ms.  Small calls
-// last as long as launch, table and one item; large ones are bound by instruction issue (seven eighths of the slots).
-//
-// The start of a call (launch, CTAs onto the SMs, table) was most of a small call's time.  The kernel is launched as a
-// dependent of whatever runs before it on the stream and waits for that before its first store only, the
-// table holds what the CTA's segments need where these are few, and a CTA has no more warps than items: 32 ranks 8.2 ->
-// 4.4 us, all ranks of 1152: 8.6 -> 4.6, of 100 003: 10.2 -> 7.6, of about 2^20: 22.7 -> 18.4 us, back to back.
-//
-// With the wide form (wide.cuh), lighter tables and a lighter path from Python, back to back: 32 ranks 3.5 us, 1152 3.4, 65 553 of
-// about 2^20 4.3, all of 100 003 6.1, of about 2^20 16.8, 8 chunks of about 2^28 2.39 ms.
+// One launch, nothing read from memory, no table of all ranks (rows.cuh).  Two forms, by size (launch_rows):
+//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp; 44 % of the issue slots at 65 553
+//     ranks of about 2^20.  Back to back 32 ranks 3.5 us, all ranks of 1152 3.6, 65 553 ranks 4.25.  The table holds what the
+//     CTA's segments need where these are few, and a CTA has no more warps than items.
+//   * wide_kernel, 16 output bytes per lane (wide.cuh).  Up to some 2^23 ranks bound by instruction issue (61 % of the slots at 2^20
+//     ranks) behind a table that every CTA builds whole; up to 2^20 ranks two CTAs fit an SM, so that the next call's table is
+//     built beside the rows, above it the 61 440 registers of a CTA leave no room and the table's time is in series.
+//     From about 2^25 ranks on bound by memory writes.  All ranks of 100 003 6.1 us, of about 2^20 17.0, 8 chunks of about
+//     2^28 2.38 to 2.48 ms (6.3 to 6.0 TB/s; the power cap shows in long runs).
+// Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
 #include <type_traits>
 
 #include "rows.cuh"
