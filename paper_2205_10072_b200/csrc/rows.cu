@@ -66,8 +66,8 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     stage_free();
 }
 
-// The same for larger tables, q >= 16 (wide.cuh), one CTA per SM; `item` is a multiple of 16.  halves: half of the warps
-// write the receive rows and half the send rows; otherwise all warps the ones before the others.
+// The same for larger tables, q >= 16 (wide.cuh), one CTA per SM; `item` is a multiple of 16.  halves: every warp has one item of
+// one table, half of the warps write the receive rows and half the send rows; otherwise all warps the ones before the others.
 // (No more than 640 threads: at the speed of the memory the write streams of 1024 cost 20 % and more.)
 template <unsigned kThreads, int kCtas, bool kAnyStep>
 __global__ void __launch_bounds__(kThreads, kCtas)
@@ -79,8 +79,16 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     const WideLayout at(rc.q);
     const RowTable t(sm, at.base);
     if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
-    if (threadIdx.x == 0) *t.wanted = (2u << (rc.q - kLow)) - 1u;
-    __syncthreads();
+    if (halves) {
+        // One run per warp, those of the CTA side by side: rows for their segments only (all ranks of 100 003: five of 11
+        // groups of rows, of about 2^20 nine of 15; 6.13 -> 5.97 and 16.8 -> 15.7 us, 1.3 million ranks 17.6 -> 16.5).
+        const uint32_t warps = (blockDim.x >> 5) / (recv != nullptr && send != nullptr ? 2u : 1u);
+        const uint32_t x0 = first + blockIdx.x * warps * item;
+        want_rows(t, rc.q, rc.inv, x0 >= rc.p ? x0 - rc.p : x0, warps * item + 1u);      // (the last vectors look at the rank behind)
+    } else {
+        if (threadIdx.x == 0) *t.wanted = (2u << (rc.q - kLow)) - 1u;
+        __syncthreads();
+    }
     build_row_table(t, rc.q, rc.odd);
     if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
     grid_dependency_wait();

@@ -306,6 +306,30 @@ __device__ __forceinline__ uint32_t wanted_rows(int q, uint32_t inv, uint32_t x0
     return __reduce_or_sync(0xffffffffu, bits);
 }
 
+// The same for any n < 2^31, into *t.wanted; by the whole CTA.  Starts and ends with a barrier.
+__device__ __forceinline__ void want_rows(const RowTable &t, int q, uint32_t inv, uint32_t x0, uint32_t n)
+{
+    const int high = q - kLow;
+    __syncthreads();
+    if (threadIdx.x == 0) *t.wanted = 0u;
+    // (where a segment has 128 ranks, the first row of the group behind its own is looked at, if not used)
+    if ((int)threadIdx.x <= high) t.rows[threadIdx.x * kLowRanks] = make_uint2(0u, 0u);
+    __syncthreads();
+    uint32_t from = __umulhi(x0, inv);                           // one before or behind, at most
+    from = from ? from - 1u : 0u;
+    const uint32_t count = __umulhi(n, inv) + 7u;                // (from is up to two before; the ends lie up to n inv / 2^32 + 3 segments apart)
+    uint32_t bits = 0;
+    for (uint32_t j = threadIdx.x; j < count; j += blockDim.x) {
+        const uint32_t g = (from + j) & ((1u << high) - 1u);
+        const int z = __ffs(~g) - 1;                             // lowest zero bit, and the next one
+        bits |= (g ? g & (0u - g) : 1u << high) | 1u << z;
+        if (z < high) bits |= 1u << (z + __ffs(~(g >> (z + 1))));
+    }
+    bits = __reduce_or_sync(0xffffffffu, bits);
+    if ((threadIdx.x & 31u) == 0u && bits != 0u) atomicOr(t.wanted, bits);
+    __syncthreads();
+}
+
 // ---------------------------------------------------------------- rows of an item, by one warp
 // How a lane's rows of q bytes lie in the words of the staging buffer, where the rows of a warp follow one another.
 // (The same for every 32 ranks of an item: 32 rows are whole words.)

@@ -50,21 +50,25 @@ struct WideLayout {
 
 // Send table: [u - 1][low], u = K - L (1..q-L) for a segment with bit L clear and lowest bit K, u = q - L + (K2 - L) for
 // one with bit L set and K2 the lowest bit of the next segment.  Entries of the rounds 0..6, baseblock as byte 7.
-// All threads of the CTA call, the row table is complete.  Ends with a barrier.
+// For the K of *t.wanted; all threads of the CTA call, the row table is complete.  Ends with a barrier.
 __device__ __forceinline__ void build_send_table(const RowTable &t, uint2 *send, int q, uint32_t odd)
 {
     const int high = q - kLow;
     const uint8_t *bytes = reinterpret_cast<const uint8_t *>(t.rows);
-    if (threadIdx.x == 0) send[2 * high * kLowRanks] = make_uint2(0u, 0u);
+    // (the first row of a group, and of the end, is looked at as the one behind a segment of 128 ranks)
+    if ((int)threadIdx.x <= 2 * high && ((int)threadIdx.x == 2 * high || ((*t.wanted >> (threadIdx.x % (uint32_t)high + 1u)) & 1u) == 0u))
+        send[threadIdx.x * kLowRanks] = make_uint2(0u, 0u);
     // Rows are 8 bytes apart, so the two halves of a warp would meet in the same banks: the upper half takes the
     // bytes 4..7 (odd words) while the lower half takes 0..3, and the other way round.
     const uint32_t turn = (threadIdx.x & 16u) ? 4u : 0u;
     int skip[8];
 #pragma unroll
     for (uint32_t j = 0; j < 8; ++j) skip[j] = (j ^ turn) < 7u ? (int)t.s[j ^ turn] : 0;
-    for (uint32_t job = threadIdx.x; job < 2u * (uint32_t)high * kLowRanks; job += blockDim.x) {
-        const int u = (int)(job / kLowRanks) + 1, low = (int)(job % kLowRanks);
-        const int own = u <= high ? u : 0, next = u <= high ? 0 : u - high;
+    const uint32_t jobs = (uint32_t)__popc(*t.wanted) * 2u * kLowRanks;
+    for (uint32_t job = threadIdx.x; job < jobs; job += blockDim.x) {
+        const int K = (int)t.list[job / (2u * kLowRanks)] - kLow, low = (int)(job % kLowRanks);
+        if (K == 0) continue;                                    // (is one of the two anyway)
+        const int own = (job & kLowRanks) ? 0 : K, next = K - own;
         const int len = (int)t.s[kLow] - (int)count_odd(odd, kLow, kLow + next);
         uint2 row = make_uint2(0u, 0u);                          // (read, but not used, behind a segment's last rank)
         if (low < len) {
@@ -78,7 +82,7 @@ __device__ __forceinline__ void build_send_table(const RowTable &t, uint2 *send,
             const uint32_t second = e[4] | e[5] << 8 | e[6] << 16 | e[7] << 24;
             row = turn ? make_uint2(second, first) : make_uint2(first, second);
         }
-        send[job] = row;
+        send[(uint32_t)((own ? K : high + K) - 1) * kLowRanks + (uint32_t)low] = row;
     }
     __syncthreads();
 }

@@ -49,3 +49,30 @@ def test_bounds_of_the_layout():
         g, low, length = form.locate(x)
         assert np.all(np.abs(guess - g) <= 1), p
         assert np.all(low < length) and np.all(length >= 41), p
+
+
+def test_rows_wanted_for_a_stretch():
+    """The kernels that build table rows for a stretch of ranks only name all that these need: the segments' own lowest bits, those of
+    the segments behind them, and where the send exceptions carry to."""
+    rng = np.random.default_rng(10)
+    for p in [129, 257, 1000, (1 << 14) + 1, (1 << 21) - 1, (1 << 23) + 1, (1 << 31) - 1] + [int(2 ** e) for e in rng.uniform(7.1, 31, 200)]:
+        form = Form(p)
+        high, inv = form.q - form.L, (1 << (form.q - form.L + 32)) // p
+        tz = lambda v: high if v == 0 else (v & -v).bit_length() - 1
+        for _ in range(8):
+            x0, n = int(rng.integers(0, p)), min(p, int(2 ** rng.uniform(0, 15)))
+            start = max((x0 * inv >> 32) - 1, 0)
+            named = 0
+            for g in range(start, start + (n * inv >> 32) + 7):
+                g &= (1 << high) - 1
+                z = tz(~g & (1 << high) - 1)
+                named |= 1 << tz(g) | 1 << z
+                if z < high:
+                    named |= 1 << z + 1 + tz(~(g >> z + 1) & (1 << high) - 1)
+            g = np.unique(form.locate(np.arange(x0, x0 + n) % p)[0]).tolist()
+            for v in g:
+                z = tz(~v & (1 << high) - 1)
+                need = 1 << tz(v) | 1 << tz(v + 1 & (1 << high) - 1)
+                if z < high:                                     # the next zero bit, a segment that the last ranks carry to
+                    need |= 1 << tz((v + 1 + (1 << z)) & (1 << high) - 1)
+                assert need & ~named == 0, (p, x0, n, v)
