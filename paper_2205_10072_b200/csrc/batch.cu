@@ -81,10 +81,10 @@ __device__ __forceinline__ void wide_piece(const RowTable &t, const uint8_t *sm,
     const uint64_t byte = job.entry0 + (uint64_t)r * (uint64_t)q;
     WideLane lane;
     lane.init<true>(q, (uint32_t)(byte & 15u));                        // (the outputs start on 16-byte boundaries)
-    wide_rows<false, true>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, recv + byte);
+    wide_rows<false, true, false>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, recv + byte);
     if (send != nullptr) {
         lane.home = -1;
-        wide_rows<true, true>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, send + byte);
+        wide_rows<true, true, false>(t, sm, at.send, ends, job.p, q, job.odd, job.inv, lane, r, n, head, tail, send + byte);
     }
 }
 
@@ -266,7 +266,7 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
             lane.init<true>(q, (uint32_t)(entry0 & 15u));
             for (uint64_t r = ((uint64_t)blockIdx.x * n_warps + warp) * item; r < p; r += (uint64_t)gridDim.x * n_warps * item) {
                 const uint32_t n = p - (uint32_t)r < item ? p - (uint32_t)r : item;
-                wide_rows<decltype(is_send)::value, true>(t, sm, at.send, sm + at.ends + warp * 32u, p, q, job.odd, job.inv, lane,
+                wide_rows<decltype(is_send)::value, true, false>(t, sm, at.send, sm + at.ends + warp * 32u, p, q, job.odd, job.inv, lane,
                                                     (uint32_t)r, n, r == 0, r + n == p, out + entry0 + r * (uint64_t)q);
             }
         };

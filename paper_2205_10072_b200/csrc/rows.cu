@@ -55,7 +55,6 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     }
     __syncthreads();
     build_row_table(t, rc.q, rc.odd);
-    grid_dependency_wait();                                      // nothing before this touches the outputs
     uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
     for (uint64_t b = begin; b < count; b += stride) {
         const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
@@ -91,7 +90,6 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     }
     build_row_table(t, rc.q, rc.odd);
     if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
-    grid_dependency_wait();
     const uint32_t warp = threadIdx.x >> 5;
     uint32_t n_warps = blockDim.x >> 5, index = warp;
     auto all = [&](auto is_send, int8_t *out) {
@@ -102,7 +100,7 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
             const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
             uint32_t x0 = first + (uint32_t)b;
             if (x0 >= rc.p) x0 -= rc.p;
-            wide_rows<decltype(is_send)::value, kAnyStep>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
+            wide_rows<decltype(is_send)::value, kAnyStep, true>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
                                                 mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
         }
     };

@@ -413,6 +413,7 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t shift = kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(dst) & 15u);
     fence_before_bulk();
+    grid_dependency_wait();                                      // (the kernel before: not until the first store)
     __syncwarp();
     const uint32_t begin = (shift + 15u) & ~15u, end = shift + len;
     uint8_t *base = reinterpret_cast<uint8_t *>(dst) - shift;

@@ -92,37 +92,39 @@ struct Pick {
     uint32_t a[4], b[4];
 };
 
+// Selectors of a row's bytes in a vector, a nibble per byte, bytes 0..7 and 8..15: its round 0 would be byte `off` of the vector
+// (-31..31), its home round is `home`, L - 1 if in the table.  A nibble is the round below L; 7 = baseblock (receive: the home
+// round, send: all rounds behind it); 15 = neither (a zero: byte 7 is below 128).
+template <bool kSend>
+__device__ __forceinline__ uint2 row_pick(int off, int q, int home)
+{
+    // nibbles n .. 7 of a word (none from n = 8 on, all for n <= 0)
+    auto from = [](int n) { return n >= 8 ? 0u : 0xffffffffu << (n > 0 ? 4 * n : 0); };
+    constexpr uint32_t low = 0xf6543210u;
+    uint32_t a = ~0u, b = ~0u;
+    if (off <= 0) {
+        if (off > -8) a = __funnelshift_r(low, ~0u, (uint32_t)(-4 * off));
+    } else if (off < 8) {
+        a = low << (4 * off) | ~from(off);
+        b = __funnelshift_l(low, ~0u, (uint32_t)(4 * off));
+    } else if (off < 16) {
+        b = low << (4 * (off - 8)) | ~from(off - 8);
+    }
+    // the baseblock's bytes: nibble 15 without its top bit
+    const int first = off + (kSend ? home + 1 : home), end = kSend ? off + q : first + (home >= kLow ? 1 : 0);
+    a &= ~(0x88888888u & from(first) & ~from(end));
+    b &= ~(0x88888888u & from(first - 8) & ~from(end - 8));
+    return make_uint2(a, b);
+}
+
 // All of a vector's selectors, 16 bits a word: A's row in x and y, the next one's in z and w.  k0: round of the
-// vector's first byte; home_a, home_b: home rounds of A and A + 1, L - 1 if in the table.  (Out of line: needed where the
+// vector's first byte; home_a, home_b: home rounds of A and A + 1.  (Out of line: needed where the
 // home round changes only, at the skips; inlined, parts of it were computed in every segment.)
 template <bool kSend>
 __device__ __noinline__ uint4 packed_pick(int k0, int q, int home_a, int home_b)
 {
-    // The nibbles of a row: its round below L; 7 = baseblock (receive: the home round, send: all
-    // rounds behind it); 15 = neither (a zero: byte 7 is below 128).
-    auto nibbles = [&](int home, uint64_t &lo, uint64_t &hi) {
-        lo = 0xfffffffff6543210ull;
-        hi = ~0ull;
-        if (kSend) {
-            const int from = home + 1;                           // L..q
-            if (from < 16) lo &= ~(0x8888888888888888ull << (4 * from));
-            hi &= from < 16 ? ~0x8888888888888888ull : (from < 32 ? ~(0x8888888888888888ull << (4 * (from - 16))) : ~0ull);
-        } else if (home >= kLow) {
-            if (home < 16) lo &= ~(8ull << (4 * home));
-            else hi &= ~(8ull << (4 * (home - 16)));
-        }
-    };
-    uint64_t lo, hi;
-    nibbles(home_a, lo, hi);
-    uint64_t a = hi >> (4 * (k0 & 15)), b = ~0ull;
-    if (k0 < 16) a = k0 ? lo >> (4 * k0) | hi << (64 - 4 * k0) : lo;
-    const int n = q - k0;                                        // bytes of A's row
-    if (n < 16) {
-        a |= ~0ull << (4 * n);
-        nibbles(home_b, lo, hi);
-        b = lo << (4 * n) | ~(~0ull << (4 * n));
-    }
-    return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+    const uint2 a = row_pick<kSend>(-k0, q, home_a), b = row_pick<kSend>(q - k0, q, home_b);
+    return make_uint4(a.x, a.y, b.x, b.y);
 }
 
 template <bool kSend>
@@ -174,6 +176,15 @@ __device__ __forceinline__ Words far_part(uint32_t g, int q, int k0)
 #pragma unroll
     for (int w = 0; w < 4; ++w) part.w[w] = __shfl_sync(0xffffffffu, e, wrap(k0 + 4 * w));
     return part;
+}
+
+// The bytes of the rows.
+__device__ __forceinline__ Words wide_rows_of(const uint2 a, const uint2 b, const Pick &pick)
+{
+    Words x;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) x.w[w] = pick_bytes(a.x, a.y, pick.a[w]) | pick_bytes(b.x, b.y, pick.b[w]);
+    return x;
 }
 
 __device__ __forceinline__ uint4 wide_vector(const uint2 a, const uint2 b, const Words &c, const Pick &pick)
@@ -236,8 +247,12 @@ struct WideLane {
 // theirs too (else n is a multiple of 16).
 // sm: the CTA's shared memory, the row table at 0, the send table at send_at; ends: 32 bytes for the two vectors that are
 // not written as a whole.
+// Waits for the kernel before (dependent launches) in front of the first store: where the run starts, some 2400 cycles, does not
+// depend on it (all ranks of 100 003 6.0 -> 5.5 us).
+// kRoom: the kernel has registers left for one computation of selectors per change of the home round instead of two (some 700 cycles each,
+// and the warp that has the first ranks has four or five such changes); the middle kernel of a batch would spill (1320 -> 1350 us).
 // kAnyStep: false where step_ranks(q) is known to be 16 (a constant: 0.2-0.3 us less for tables of up to 2 million ranks).
-template <bool kSend, bool kAnyStep>
+template <bool kSend, bool kAnyStep, bool kRoom>
 __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, uint32_t send_at, uint8_t *ends, uint32_t p,
                                           int q, uint32_t odd, uint32_t inv, WideLane &mine, uint32_t x0, uint32_t n,
                                           bool head, bool tail, int8_t *dst)
@@ -372,6 +387,7 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
             if (home != mine.home) mine.pick = make_pick<kSend>(mine.k0, q, home, home);
             mine.home = home;
             begun = true;
+            grid_dependency_wait();                              // (the kernel before: not until the first store)
         } else {
             base = __shfl_sync(0xffffffffu, pos, 0) - (uint32_t)start;
             next = (int)(__shfl_sync(0xffffffffu, pos, 1) - base);
@@ -410,22 +426,36 @@ __device__ __forceinline__ void wide_rows(const RowTable &t, const uint8_t *sm, 
             const int A = step + mine.a;
             const uint32_t new_at = (inf2 & 0xffffffu) + (uint32_t)((A - next) * 8);
             const bool behind = A >= next, behind_b = A + 1 >= next;
-            if (mine.home != home2)
-                mine.pick = make_pick<kSend>(mine.k0, q, behind ? home2 : mine.home, behind_b ? home2 : mine.home);
-            if (to < len) {
-                Words c;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const uint32_t keep = behind_b ? (behind ? 0u : mine.own[w]) : 0xffffffffu;
-                    c.w[w] = (part.w[w] & keep) | (coming.w[w] & ~keep);
-                }
+            auto segment_part = [&](int w) {                     // of the two segments
+                const uint32_t keep = behind_b ? (behind ? 0u : mine.own[w]) : 0xffffffffu;
+                return (part.w[w] & keep) | (coming.w[w] & ~keep);
+            };
+            if (kRoom && mine.home != home2) {
+                // the rows in front by the selectors so far, those behind by the new ones
+                const uint2 none = make_uint2(0u, 0u);
                 const uint2 ra = *reinterpret_cast<const uint2 *>(sm + (behind ? new_at : at));
                 const uint2 rb = *reinterpret_cast<const uint2 *>(sm + (uint32_t)((behind_b ? new_at : at) + 8u));
-                store(to, wide_vector(ra, rb, c, mine.pick));
+                Words c = wide_rows_of(behind ? none : ra, behind_b ? none : rb, mine.pick);
+                mine.pick = make_pick<kSend>(mine.k0, q, home2, home2);
+                const Words d = wide_rows_of(behind ? ra : none, behind_b ? rb : none, mine.pick);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) c.w[w] |= d.w[w] | segment_part(w);
+                if (to < len) store(to, make_uint4(c.w[0], c.w[1], c.w[2], c.w[3]));
+            } else {
+                if (!kRoom && mine.home != home2)
+                    mine.pick = make_pick<kSend>(mine.k0, q, behind ? home2 : mine.home, behind_b ? home2 : mine.home);
+                if (to < len) {
+                    Words c;
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) c.w[w] = segment_part(w);
+                    const uint2 ra = *reinterpret_cast<const uint2 *>(sm + (behind ? new_at : at));
+                    const uint2 rb = *reinterpret_cast<const uint2 *>(sm + (uint32_t)((behind_b ? new_at : at) + 8u));
+                    store(to, wide_vector(ra, rb, c, mine.pick));
+                }
+                if (!kRoom && mine.home != home2) mine.pick = make_pick<kSend>(mine.k0, q, home2, home2);
             }
-            part = coming;
-            if (mine.home != home2) mine.pick = make_pick<kSend>(mine.k0, q, home2, home2);
             mine.home = home2;
+            part = coming;
             at = new_at + 8u * ranks;
             to += step_bytes;
             step += (int)ranks;
