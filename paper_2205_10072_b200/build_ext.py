@@ -12,6 +12,9 @@ LIB_PATH = os.path.join(_PKG, "libbcs.so")
 SOURCES = sorted(glob.glob(os.path.join(_PKG, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(_ROOT, "include", "*.h")) +
                  glob.glob(os.path.join(_PKG, "csrc", "*.cuh")))
+# The packed rows of all shapes of segments, written by a small program at build time.
+ROW_TABLE = os.path.join(_PKG, "csrc", "row_table.inc")
+ROW_TABLE_SOURCE = os.path.join(_PKG, "csrc", "gen", "row_table.c")
 # The calls of the library for Python (csrc/calls.c), linked to it.
 CALLS_PATH = os.path.join(_PKG, "_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 CALLS_SOURCE = os.path.join(_PKG, "csrc", "calls.c")
@@ -37,7 +40,7 @@ def _stale(lib: str, deps: list) -> bool:
 
 
 def stale() -> bool:
-    return _stale(LIB_PATH, SOURCES + HEADERS)
+    return _stale(LIB_PATH, SOURCES + HEADERS + [ROW_TABLE_SOURCE])
 
 
 def _nvcc(lib: str, sources: list, verbose: bool, extra: list = ()) -> None:
@@ -48,8 +51,25 @@ def _nvcc(lib: str, sources: list, verbose: bool, extra: list = ()) -> None:
     os.replace(tmp, lib)
 
 
+def build_row_table(force: bool = False) -> str:
+    """Compiles and runs csrc/gen/row_table.c, which writes the constants that the row kernels include."""
+    if force or _stale(ROW_TABLE, [ROW_TABLE_SOURCE]):
+        tmp = ROW_TABLE + ".%d.tmp" % os.getpid()
+        exe = tmp + ".exe"
+        try:
+            subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-o", exe, ROW_TABLE_SOURCE])
+            with open(tmp, "wb") as out:
+                subprocess.check_call([exe], stdout=out)
+        finally:
+            if os.path.exists(exe):
+                os.remove(exe)
+        os.replace(tmp, ROW_TABLE)
+    return ROW_TABLE
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Runs nvcc (cross-compiles without a GPU).  Returns the path of the shared library."""
+    build_row_table(force)
     if force or stale():
         _nvcc(LIB_PATH, SOURCES, verbose)
     build_calls(force)

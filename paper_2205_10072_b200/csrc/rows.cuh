@@ -28,9 +28,8 @@
 // close behind a segment's start.
 //
 // Rounds below L.  The entries of a rank depend on (K, low) only, low < skips[L] <= 128: a table of at most
-// 25 x 128 rows of 8 bytes.  The CTA fills it by running Algorithm 4 itself on those rows, the windows read
-// from the baseblocks of the ranks around a segment's start: what lies d ranks below the rank skips[K] is what lies
-// d + C(7, K) ranks below skips[7].
+// 25 x 128 rows of 8 bytes in the CTA's shared memory.  What lies d ranks below the rank skips[K] is what lies
+// d + C(7, K) ranks below skips[7], so there are few shapes of such rows in all: they are kept as constants.
 //
 // All of this is checked entry by entry against the CPU oracle by the tests.
 #pragma once
@@ -40,8 +39,6 @@ namespace bcs {
 
 constexpr int kLow = 7;                       // rounds whose entries come from the table
 constexpr int kLowRanks = 128;                // skips[7] <= 128
-constexpr int kRunLevels = 6;                 // runs of 1, 2, 4, ..., 32 ranks
-constexpr int kAround = 160, kBehind = 80;    // ranks around a segment's start that windows are read from, those before it
 constexpr int kMissRanks = 32;                // ranks behind a segment's start that can be exceptions (<= 25)
 constexpr uint32_t kRootMark = 0x7f;          // in place of the root's baseblock in the table
 constexpr uint32_t kItemRanks = 128;          // ranks that a warp takes at a time
@@ -77,16 +74,12 @@ static_assert(kItemSegments * 8u <= 48u && kWarpStage % 16u == 0, "layout of a w
 
 // Byte offsets in the CTA's dynamic shared memory.
 struct RowLayout {
-    uint32_t miss, bits, codes, rounds, six, s, flags, warps, warp_bytes;
+    uint32_t miss, s, flags, warps, warp_bytes;
     __host__ __device__ explicit RowLayout(int q)
     {
         const uint32_t rows = (uint32_t)(q - low_levels(q) + 1);
         miss = rows * kLowRanks * 8u;
-        bits = miss + rows * kMissRanks;
-        codes = bits + kLowRanks;
-        rounds = codes + kLowRanks;
-        six = rounds + 8u * 8u;
-        s = six + 64u * 8u;
+        s = miss + rows * kMissRanks;
         flags = s + (kRow + kLow + 1) * 4u;
         warps = flags + 16u + 32u;
         warps = (warps + 127u) & ~127u;
@@ -98,192 +91,75 @@ struct RowLayout {
 struct RowTable {
     uint2 *rows;          // [K - L][low]: entries of rounds 0..6 as bytes 0..6, baseblock as byte 7
     uint8_t *miss;        // [K - L][low < 32]: the block of 0..7 that is not taken before round 7
-    uint8_t *bits;        // [x]: baseblock bit of x < skips[L]
-    uint8_t *codes;       // [x]: skip code of x < skips[L]
-    uint2 *rounds;        // [i]: where round i < 6 finds its windows, see below
-    uint2 *six;           // rows of the ranks with bit 6 set, without round 6
     uint32_t *s;
     uint32_t *wanted;     // bit K - L: the rows of K are wanted
     uint8_t *list;        // the wanted K
-    uint8_t *runs;        // [K of the list, then K = 6][level][x + 80]: baseblock bits of the 2^level ranks that end x ranks
-                          // from the start of a segment whose lowest bit is K; used while the table is built only, in
-                          // the place of what comes behind it (at most 26 x 960 bytes; eight warps' parts are 34 KB
-                          // from q = 17 on, and 17 KB where q <= 16 needs 11 KB)
     __device__ RowTable(uint8_t *sm, const RowLayout &at)
-        : rows(reinterpret_cast<uint2 *>(sm)), miss(sm + at.miss), bits(sm + at.bits), codes(sm + at.codes),
-          rounds(reinterpret_cast<uint2 *>(sm + at.rounds)), six(reinterpret_cast<uint2 *>(sm + at.six)),
-          s(reinterpret_cast<uint32_t *>(sm + at.s)), wanted(reinterpret_cast<uint32_t *>(sm + at.flags)),
-          list(sm + at.flags + 16), runs(sm + at.warps)
+        : rows(reinterpret_cast<uint2 *>(sm)), miss(sm + at.miss), s(reinterpret_cast<uint32_t *>(sm + at.s)),
+          wanted(reinterpret_cast<uint32_t *>(sm + at.flags)), list(sm + at.flags + 16)
     {
     }
 };
 
-// One warp: the runs around the start of a segment whose lowest bit is K, eight ranks per lane.
-__device__ __forceinline__ void build_runs(const RowTable &t, int q, uint32_t odd, int K, uint8_t *runs)
+// The rows of all shapes of segments (gen/row_table.c writes them at build time and says how they are packed): 1.7 MB, of which a
+// CTA reads 512 bytes for each K that it wants, by one load per row.
+#include "row_table.inc"
+
+// A packed row: entries are block - q, K for 8, blocks of 16 and more the rank's own.
+__device__ __forceinline__ uint2 unpack_row(unsigned long long v, int q, int K)
 {
-    const uint32_t lane = threadIdx.x & 31u;
-    // the ranks below the rank skips[K] are those below `top`
-    const int top = K >= kLow ? (int)t.s[kLow] - (int)count_odd(odd, kLow, K) : (int)t.s[K];
-    const int lows = (int)t.s[low_levels(q)];
-    unsigned long long r = 0;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const int x = (int)lane * 8 + b - kBehind;
-        const int z = x < 0 ? top + x : x;
-        uint32_t bit = z >= 1 && z < lows ? t.bits[z] : 0u;
-        if (x == 0) bit = K < q ? 1u << (K < kLow ? K : kLow) : 0u;  // block K, as bit 7 from K = 7 on
-        r |= (unsigned long long)bit << (8 * b);
-    }
-    unsigned long long *at = reinterpret_cast<unsigned long long *>(runs) + lane;
-    auto before = [&](uint32_t lanes) {
-        const unsigned long long up = __shfl_up_sync(0xffffffffu, r, lanes);
-        return lane >= lanes ? up : 0ull;
+    auto word = [&](uint32_t x, uint32_t ones) {
+        x += ((x >> 3) & 0x01010101u) * (uint32_t)(K - 8) + ((x >> 4) & 0x01010101u) * (uint32_t)(q - 16);
+        return ((x | 0x80808080u) - (uint32_t)q * ones) ^ 0x80808080u;          // (no byte borrows)
     };
-    auto store = [&](int level) {
-        if (lane < kAround / 8) at[level * (kAround / 8)] = r;
-    };
-    store(0);
-    r |= r << 8 | before(1) >> 56;
-    store(1);
-    r |= r << 16 | before(1) >> 48;
-    store(2);
-    r |= r << 32 | before(1) >> 32;
-    store(3);
-    r |= before(1);
-    store(4);
-    r |= before(2);
-    store(5);
+    return make_uint2(word((uint32_t)v, 0x01010101u), word((uint32_t)(v >> 32) & 0x1fffffffu, 0x00010101u));
 }
 
-// Rounds 0 .. kRounds-1 (at most six) of rank `low` of a segment whose lowest bit is K: Algorithm 4 with its
-// windows looked up in the runs of K.  Returns the entries as bytes 0..5 and the baseblock as byte 7; B: the blocks
-// taken, K as bit 7 from K = 7 on.  (Both windows of all rounds are loaded at once; the chain from round to round is
-// a few operations on B.)
-template <int kRounds>
-__device__ __forceinline__ uint2 table_row(const RowTable &t, const uint8_t *runs, int q, int K, int low, uint32_t &B)
-{
-    const uint32_t c = t.codes[low];
-    const int flag = K < kLow ? K : kLow;
-    uint32_t first[kRounds], second[kRounds];
-#pragma unroll
-    for (int i = 0; i < kRounds; ++i) {
-        const uint2 r = t.rounds[i];                             // ends of the two runs of either window
-        first[i] = runs[(r.x & 0xffffu) + (uint32_t)low] | runs[(r.x >> 16) + (uint32_t)low];
-        second[i] = r.y ? runs[(r.y & 0xffffu) + (uint32_t)low] | runs[(r.y >> 16) + (uint32_t)low] : 0u;
-    }
-    const int bb = c ? __ffs(c) - 1 : (K < q ? K : -1);
-    B = c ? c & (0u - c) : (K < q ? 1u << flag : 0u);
-    uint32_t entry[8] = {0, 0, 0, 0, 0, 0, 0, bb >= 0 ? (uint32_t)bb : kRootMark};
-#pragma unroll
-    for (int i = 0; i < kRounds; ++i) {
-        const uint32_t above = c >> (i + 1);
-        const bool set = ((c >> i) & 1u) != 0u;
-        uint32_t U = first[i] & ~B;
-        if (U == 0u) U = second[i] & ~B;
-        if (set) U = above ? (above & (0u - above)) << (i + 1) : 1u << flag;
-        const bool home = set && above == 0u && K == q;          // the home round: its own block
-        const int blk = top_bit(U);
-        if (U != 0u && !home) B |= U & (0x80000000u >> __clz(U));
-        const int label = blk == kLow ? K : blk;
-        entry[i] = (uint32_t)(uint8_t)(home ? bb : (U ? label - q : BCS_BAD_ENTRY));
-    }
-    return make_uint2(entry[0] | entry[1] << 8 | entry[2] << 16 | entry[3] << 24,
-                      entry[4] | entry[5] << 8 | entry[6] << 16 | entry[7] << 24);
-}
-
-template <int kRounds>
-__device__ __forceinline__ void build_whole_table(const RowTable &t, int q)
-{
-    if (q != kRounds) return;
-    for (uint32_t low = threadIdx.x; low < t.s[kRounds]; low += blockDim.x) {
-        uint32_t B;
-        t.rows[low] = table_row<kRounds>(t, t.runs, q, q, (int)low, B);
-    }
-}
-
-// Fills the table of a p, for the K whose bits in *t.wanted are set (q > 7); all threads of the CTA call (at least
-// 128), after a barrier behind the writes of t.s (the skips, then zeros) and *t.wanted.  Ends with a barrier.
+// Fills the table of a p, for the K whose bits in *t.wanted are set (q > 7); all threads of the CTA call, after a barrier behind the
+// writes of t.s (the skips, then zeros) and *t.wanted.  Ends with a barrier.
+// (One load and some twenty instructions a row.  Computed by Algorithm 4 in every CTA it took 5000 cycles before the first row: 65 553 ranks
+// 4.2 -> 3.3 us, all ranks of 100 003 5.5 -> 4.3, of about 2^20 15.6 -> 13.6, every p up to 1024 18.3 -> 16.7, back to back; a call alone 2 us
+// less.)
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {
     const int L = low_levels(q);
     const uint32_t lows = t.s[L];
-    if (threadIdx.x < kLowRanks) {
-        uint32_t x = threadIdx.x, c = 0;
-#pragma unroll
-        for (int k = kLow - 1; k >= 0; --k) {
-            const uint32_t skip = t.s[k];
-            if (k < L && x >= skip) {
-                x -= skip;
-                c |= 1u << k;
-            }
-        }
-        t.codes[threadIdx.x] = (uint8_t)c;
-        t.bits[threadIdx.x] = (uint8_t)(threadIdx.x < lows ? c & (0u - c) : 0u);
-    }
-    const uint32_t round = blockDim.x > kLowRanks ? threadIdx.x - kLowRanks : threadIdx.x;
-    if (round < kLow - 1u) {
-        // Windows of round i, as ends of runs counted from the rank (`len` ranks are two runs of 2^floor(log2 len)): the
-        // first skips[i+1] - skips[i] ranks that end skips[i] below it, the second those from there to the sum of
-        // the skips 0..i below it.
-        const int i = (int)round;
-        const int lo = (int)t.s[i], hi = (int)t.s[i + 1];
-        int sum = 0;
-        for (int k = 0; k <= i; ++k) sum += (int)t.s[k];
-        auto ends = [](int end, int len) {
-            const int level = 31 - __clz(len);
-            const uint32_t at = (uint32_t)(level * kAround + kBehind - end);
-            return at | (at - (uint32_t)(len - (1 << level))) << 16;
-        };
-        t.rounds[i] = i < L ? make_uint2(ends(lo, hi > lo ? hi - lo : 1), sum >= hi ? ends(hi, sum - hi + 1) : 0u) : make_uint2(0u, 0u);
-    }
-    if (threadIdx.x < 32u) {                                     // list of the K
-        const uint32_t wanted = q > kLow ? *t.wanted : 1u;
-        if ((wanted >> threadIdx.x) & 1u) t.list[__popc(wanted & ((1u << threadIdx.x) - 1u))] = (uint8_t)(L + threadIdx.x);
-    }
-    __syncthreads();
-    const int n_list = q > kLow ? __popc(*t.wanted) : 1;
-    for (int k = (int)(threadIdx.x >> 5); k < n_list + (q >= kLow ? 1 : 0); k += (int)(blockDim.x >> 5))
-        build_runs(t, q, odd, k < n_list ? t.list[k] : 6, t.runs + k * kRunLevels * kAround);
-    __syncthreads();
     if (q < kLow) {                                              // one segment, all rounds in the table
-        build_whole_table<1>(t, q);
-        build_whole_table<2>(t, q);
-        build_whole_table<3>(t, q);
-        build_whole_table<4>(t, q);
-        build_whole_table<5>(t, q);
-        build_whole_table<6>(t, q);
-    } else {
-        // ranks without bit 6: rounds 0..5 as above, round 6 from the distances of the ranks with
-        // baseblock 7 and 6.  Ranks with it (K = 6 here): rounds 0..5 do not depend on what comes before
-        // that bit, round 6 receives the next higher one.
-        const int n = n_list * 64;
-        for (int job = (int)threadIdx.x; job < n + 64; job += (int)blockDim.x) {
-            const int K = job < n ? t.list[job >> 6] : 6, low = job & 63;
-            if (low >= (int)t.s[6]) continue;
-            uint32_t B;
-            uint2 row = table_row<6>(t, t.runs + (job >> 6) * kRunLevels * kAround, q, K, low, B);
-            if (K == 6) {
-                t.six[low] = row;
-            } else {
-                const int m = __ffs(~B) - 1;                     // the block of 0..6 not taken so far
-                const bool seven = low < (int)count_odd(odd, kLow, K) ||
-                                   (m == 6 && K > kLow && low < (int)count_odd(odd, 6, K));
-                row.y |= (uint32_t)(uint8_t)((seven ? kLow : m) - q) << 16;
-                t.rows[(K - kLow) * kLowRanks + low] = row;
-                if (low < kMissRanks) t.miss[(K - kLow) * kMissRanks + low] = (uint8_t)(seven ? m : kLow);
-            }
+        for (uint32_t low = threadIdx.x; low < lows; low += blockDim.x) {
+            uint2 row = unpack_row(__ldg(row_small + lows * (lows - 1u) / 2u + low), q, 0x7f);
+            row.y &= 0xff000000u | (q > 4 ? (1u << (8 * (q - 4))) - 1u : 0u);
+            if (low == 0u) row.y |= kRootMark << 24;
+            t.rows[low] = row;
         }
         __syncthreads();
-        for (int job = (int)threadIdx.x; job < n; job += (int)blockDim.x) {
-            const int K = t.list[job >> 6], low = job & 63;
-            const int at = low + (int)t.s[6];
-            uint2 row = make_uint2(0u, 0u);                      // (read, but not used, behind the last one)
-            if (at < (int)t.s[7]) {
-                row = t.six[low];
-                row.y |= (uint32_t)(uint8_t)(K < q ? K - q : (int)(row.y >> 24)) << 16;
-            }
-            if (at < kLowRanks) t.rows[(K - kLow) * kLowRanks + at] = row;
+        return;
+    }
+    const uint32_t wanted = q > kLow ? *t.wanted : 1u;
+    if (threadIdx.x < 32u && ((wanted >> threadIdx.x) & 1u))     // list of the K
+        t.list[__popc(wanted & ((1u << threadIdx.x) - 1u))] = (uint8_t)(L + threadIdx.x);
+    __syncthreads();
+    const uint32_t six = t.s[6];
+    const unsigned long long *shapes = row_shapes + (lows - 65u) * (52u * 64u), *sixes = row_six + (lows - 65u) * 64u;
+    const int n = __popc(wanted) * 64;
+    for (int job = (int)threadIdx.x; job < n; job += (int)blockDim.x) {
+        const int K = t.list[job >> 6];
+        const uint32_t low = (uint32_t)job & 63u, shape = (K == q ? 26u : 0u) + (K == kLow ? 0u : 1u + count_odd(odd, kLow, K));
+        const unsigned long long v = __ldg(shapes + shape * 64u + low), w = __ldg(sixes + low);
+        uint2 *rows = t.rows + (K - kLow) * kLowRanks;
+        if (low < six) {
+            uint2 row = unpack_row(v, q, K);
+            if (K == q && low == 0u) row.y |= kRootMark << 24;
+            rows[low] = row;
+            if (low < (uint32_t)kMissRanks) t.miss[(K - kLow) * kMissRanks + (int)low] = (uint8_t)(v >> 61);
         }
+        // ranks with bit 6: the rounds before that do not depend on K, round 6 receives the next higher bit
+        const uint32_t at = low + six;
+        uint2 row = make_uint2(0u, 0u);                          // (read, but not used, behind the last one)
+        if (at < lows) {
+            row = unpack_row(w, q, K);
+            row.y = (row.y & 0xff00ffffu) | (uint32_t)(uint8_t)(K < q ? K - q : (int)(row.y >> 24)) << 16;
+        }
+        if (at < kLowRanks) rows[at] = row;
     }
     __syncthreads();
 }

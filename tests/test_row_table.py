@@ -1,0 +1,57 @@
+"""The constants that the row kernels include (written by csrc/gen/row_table.c when the library is built), unpacked as the kernels
+do it, are the rows of the rule restated in tests/segment_form.py and, for the smallest p, of the oracle."""
+import re
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2205_10072_b200 import build_ext
+from tests.segment_form import Form
+
+
+@pytest.fixture(scope="module")
+def packed():
+    with open(build_ext.build_row_table()) as f:
+        parts = re.split(r"static __device__ const unsigned long long (\w+)", f.read())[1:]
+    return {name: np.array([int(v, 16) for v in re.findall(r"0x[0-9a-f]+", body)], dtype=np.uint64).view(np.uint8).reshape(-1, 8).astype(int)
+            for name, body in zip(parts[::2], parts[1::2])}
+
+
+def _unpack(rows, q, K):
+    """Entries of the rounds 0..6, baseblock, missing block."""
+    block, own = np.where(rows == 8, K, rows & 15), rows >= 16
+    base = rows[:, 7] & 15
+    return np.where(own, block, block - q)[:, :7], np.where(base == 8, K, base), rows[:, 7] >> 5
+
+
+def test_rows_of_every_shape(packed):
+    rng = np.random.default_rng(11)
+    shapes = packed["row_shapes"].reshape(64, 52, 64, 8)
+    sixes = packed["row_six"].reshape(64, 64, 8)
+    seen = set()
+    for p in [*range(65, 1400, 7), (1 << 30) + 1, (1 << 31) - 1] + [int(2 ** e) for e in rng.uniform(10, 31, 300)]:
+        form = Form(p)
+        q, six, lows = form.q, form.s[6], form.s[7]
+        for K in range(7, q + 1):
+            shape = (26 if K == q else 0) + (0 if K == 7 else 1 + int(form.C(7, K)))
+            if (lows, shape) in seen:
+                continue
+            seen.add((lows, shape))
+            want, base, missing = form.table(K)
+            got, bb, miss = _unpack(shapes[lows - 65, shape, :six], q, K)
+            assert np.array_equal(got, want[:six]) and np.array_equal(miss, missing[:six]), (p, K)
+            if K == q:
+                base, bb = base[1:], bb[1:]                      # (the root has none)
+            assert np.array_equal(bb, base[:six - (K == q)]), (p, K)
+            got, bb, _ = _unpack(sixes[lows - 65, :lows - six], q, K)
+            assert np.array_equal(got[:, :6], want[six:, :6]) and np.array_equal(bb, form.table(K)[1][six:]), (p, K)
+    assert len(seen) > 900
+
+
+def test_rows_of_small_p(packed):
+    rows = packed["row_small"]
+    for p in range(2, 65):
+        q = Form(p).q
+        got, _, _ = _unpack(rows[p * (p - 1) // 2:p * (p + 1) // 2], q, 0)
+        assert np.array_equal(got[:, :q], oracle.full_table(p)[0]), p
