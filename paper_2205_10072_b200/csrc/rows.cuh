@@ -211,54 +211,41 @@ __device__ __forceinline__ void want_rows(const RowTable &t, int q, uint32_t inv
 // (The same for every 32 ranks of an item: 32 rows are whole words.)
 struct RowPlace {
     uint32_t sh;       // bits by which the row is off a word
-    bool longer;       // it reaches into word ceil(q / 4), counted from the word it begins in
+    bool longer;       // it ends in or behind word ceil(q / 4), counted from the word it begins in
     uint32_t shared;   // all ones if the next row begins in this row's last word
     __device__ RowPlace(uint32_t first_byte, int q)
     {
         const uint32_t mis = (first_byte + (threadIdx.x & 31u) * (uint32_t)q) & 3u;
         sh = 8u * mis;
-        longer = mis + (uint32_t)q > 4u * (((uint32_t)q + 3u) / 4u);
+        longer = mis + (uint32_t)q >= 4u * (((uint32_t)q + 3u) / 4u);
         shared = ((mis + (uint32_t)q) & 3u) != 0u ? 0xffffffffu : 0u;
     }
 };
 
 // Stores the rows (words W, zero beyond byte q) of 32 ranks at once, this lane's at `at`.  A word that two rows share is
-// put together by the lane it begins in.  kAligned: the first row begins on a word.  Where it
-// does not, the first lane's head and the last lane's tail go out as bytes.  Lanes without a rank store
+// stored by the lane it ends in.  kAligned: the first row begins on a word.  Else the last lane stores what it has of a shared word, too, and the first
+// lane of the next 32 ranks (`more`) completes that.  Lanes without a rank store
 // too (the buffer has room for them, and nobody reads it).
+// (With the words at either end written byte by byte every p up to 1024 took 16.5 us and not 13.8, 1024 p up to 2^20 1257 and not 1250.)
 template <int kWords, bool kAligned>
-__device__ __forceinline__ void stage_row(uint8_t *at, const uint32_t (&W)[kWords], int q, const RowPlace &pl)
+__device__ __forceinline__ void stage_row(uint8_t *at, const uint32_t (&W)[kWords], int q, const RowPlace &pl, bool more)
 {
     if (kWords == 1 && q < 4) {
         for (int k = 0; k < q; ++k) at[k] = (uint8_t)(W[0] >> (8 * k));
         return;
     }
+    const uint32_t lane = threadIdx.x & 31u;
     uint32_t V[kWords + 1];
 #pragma unroll
     for (int w = 0; w <= kWords; ++w) V[w] = __funnelshift_l(w ? W[w - 1] : 0u, w < kWords ? W[w] : 0u, pl.sh);
-    uint32_t next = __shfl_down_sync(0xffffffffu, V[0], 1) & pl.shared;
     uint32_t *words = reinterpret_cast<uint32_t *>(at - (pl.sh >> 3));
-    bool tail_bytes = false;
-    if (!kAligned) {
-        const uint32_t lane = threadIdx.x & 31u;
-        tail_bytes = lane == 31u && pl.shared != 0u;
-        if (lane == 0u && pl.sh != 0u)
-            for (uint32_t e = pl.sh; e < 32u; e += 8u) at[(e - pl.sh) >> 3] = (uint8_t)(V[0] >> e);
-        if (tail_bytes) {
-            const uint32_t v = pl.longer ? V[kWords] : V[kWords - 1];
-            uint8_t *tail = reinterpret_cast<uint8_t *>(words + (pl.longer ? kWords : kWords - 1));
-            for (uint32_t e = 0; e < (((pl.sh >> 3) + (uint32_t)q) & 3u); ++e) tail[e] = (uint8_t)(v >> (8u * e));
-        }
-    }
-    if (kWords > 1) {
-        if (pl.sh == 0u) words[0] = V[0];
+    const uint32_t rest = (pl.longer ? V[kWords] : V[kWords - 1]) & pl.shared;
+    const uint32_t before = __shfl_sync(0xffffffffu, rest, (lane - 1u) & 31u);
+    V[0] |= kAligned || lane != 0u ? before : (more && pl.sh ? words[0] : 0u);       // (aligned: lane 31 shares no word)
 #pragma unroll
-        for (int w = 1; w < kWords - 1; ++w) words[w] = V[w];
-        if (kAligned || pl.longer || !tail_bytes) words[kWords - 1] = V[kWords - 1] | (pl.longer ? 0u : next);
-    } else if (pl.sh == 0u) {
-        words[0] = V[0];
-    }
-    if (pl.longer && (kAligned || !tail_bytes)) words[kWords] = V[kWords] | next;
+    for (int w = 0; w < kWords - 1; ++w) words[w] = V[w];
+    if (pl.longer) words[kWords - 1] = V[kWords - 1];
+    if (!kAligned && lane == 31u && pl.shared) words[pl.longer ? kWords : kWords - 1] = rest;
 }
 
 // Row of a rank: its rounds below L from the table, the others from its segment.
@@ -420,7 +407,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
             const uint32_t note = notes[b + lane];
             uint32_t W[kWords];
             join_row<kWords>(row.x, row.y, entries + (note & 7u) * 64u, W);
-            stage_row<kWords, kAligned>(at, W, q, place);
+            stage_row<kWords, kAligned>(at, W, q, place, b != 0u);
             __syncwarp();
             const uint32_t from = (note >> kNoteFrom) & 31u;
             if (from > (uint32_t)L) at[from - 1u] = (uint8_t)(row.y >> 24);     // home round
@@ -432,6 +419,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
                 for (; low < (int)count_odd(odd, k + 1, K); ++k) at[k] = (uint8_t)(k + 1 - q);
                 at[k] = (uint8_t)((int)t.miss[(K - L) * kMissRanks + low] - q);
             }
+            if (!kAligned) __syncwarp();                         // (bytes of a word that the first lane completes next)
         }
         flush_item<kAligned>(stage, recv, n * (uint32_t)q);
     }
@@ -458,7 +446,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
             }
             uint32_t W[kWords];
             join_row<kWords>(lo, hi, entries + (note & 7u) * 64u + 32u, W);
-            stage_row<kWords, kAligned>(at, W, q, place);
+            stage_row<kWords, kAligned>(at, W, q, place, b != 0u);
             __syncwarp();
             const int from = (int)((note >> kNoteFrom) & 31u);
             if (from < q) {                                      // rounds past the home round: the baseblock
@@ -481,6 +469,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
                     at[k] = (uint8_t)(block - q);
                 }
             }
+            if (!kAligned) __syncwarp();
         }
         flush_item<kAligned>(stage, send, n * (uint32_t)q);
     }
