@@ -12,6 +12,8 @@ constexpr int kAgThreads = 256;   // threads per CTA; a CTA writes 256 consecuti
 constexpr int kAgLine = 32;       // int32 elements per 128-byte line
 constexpr int kAgCols = kAgThreads + kAgLine;   // buffers staged per CTA: its window slides by up to 31 from row to row
 constexpr int kAgCtas = 148 * 32; // CTAs that a call aims for: the rounds are cut into as many chunks as that takes
+constexpr uint32_t kAgRounds = 64;          // rounds that make up for the staging of a CTA's rows,
+constexpr uint32_t kAgFewCtas = 148 * 4;  // as far as that leaves so many CTAs
 constexpr int kAgRowBytes = kAgCols * BCS_MAX_Q + 48;
 
 // Where the rows of a CTA's columns lie in its copy of a schedule table: column c (buffer j0 + c,
@@ -253,10 +255,14 @@ bcs_status bcs_allgather_tables(uint32_t p, uint32_t n, uint32_t r, const int8_t
     // A CTA stages the schedule rows of its buffers once and then streams rows of the output: the
     // rounds are cut into as many chunks (a multiple of four rounds each) as it takes to have
     // about kAgCtas CTAs (measured best on p = 100 003, n = 1000: 5.9 TB/s; a quarter or four times
-    // as many CTAs 5.1 resp. 4.5 TB/s).
+    // as many CTAs 5.1 resp. 4.5 TB/s).  Where that would leave a CTA less than some 64 rounds, staging 288 rows costs more than
+    // writing: fewer chunks then, down to four CTAs per SM (us before / like this: p = 20 262, n = 116 21.4 / 12.9; 261 597, 7 28.3 / 17.3;
+    // 5000, 500 17.0 / 11.7; 50 000, 20 15.0 / 10.8; 260 000, 100 59 / 46, with 32 rounds 54).
     const uint32_t rounds = n - 1u + (uint32_t)tab.q;
     const uint32_t col_blocks = (p + kAgThreads - 1) / kAgThreads;
     uint32_t chunks = (kAgCtas + col_blocks - 1) / col_blocks;
+    const uint32_t few = (kAgFewCtas + col_blocks - 1) / col_blocks, many = (rounds + kAgRounds - 1) / kAgRounds;
+    if (chunks > many) chunks = many > few ? many : few;
     uint32_t per_cta = ((rounds + chunks - 1) / chunks + 3u) & ~3u;
     chunks = (rounds + per_cta - 1) / per_cta;
     dim3 grid(col_blocks, chunks);
