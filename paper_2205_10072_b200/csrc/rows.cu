@@ -1,14 +1,15 @@
 // Receive and send rows of a stretch of ranks of one p: the kernels behind bcs_build and its relatives.
 //
-// One launch, nothing read from memory, no table of all ranks (rows.cuh).  Two forms, by size (launch_rows):
-//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp; 44 % of the issue slots at 65 553
-//     ranks of about 2^20.  Back to back 32 ranks 3.5 us, all ranks of 1152 3.6, 65 553 ranks 4.25.  The table holds what the
+// One launch, nothing read from memory but constants, no table of all ranks (rows.cuh).  Two forms, by size (launch_rows):
+//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp.  From Python 32 ranks 3.2 us back to
+//     back, all ranks of 1152 3.3, 65 553 ranks 3.3 (2.7 on the device).  The table holds what the
 //     CTA's segments need where these are few, and a CTA has no more warps than items.
-//   * wide_kernel, 16 output bytes per lane (wide.cuh).  Up to some 2^23 ranks bound by instruction issue (61 % of the slots at 2^20
-//     ranks) behind a table that every CTA builds whole; up to 2^20 ranks two CTAs fit an SM, so that the next call's table is
-//     built beside the rows, above it the 61 440 registers of a CTA leave no room and the table's time is in series.
-//     From about 2^25 ranks on bound by memory writes.  All ranks of 100 003 6.1 us, of about 2^20 17.0, 8 chunks of about
-//     2^28 2.38 to 2.48 ms (6.3 to 6.0 TB/s; the power cap shows in long runs).
+//   * wide_kernel, 16 output bytes per lane (wide.cuh).  Up to some 2^23 ranks bound by instruction issue and latency: a segment of 65 ranks
+//     takes a warp 1250 cycles, most of them in the step in which it ends.  Up to 2^20 ranks two CTAs fit an SM, so that the next call's table is
+//     built beside the rows, above it the 61 440 registers of a CTA leave no room and the table's time (some 4800 cycles, half of
+//     them for the send table) is in series.
+//     From about 2^25 ranks on bound by memory writes.  All ranks of 100 003 4.3 to 4.7 us, of 1.06 million 13.5, 8 chunks of about
+//     2^28 2.34 to 2.46 ms (6.4 to 6.1 TB/s; the power cap shows in long runs).
 // Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
 #include <type_traits>
 
@@ -170,21 +171,20 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     // The wide kernel where the per-rank form is the slower one back to back.  That gets slower in steps: above 148 x 16 x 32 ranks
     // (75 776) a CTA has more than 16 warps and the next call's does not fit beside it, above 148 x 32 x 32 (151 552) items have
     // more than 32 ranks.  The wide kernel's tables cost more the larger q is.  Both tables, us, per rank / wide:
-    //     ranks      q = 17    q = 19    q = 21    q = 22    q = 24    q = 26    q = 30
-    //     65 536    4.2/5.8   4.3/6.2   4.4/6.7   4.4/6.8   4.4/7.5   4.3/7.8   4.1/8.2
-    //     81 920    4.8/6.0   4.7/6.3   4.8/7.0   4.8/7.1   4.8/7.9   7.2/7.9   6.8/8.4
-    //     90 112    6.9/6.0   6.9/6.3   7.2/6.9   7.2/7.1   7.2/7.8   7.2/8.0   6.7/8.3
-    //     98 304    7.5/6.1   7.5/6.4   7.4/7.0   7.4/7.2   7.4/8.0   7.5/8.1   7.1/8.5
-    //    131 072              7.4/6.7   7.5/7.4   7.5/7.5   7.6/8.2   7.5/8.3   7.2/8.7
-    //    163 840              9.4/6.9   9.7/7.6  10.5/7.8  10.8/8.5  11.0/8.6  10.7/8.9
-    // Without send rows there is no send table: 98 304 ranks of q = 26 then take 6.5 and 5.9 us.  (One call with both and a wait for
-    // it: the per-rank form 18 us, the wide one 20 at q = 17, 22 at 21, 24 from 24 on.)  Up to
+    //     ranks      q = 18    q = 19    q = 21    q = 22    q = 24    q = 26    q = 30
+    //     65 536    2.6/4.1   2.7/4.3   2.7/4.6   2.7/4.9   2.7/4.7   2.7/4.4   2.6/4.1
+    //     90 112    4.5/4.7   4.6/5.0   4.8/5.2   4.9/5.2   5.0/5.5   4.7/4.7   4.7/4.4
+    //     98 304    4.7/4.4   4.7/4.8   4.8/5.0   5.0/5.0   5.1/5.4   4.9/4.5   4.9/4.1
+    //    131 072    5.1/4.8   5.3/5.4   5.4/5.4   5.3/5.7   5.4/5.7   5.4/5.4   5.5/4.8
+    //    163 840    6.6/5.2   7.0/5.7   7.2/5.9   7.1/6.0   7.4/6.0   7.7/5.8   7.6/5.0
+    // One table, receive (send) rows of q = 21: 75 776 ranks 2.4/3.4 (2.7/3.4), 90 112 3.9/3.4 (4.4/3.5), 131 072 4.1/3.7 (5.0/3.6).  Up to
     // 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
-    // are built beside it (with steps of 16 ranks: 700 001 ranks 12.3 us, 13.7 with 640 threads, 14.9 per rank; 1.3 million 18.2, 18.0, 23.4; 2.1
-    // million 21.4, 20.6, 29.3).  Beyond, all receive rows before the send rows, item by item: an item's start costs as
+    // are built beside it.  (Above, 640 threads in one CTA: 1.06 million 13.5 us, with 768 13.7, with two CTAs of 448 15.1, of 384 15.3.)
+    // Beyond, all receive rows before the send rows, item by item: an item's start costs as
     // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
     // faster (12.3 million ranks 54 us a table with items of 800, 61 with 400; 2^25: 151 and 146 us).
-    if (rc.q >= kWideMinQ && count >= (rc.q <= 22 || send == nullptr ? 98304u : kSms * 32u * 32u + 1u)) {
+    const bool one = recv == nullptr || send == nullptr;
+    if (rc.q >= kWideMinQ && count >= (one ? kSms * 16u * 32u + 1u : (rc.q <= 22 ? 98304u : kSms * 32u * 32u + 1u))) {
         const bool halves = count < (1u << 23);
         auto run = [&](uint32_t warps) {
             if (recv != nullptr && send != nullptr) warps /= 2;

@@ -71,6 +71,15 @@ def test_rows_where_the_split_changes(bcs, p, n):
     _check(bcs, p, r0, r0 + n)
 
 
+# one table alone changes kernels earlier
+@pytest.mark.parametrize("n", [148 * 16 * 32, 148 * 16 * 32 + 1, 90001])
+@pytest.mark.parametrize("p", [148 * 16 * 32 + 15000, (1 << 20) + 1, (1 << 23) - 1, 40000003])
+def test_rows_of_one_table_where_the_split_changes(bcs, p, n):
+    r0 = 1234567 % (p - n + 1)
+    _check(bcs, p, r0, r0 + n, send=False)
+    _check(bcs, p, r0, r0 + n, recv=False)
+
+
 # steps of 24, 16 and 20 ranks (32 for q = 16: the batches below), runs and items that end inside one
 @pytest.mark.parametrize("p,r0,n", [(140001, 0, 140001), (262144, 100000, 98311), (600011, 0, 600011), (1 << 20, 777, 98304 + 24),
                                     ((1 << 23) + 1, (1 << 22) + 12345, 100001), (1 << 24, (1 << 23) - 200000, 400009)])
