@@ -15,8 +15,9 @@
  *     "host" pointers are ordinary host addresses.  The caller owns every buffer.
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = default stream).
  *     Calls only enqueue work on that stream; they do not synchronise, and the
- *     library holds no device memory of its own unless an entry point says so
- *     (scratch memory is passed in by the caller as a `workspace`).
+ *     library holds no device memory of its own but its code and constants (some 4 MB)
+ *     unless an entry point says so (scratch memory is passed in by the caller as a
+ *     `workspace`).
  *   - Schedule tables are int8, rank-major and unpadded: the row of rank r of a
  *     call for ranks r_begin..r_end-1 starts at byte (r - r_begin) * q.
  *   - Errors are return codes.  Arguments are checked before the first CUDA call: when
