@@ -11,11 +11,11 @@
 // alone, and the one that the guess asks for is built while the wait lasts.  Any p in a kernel's range gives a table
 // within bounds, the search stays inside the plan's arrays whatever they hold, and nothing else is done.  Behind the wait all is
 // read again (past the L1 cache, which may hold what the guess has read), and the table is built again if p is another.
-// (Back to back, every p up to 1024: 17.7 us with the guess taken as it is, 18.3 like this, 25.4 with the first load behind the
+// (With row tables computed in place, back to back, every p up to 1024: 17.7 us with the guess taken as it is, 18.3 like this, 25.4 with the first load behind the
 // wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8, 18.7.)
 //
-// Up to 1024 ranks the tables are most of the work: every p up to 1024 18.4 us, 57 % of the issue slots.  Above, instruction issue
-// and the integer pipe bound it: 1024 p of 2^10..2^20 1288 us (both tables 4.6 TB/s).  That kernel holds two narrow and two wide
+// Up to 1024 ranks instruction issue bounds it, 58 % of the slots: every p up to 1024 13.8 us.  Above, instruction issue
+// and the integer pipe: 1024 p of 2^10..2^20 1250 us (both tables 4.7 TB/s).  That kernel holds two narrow and two wide
 // forms in 80 registers and spills a few bytes at its three CTAs per SM; two per SM take 1368 us, four 1490.
 #include <type_traits>
 
