@@ -336,10 +336,10 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         const RowLayout narrow(kWideMinQ - 1);
         const uint32_t shared = wide.bytes > narrow.total(kBatchWarps) ? wide.bytes : narrow.total(kBatchWarps);
         if (!allow_shared<batch_middle_kernel>()) return BCS_ERR_CUDA;
-        // Up to 2^23 ranks a share per resident CTA: every share costs a search and a table or two, some 10 us (16 p
-        // of 2^10..2^20 79 us with three, 75 with one; 3000 of 2^10..2^11 167, 154).  Beyond, three, so that none
-        // ends last by much (150 p of 2^12..2^18 164 us, with one 168; 300 of 2^14..2^18 326, 348; 3000 of 2^12..2^13 383, 485;
-        // but 64 of 2^17..2^18, few tables, 165, 143).  At most 32768 ranks, at least 1024 (a table costs as much as some
+        // Up to 2^23 ranks a share per resident CTA: every share costs a search and a table or two (16 p
+        // of 2^10..2^20 83 us with three, 76 with one; 3000 of 2^10..2^11 115, 106).  Beyond, three, so that none
+        // ends last by much (150 p of 2^12..2^18 146 us, with one 152; 300 of 2^14..2^18 286, 296; 3000 of 2^12..2^13 277, 341;
+        // but 64 of 2^17..2^18, few tables, 140, 137).  At most 32768 ranks, at least 1024 (a table costs as much as some
         // hundred ranks of each warp).
         const uint64_t ctas = kSms * kMiddleCtas * (total_ranks <= (1u << 23) ? 1u : 3u);
         uint64_t share = align_up(total_ranks / ctas, 128);
@@ -354,8 +354,9 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         }
     }
     // CTAs of 256 threads while all are resident at once (the shorter chain counts), else of 128 (less waiting at
-    // barriers, longer items): us with 256 / 128, 300 p of 3..900 8.4/11.7, 700 of 3..702 11.5/12.1, 740 of 280..1019 13.4/14.6;
-    // 800 of 1000 17.3/16.0, 1000 of 33 8.6/5.3, 1000 of 3..1002 16.2/18.2, 2000 of 2..1024 36.8/36.4, 5000 of 777 96/93.
+    // barriers, longer items): us with 256 / 128, 300 p of 3..900 7.0/8.8, 700 of 3..702 9.4/10.2, 740 of 280..1019 9.7/12.0;
+    // 800 of 1000 13.4/12.9, 900 of 64..256 8.4/6.0, 1000 of 33 6.4/3.7, every p up to 1024 in any order 14.6/13.9 (but in ascending
+    // order 11.8/15.3), 2000 of 2..1024 20.7/20.7, 5000 of 777 62/61.
     if (num_p <= kSms * 5u) return launch_small<256, 5>(ba, small_only, recv_out, send_out, stream);
     return launch_small<128, 8>(ba, small_only, recv_out, send_out, stream);
 }
