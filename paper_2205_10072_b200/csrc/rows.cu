@@ -137,6 +137,14 @@ bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, uint
     return launch_status();
 }
 
+// Warps of a CTA of the per-rank form of which two fit an SM, 16 to 18: 56 registers a thread, 228 KB (1 KB of each CTA the system's).
+uint32_t paired_warps(int q)
+{
+    const RowLayout at(q);
+    const uint32_t warps = (228u * 512u - 1024u - at.warps) / at.warp_bytes;
+    return warps > 18u ? 18u : (warps < 16u ? 16u : warps);
+}
+
 template <int kWords>
 bcs_status launch(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
@@ -175,23 +183,31 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     for (int k = 1; k <= rc.q; ++k) rc.odd |= (2u * rc.s[k - 1] - rc.s[k]) << k;
     rc.inv = (uint32_t)((1ull << (rc.q - low_levels(rc.q) + 32)) / p);
     const uint32_t ranks = (uint32_t)count, x0 = (uint32_t)first;
-    // The wide kernel where the per-rank form is the slower one back to back.  That gets slower in steps: above 148 x 16 x 32 ranks
-    // (75 776) a CTA has more than 16 warps and the next call's does not fit beside it, above 148 x 32 x 32 (151 552) items have
-    // more than 32 ranks.  The wide kernel's tables cost more the larger q is.  Both tables, us, per rank / wide:
-    //     ranks      q = 18    q = 19    q = 21    q = 22    q = 24    q = 26    q = 30
-    //     65 536    2.6/4.1   2.7/4.3   2.7/4.6   2.7/4.9   2.7/4.7   2.7/4.4   2.6/4.1
-    //     90 112    4.5/4.7   4.6/5.0   4.8/5.2   4.9/5.2   5.0/5.5   4.7/4.7   4.7/4.4
-    //     98 304    4.7/4.4   4.7/4.8   4.8/5.0   5.0/5.0   5.1/5.4   4.9/4.5   4.9/4.1
-    //    131 072    5.1/4.8   5.3/5.4   5.4/5.4   5.3/5.7   5.4/5.7   5.4/5.4   5.5/4.8
-    //    163 840    6.6/5.2   7.0/5.7   7.2/5.9   7.1/6.0   7.4/6.0   7.7/5.8   7.6/5.0
-    // One table, receive (send) rows of q = 21: 75 776 ranks 2.4/3.4 (2.7/3.4), 90 112 3.9/3.4 (4.4/3.5), 131 072 4.1/3.7 (5.0/3.6).  Up to
-    // 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
+    // The wide kernel for larger tables.  The per-rank form gets slower in steps: where the next call's CTA no longer fits beside one
+    // (paired_warps) and above 148 x 32 x 32 ranks (151 552), where items have more than 32.  Both tables, us, per rank / wide, back to back:
+    //     ranks     q = 18, 20   q = 19, 21, 22    q = 24     q = 26     q = 30
+    //     65 536     2.8/4.5        2.7/4.3       2.8/4.2    2.8/4.4    2.9/4.4
+    //     90 112     4.7/5.3        4.8/5.1       4.8/5.4    4.9/5.1    5.0/5.2
+    //     98 304     4.7/5.3        4.8/5.0       4.9/5.5    4.9/5.1    5.0/5.0
+    //    120 000     5.4/5.4        5.5/5.4       5.6/5.7    5.6/5.4    5.7/5.4
+    //    140 000     5.8/5.2        5.9/5.3       6.0/5.4    6.1/5.3    6.2/5.4
+    //    151 552     5.8/5.6        5.9/5.5       6.1/5.7    6.3/5.5    6.4/5.6
+    // A call that is waited for takes 15.7 us per rank and 17.6 wide at 98 304 ranks, 15.9 and 17.7 at 131 072.  The lines, 98 304 up to
+    // q = 22 and 151 552 above, are a compromise of the two: back to back the forms cross at some 105 000 (q = 18, 20, 24: 125 000) ranks.
+    // One table alone: the wide form where the per-rank form's CTAs no longer fit an SM in pairs, above 85 248 ranks up to q = 24, 80 512 up
+    // to 26, 75 776 for larger q.  Receive (send) rows, us, per rank / wide:
+    //     ranks             q = 18               q = 24               q = 26               q = 30
+    //     75 777    2.3/3.5 (2.7/3.4)    2.3/3.6 (2.7/3.6)    2.3/3.5 (2.8/3.4)    3.8/3.5 (4.5/3.4)
+    //     83 000    2.5/3.5 (2.8/3.5)    2.5/3.7 (2.9/3.6)    4.1/3.6 (4.5/3.4)    4.0/3.6 (4.6/3.4)
+    //     90 112    3.8/3.7 (4.3/3.5)    3.8/3.7 (4.4/3.6)    3.8/3.5 (4.4/3.4)    3.8/3.5 (4.5/3.4)
+    //    131 072    4.3/3.6 (4.8/3.7)    4.3/3.6 (5.0/3.7)    4.4/3.6 (5.1/3.5)    4.4/3.6 (5.3/3.5)
+    // Up to 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
     // are built beside it.  (Above, 640 threads in one CTA: 1.06 million 13.5 us, with 768 13.7, with two CTAs of 448 15.1, of 384 15.3.)
     // Beyond, all receive rows before the send rows, item by item: an item's start costs as
     // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
     // faster (12.3 million ranks 54 us a table with items of 800, 61 with 400; 2^25: 151 and 146 us).
     const bool one = recv == nullptr || send == nullptr;
-    if (rc.q >= kWideMinQ && count >= (one ? kSms * 16u * 32u + 1u : (rc.q <= 22 ? 98304u : kSms * 32u * 32u + 1u))) {
+    if (rc.q >= kWideMinQ && count >= (one ? kSms * paired_warps(rc.q) * 32u + 1u : (rc.q <= 22 ? 98304u : kSms * 32u * 32u + 1u))) {
         const bool halves = count < (1u << 23);
         auto run = [&](uint32_t warps) {
             if (recv != nullptr && send != nullptr) warps /= 2;

@@ -236,3 +236,18 @@ def _back_to_back(bcs, p, n, recv=True, send=True, calls=200):
 def test_ctas_without_ranks_do_not_hold_up_a_row_of_calls(bcs, recv, send):
     p = 1398101
     assert _back_to_back(bcs, p, 1000003, recv, send) < 1.1 * _back_to_back(bcs, p, 1 << 20, recv, send)
+
+
+# One table alone stays with the per-rank form while two of its CTAs fit an SM: 80 000 ranks of q = 21 take 2.4 us (send rows 2.8), a
+# twentieth more than 75 776, and took 3.5 (3.4) in the wide form.
+@pytest.mark.parametrize("recv", [True, False])
+def test_one_table_keeps_the_faster_form(bcs, recv):
+    assert _back_to_back(bcs, 1398101, 80000, recv, not recv) < 1.15 * _back_to_back(bcs, 1398101, 75776, recv, not recv)
+
+
+@pytest.mark.parametrize("p,n", [((1 << 20) + 1, 148 * 18 * 32), ((1 << 20) + 1, 148 * 18 * 32 + 1), (100001, 148 * 18 * 32),
+                                 ((1 << 24) - 1, 148 * 18 * 32 + 1), (40000003, 148 * 17 * 32), (40000003, 148 * 17 * 32 + 1)])
+def test_rows_of_one_table_at_the_end_of_pairs(bcs, p, n):
+    r0 = 1234567 % (p - n + 1)
+    _check(bcs, p, r0, r0 + n, send=False)
+    _check(bcs, p, r0, r0 + n, recv=False)
