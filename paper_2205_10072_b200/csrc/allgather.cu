@@ -13,7 +13,9 @@ constexpr int kAgLine = 32;       // int32 elements per 128-byte line
 constexpr int kAgCols = kAgThreads + kAgLine;   // buffers staged per CTA: its window slides by up to 31 from row to row
 constexpr int kAgCtas = 148 * 32; // CTAs that a call aims for: the rounds are cut into as many chunks as that takes
 constexpr uint32_t kAgRounds = 64;          // rounds that make up for the staging of a CTA's rows,
-constexpr uint32_t kAgFewCtas = 148 * 4;  // as far as that leaves so many CTAs
+constexpr uint32_t kAgFewCtas = 148 * 4;    // as far as that leaves so many CTAs
+constexpr uint32_t kAgFitBoth = 148 * 6;    // CTAs that run at once (36 KB of shared memory each);
+constexpr uint32_t kAgFitOne = 148 * 7;     // with one table eight per SM would fit, but seven are as fast
 constexpr int kAgRowBytes = kAgCols * BCS_MAX_Q + 48;
 
 // Where the rows of a CTA's columns lie in its copy of a schedule table: column c (buffer j0 + c,
@@ -256,14 +258,20 @@ bcs_status bcs_allgather_tables(uint32_t p, uint32_t n, uint32_t r, const int8_t
     // rounds are cut into as many chunks (a multiple of four rounds each) as it takes to have
     // about kAgCtas CTAs (measured best on p = 100 003, n = 1000: 5.9 TB/s; a quarter or four times
     // as many CTAs 5.1 resp. 4.5 TB/s).  Where that would leave a CTA less than some 64 rounds, staging 288 rows costs more than
-    // writing: fewer chunks then, down to four CTAs per SM (us before / like this: p = 20 262, n = 116 21.4 / 12.9; 261 597, 7 28.3 / 17.3;
-    // 5000, 500 17.0 / 11.7; 50 000, 20 15.0 / 10.8; 260 000, 100 59 / 46, with 32 rounds 54).
+    // writing: fewer chunks then, down to four CTAs per SM (us before / like this: p = 20 262, n = 116 21.3 / 13.0; 261 597, 7 28.2 / 17.2;
+    // 5000, 500 17.0 / 11.7; 50 000, 20 15.0 / 10.8).  But not where all CTAs run at once anyway: all stage at the same time then (p = 2000,
+    // n = 300 7.5, with half as many CTAs of twice the rounds 8.5; 5000, 116 7.45, 8.4; 20 262, 20 9.1, 10.1; one table of 35 000, 12 6.1, 6.5.
+    // Half as many, drawn sizes, on average: 700 to 888 CTAs 4 % slower, one table 900 to 1036 2 % slower, 1050 to 1184 5 % faster).
     const uint32_t rounds = n - 1u + (uint32_t)tab.q;
     const uint32_t col_blocks = (p + kAgThreads - 1) / kAgThreads;
     uint32_t chunks = (kAgCtas + col_blocks - 1) / col_blocks;
-    const uint32_t few = (kAgFewCtas + col_blocks - 1) / col_blocks, many = (rounds + kAgRounds - 1) / kAgRounds;
-    if (chunks > many) chunks = many > few ? many : few;
     uint32_t per_cta = ((rounds + chunks - 1) / chunks + 3u) & ~3u;
+    const uint32_t fit = pack_out && unpack_out ? kAgFitBoth : kAgFitOne;
+    const uint32_t few = (kAgFewCtas + col_blocks - 1) / col_blocks, many = (rounds + kAgRounds - 1) / kAgRounds;
+    if (chunks > many && (uint64_t)col_blocks * ((rounds + per_cta - 1) / per_cta) > fit) {
+        chunks = many > few ? many : few;
+        per_cta = ((rounds + chunks - 1) / chunks + 3u) & ~3u;
+    }
     chunks = (rounds + per_cta - 1) / per_cta;
     dim3 grid(col_blocks, chunks);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);

@@ -185,3 +185,65 @@ def test_a_refused_call_leaves_no_error_behind(tmp_path):
     subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + flags +
                           ["-I", os.path.join(os.path.dirname(build_ext.LIB_PATH), "csrc"), "-o", str(tmp_path / "refused"), str(source)])
     assert subprocess.check_output([str(tmp_path / "refused")], text=True) == "0 0 0 0 "
+
+
+FAKE_LAUNCH = r"""
+#include <cuda_runtime.h>
+#include <stdio.h>
+static int4 split;
+template <class... P, class... A>
+static cudaError_t fake_launch(const cudaLaunchConfig_t *cfg, void (*)(P...), A &&...)
+{
+    split = make_int4(cfg->gridDim.x, cfg->gridDim.y, 0, 0);
+    return cudaSuccess;
+}
+#define cudaLaunchKernelEx fake_launch
+#include "allgather.cu"
+namespace bcs {
+bcs_status make_table(uint32_t p, PTable *tab)
+{
+    tab->p = p;
+    for (tab->q = 0; (1ull << tab->q) < p; ++tab->q) {}
+    return BCS_OK;
+}
+}
+int main()
+{
+    alignas(16) static int8_t rows[16];
+    alignas(16) static int32_t out[4];
+    unsigned p, n;
+    int both;
+    while (scanf("%u %u %d", &p, &n, &both) == 3) {
+        (void)bcs_allgather_tables(p, n, 0, rows, rows, out, both ? out : nullptr, nullptr);
+        printf("%d %d\n", split.x, split.y);
+    }
+}
+"""
+
+
+def test_allgather_grids_that_fit_the_card_are_not_made_smaller(tmp_path):
+    """Where CTAs of four rounds each are on the card at once (six per SM with both tables, seven with one), the launch has those; longer
+    ones took a tenth more time.  Where they are not, it has fewer CTAs with up to 64 rounds, four per SM or more.  (The launch is a fake.)"""
+    import subprocess
+    from paper_2205_10072_b200 import build_ext
+    source = tmp_path / "split.cu"
+    source.write_text(FAKE_LAUNCH)
+    flags = [f for f in build_ext.NVCC_FLAGS if f != "--shared"]
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + flags +
+                          ["-I", os.path.join(os.path.dirname(build_ext.LIB_PATH), "csrc"), "-o", str(tmp_path / "split"), str(source)])
+    sizes = [(p, n, both) for p in (300, 1152, 2000, 5000, 9000, 12000, 20262, 35000, 50000, 70000, 261597)
+             for n in (2, 7, 20, 64, 116, 300, 500, 1500, 6000) for both in (0, 1)]
+    out = subprocess.run([str(tmp_path / "split")], input="".join("%d %d %d\n" % s for s in sizes), text=True, check=True, capture_output=True)
+    whole = 0
+    for (p, n, both), line in zip(sizes, out.stdout.splitlines(), strict=True):
+        x, y = map(int, line.split())
+        rounds, blocks = n - 1 + (p - 1).bit_length(), -(-p // 256)
+        finest = -(-rounds // 4)
+        assert x == blocks and y <= finest, (p, n, both)
+        if x * finest <= 148 * (6 if both else 7):
+            assert y == finest, (p, n, both, y)
+            whole += 1
+        elif y != finest:                                        # the last chunk may be short
+            per_cta = -(-rounds // y)
+            assert per_cta <= 64 + 3 or x * (-(-rounds // (per_cta - 4))) > 148 * 4, (p, n, both, y)
+    assert whole > 60 and len(sizes) - whole > 60

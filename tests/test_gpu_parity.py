@@ -602,6 +602,24 @@ def test_expansion_builds_its_rows_when_given_no_tables(bcs):
     assert L.bcs_expand(10, 4, 0, 10, None, tab.data_ptr(), tab.data_ptr(), None) == 1   # one table only
 
 
+# whole tables at each kind of split: four rounds a CTA because that fits the card (2000, 9000, 20262), rounds for some four CTAs per SM
+# with a short last chunk (5000: 20 rounds and 12, 20262: 20 and 10), all rounds in one chunk (261597); outputs off a 16-byte boundary
+@pytest.mark.parametrize("p,n", [(2000, 300), (9000, 64), (20262, 20), (5000, 500), (20262, 116), (261597, 7)])
+def test_allgather_tables_of_every_split(bcs, p, n):
+    want_r, want_s = oracle.full_table(p)
+    recv, send = torch.from_numpy(want_r).cuda(), torch.from_numpy(want_s).cuda()
+    size = (n - 1 + oracle.q_of(p)) * p
+    for r, off in ((p // 3, 32), (p - 1, 33)):
+        want = [torch.from_numpy(t).cuda().view(-1) for t in oracle.allgather_rank(p, n, r, want_r, want_s)]
+        for pack, unpack in ((True, True), (True, False), (False, True)):
+            raw = torch.full((2, size + 96), -77, dtype=torch.int32, device="cuda")
+            outs = [raw[i, off + i:off + i + size] if asked else None for i, asked in enumerate((pack, unpack))]
+            bcs.bcs_allgather_tables(p, n, r, recv, send, *outs)
+            for i, out in enumerate(outs):
+                assert bool((raw[i, :off + i] == -77).all()) and bool((raw[i, off + i + size:] == -77).all()), (r, off)
+                assert bool((raw[i] == -77).all()) if out is None else torch.equal(out, want[i]), (r, off, i)
+
+
 def test_allgather_tables_match_oracle(bcs):
     """Algorithm 9's pack / unpack block numbers: every entry against the oracle's literal loops
     for small p, the library's own tables simulated (all p processors) for tiny p, and the
