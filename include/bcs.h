@@ -15,7 +15,7 @@
  *     "host" pointers are ordinary host addresses.  The caller owns every buffer.
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = default stream).
  *     Calls only enqueue work on that stream; they do not synchronise, and the
- *     library holds no device memory of its own but its code and constants (some 4 MB)
+ *     library holds no device memory of its own but its code and constants (some 2 MB)
  *     unless an entry point says so (scratch memory is passed in by the caller as a
  *     `workspace`).
  *   - Schedule tables are int8, rank-major and unpadded: the row of rank r of a

@@ -17,6 +17,7 @@
 // Up to 1024 ranks instruction issue bounds it, 58 % of the slots: every p up to 1024 13.8 us.  Above, instruction issue
 // and the integer pipe: 1024 p of 2^10..2^20 1250 us (both tables 4.7 TB/s).  That kernel holds two narrow and two wide
 // forms in 80 registers and spills a few bytes at its three CTAs per SM; two per SM take 1368 us, four 1490.
+#pragma once
 #include <type_traits>
 
 #include "rows.cuh"
@@ -25,7 +26,6 @@
 namespace bcs {
 namespace {
 
-constexpr unsigned kSms = 148;
 constexpr uint32_t kSmallP = 1024;
 constexpr int kSmallQ = 10;
 constexpr int kMiddleQ = 21;

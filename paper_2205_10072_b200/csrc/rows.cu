@@ -13,13 +13,13 @@
 // Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
 #include <type_traits>
 
+#include "batch.cuh"     // (in this unit, too: the constants of rows.cuh are in the module once)
 #include "rows.cuh"
 #include "wide.cuh"
 
 namespace bcs {
 namespace {
 
-constexpr unsigned kSms = 148;
 constexpr unsigned kRowThreads = 1024;
 constexpr uint32_t kShortRun = 192;               // see wide_kernel
 

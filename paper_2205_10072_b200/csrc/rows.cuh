@@ -37,6 +37,7 @@
 
 namespace bcs {
 
+constexpr unsigned kSms = 148;
 constexpr int kLow = 7;                       // rounds whose entries come from the table
 constexpr int kLowRanks = 128;                // skips[7] <= 128
 constexpr int kMissRanks = 32;                // ranks behind a segment's start that can be exceptions (<= 25)

@@ -1,5 +1,5 @@
 // The calls that build schedules of one p (arXiv 2205.10072, Algorithms 1-5 and the lookup of Algorithm 9): they check
-// their arguments and launch the kernels of rows.cu.  Many p at once: batch.cu.
+// their arguments and launch the kernels of rows.cu.  Many p at once: batch.cuh.
 #include "bcs_common.cuh"
 
 namespace bcs {

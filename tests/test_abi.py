@@ -17,6 +17,12 @@ def lib():
     return bcs
 
 
+def test_the_library_holds_its_constants_once(lib):
+    """1.75 MB of row constants, once for the device and once for the host, and kernels: 5.8 MB.  In two units, with line information
+    (nvcc adds the constants as text) it was 23 MB, and a process's first calls took twice as long."""
+    assert os.path.getsize(lib.lib_path()) < 8 << 20
+
+
 def _declared_symbols():
     names = set()
     for fn in os.listdir(os.path.join(ROOT, "include")):
