@@ -84,6 +84,15 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
         // One run per warp, those of the CTA side by side: rows for their segments only (all ranks of 100 003: five of 11
         // groups of rows, of about 2^20 nine of 15; 6.13 -> 5.97 and 16.8 -> 15.7 us, 1.3 million ranks 17.6 -> 16.5).
         const uint32_t warps = (blockDim.x >> 5) / (recv != nullptr && send != nullptr ? 2u : 1u);
+        // A CTA that has no ranks stays until the kernel before is done, too.  If it left at once, CTAs of the call after next would
+        // take its place, two of one call on some SMs, and the whole call would wait for those: in a row of calls 700 001 ranks 12.5 us
+        // and not 9.65, 1 000 003 16.7 and not 12.0, receive rows of 1 000 003 9.8 and not 7.5 (none is without ranks at 1 048 576: 12.4 both
+        // ways).  Runs of both tables of kShortRun ranks and less take no longer than what comes before them, and the call after next is
+        // welcome: 98 304 ranks 5.0 us, 5.15 with the wait, 140 000 ranks of q = 20 5.05, 5.5; but 180 000 6.0, 5.95, 300 001 7.0, 6.7.
+        if (blockIdx.x * warps * item >= count) {
+            if (item > kShortRun || recv == nullptr || send == nullptr) grid_dependency_wait();
+            return;
+        }
         const uint32_t x0 = first + blockIdx.x * warps * item;
         want_rows(t, rc.q, rc.inv, x0 >= rc.p ? x0 - rc.p : x0, warps * item + 1u);      // (the last vectors look at the rank behind)
     } else {
@@ -115,12 +124,6 @@ wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     }
     if (receives) all(std::false_type(), recv);
     if (sends) all(std::true_type(), send);
-    // A CTA that has no ranks stays until the kernel before is done, too.  If it left at once, CTAs of the call after next would take
-    // its place, two of one call on some SMs, and the whole call would wait for those: in a row of calls 700 001 ranks 12.5 us and not
-    // 9.65, 1 000 003 16.7 and not 12.0, receive rows of 1 000 003 9.8 and not 7.5 (none is without ranks at 1 048 576: 12.4 both ways).
-    // Runs of both tables of kShortRun ranks and less take no longer than what comes before them, and the call after next is welcome:
-    // 98 304 ranks 5.0 us, 5.15 with the wait, 140 000 ranks of q = 20 5.05, 5.5; but 180 000 6.0, 5.95, 300 001 7.0, 6.7.
-    if (item > kShortRun || recv == nullptr || send == nullptr) grid_dependency_wait();
 }
 
 template <unsigned kThreads, int kCtas, bool kAnyStep = false>
