@@ -73,10 +73,11 @@ def build_row_table(force: bool = False) -> str:
             subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-o", exe, ROW_TABLE_SOURCE])
             with open(tmp, "wb") as out:
                 subprocess.check_call([exe], stdout=out)
+            os.replace(tmp, ROW_TABLE)
         finally:
-            if os.path.exists(exe):
-                os.remove(exe)
-        os.replace(tmp, ROW_TABLE)
+            for left in (exe, tmp):
+                if os.path.exists(left):
+                    os.remove(left)
     return ROW_TABLE
 
 

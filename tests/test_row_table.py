@@ -55,3 +55,20 @@ def test_rows_of_small_p(packed):
         q = Form(p).q
         got, _, _ = _unpack(rows[p * (p - 1) // 2:p * (p + 1) // 2], q, 0)
         assert np.array_equal(got[:, :q], oracle.full_table(p)[0]), p
+
+
+def test_a_failed_generator_leaves_nothing_behind(tmp_path, monkeypatch):
+    """The constants as they were, and no part of others beside them."""
+    import os
+    import subprocess
+    compiler = tmp_path / "cc"
+    compiler.write_text('#!/bin/sh\nfor a; do [ "$was" = -o ] && out=$a; was=$a; done\n'
+                        'printf "#!/bin/sh\\necho half of it\\nexit 3\\n" > "$out"; chmod +x "$out"\n')
+    compiler.chmod(0o755)
+    monkeypatch.setattr(build_ext, "ROW_TABLE", str(tmp_path / "row_table.inc"))
+    (tmp_path / "row_table.inc").write_text("as it was")
+    monkeypatch.setenv("CC", str(compiler))
+    with pytest.raises(subprocess.CalledProcessError):
+        build_ext.build_row_table(force=True)
+    assert sorted(os.listdir(tmp_path)) == ["cc", "row_table.inc"]
+    assert (tmp_path / "row_table.inc").read_text() == "as it was"
