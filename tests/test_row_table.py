@@ -25,12 +25,21 @@ def _unpack(rows, q, K):
     return np.where(own, block, block - q)[:, :7], np.where(base == 8, K, base), rows[:, 7] >> 5
 
 
+def _every_shape():
+    """Counts p that between them have segments of every kind: for each skips[7], all halvings above it rounding up, for every q, and none."""
+    for s7 in range(65, 129):
+        yield s7 << 2
+        p = s7
+        while p < 1 << 31:
+            yield p
+            p = 2 * p - 1
+
+
 def test_rows_of_every_shape(packed):
-    rng = np.random.default_rng(11)
     shapes = packed["row_shapes"].reshape(64, 52, 64, 8)
     sixes = packed["row_six"].reshape(64, 64, 8)
     seen = set()
-    for p in [*range(65, 1400, 7), (1 << 30) + 1, (1 << 31) - 1] + [int(2 ** e) for e in rng.uniform(10, 31, 300)]:
+    for p in _every_shape():
         form = Form(p)
         q, six, lows = form.q, form.s[6], form.s[7]
         for K in range(7, q + 1):
@@ -46,7 +55,36 @@ def test_rows_of_every_shape(packed):
             assert np.array_equal(bb, base[:six - (K == q)]), (p, K)
             got, bb, _ = _unpack(sixes[lows - 65, :lows - six], q, K)
             assert np.array_equal(got[:, :6], want[six:, :6]) and np.array_equal(bb, form.table(K)[1][six:]), (p, K)
-    assert len(seen) > 900
+    assert len(seen) == 64 * 51                                  # 25 kinds of segments and the root's 26 for each skips[7]
+
+
+def test_rows_of_every_shape_against_the_oracle(packed):
+    """The rounds 0..6 of the ranks of one segment of each kind, as the oracle computes them rank by rank."""
+    shapes = packed["row_shapes"].reshape(64, 52, 64, 8)
+    sixes = packed["row_six"].reshape(64, 64, 8)
+    seen = set()
+    for p in _every_shape():
+        q = (p - 1).bit_length()
+        s = oracle.skips(p).tolist()
+        odd = [0] + [2 * s[t - 1] - s[t] for t in range(1, q + 1)]
+        lows, six, ranks, kinds = s[7], s[6], [], []
+        for K in range(7, q + 1):
+            shape = (26 if K == q else 0) + (0 if K == 7 else 1 + sum(odd[8:K + 1]))
+            if (lows, shape) in seen:
+                continue
+            seen.add((lows, shape))
+            # the segment of the rank skips[K] (rank 0) ends where the next one starts: bit 7 is clear unless K = 7
+            n = lows - (sum(odd[8:9]) if K == 7 and q > 7 else 0)
+            kinds.append((K, shape, n))
+            ranks += [(0 if K == q else s[K]) + low for low in range(n)]
+        got = oracle.build_ranks(p, np.array(ranks, dtype=np.uint32))[0][:, :7]
+        for K, shape, n in kinds:
+            rows, got = got[:n], got[n:]
+            want = _unpack(shapes[lows - 65, shape, :six], q, K)[0]
+            assert np.array_equal(rows[:six], want), (p, K)
+            want = _unpack(sixes[lows - 65, :n - six], q, K)[0][:, :6]
+            assert np.array_equal(rows[six:, :6], want), (p, K)
+    assert len(seen) == 64 * 51
 
 
 def test_rows_of_small_p(packed):
