@@ -251,3 +251,50 @@ def test_rows_of_one_table_at_the_end_of_pairs(bcs, p, n):
     r0 = 1234567 % (p - n + 1)
     _check(bcs, p, r0, r0 + n, send=False)
     _check(bcs, p, r0, r0 + n, recv=False)
+
+
+# A call into tables that the kernel in front of it still reads: the row kernels are launched while that one runs, and wait for it in
+# front of their first store, warp by warp; warps and CTAs without ranks need not.  `between`: with a call of one CTA into other
+# tables in the middle, which must not be done before the one in front of it is.
+@pytest.mark.parametrize("between", [False, True])
+@pytest.mark.parametrize("n", [32, 20000, 100003, 700001])
+@pytest.mark.parametrize("reader", ["expand", "allgather"])
+def test_tables_are_not_written_before_they_are_read(bcs, reader, n, between):
+    p, blocks, next_p = 100003, 150, 1398101
+    q, next_q = bcs.bcs_q(p), bcs.bcs_q(next_p)
+    tables = [torch.from_numpy(t).cuda().view(-1) for t in oracle.full_table(p)]
+    size, written = p * q, n * next_q
+    at = max(size - written, 0) // 16 * 16                       # over the end of the tables, where reading ends
+    memory = [torch.empty(max(size, at + written), dtype=torch.int8, device="cuda") for _ in range(2)]
+    other = [torch.empty(32 * next_q, dtype=torch.int8, device="cuda") for _ in range(2)]
+    out = torch.empty(4 * p * (blocks - 1 + q), dtype=torch.int32, device="cuda")
+    busy = torch.empty(1 << 29, dtype=torch.int8, device="cuda")
+    rows = [torch.empty(written, dtype=torch.int8, device="cuda") for _ in range(2)]
+    bcs.bcs_build(next_p, 0, n, *rows)
+
+    def read():
+        if reader == "expand":
+            bcs.bcs_expand(p, blocks, 0, p, memory[0][:size], memory[1][:size], out.view(p, -1, 4))
+        else:
+            half = len(out) // 4
+            bcs.bcs_allgather_tables(p, blocks, 7, memory[0][:size], memory[1][:size], out[:half], out[half:2 * half])
+
+    want = None
+    for _ in range(5):
+        for m, t in zip(memory, tables):
+            m[:size] = t
+        out.fill_(-9)
+        torch.cuda.synchronize()
+        if want is None:                                         # nothing behind it
+            read()
+            want = out.clone()
+            continue
+        for _ in range(4):
+            busy.zero_()                                         # (all that follows is enqueued while this lasts)
+        read()
+        if between:
+            bcs.bcs_build(next_p, 0, 32, *other)
+        bcs.bcs_build(next_p, 0, n, memory[0][at:at + written], memory[1][at:at + written])
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        assert all(torch.equal(m[at:at + written], r) for m, r in zip(memory, rows))
