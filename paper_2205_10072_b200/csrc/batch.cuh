@@ -11,11 +11,12 @@
 // alone, and the one that the guess asks for is built while the wait lasts.  Any p in a kernel's range gives a table
 // within bounds, the search stays inside the plan's arrays whatever they hold, and nothing else is done.  Behind the wait all is
 // read again (past the L1 cache, which may hold what the guess has read), and the table is built again if p is another.
-// (With row tables computed in place, back to back, every p up to 1024: 17.7 us with the guess taken as it is, 18.3 like this, 25.4 with the first load behind the
-// wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8, 18.7.)
+// (With row tables computed in place, back to back, every p up to 1024, in any order: 17.7 us with the guess taken as it is, 18.3 like
+// this, 25.4 with the first load behind the wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8,
+// 18.7.)
 //
-// Up to 1024 ranks instruction issue bounds it, 58 % of the slots: every p up to 1024 13.8 us.  Above, instruction issue
-// and the integer pipe: 1024 p of 2^10..2^20 1250 us (both tables 4.7 TB/s).  That kernel holds two narrow and two wide
+// Up to 1024 ranks instruction issue bounds it, 58 % of the slots: every p up to 1024 13.9 us in any order, 15.2 ascending, 12.4 descending.
+// Above, instruction issue and the integer pipe: 1024 p of 2^10..2^20 1250 us (both tables 4.7 TB/s).  That kernel holds two narrow and two wide
 // forms in 80 registers and spills a few bytes at its three CTAs per SM; two per SM take 1368 us, four 1490.
 #pragma once
 #include <type_traits>
@@ -355,8 +356,8 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
     }
     // CTAs of 256 threads while all are resident at once (the shorter chain counts), else of 128 (less waiting at
     // barriers, longer items): us with 256 / 128, 300 p of 3..900 7.0/8.8, 700 of 3..702 9.4/10.2, 740 of 280..1019 9.7/12.0;
-    // 800 of 1000 13.4/12.9, 900 of 64..256 8.4/6.0, 1000 of 33 6.4/3.7, every p up to 1024 in any order 14.6/13.9 (but in ascending
-    // order 11.8/15.3), 2000 of 2..1024 20.7/20.7, 5000 of 777 62/61.
+    // 800 of 1000 13.4/12.9, 900 of 64..256 8.4/6.0, 1000 of 33 6.4/3.7, 2000 of 2..1024 20.7/20.7, 5000 of 777 62/61.  The number alone
+    // does not tell: every p up to 1024 takes 14.6/13.9 in any order, but 11.8/15.3 in ascending order (neighbours of like size).
     if (num_p <= kSms * 5u) return launch_small<256, 5>(ba, small_only, recv_out, send_out, stream);
     return launch_small<128, 8>(ba, small_only, recv_out, send_out, stream);
 }

@@ -2,8 +2,10 @@
  *
  * The entries of the rounds 0..6 of a rank depend on its place `low` in its segment, on skips[7] (65..128, which gives the skips below
  * it), and on the segment's lowest set bit K by way of three things: the number c = C(7, K) of halvings that rounded up between 7 and
- * K, whether K is 7, and whether it is the root's segment (K = q).  They are computed here by Algorithm 4 (arXiv 2205.10072) as it
- * is written: windows of baseblocks, the largest new one.  Baseblock K stands for itself as 8.
+ * K, whether K is 7, and whether it is the root's segment (K = q).  The rounds 0..5 in which the rank's skip code has no bit are
+ * computed here by Algorithm 4 (arXiv 2205.10072) as it is written: windows of baseblocks, the largest new one.  Where the code has the bit,
+ * and in round 6, it is the closed form of csrc/rows.cuh: the next higher bit, or the block that is left, with the exceptions behind a
+ * segment's start.  Baseblock K stands for itself as 8.
  *
  * A row is 8 bytes.  Rounds 0..6: the block, 8 for K, 16 + the block where it is the rank's own (the home round, entry without
  * - q).  Byte 7: baseblock (8 for K, 0 for the root) in bits 0..3, and in bits 5..7 the block of 0..7 that is not taken before round 7.
@@ -135,7 +137,7 @@ int main(void)
         }
         printf("\n");
     }
-    printf("};\nstatic __device__ const unsigned long long row_small[64 * 65 / 2 + 64] = {\n");
+    printf("};\nstatic __device__ const unsigned long long row_small[64 * 65 / 2] = {\n");
     for (int p = 1; p <= 64; ++p) {
         int q = 0;
         while (1 << q < p) ++q;

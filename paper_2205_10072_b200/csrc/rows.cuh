@@ -103,7 +103,7 @@ struct RowTable {
 };
 
 // The rows of all shapes of segments (gen/row_table.c writes them at build time and says how they are packed): 1.7 MB, of which a
-// CTA reads 512 bytes for each K that it wants, by one load per row.
+// CTA reads 512 bytes for each K that it wants, and the same 512 bytes of row_six each time.
 #include "row_table.inc"
 
 // A packed row: entries are block - q, K for 8, blocks of 16 and more the rank's own.
@@ -118,9 +118,9 @@ __device__ __forceinline__ uint2 unpack_row(unsigned long long v, int q, int K)
 
 // Fills the table of a p, for the K whose bits in *t.wanted are set (q > 7); all threads of the CTA call, after a barrier behind the
 // writes of t.s (the skips, then zeros) and *t.wanted.  Ends with a barrier.
-// (One load and some twenty instructions a row.  Computed by Algorithm 4 in every CTA it took 5000 cycles before the first row: 65 553 ranks
-// 4.2 -> 3.3 us, all ranks of 100 003 5.5 -> 4.3, of about 2^20 15.6 -> 13.6, every p up to 1024 18.3 -> 16.7, back to back; a call alone 2 us
-// less.)
+// (Two loads and some twenty instructions for two rows.  Computed by Algorithm 4 in every CTA it took 5000 cycles before the first row:
+// 65 553 ranks 4.2 -> 3.5 us, all ranks of 100 003 5.5 -> 4.8, of about 2^20 15.6 -> 13.6, every p up to 1024 in any order 18.3 -> 16.7, back
+// to back; a call alone 2 us less.)
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {
     const int L = low_levels(q);
@@ -129,8 +129,7 @@ __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32
         for (uint32_t low = threadIdx.x; low < lows; low += blockDim.x) {
             uint2 row = unpack_row(__ldg(row_small + lows * (lows - 1u) / 2u + low), q, 0x7f);
             row.y &= 0xff000000u | (q > 4 ? (1u << (8 * (q - 4))) - 1u : 0u);
-            if (low == 0u) row.y |= kRootMark << 24;
-            t.rows[low] = row;
+            t.rows[low] = row;                                   // (the root's baseblock is 8 in the constants: 0x7f)
         }
         __syncthreads();
         return;
@@ -224,9 +223,9 @@ struct RowPlace {
 };
 
 // Stores the rows (words W, zero beyond byte q) of 32 ranks at once, this lane's at `at`.  A word that two rows share is
-// stored by the lane it ends in.  kAligned: the first row begins on a word.  Else the last lane stores what it has of a shared word, too, and the first
-// lane of the next 32 ranks (`more`) completes that.  Lanes without a rank store
-// too (the buffer has room for them, and nobody reads it).
+// stored by the lane it ends in.  kAligned: the first row begins on a word.  Else the last lane stores what it has of a shared word,
+// too, and the first lane of the next 32 ranks (`more`) completes that.  Lanes without a rank store too (the buffer has room for
+// them, and nobody reads it).
 // (With the words at either end written byte by byte every p up to 1024 took 16.5 us and not 13.8, 1024 p up to 2^20 1257 and not 1250.)
 template <int kWords, bool kAligned>
 __device__ __forceinline__ void stage_row(uint8_t *at, const uint32_t (&W)[kWords], int q, const RowPlace &pl, bool more)
