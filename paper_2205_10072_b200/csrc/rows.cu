@@ -1,14 +1,14 @@
 // Receive and send rows of a stretch of ranks of one p: the kernels behind bcs_build and its relatives.
 //
 // One launch, nothing read from memory but constants, no table of all ranks (rows.cuh).  Two forms, by size (launch_rows):
-//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp.  From Python 32 ranks 3.2 us back to
-//     back, all ranks of 1152 3.3, 65 553 ranks 3.3 (2.7 on the device).  The table holds what the
+//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp.  From Python 32 ranks 3.2 to 3.5 us back to
+//     back, all ranks of 1152 3.3 to 3.7, 65 553 ranks 3.5 (2.7 on the device).  The table holds what the
 //     CTA's segments need where these are few, and a CTA has no more warps than items.
 //   * wide_kernel, 16 output bytes per lane (wide.cuh).  Up to some 2^23 ranks bound by instruction issue and latency: a segment of 65 ranks
 //     takes a warp 1250 cycles, most of them in the step in which it ends.  Up to 2^20 ranks two CTAs fit an SM, so that the next call's table is
 //     built beside the rows, above it the 61 440 registers of a CTA leave no room and the table's time (some 4800 cycles, half of
 //     them for the send table) is in series.
-//     From about 2^25 ranks on bound by memory writes.  All ranks of 100 003 4.3 to 4.7 us, of 1.06 million 13.5, 8 chunks of about
+//     From about 2^25 ranks on bound by memory writes.  All ranks of 100 003 4.6 to 5.1 us by the card, of 1.06 million 13.7, 8 chunks of about
 //     2^28 2.34 to 2.46 ms (6.4 to 6.1 TB/s; the power cap shows in long runs).
 // Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
 #include <type_traits>
