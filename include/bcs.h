@@ -271,8 +271,8 @@ bcs_status bcs_simulate(uint32_t p, uint32_t n, const int8_t *recv, const int8_t
                         uint64_t *state_dev, uint64_t *counts_dev, void *cuda_stream);
 
 /* Waits for all work of the current device (cudaDeviceSynchronize) and stores in *count_host (host) how
- * many waits of the library's kernels ran out: 0, since none of them waits with a limit.  (Kept for
- * callers of earlier versions, whose transposition kernels did.) */
+ * many waits of the library's kernels on it ran out since the process began (tables of ranges that are
+ * handed out turn by turn: a turn that was asked for, but not answered in two seconds).  Other than 0: rows are missing. */
 bcs_status bcs_wait_expired(uint64_t *count_host);
 
 /* Position-weighted 64-bit checksum of a stretch of schedule entries, additive

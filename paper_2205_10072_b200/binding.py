@@ -351,7 +351,7 @@ def bcs_simulate(p: int, n: int, recv, send, state, counts_out, stream=None) -> 
 
 
 def bcs_wait_expired() -> int:
-    """Waits that ran out, 0: no kernel waits with a limit.  Synchronises the device."""
+    """Waits of the kernels that ran out on the current device; other than 0: rows are missing.  Synchronises the device."""
     v = _c.c_uint64(0)
     _check(lib().bcs_wait_expired(_c.byref(v)), "bcs_wait_expired")
     return v.value

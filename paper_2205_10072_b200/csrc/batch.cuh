@@ -208,7 +208,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
             built = 0u;
             if (p != 0u && r0 < r1) {
                 build_row_table(t, q, job.odd);
-                if (!narrow && send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
+                if (!narrow && send != nullptr) build_send_table_wide(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
                 built = p;
             }
         }
@@ -260,7 +260,7 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         const uint64_t entry0 = ba.entry_off[j];
         __syncthreads();
         build_row_table(t, q, job.odd);
-        if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
+        if (send != nullptr) build_send_table_wide(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
         const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
         auto all = [&](auto is_send, int8_t *out) {
             WideLane lane;

@@ -125,6 +125,9 @@ bcs_status make_table(uint32_t p, PTable *tab);
 // Rows of the count <= p ranks first, first+1, ... (mod p; first < p, p > 1): rows.cu.  Either output may be null.
 bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv, int8_t *send, cudaStream_t stream);
 
+// Waits with a limit that ran out in the row kernels of the current device: rows.cu.
+bool expired_wait_count(unsigned long long *count);
+
 // Launch with programmatic stream serialisation (see above); `dependent` false: ordinary launch.
 template <class... Params, class... Args>
 inline void launch_dependent(bool dependent, void (*kernel)(Params...), dim3 grid, unsigned block, size_t shared,

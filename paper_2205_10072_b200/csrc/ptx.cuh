@@ -48,7 +48,60 @@ __device__ __forceinline__ void bulk_store(void *dst, const void *from_shared, u
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// True for one lane of a full warp, the same one each time (the compiler then knows that what follows is done by one thread).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(one) :: "memory");
+    return one != 0u;
+}
+
 // The copies that this thread has started have read their shared memory.
 __device__ __forceinline__ void bulk_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
+// ---------------------------------------------------------------- work that CTAs take from one another
+// A CTA that asks for the work of one that has not started yet gets its index, and that one is not launched (cluster launch control).  The answer
+// (16 bytes) arrives in shared memory and completes a phase of the barrier.
+__device__ __forceinline__ void barrier_init(uint64_t *bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"((uint32_t)__cvta_generic_to_shared(bar)) : "memory");
+}
+
+__device__ __forceinline__ void ask_for_work(uint4 *answer, uint64_t *bar)
+{
+    const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 16;" :: "r"(b) : "memory");
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(answer)), "r"(b) : "memory");
+}
+
+// Waits for the phase of the given parity, two seconds at most; false: it has not come.
+__device__ __forceinline__ bool barrier_wait(uint64_t *bar, uint32_t parity)
+{
+    const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
+    uint64_t begin = 0, now = 0;
+    for (;;) {
+        uint32_t done;
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(done) : "r"(b), "r"(parity) : "memory");
+        if (done) return true;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now) :: "memory");
+        if (begin == 0) begin = now;
+        if (now - begin > 2000000000ull) return false;
+    }
+}
+
+// Whether an answer names a CTA, and which.
+__device__ __forceinline__ bool work_given(const uint4 *answer, uint32_t *cta)
+{
+    const uint4 a = *answer;
+    uint32_t given, x;
+    asm volatile("{\n.reg .b128 r;\n.reg .pred p;\n.reg .b64 lo, hi;\nmov.b64 lo, {%2, %3};\nmov.b64 hi, {%4, %5};\nmov.b128 r, {lo, hi};\n"
+                 "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\nselp.u32 %0, 1, 0, p;\nmov.u32 %1, 0;\n"
+                 "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, _, _, _}, r;\n}"
+                 : "=r"(given), "=r"(x) : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w) : "memory");
+    *cta = x;
+    return given != 0u;
+}
 
 }  // namespace bcs

@@ -1,27 +1,21 @@
 // Receive and send rows of a stretch of ranks of one p: the kernels behind bcs_build and its relatives.
 //
 // One launch, nothing read from memory but constants, no table of all ranks (rows.cuh).  Two forms, by size (launch_rows):
-//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp.  From Python 32 ranks 3.2 to 3.5 us back to
-//     back, all ranks of 1152 3.3 to 3.7, 65 553 ranks 3.5 (2.7 on the device).  The table holds what the
+//   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp.  From Python 32 ranks 3.2 us back to
+//     back, all ranks of 1152 3.3, 65 553 ranks 3.2 (2.7 on the device).  The table holds what the
 //     CTA's segments need where these are few, and a CTA has no more warps than items.
-//   * wide_kernel, 16 output bytes per lane (wide.cuh).  Up to some 2^23 ranks bound by instruction issue and latency: a segment of 65 ranks
-//     takes a warp 1250 cycles, most of them in the step in which it ends.  Up to 2^20 ranks two CTAs fit an SM, so that the next call's table is
-//     built beside the rows, above it the 61 440 registers of a CTA leave no room and the table's time (some 4800 cycles, half of
-//     them for the send table) is in series.
-//     From about 2^25 ranks on bound by memory writes.  All ranks of 100 003 4.6 to 5.1 us by the card, of 1.06 million 13.7, 8 chunks of about
-//     2^28 2.34 to 2.46 ms (6.4 to 6.1 TB/s; the power cap shows in long runs).
+//   * quad_kernel, four ranks per lane (quad.cuh).  Up to some 2^21 ranks bound by instruction issue, the integer pipe with it, above by
+//     memory writes.  All ranks of 100 003 2.4 us, of 1.06 million 10.2, 2^24 ranks of q = 28 132, 2^25 receive rows 134 (7.0 TB/s).  With vectors
+//     of 16 output bytes per lane in its place, some 40 warp instructions for every 32 of them where a segment ends: 4.9, 13.6, 146 and 149.
 // Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
-#include <type_traits>
-
 #include "batch.cuh"     // (in this unit, too: the constants of rows.cuh are in the module once)
 #include "rows.cuh"
-#include "wide.cuh"
+#include "quad.cuh"
 
 namespace bcs {
 namespace {
 
 constexpr unsigned kRowThreads = 1024;
-constexpr uint32_t kShortRun = 192;               // see wide_kernel
 
 // One CTA per SM at most; every warp takes items of `item` (32, 64 or 128) consecutive ranks, in turn over the CTAs.
 // first: rank of the first row (< p); the count <= p ranks go on at 0 behind p - 1.
@@ -67,85 +61,110 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     stage_free();
 }
 
-// The same for larger tables, q >= 16 (wide.cuh), one CTA per SM; `item` is a multiple of 16.  halves: every warp has one item of
-// one table, half of the warps write the receive rows and half the send rows; otherwise all warps the ones before the others.
-// (No more than 640 threads: at the speed of the memory the write streams of 1024 cost 20 % and more.)
-template <unsigned kThreads, int kCtas, bool kAnyStep>
-__global__ void __launch_bounds__(kThreads, kCtas)
-wide_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t item, bool halves,
-            int8_t *recv, int8_t *send)
+constexpr unsigned kQuadThreads = 320;
+
+__device__ unsigned long long expired_waits;      // waits with a limit that ran out
+
+// Two CTAs per SM.  A turn of a CTA is a run per warp.  once: a CTA for each turn, all of them run at once.  Otherwise the CTAs that run take the turns of
+// those that have not started yet: SMs do not write equally fast (a fill by CTAs of equal shares reaches 6.3 TB/s, by CTAs of 16 KB in
+// any order 7.5), and one table serves all turns of a CTA.
+template <int Q, bool kTable>
+__global__ void __launch_bounds__(kQuadThreads, 2)
+quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t run, bool once, int8_t *recv, int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ __align__(16) uint4 answer;
     grid_launch_dependents();
-    const WideLayout at(rc.q);
+    __shared__ uint64_t answered;
+    const QuadLayout<kTable> at(Q, run);
+    const uint32_t warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const RowTable t(sm, at.base);
     if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
-    if (halves) {
-        // One run per warp, those of the CTA side by side: rows for their segments only (all ranks of 100 003: five of 11
-        // groups of rows, of about 2^20 nine of 15; 6.13 -> 5.97 and 16.8 -> 15.7 us, 1.3 million ranks 17.6 -> 16.5).
-        const uint32_t warps = (blockDim.x >> 5) / (recv != nullptr && send != nullptr ? 2u : 1u);
-        // A CTA that has no ranks stays until the kernel before is done, too.  If it left at once, CTAs of the call after next would
-        // take its place, two of one call on some SMs, and the whole call would wait for those: in a row of calls 700 001 ranks 12.5 us
-        // and not 9.65, 1 000 003 16.7 and not 12.0, receive rows of 1 000 003 9.8 and not 7.5 (none is without ranks at 1 048 576: 12.4 both
-        // ways).  Runs of both tables of kShortRun ranks and less take no longer than what comes before them, and the call after next is
-        // welcome: 98 304 ranks 5.0 us, 5.15 with the wait, 140 000 ranks of q = 20 5.05, 5.5; but 180 000 6.0, 5.95, 300 001 7.0, 6.7.
-        if (blockIdx.x * warps * item >= count) {
-            if (item > kShortRun || recv == nullptr || send == nullptr) grid_dependency_wait();
-            return;
-        }
-        const uint32_t x0 = first + blockIdx.x * warps * item;
-        want_rows(t, rc.q, rc.inv, x0 >= rc.p ? x0 - rc.p : x0, warps * item + 1u);      // (the last vectors look at the rank behind)
+    if (once) {
+        const uint32_t x0 = first + blockIdx.x * warps * run;
+        want_rows(t, Q, rc.inv, x0 >= rc.p ? x0 - rc.p : x0, warps * run + kHalo);
     } else {
-        if (threadIdx.x == 0) *t.wanted = (2u << (rc.q - kLow)) - 1u;
+        if (threadIdx.x == 0) {
+            *t.wanted = (2u << (Q - kLow)) - 1u;
+            barrier_init(&answered);
+        }
         __syncthreads();
     }
-    build_row_table(t, rc.q, rc.odd);
-    if (send != nullptr) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
-    const uint32_t warp = threadIdx.x >> 5;
-    uint32_t n_warps = blockDim.x >> 5, index = warp;
-    auto all = [&](auto is_send, int8_t *out) {
-        WideLane mine;
-        mine.template init<kAnyStep>(rc.q, 0u);
-        const uint64_t stride = (uint64_t)gridDim.x * n_warps * item;
-        for (uint64_t b = ((uint64_t)blockIdx.x * n_warps + index) * item; b < count; b += stride) {
-            const uint32_t n = count - (uint32_t)b < item ? count - (uint32_t)b : item;
+    build_row_table<true>(t, Q, rc.odd);
+    if constexpr (kTable) build_send_table(t, reinterpret_cast<uint2 *>(sm + at.table), Q, rc.odd);
+    uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
+    uint32_t turn = blockIdx.x, parity = 0;
+    for (;;) {
+        if (!once && threadIdx.x == 0) ask_for_work(&answer, &answered);
+        const uint64_t b = ((uint64_t)turn * warps + warp) * run;
+        if (b < count) {
+            const uint32_t n = count - (uint32_t)b < run ? count - (uint32_t)b : run;
             uint32_t x0 = first + (uint32_t)b;
             if (x0 >= rc.p) x0 -= rc.p;
-            wide_rows<decltype(is_send)::value, kAnyStep, true>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv,
-                                                mine, x0, n, b == 0, b + n == count, out + b * (uint64_t)rc.q);
+            const uint64_t byte = b * Q;
+            quad_run<Q, kTable>(t, sm + at.table, mine, at, rc.s, rc.odd, rc.inv, x0, n, recv ? recv + byte : nullptr, send ? send + byte : nullptr);
         }
-    };
-    bool receives = recv != nullptr, sends = send != nullptr;
-    if (halves && receives && sends) {
-        n_warps /= 2;
-        sends = warp >= n_warps;
-        receives = !sends;
-        if (sends) index -= n_warps;
+        if (once) break;
+        if (!barrier_wait(&answered, parity)) {
+            if (threadIdx.x == 0) atomicAdd(&expired_waits, 1ull);       // (bcs_wait_expired)
+            break;
+        }
+        parity ^= 1u;
+        const bool more = work_given(&answer, &turn);
+        if (!more) break;
+        fence_before_bulk();                                     // (the answer is written by the asynchronous proxy: it has been read)
+        __syncthreads();
     }
-    if (receives) all(std::false_type(), recv);
-    if (sends) all(std::true_type(), send);
+    stage_free();
 }
 
-template <unsigned kThreads, int kCtas, bool kAnyStep = false>
-bcs_status launch_wide(const RowConsts &rc, uint32_t first, uint32_t count, uint32_t item, bool halves, int8_t *recv, int8_t *send,
-                       cudaStream_t stream)
+// Turns and CTAs.  Runs are whole look-ups (128 ranks): partly filled ones cost as much.  The shortest run with which at most 296 CTAs of up to ten warps
+// (as many as two CTAs per SM have shared memory for) have all ranks at once; and no more warps than make 148 CTAs, which leave room for the
+// next call's (back to back, us: all ranks of 100 003 2.4, with the ranks spread over 296 CTAs 4.5; 200 000 ranks of q = 21 4.2 and 4.9, 524 288 6.6
+// and 6.5, 1.06 million 10.2 and 10.3).  One table: two look-ups as soon as 148 CTAs do not do with one (200 000 receive rows 2.6 us, with runs of 128 3.0).
+// The shared memory is filled up to half an SM, lest three CTAs of one call meet on an SM while another one has one.
+// Longer ranges: turns of 512 ranks per warp, of 768 for one table from 3.5 million on (2^24 send rows of q = 28 71 us, with 512 74; receive rows of 3
+// million 15.6, with 512 14.9).
+template <int Q, bool kTable>
+bcs_status launch_quad(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
-    if constexpr (!kAnyStep) {
-        if (step_ranks(rc.q) != 16u) return launch_wide<kThreads, kCtas, true>(rc, first, count, item, halves, recv, send, stream);
+    if (!allow_shared<quad_kernel<Q, kTable>>()) return BCS_ERR_CUDA;
+    constexpr uint32_t half = (228u * 512u - 1024u - 128u) & ~127u, most = kQuadThreads / 32u;
+    auto bytes = [](uint32_t warps, uint32_t run) { return QuadLayout<kTable>(Q, run).total(warps); };
+    auto fit = [&](uint32_t run) {
+        uint32_t w = most;
+        while (w > 4u && bytes(w, run) > half) --w;
+        return w;
+    };
+    const uint32_t quads = (count + kQuads - 1u) / kQuads;
+    const bool one = recv == nullptr || send == nullptr;
+    uint32_t k = 1;
+    while (k * kQuads <= kMostRun && fit(k * kQuads) * k * kSms * (one && k == 1u ? 1u : 2u) < quads) ++k;
+    const bool once = k * kQuads <= kMostRun;
+    if (!once) k = one && count >= 3500000u ? 6u : 4u;
+    const uint32_t run = k * kQuads;
+    uint32_t warps = fit(run);
+    if (once) {
+        const uint32_t enough = (quads + k * kSms - 1u) / (k * kSms);
+        warps = warps < enough ? warps : (enough < 4u ? 4u : enough);
     }
-    if (!allow_shared<wide_kernel<kThreads, kCtas, kAnyStep>>()) return BCS_ERR_CUDA;
-    const unsigned items = (count + item - 1) / item;
-    launch_dependent(true, wide_kernel<kThreads, kCtas, kAnyStep>, items < kSms ? items : kSms, kThreads,
-                     WideLayout(rc.q).bytes, stream, rc, first, count, item, halves, recv, send);
+    const uint32_t need = bytes(warps, run), turn = warps * run;
+    launch_dependent(true, quad_kernel<Q, kTable>, (unsigned)(((uint64_t)count + turn - 1u) / turn), 32u * warps, need < half ? half : need, stream, rc, first,
+                     count, run, once, recv, send);
     return launch_status();
 }
 
-// Warps of a CTA of the per-rank form of which two fit an SM, 16 to 18: 56 registers a thread, 228 KB (1 KB of each CTA the system's).
-uint32_t paired_warps(int q)
+// kTable from 2^22 ranks on: building the table of send rows pays (send rows of q = 28, us, without / with it: 1 million 7.1/8.0, 3 million 17.6/17.4, 8 million
+// 43/37, 2^25 164/137; both tables 4 million 33.9/35.0, 8 million 66.6/65.7).
+template <int Q>
+bcs_status launch_quads(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
-    const RowLayout at(q);
-    const uint32_t warps = (228u * 512u - 1024u - at.warps) / at.warp_bytes;
-    return warps > 18u ? 18u : (warps < 16u ? 16u : warps);
+    if constexpr (Q > BCS_MAX_Q) return BCS_ERR_UNSUPPORTED;
+    else {
+        if (rc.q != Q) return launch_quads<Q + 1>(rc, first, count, recv, send, stream);
+        if (send != nullptr && count >= (1u << 22)) return launch_quad<Q, true>(rc, first, count, recv, send, stream);
+        return launch_quad<Q, false>(rc, first, count, recv, send, stream);
+    }
 }
 
 template <int kWords>
@@ -173,6 +192,11 @@ bcs_status launch(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *r
 
 }  // namespace
 
+bool expired_wait_count(unsigned long long *count)
+{
+    return cudaMemcpyFromSymbol(count, expired_waits, sizeof *count) == cudaSuccess;
+}
+
 bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
     RowConsts rc = {};
@@ -186,41 +210,14 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     for (int k = 1; k <= rc.q; ++k) rc.odd |= (2u * rc.s[k - 1] - rc.s[k]) << k;
     rc.inv = (uint32_t)((1ull << (rc.q - low_levels(rc.q) + 32)) / p);
     const uint32_t ranks = (uint32_t)count, x0 = (uint32_t)first;
-    // The wide kernel for larger tables.  The per-rank form gets slower in steps: where the next call's CTA no longer fits beside one
-    // (paired_warps) and above 148 x 32 x 32 ranks (151 552), where items have more than 32.  Both tables, us, per rank / wide, back to back:
-    //     ranks     q = 18, 20   q = 19, 21, 22    q = 24     q = 26     q = 30
-    //     65 536     2.8/4.5        2.7/4.3       2.8/4.2    2.8/4.4    2.9/4.4
-    //     90 112     4.7/5.3        4.8/5.1       4.8/5.4    4.9/5.1    5.0/5.2
-    //     98 304     4.7/5.3        4.8/5.0       4.9/5.5    4.9/5.1    5.0/5.0
-    //    120 000     5.4/5.4        5.5/5.4       5.6/5.7    5.6/5.4    5.7/5.4
-    //    140 000     5.8/5.2        5.9/5.3       6.0/5.4    6.1/5.3    6.2/5.4
-    //    151 552     5.8/5.6        5.9/5.5       6.1/5.7    6.3/5.5    6.4/5.6
-    // A call that is waited for takes 15.7 us per rank and 17.6 wide at 98 304 ranks, 15.9 and 17.7 at 131 072.  The lines, 98 304 up to
-    // q = 22 and 151 552 above, are a compromise of the two: back to back the forms cross at some 105 000 (q = 18, 20, 24: 125 000) ranks.
-    // One table alone: the wide form where the per-rank form's CTAs no longer fit an SM in pairs, above 85 248 ranks up to q = 24, 80 512 up
-    // to 26, 75 776 for larger q.  Receive (send) rows, us, per rank / wide:
-    //     ranks             q = 18               q = 24               q = 26               q = 30
-    //     75 777    2.3/3.5 (2.7/3.4)    2.3/3.6 (2.7/3.6)    2.3/3.5 (2.8/3.4)    3.8/3.5 (4.5/3.4)
-    //     83 000    2.5/3.5 (2.8/3.5)    2.5/3.7 (2.9/3.6)    4.1/3.6 (4.5/3.4)    4.0/3.6 (4.6/3.4)
-    //     90 112    3.8/3.7 (4.3/3.5)    3.8/3.7 (4.4/3.6)    3.8/3.5 (4.4/3.4)    3.8/3.5 (4.5/3.4)
-    //    131 072    4.3/3.6 (4.8/3.7)    4.3/3.6 (5.0/3.7)    4.4/3.6 (5.1/3.5)    4.4/3.6 (5.3/3.5)
-    // Up to 2^23 ranks every warp has one run of one table; up to 2^20 the CTA is half an SM, so that the next call's tables
-    // are built beside it.  (Above, 640 threads in one CTA: 1.06 million 13.5 us, with 768 13.7, with two CTAs of 448 15.1, of 384 15.3.)
-    // Beyond, all receive rows before the send rows, item by item: an item's start costs as
-    // much as some 50 ranks, but from 2^25 ranks on the memory bounds it, and items close together are written
-    // faster (12.3 million ranks 54 us a table with items of 800, 61 with 400; 2^25: 151 and 146 us).
-    const bool one = recv == nullptr || send == nullptr;
-    if (rc.q >= kWideMinQ && count >= (one ? kSms * paired_warps(rc.q) * 32u + 1u : (rc.q <= 22 ? 98304u : kSms * 32u * 32u + 1u))) {
-        const bool halves = count < (1u << 23);
-        auto run = [&](uint32_t warps) {
-            if (recv != nullptr && send != nullptr) warps /= 2;
-            return (ranks + kSms * warps * kStep - 1u) / (kSms * warps * kStep) * kStep;
-        };
-        if (count <= (1u << 20)) return launch_wide<384, 2>(rc, x0, ranks, run(12), halves, recv, send, stream);
-        if (halves) return launch_wide<640, 1>(rc, x0, ranks, run(20), halves, recv, send, stream);
-        const uint32_t item = count >= (1u << 25) ? 384u : 768u;            // (whole steps: 400 and 800 where these have 20 ranks)
-        return launch_wide<640, 1>(rc, x0, ranks, step_ranks(rc.q) == 20u ? item / 24u * 25u : item, halves, recv, send, stream);
-    }
+    // Four ranks per lane where two of the per-rank form's CTAs no longer fit an SM (148 x 16 x 32 ranks).  Both tables, us back to back, per rank / four
+    // per lane (a call that is waited for):
+    //     ranks          q = 20                 q = 24                 q = 28                 q = 31
+    //     32 768    2.0/2.2 (14.3/16.0)    2.1/2.5 (14.3/15.0)    2.1/2.6 (14.3/15.2)    2.1/2.9 (14.6/15.5)
+    //     65 553    2.7/2.4 (14.6/15.4)    2.7/2.6 (14.6/15.1)    2.8/2.7 (14.6/15.0)    2.8/2.9 (14.9/15.5)
+    //     75 777    2.9/2.4 (14.6/14.9)    3.0/2.6 (14.5/15.2)    4.6/2.8 (14.6/15.3)    4.7/3.1 (14.7/15.4)
+    //     98 304    5.2/2.5 (17.6/15.1)    4.9/2.8 (15.1/15.0)    4.8/3.2 (14.8/15.2)    5.0/3.5 (15.4/14.9)
+    if (rc.q >= kQuadMinQ && count > kSms * 16u * 32u) return launch_quads<kQuadMinQ>(rc, x0, ranks, recv, send, stream);
     return launch<1>(rc, x0, ranks, recv, send, stream);
 }
 

@@ -106,6 +106,9 @@ struct RowTable {
 // CTA reads 512 bytes for each K that it wants, and the same 512 bytes of row_six each time.
 #include "row_table.inc"
 
+// Place of row `low` in a table whose readers are four rows apart: 16 lanes meet in no bank.
+__device__ __forceinline__ uint32_t permuted_row(uint32_t low) { return low ^ ((low >> 4) & 3u); }
+
 // A packed row: entries are block - q, K for 8, blocks of 16 and more the rank's own.
 __device__ __forceinline__ uint2 unpack_row(unsigned long long v, int q, int K)
 {
@@ -121,15 +124,17 @@ __device__ __forceinline__ uint2 unpack_row(unsigned long long v, int q, int K)
 // (Two loads and some twenty instructions for two rows.  Computed by Algorithm 4 in every CTA it took 5000 cycles before the first row:
 // 65 553 ranks 4.2 -> 3.5 us, all ranks of 100 003 5.5 -> 4.8, of about 2^20 15.6 -> 13.6, every p up to 1024 in any order 18.3 -> 16.7, back
 // to back; a call alone 2 us less.)
+template <bool kPermuted = false>
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {
+    auto place = [](uint32_t low) { return kPermuted ? permuted_row(low) : low; };
     const int L = low_levels(q);
     const uint32_t lows = t.s[L];
     if (q < kLow) {                                              // one segment, all rounds in the table
         for (uint32_t low = threadIdx.x; low < lows; low += blockDim.x) {
             uint2 row = unpack_row(__ldg(row_small + lows * (lows - 1u) / 2u + low), q, 0x7f);
             row.y &= 0xff000000u | (q > 4 ? (1u << (8 * (q - 4))) - 1u : 0u);
-            t.rows[low] = row;                                   // (the root's baseblock is 8 in the constants: 0x7f)
+            t.rows[place(low)] = row;                            // (the root's baseblock is 8 in the constants: 0x7f)
         }
         __syncthreads();
         return;
@@ -141,25 +146,43 @@ __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32
     const uint32_t six = t.s[6];
     const unsigned long long *shapes = row_shapes + (lows - 65u) * (52u * 64u), *sixes = row_six + (lows - 65u) * 64u;
     const int n = __popc(wanted) * 64;
-    for (int job = (int)threadIdx.x; job < n; job += (int)blockDim.x) {
-        const int K = t.list[job >> 6];
-        const uint32_t low = (uint32_t)job & 63u, shape = (K == q ? 26u : 0u) + (K == kLow ? 0u : 1u + count_odd(odd, kLow, K));
-        const unsigned long long v = __ldg(shapes + shape * 64u + low), w = __ldg(sixes + low);
-        uint2 *rows = t.rows + (K - kLow) * kLowRanks;
-        if (low < six) {
-            uint2 row = unpack_row(v, q, K);
-            if (K == q && low == 0u) row.y |= kRootMark << 24;
-            rows[low] = row;
-            if (low < (uint32_t)kMissRanks) t.miss[(K - kLow) * kMissRanks + (int)low] = (uint8_t)(v >> 61);
+    // (the loads of up to four jobs at once: their latency is most of the time)
+    constexpr int kJobs = 4;
+    for (int job0 = (int)threadIdx.x; job0 < n; job0 += kJobs * (int)blockDim.x) {
+        unsigned long long v[kJobs], w[kJobs];
+#pragma unroll
+        for (int j = 0; j < kJobs; ++j) {
+            const int job = job0 + j * (int)blockDim.x;
+            v[j] = w[j] = 0;
+            if (job < n) {
+                const int K = t.list[job >> 6];
+                const uint32_t low = (uint32_t)job & 63u, shape = (K == q ? 26u : 0u) + (K == kLow ? 0u : 1u + count_odd(odd, kLow, K));
+                v[j] = __ldg(shapes + shape * 64u + low);
+                w[j] = __ldg(sixes + low);
+            }
         }
-        // ranks with bit 6: the rounds before that do not depend on K, round 6 receives the next higher bit
-        const uint32_t at = low + six;
-        uint2 row = make_uint2(0u, 0u);                          // (read, but not used, behind the last one)
-        if (at < lows) {
-            row = unpack_row(w, q, K);
-            row.y = (row.y & 0xff00ffffu) | (uint32_t)(uint8_t)(K < q ? K - q : (int)(row.y >> 24)) << 16;
+#pragma unroll
+        for (int j = 0; j < kJobs; ++j) {
+            const int job = job0 + j * (int)blockDim.x;
+            if (job >= n) break;
+            const int K = t.list[job >> 6];
+            const uint32_t low = (uint32_t)job & 63u;
+            uint2 *rows = t.rows + (K - kLow) * kLowRanks;
+            if (low < six) {
+                uint2 row = unpack_row(v[j], q, K);
+                if (K == q && low == 0u) row.y |= kRootMark << 24;
+                rows[place(low)] = row;
+                if (low < (uint32_t)kMissRanks) t.miss[(K - kLow) * kMissRanks + (int)low] = (uint8_t)(v[j] >> 61);
+            }
+            // ranks with bit 6: the rounds before that do not depend on K, round 6 receives the next higher bit
+            const uint32_t at = low + six;
+            uint2 row = make_uint2(0u, 0u);                      // (read, but not used, behind the last one)
+            if (at < lows) {
+                row = unpack_row(w[j], q, K);
+                row.y = (row.y & 0xff00ffffu) | (uint32_t)(uint8_t)(K < q ? K - q : (int)(row.y >> 24)) << 16;
+            }
+            if (at < kLowRanks) rows[place(at)] = row;
         }
-        if (at < kLowRanks) rows[at] = row;
     }
     __syncthreads();
 }
@@ -281,7 +304,7 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
     const uint32_t begin = (shift + 15u) & ~15u, end = shift + len;
     uint8_t *base = reinterpret_cast<uint8_t *>(dst) - shift;
     const uint32_t stop = end & ~15u;
-    if (lane == 0u && stop > begin) bulk_store(base + begin, stage + begin, stop - begin);
+    if (elect_one() && stop > begin) bulk_store(base + begin, stage + begin, stop - begin);
     if (!kAligned || (end & 15u) != 0u) {                        // bytes [shift, head) and [tail, end) one by one
         const uint32_t head = begin < end ? begin : end;
         if (shift + lane < head) base[shift + lane] = stage[shift + lane];
@@ -293,7 +316,7 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
 // The staging buffer may be written again.
 __device__ __forceinline__ void stage_free()
 {
-    if ((threadIdx.x & 31u) == 0u) bulk_stores_read();
+    if (elect_one()) bulk_stores_read();
     __syncwarp();
 }
 

@@ -182,7 +182,9 @@ bcs_status bcs_wait_expired(uint64_t *count_host)
 {
     if (count_host == nullptr) return BCS_ERR_ARG;
     if (cudaDeviceSynchronize() != cudaSuccess) return BCS_ERR_CUDA;
-    *count_host = 0;                         // no kernel of the library waits with a limit
+    unsigned long long count = 0;            // (the kernel that hands out turns waits for its answers with a limit)
+    if (!expired_wait_count(&count)) return BCS_ERR_CUDA;
+    *count_host = count;
     return BCS_OK;
 }
 

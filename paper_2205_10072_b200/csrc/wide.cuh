@@ -51,7 +51,7 @@ struct WideLayout {
 // Send table: [u - 1][low], u = K - L (1..q-L) for a segment with bit L clear and lowest bit K, u = q - L + (K2 - L) for
 // one with bit L set and K2 the lowest bit of the next segment.  Entries of the rounds 0..6, baseblock as byte 7.
 // For the K of *t.wanted; all threads of the CTA call, the row table is complete.  Ends with a barrier.
-__device__ __forceinline__ void build_send_table(const RowTable &t, uint2 *send, int q, uint32_t odd)
+__device__ __forceinline__ void build_send_table_wide(const RowTable &t, uint2 *send, int q, uint32_t odd)
 {
     const int high = q - kLow;
     const uint8_t *bytes = reinterpret_cast<const uint8_t *>(t.rows);

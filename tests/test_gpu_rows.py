@@ -253,6 +253,24 @@ def test_rows_of_one_table_at_the_end_of_pairs(bcs, p, n):
     _check(bcs, p, r0, r0 + n, recv=False)
 
 
+# Four ranks per lane: every q, ranges with one run per warp, longer runs, and turns that CTAs take from one another (with the table of send rows); from
+# rank 0 on (home rounds in any word of a row) and to the last one; each table alone, and every row and pair of both.
+@pytest.mark.parametrize("q", range(17, 32))
+def test_four_ranks_per_lane(bcs, q):
+    p = min((3 << q - 2) + 12345, (1 << 31) - 1)
+    for i, n in enumerate((148 * 16 * 32 + 1, 148 * 10 * 128 + 1, 148 * 20 * 256 + 129, (1 << 22) + 77)):
+        if n > p:
+            continue
+        for r0 in (0, p - n):
+            _check(bcs, p, r0, r0 + n, recv=i % 2 == 0 or r0 == 0, send=i % 2 == 1 or r0 == 0)
+        recv, send = (torch.empty(n * q, dtype=torch.int8, device="cuda") for _ in range(2))
+        counts = torch.ones(3, dtype=torch.int64, device="cuda")
+        bcs.bcs_build(p, p - n, p, recv, send)
+        bcs.bcs_validate(p, p - n, p, recv, send, counts)
+        assert counts.tolist() == [0, 0, 0], n
+    assert bcs.bcs_wait_expired() == 0
+
+
 # A call into tables that the kernel in front of it still reads: the row kernels are launched while that one runs, and wait for it in
 # front of their first store, warp by warp; warps and CTAs without ranks need not.  `between`: with a call of one CTA into other
 # tables in the middle, which must not be done before the one in front of it is.
