@@ -574,6 +574,26 @@ def test_expansion_small_cases_and_simulation(bcs):
                 assert bcast_sim.simulate(p, n, got) is None
 
 
+# CTAs begin anywhere in a rank's rounds: rows about as long as a CTA's records (512, 1024), longer and much longer, many to a CTA; numbers of records on
+# both sides of the rule's lines (1.2 and 4 million); tables that do not start on a line
+@pytest.mark.parametrize("p,n,skew", [(9, 509, 0), (9, 510, 1), (1000, 503, 0), (2, 1023, 7), (2, 1025, 3), (1200, 1014, 0), (4000, 1013, 5), (3, 100000, 0),
+                                      (300, 14000, 2), (5, 900000, 0), (40000, 15, 1), (70000, 2, 4), (200000, 5, 0)])
+def test_expansion_wherever_ctas_begin(bcs, p, n, skew):
+    q = oracle.q_of(p)
+    rounds = n - 1 + q
+    want_r, want_s = oracle.full_table(p)
+    recv, send = torch.from_numpy(want_r).cuda(), torch.from_numpy(want_s).cuda()
+    raw = torch.full((p * rounds * 4 + 128,), -77, dtype=torch.int32, device="cuda")
+    tab = raw[64 + 4 * skew:64 + 4 * skew + p * rounds * 4].view(p, rounds, 4)
+    want = torch.from_numpy(oracle.expand(p, n, want_r, want_s)).cuda()
+    for tables in ((recv, send), (None, None)) if p <= 1000 else ((recv, send),):
+        raw.fill_(-77)
+        bcs.bcs_expand(p, n, 0, p, *tables, tab)
+        torch.cuda.synchronize()
+        assert torch.equal(tab, want)
+        assert bool((raw[:64 + 4 * skew] == -77).all()) and bool((raw[64 + 4 * skew + p * rounds * 4:] == -77).all())
+
+
 def test_expansion_builds_its_rows_when_given_no_tables(bcs):
     """bcs_expand with both tables NULL computes the rows of its ranks itself (Algorithm 6 calls
     recvsched and sendsched): same records as the oracle's literal loop, for whole small p, for
