@@ -118,11 +118,13 @@ def _stream(stream) -> int | None:
 
 
 class _Calls:
-    """The calls that enqueue work, by name without "bcs_"; the first use of one loads the library."""
+    """The calls that enqueue work, by name without "bcs_"; the first use of one loads the library.  With "on_" in front they take
+    tensors (None for none) and a stream or None where the others take addresses, sizes and a handle."""
 
     def __getattr__(self, name):
         library = lib()
-        call = getattr(_extension(library), name, None) or getattr(library, "bcs_" + name)
+        plain = _PLAIN[name[3:]] if name.startswith("on_") else getattr(library, "bcs_" + name)
+        call = getattr(_extension(library), name, None) or plain
         setattr(self, name, call)
         return call
 
@@ -138,10 +140,29 @@ def _extension(library):
     except ImportError:
         return None
     _calls.set_library(library)
+    _calls.set_torch(torch.cuda.is_initialized, _device, _raw_stream, _stream, _PLAIN)
     return _calls
 
 
 _call = _Calls()
+
+# What the extension module does for the calls with tensors, through the calls with numbers.
+_PLAIN = {
+    "build": lambda p, r0, r1, recv, send, ws, stream:
+        _call.build(p, r0, r1, _ptr(recv), _ptr(send), _ptr(ws), _nbytes(ws), _stream(stream)),
+    "build_rooted": lambda p, root, r0, r1, recv, send, ws, stream:
+        _call.build_rooted(p, root, r0, r1, _ptr(recv), _ptr(send), _ptr(ws), _nbytes(ws), _stream(stream)),
+    "prepare_rows": lambda p, r0, r1, recv, ws, stream:
+        _call.prepare_rows(p, r0, r1, _ptr(recv), _ptr(ws), _nbytes(ws), _stream(stream)),
+    "build_prepared": lambda p, r0, r1, recv, send, ws, stream:
+        _call.build_prepared(p, r0, r1, _ptr(recv), _ptr(send), _ptr(ws), _nbytes(ws), _stream(stream)),
+    "build_static": lambda p, r0, r1, recv, send, stream:
+        _call.build_static(p, r0, r1, _ptr(recv), _ptr(send), _stream(stream)),
+    "expand": lambda p, n, r0, r1, recv, send, out, stream:
+        _call.expand(p, n, r0, r1, _ptr(recv), _ptr(send), _ptr(out), _stream(stream)),
+    "allgather_tables": lambda p, n, r, recv, send, pack, unpack, stream:
+        _call.allgather_tables(p, n, r, _ptr(recv), _ptr(send), _ptr(pack), _ptr(unpack), _stream(stream)),
+}
 
 
 def bcs_status_str(status: int) -> str:
@@ -170,8 +191,7 @@ def bcs_build(p: int, r_begin: int, r_end: int, recv_out, send_out, workspace=No
               stream=None) -> None:
     """recv_out / send_out: CUDA int8 tensors of (r_end-r_begin)*q elements, or None;
     workspace: CUDA tensor of bcs_build_workspace_bytes(...) bytes or None (not touched)."""
-    _check(_call.build(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out), _ptr(workspace),
-                           _nbytes(workspace), _stream(stream)), "bcs_build")
+    _check(_call.on_build(p, r_begin, r_end, recv_out, send_out, workspace, stream), "bcs_build")
 
 
 def bcs_build_rooted_workspace_bytes(p: int, root: int, r_begin: int, r_end: int) -> int:
@@ -182,8 +202,7 @@ def bcs_build_rooted(p: int, root: int, r_begin: int, r_end: int, recv_out, send
                      workspace=None, stream=None) -> None:
     """As bcs_build for a broadcast rooted at `root`: row r is the rank-0-rooted row of virtual
     rank (r - root) mod p."""
-    _check(_call.build_rooted(p, root, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
-                                  _ptr(workspace), _nbytes(workspace), _stream(stream)),
+    _check(_call.on_build_rooted(p, root, r_begin, r_end, recv_out, send_out, workspace, stream),
            "bcs_build_rooted")
 
 
@@ -206,23 +225,20 @@ def bcs_prepare_codes(p: int, workspace, stream=None) -> None:
 def bcs_prepare_rows(p: int, r_begin: int, r_end: int, recv_out, workspace, stream=None) -> None:
     """Second half, for one range (r_begin a multiple of 16): its receive rows into recv_out, if
     that is not None."""
-    _check(_call.prepare_rows(p, r_begin, r_end, _ptr(recv_out), _ptr(workspace),
-                                  _nbytes(workspace), _stream(stream)), "bcs_prepare_rows")
+    _check(_call.on_prepare_rows(p, r_begin, r_end, recv_out, workspace, stream), "bcs_prepare_rows")
 
 
 def bcs_build_prepared(p: int, r_begin: int, r_end: int, recv_out, send_out, workspace,
                        stream=None) -> None:
     """Rank-major receive / send rows of a range of a p that bcs_prepare was called for."""
-    _check(_call.build_prepared(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
-                                    _ptr(workspace), _nbytes(workspace), _stream(stream)),
+    _check(_call.on_build_prepared(p, r_begin, r_end, recv_out, send_out, workspace, stream),
            "bcs_build_prepared")
 
 
 def bcs_build_static(p: int, r_begin: int, r_end: int, recv_out, send_out, stream=None) -> None:
     """bcs_build for callers that cannot allocate or pass a workspace.  Raises BcsError
     (BCS_ERR_UNSUPPORTED) when bcs_build_workspace_bytes of the range is above 8 MiB."""
-    _check(_call.build_static(p, r_begin, r_end, _ptr(recv_out), _ptr(send_out),
-                                  _stream(stream)), "bcs_build_static")
+    _check(_call.on_build_static(p, r_begin, r_end, recv_out, send_out, stream), "bcs_build_static")
 
 
 def bcs_build_to_host(p: int, r_begin: int, r_end: int, recv_host, send_host, stage_dev,
@@ -316,8 +332,7 @@ def bcs_build_batch(plan_dev: BatchPlan, recv_out, send_out, workspace=None, str
 def bcs_expand(p: int, n: int, r_begin: int, r_end: int, recv, send, table_out, stream=None) -> None:
     """recv/send: CUDA int8 rows of ranks r_begin..r_end-1; table_out: CUDA int32
     [(r_end-r_begin), n-1+q, 4]."""
-    _check(_call.expand(p, n, r_begin, r_end, _ptr(recv), _ptr(send), _ptr(table_out),
-                            _stream(stream)), "bcs_expand")
+    _check(_call.on_expand(p, n, r_begin, r_end, recv, send, table_out, stream), "bcs_expand")
 
 
 def bcs_validate(p: int, r_begin: int, r_end: int, recv, send, violations_out, stream=None) -> None:
@@ -339,8 +354,7 @@ def bcs_allgather_tables(p: int, n: int, r: int, recv, send, pack_out, unpack_ou
                          stream=None) -> None:
     """recv/send: full [p][q] CUDA int8 tables; pack_out/unpack_out: CUDA int32 [n-1+q, p]
     (or None): blocks of buffer[j] processor r packs / unpacks per round (Algorithm 9)."""
-    _check(_call.allgather_tables(p, n, r, _ptr(recv), _ptr(send), _ptr(pack_out),
-                                      _ptr(unpack_out), _stream(stream)), "bcs_allgather_tables")
+    _check(_call.on_allgather_tables(p, n, r, recv, send, pack_out, unpack_out, stream), "bcs_allgather_tables")
 
 
 def bcs_simulate(p: int, n: int, recv, send, state, counts_out, stream=None) -> None:

@@ -155,6 +155,42 @@ def test_arguments_that_the_fast_calls_take_are_those_of_ctypes(lib):
         binding._call.build(10, 0, 0)
 
 
+def test_calls_with_tensors_are_those_with_numbers(lib):
+    """What the extension module makes of tensors and streams is what binding.py makes of them: each argument in its place (told by the
+    refusals), the errors of a tensor, and the workspace's size."""
+    from types import SimpleNamespace
+    from paper_2205_10072_b200 import binding
+    stream = SimpleNamespace(cuda_stream=0)
+    at = lambda address, size=0: SimpleNamespace(data_ptr=lambda: address, nbytes=size)
+    good, off, ws, small = at(64), at(72), at(64, 1 << 20), at(64, 64)
+    cases = [("build", (10, 0, 10, None, None, None, stream)), ("build", (10, 0, 10, off, None, None, stream)), ("build", (10, 0, 10, good, off, None, stream)),
+             ("build", (10, 0, 10, good, None, off, stream)), ("build", (10, 3, 2, good, good, good, stream)), ("build", (10, 3, 3, None, None, None, stream)),
+             ("build_rooted", (10, 10, 0, 10, good, good, None, stream)), ("build_rooted", (10, 3, 0, 11, good, good, None, stream)),
+             ("build_rooted", (1001, 3, 0, 1001, good, good, small, stream)), ("prepare_rows", (1000, 16, 100, good, small, stream)),
+             ("prepare_rows", (1000, 16, 100, off, ws, stream)), ("prepare_rows", (1000, 8, 100, good, ws, stream)),
+             ("build_prepared", (1000, 0, 100, good, off, ws, stream)), ("build_prepared", (1000, 0, 100, good, good, small, stream)),
+             ("build_prepared", (1000, 0, 100, None, None, ws, stream)), ("build_static", (10, 0, 10, None, off, stream)),
+             ("build_static", (10, 0, 11, good, good, stream)), ("expand", (10, 4, 0, 10, good, None, good, stream)), ("expand", (10, 4, 0, 10, good, good, off, stream)),
+             ("expand", (10, 0, 0, 10, good, good, good, stream)), ("allgather_tables", (10, 4, 10, good, good, good, good, stream)),
+             ("allgather_tables", (10, 4, 3, off, good, good, None, stream)), ("allgather_tables", (10, 4, 3, good, off, None, good, stream)),
+             ("allgather_tables", (10, 4, 3, good, good, at(66), None, stream)), ("allgather_tables", (10, 4, 3, good, good, None, None, stream))]
+    statuses = set()
+    for name, args in cases:
+        status = getattr(binding._call, "on_" + name)(*args)
+        assert status == binding._PLAIN[name](*args), (name, args)
+        statuses.add(status)
+    assert statuses == {0, 1, 2, 3}
+    for bad in (3, SimpleNamespace(), "x"):
+        with pytest.raises(AttributeError):
+            lib.bcs_build(10, 0, 10, good, bad, stream=stream)
+    with pytest.raises(AttributeError):                          # a workspace without a size
+        lib.bcs_build(10, 0, 10, good, good, SimpleNamespace(data_ptr=lambda: 64), stream=stream)
+    with pytest.raises(ZeroDivisionError):
+        lib.bcs_build(10, 0, 10, SimpleNamespace(data_ptr=lambda: 1 // 0), good, stream=stream)
+    with pytest.raises(AttributeError):
+        lib.bcs_build(10, 0, 10, good, good, stream=3)
+
+
 FAKE_RUNTIME = r"""
 #include <cuda_runtime.h>
 #include <stdio.h>
