@@ -640,6 +640,25 @@ def test_allgather_tables_of_every_split(bcs, p, n):
                 assert bool((raw[i] == -77).all()) if out is None else torch.equal(out, want[i]), (r, off, i)
 
 
+# rows copied as they lie (odd q) or with a gap behind every fourth (even q), in short and in long CTAs; the ranks of a CTA that go on at 0 (r anywhere), tables
+# that end inside a word, q = 1, and a row of one buffer group more or less
+@pytest.mark.parametrize("p,n", [(2, 5), (3, 9), (6, 40), (255, 90), (256, 90), (257, 90), (1001, 600), (2047, 70), (3000, 2600), (9999, 500), (20001, 60), (20001, 500),
+                                 (40001, 30), (40001, 250), (70001, 130)])
+def test_allgather_rows_as_they_lie(bcs, p, n):
+    want_r, want_s = oracle.full_table(p)
+    recv, send = torch.from_numpy(want_r).cuda(), torch.from_numpy(want_s).cuda()
+    size = (n - 1 + oracle.q_of(p)) * p
+    for r, off in ((0, 32), (p // 2, 33), (p - 1, 34)):
+        want = [torch.from_numpy(t).cuda().view(-1) for t in oracle.allgather_rank(p, n, r, want_r, want_s)]
+        for asked in ((True, True), (True, False), (False, True)):
+            raw = torch.full((2, size + 96), -77, dtype=torch.int32, device="cuda")
+            outs = [raw[i, off + i:off + i + size] if a else None for i, a in enumerate(asked)]
+            bcs.bcs_allgather_tables(p, n, r, recv, send, *outs)
+            for i, out in enumerate(outs):
+                assert bool((raw[i, :off + i] == -77).all()) and bool((raw[i, off + i + size:] == -77).all()), (r, off)
+                assert bool((raw[i] == -77).all()) if out is None else torch.equal(out, want[i]), (r, off, i)
+
+
 def test_allgather_tables_match_oracle(bcs):
     """Algorithm 9's pack / unpack block numbers: every entry against the oracle's literal loops
     for small p, the library's own tables simulated (all p processors) for tiny p, and the
