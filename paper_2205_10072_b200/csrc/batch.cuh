@@ -2,7 +2,7 @@
 //
 // A CTA builds the row table of a p (rows.cuh) and computes rows from it; where several CTAs share an SM, one builds a
 // table while the others compute.  Three kernels take a p by its size:
-//   * up to 1024 ranks: a CTA of 128 or 256 threads per p;
+//   * up to 1024 ranks: a CTA of 128 or 256 threads per p, a rank per lane or four (rule at the end of this file);
 //   * up to 2^21 ranks: CTAs of 256 threads take equal shares of the flattened ranks of the list, p by p;
 //   * more: CTAs of 640 threads, one per SM, work on one p after another (launched only when the list is long enough to hold one).
 // Each is launched as a dependent of the kernel before it on the stream and may run beside it until it waits for it.
@@ -15,12 +15,14 @@
 // this, 25.4 with the first load behind the wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8,
 // 18.7.)
 //
-// Up to 1024 ranks instruction issue bounds it, 58 % of the slots: every p up to 1024 13.9 us in any order, 15.2 ascending, 12.4 descending.
+// Up to 1024 ranks: instruction issue, and a CTA's chain from its p to its last row.  Every p up to 1024, four ranks per lane, 11.7 us in any order, 10.9
+// ascending, 11.1 descending (a rank per lane 13.9, 15.4, 12.4).
 // Above, instruction issue and the integer pipe: 1024 p of 2^10..2^20 1250 us (both tables 4.7 TB/s).  That kernel holds two narrow and two wide
 // forms in 80 registers and spills a few bytes at its three CTAs per SM; two per SM take 1368 us, four 1490.
 #pragma once
 #include <type_traits>
 
+#include "quad.cuh"
 #include "rows.cuh"
 #include "wide.cuh"
 
@@ -89,8 +91,30 @@ __device__ __forceinline__ void wide_piece(const RowTable &t, const uint8_t *sm,
     }
 }
 
-// p <= 1024: a CTA per p.
-template <unsigned kThreads, int kCtas>
+constexpr uint32_t kSmallRun = 256;               // ranks of a warp's run
+
+// All ranks of a p of 129..1024 by the warps of the CTA, four ranks per lane.  Runs begin where rows begin (nearly) on a 16-byte boundary.
+template <int Q>
+__device__ __forceinline__ void quad_small(const RowTable &t, uint8_t *sm, const BatchJob &job, uint64_t entry0, int8_t *recv, int8_t *send)
+{
+    const QuadLayout<false> at(Q, kSmallRun);
+    const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
+    const uint32_t best = quad_shift(entry0, Q), up = best & 15u, shift = best >> 4;
+    const int begin = up ? (int)up - 16 : 0, p = (int)job.p;
+    const int share = (int)(((uint32_t)(p - begin) + warps * kQuads - 1u) / (warps * kQuads) * kQuads);
+    const int stop = begin + ((int)warp + 1) * share < p ? begin + ((int)warp + 1) * share : p;
+    for (int a = begin + (int)warp * share; a < stop; a += (int)kSmallRun) {
+        const uint32_t n = stop - a < (int)kSmallRun ? (uint32_t)(stop - a) : kSmallRun;
+        const uint32_t lead = a < 0 ? (uint32_t)-a : 0u;
+        const int64_t byte = (int64_t)entry0 + (int64_t)a * Q;
+        quad_run<Q, false, false>(t, sm + at.table, mine, at, t.s, job.odd, job.inv, a < 0 ? job.p - lead : (uint32_t)a, n, lead, shift, recv + byte,
+                                  send ? send + byte : nullptr);
+    }
+}
+
+// p <= 1024: a CTA per p.  kQuad: four ranks per lane for p > 128.
+template <unsigned kThreads, int kCtas, bool kQuad>
 __global__ void __launch_bounds__(kThreads, kCtas)
 batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *send)
 {
@@ -105,7 +129,8 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         const RowTable t(sm, RowLayout(q));
         if (threadIdx.x < 32u) load_p(p, t, job);
         __syncthreads();
-        build_row_table(t, q, job.odd);
+        if (kQuad && q > kLow) build_row_table<true>(t, q, job.odd);
+        else build_row_table(t, q, job.odd);
     };
     auto fits = [](uint32_t p) { return p > 1u && p <= kSmallP; };
     if (threadIdx.x == 0) guess = load_relaxed(ba.p_list + j);
@@ -120,13 +145,19 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
     const int q = ceil_log2_fast(p);
     const RowLayout at(q);
     const RowTable t(sm, at);
-    uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
-    constexpr uint32_t warps = kThreads / 32;
-    const uint32_t turns = (p + warps * kItemRanks - 1u) / (warps * kItemRanks) * warps;
-    const uint32_t item = ((p + turns - 1u) / turns + 31u) & ~31u;
-    if (q <= 4) narrow_piece<1>(t, mine, job, entry0, q, 0u, p, item, recv, send);
-    else if (q <= 8) narrow_piece<2>(t, mine, job, entry0, q, 0u, p, item, recv, send);
-    else narrow_piece<3>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+    if (kQuad && q > kLow) {
+        if (q == 8) quad_small<8>(t, sm, job, entry0, recv, send);
+        else if (q == 9) quad_small<9>(t, sm, job, entry0, recv, send);
+        else quad_small<10>(t, sm, job, entry0, recv, send);
+    } else {
+        uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
+        constexpr uint32_t warps = kThreads / 32;
+        const uint32_t turns = (p + warps * kItemRanks - 1u) / (warps * kItemRanks) * warps;
+        const uint32_t item = ((p + turns - 1u) / turns + 31u) & ~31u;
+        if (q <= 4) narrow_piece<1>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+        else if (q <= 8) narrow_piece<2>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+        else if constexpr (!kQuad) narrow_piece<3>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+    }
     stage_free();
 }
 
@@ -280,17 +311,17 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
 // A CTA per p of the list, up to kCtas of them per SM.  alone: no larger p, nothing runs beside them.  Where the list is then
 // too short to fill the card, they ask for so much shared memory that they spread over all SMs (else some held five and
 // others one: 300 p of 3..900 11.9 -> 8.4 us).
-template <unsigned kThreads, int kCtas>
+template <unsigned kThreads, int kCtas, bool kQuad>
 bcs_status launch_small(const BatchArgs &ba, bool alone, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
-    uint32_t shared = RowLayout(kSmallQ).total(kThreads / 32);
+    uint32_t shared = kQuad ? QuadLayout<false>(kSmallQ, kSmallRun).total(kThreads / 32) : RowLayout(kSmallQ).total(kThreads / 32);
     const uint32_t per_sm = (ba.num_p + kSms - 1) / kSms;
     if (alone && per_sm < (uint32_t)kCtas) {
         const uint32_t spread = (226u * 1024u / per_sm - 1280u) & ~127u;     // (1 KB of each CTA is the system's)
         if (shared < spread) shared = spread;
     }
-    if (!allow_shared<batch_small_kernel<kThreads, kCtas>>()) return BCS_ERR_CUDA;
-    launch_dependent(true, batch_small_kernel<kThreads, kCtas>, ba.num_p, kThreads, shared, stream, ba, recv, send);
+    if (!allow_shared<batch_small_kernel<kThreads, kCtas, kQuad>>()) return BCS_ERR_CUDA;
+    launch_dependent(true, batch_small_kernel<kThreads, kCtas, kQuad>, ba.num_p, kThreads, shared, stream, ba, recv, send);
     return launch_status();
 }
 
@@ -354,12 +385,19 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
                              send_out);
         }
     }
-    // CTAs of 256 threads while all are resident at once (the shorter chain counts), else of 128 (less waiting at
-    // barriers, longer items): us with 256 / 128, 300 p of 3..900 7.0/8.8, 700 of 3..702 9.4/10.2, 740 of 280..1019 9.7/12.0;
-    // 800 of 1000 13.4/12.9, 900 of 64..256 8.4/6.0, 1000 of 33 6.4/3.7, 2000 of 2..1024 20.7/20.7, 5000 of 777 62/61.  The number alone
-    // does not tell: every p up to 1024 takes 14.6/13.9 in any order, but 11.8/15.3 in ascending order (neighbours of like size).
-    if (num_p <= kSms * 5u) return launch_small<256, 5>(ba, small_only, recv_out, send_out, stream);
-    return launch_small<128, 8>(ba, small_only, recv_out, send_out, stream);
+    // Four ranks per lane for lists without a larger p whose p are 400 on average or more; us with it / the per-rank form: every p up to 1024 in any order
+    // 11.7/13.9, ascending 10.8/15.4, 5000 of 777 43.6/60.8, 800 of 1000 8.1/12.9, 740 of 280..1019 8.8/9.8.  A CTA takes one p, and CTAs whose p
+    // have other q run other code, which counts where there is little to do for each: 900 of 64..256 6.3/5.9, 300 of 64..1000 7.5/6.7, 700 of 2^6..2^12
+    // (beside the kernel for larger p) 33.3/29.8.  CTAs of 256 threads while three of them per SM take the list (140 of 900 4.6, with 128 threads 5.1).
+    if (small_only && total_ranks >= 400ull * num_p) {
+        if (num_p <= kSms * 3u) return launch_small<256, 3, true>(ba, true, recv_out, send_out, stream);
+        return launch_small<128, 8, true>(ba, true, recv_out, send_out, stream);
+    }
+    // Per rank: CTAs of 256 threads while all are resident at once (the shorter chain counts), else of 128 (less waiting at
+    // barriers, longer items): us with 256 / 128, 300 p of 3..900 7.0/8.8, 700 of 3..702 9.4/10.2;
+    // 900 of 64..256 8.4/6.0, 1000 of 33 6.4/3.7, 2000 of 2..1024 20.7/20.7.
+    if (num_p <= kSms * 5u) return launch_small<256, 5, false>(ba, small_only, recv_out, send_out, stream);
+    return launch_small<128, 8, false>(ba, small_only, recv_out, send_out, stream);
 }
 
 }  // extern "C"

@@ -84,7 +84,7 @@ struct QuadLayout {
         entries = segments * 16u;
         columns = entries + segments * 64u;
         stage = (columns + (kTable ? 0u : kLow * kColumn) + 15u) & ~15u;
-        warp_bytes = stage + kPass * (uint32_t)q + 16u;
+        warp_bytes = stage + kPass * (uint32_t)q + 16u;      // (rows that are shifted end in the last 16 bytes)
     }
     __host__ __device__ uint32_t total(uint32_t n_warps) const { return warps + n_warps * warp_bytes; }
 };
@@ -133,7 +133,7 @@ __device__ __forceinline__ int locate_run(const RowTable &t, Segment *segments, 
         seg.start = start;
         seg.key = (K * kLowRanks - start) * 8;
         const uint32_t home = g ? (uint32_t)(31 - __clz(g) + kLow) : 0u;
-        seg.recv = (K ? count_odd(odd, kLow, kLow + K) + 1u : 0u) | (uint32_t)K << 5 | home << 10 | (home < (uint32_t)(4 * ((Q + 3) / 4 - 2)) ? 1u << 15 : 0u);
+        seg.recv = (K ? count_odd(odd, kLow, kLow + K) + 1u : 0u) | (uint32_t)K << 5 | home << 10 | ((int)(home ? home : kLow) < 4 * ((Q + 3) / 4 - 2) ? 1u << 15 : 0u);
         seg.send = g ? 0u : 1u << 21;
         if (g & 1u)                                              // its first rank carries into one close behind a start
             seg.send = 1u << 20 | (uint32_t)((int)t.miss[tz * kMissRanks + (int)count_odd(odd, kLow, kLow + tz)] - Q) << 24;
@@ -180,6 +180,8 @@ __device__ __forceinline__ int locate_run(const RowTable &t, Segment *segments, 
                 if (home >= 0) {
                     received |= 7u << (4 * home);
                     sent |= home < 7 ? 0x77777777u << (4 * home + 4) : 0u;
+                } else if constexpr (kLow >= tail) {             // the root's segment, rounds from L on
+                    if (code == 0u) sent |= 0x77777777u << (4 * (kLow - tail));
                 }
             }
             e[0] = received;
@@ -243,6 +245,115 @@ __device__ __forceinline__ void stage_words(uint8_t *at, const uint32_t (&R)[4][
     }
 }
 
+// The same for rows that begin `bits` / 8 bytes behind `at`, 3 at most: the words are shifted, the last one runs into the next lane's first.
+// prev: the word in front of the lane's.
+template <int Q, int o, int kWords>
+__device__ __forceinline__ void stage_words_shifted(uint8_t *at, const uint32_t (&R)[4][kWords], uint32_t prev, uint32_t bits)
+{
+    if constexpr (o < Q) {
+        constexpr int step = Q % 4 == 0 ? 4 : (Q % 2 == 0 ? 2 : 1);
+        const uint32_t a = joined<Q, o>(R);
+        if constexpr (step == 4) {
+            const uint32_t b = joined<Q, o + 1>(R), c = joined<Q, o + 2>(R), d = joined<Q, o + 3>(R);
+            *reinterpret_cast<uint4 *>(at + 4 * o) = make_uint4(__funnelshift_l(prev, a, bits), __funnelshift_l(a, b, bits),
+                                                                __funnelshift_l(b, c, bits), __funnelshift_l(c, d, bits));
+            stage_words_shifted<Q, o + 4>(at, R, d, bits);
+        } else if constexpr (step == 2) {
+            const uint32_t b = joined<Q, o + 1>(R);
+            *reinterpret_cast<uint2 *>(at + 4 * o) = make_uint2(__funnelshift_l(prev, a, bits), __funnelshift_l(a, b, bits));
+            stage_words_shifted<Q, o + 2>(at, R, b, bits);
+        } else {
+            *reinterpret_cast<uint32_t *>(at + 4 * o) = __funnelshift_l(prev, a, bits);
+            stage_words_shifted<Q, o + 1>(at, R, a, bits);
+        }
+    }
+}
+
+// How the rows of a run lie in memory, and the words that a lane hands on.  Where q is a multiple of 8 the rows of all ranks begin at the same or at two places
+// of a 16-byte group, so up to 15 bytes of shift are left, else 3 (quad_shift()).
+template <int Q>
+struct Shifted {
+    static constexpr int kCarry = Q % 8 == 0 ? 4 : 1;
+    uint32_t bytes;                                    // by which the run's first row is off a 16-byte group
+    uint32_t carry[kCarry];                            // the last words of the 128 ranks before, the last one first
+};
+
+template <int Q, int o, int kWords>
+__device__ __forceinline__ void join_words(const uint32_t (&R)[4][kWords], uint32_t (&V)[Q + 4])
+{
+    if constexpr (o < Q) {
+        V[o + 4] = joined<Q, o>(R);
+        join_words<Q, o + 1>(R, V);
+    }
+}
+
+template <int Q, int kWords>
+__device__ __forceinline__ void stage_shifted(uint8_t *at, const uint32_t (&R)[4][kWords], Shifted<Q> &sh)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    if constexpr (Q % 8 == 0) {
+        uint32_t V[Q + 4];                             // V[w + 4]: word w
+        join_words<Q, 0>(R, V);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t before = __shfl_up_sync(0xffffffffu, V[Q + 3 - j], 1);
+            V[3 - j] = lane ? before : sh.carry[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sh.carry[j] = __shfl_sync(0xffffffffu, V[Q + 3 - j], 31);
+        const uint32_t bits = 8u * (sh.bytes & 3u);
+#pragma unroll
+        for (int w = Q + 3; w > 0; --w) V[w] = __funnelshift_l(V[w - 1], V[w], bits);
+        if (sh.bytes & 4u) {
+#pragma unroll
+            for (int w = Q + 3; w > 1; --w) V[w] = V[w - 1];
+        }
+        if (sh.bytes & 8u) {
+#pragma unroll
+            for (int w = Q + 3; w > 3; --w) V[w] = V[w - 2];
+        }
+#pragma unroll
+        for (int w = 0; w < Q; w += 4) *reinterpret_cast<uint4 *>(at + 4 * w) = make_uint4(V[w + 4], V[w + 5], V[w + 6], V[w + 7]);
+    } else {
+        const uint32_t last = joined<Q, Q - 1>(R), before = __shfl_up_sync(0xffffffffu, last, 1);
+        stage_words_shifted<Q, 0>(at, R, lane ? before : sh.carry[0], 8u * sh.bytes);
+        sh.carry[0] = __shfl_sync(0xffffffffu, last, 31);
+    }
+}
+
+// What the rows of the last lane leave for the 16 bytes behind them.
+template <int Q>
+__device__ __forceinline__ void stage_rest(uint8_t *at, const Shifted<Q> &sh)
+{
+    if ((threadIdx.x & 31u) != 0u || sh.bytes == 0u) return;
+    if constexpr (Q % 8 == 0) {
+        const uint32_t bits = 8u * (sh.bytes & 3u), s = sh.bytes >> 2;
+        uint32_t F[5];                                 // words -4 .. 0 behind the end, shifted by `bits`
+        F[0] = 0u;
+#pragma unroll
+        for (int j = 1; j < 4; ++j) F[j] = __funnelshift_l(sh.carry[4 - j], sh.carry[3 - j], bits);
+        F[4] = __funnelshift_l(sh.carry[0], 0u, bits);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {                  // word w: word w - s of these
+            uint32_t v = 0u;
+#pragma unroll
+            for (int j = 0; j < 5; ++j)
+                if (w - (int)s == j - 4) v = F[j];
+            reinterpret_cast<uint32_t *>(at)[w] = v;
+        }
+    } else {
+        *reinterpret_cast<uint32_t *>(at) = __funnelshift_l(sh.carry[0], 0u, 8u * sh.bytes);
+    }
+}
+
+// Of 16 consecutive ranks of a p whose rows begin at byte `entry`, one whose row begins the least behind a 16-byte boundary: 0 bytes for odd q, 1 at most
+// for q = 2 (mod 4), 3 for 4 (mod 8).  Returns rank + 16 bytes.  By a warp.
+__device__ __forceinline__ uint32_t quad_shift(uint64_t entry, int q)
+{
+    const uint32_t rank = threadIdx.x & 15u;
+    return __reduce_min_sync(0xffffffffu, (((uint32_t)entry + rank * (uint32_t)q) & 15u) << 4 | rank);
+}
+
 // What a look-up leaves about four ranks for the rows that are made from them.
 struct QuadState {
     uint32_t slot;         // segment of the first of them
@@ -253,8 +364,9 @@ struct QuadState {
 
 // Stages four rows at `at`: words 0 and 1 from the rounds below L (eight bytes a row, the last one the baseblock), the others from the entries of
 // their segment and of the next one; in the home round (kSend: in all rounds behind it) the baseblock.
-template <int Q, bool kSend>
-__device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4], const uint32_t (&hi)[4], const uint8_t *entries, const QuadState &s)
+template <int Q, bool kSend, bool kAligned>
+__device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4], const uint32_t (&hi)[4], const uint8_t *entries, const QuadState &s,
+                                           Shifted<Q> &shifted)
 {
     constexpr int kWords = (Q + 3) / 4;
     uint32_t R[4][kWords], S[8], T[8];
@@ -313,20 +425,22 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
             for (int i = 0; i < 4; ++i) R[i][w] = __byte_perm(R[i][w], hi[i], i == 0 || i < s.room ? here : next);
         }
     }
-    stage_words<Q, 0>(at, R);
+    if constexpr (kAligned) stage_words<Q, 0>(at, R);
+    else stage_shifted<Q>(at, R, shifted);
 }
 
 // Receive and send rows (either pointer may be null) of the n ranks x0, x0 + 1, ... (mod p; x0 < p, n <= the run of `at`, n <= p) by one warp.
-// recv, send: where the row of x0 goes, 16-byte aligned.  mine: the warp's shared memory; skips: those of p.  kTable: send rows from
-// their table, at send_rows.
-template <int Q, bool kTable>
+// recv, send: where the row of x0 goes: kAligned, on a 16-byte boundary; else `bytes` behind one (quad_shift()), and the first `lead` ranks are not written.
+// mine: the warp's shared memory; skips: those of p.  kTable: send rows from their table, at send_rows.
+template <int Q, bool kTable, bool kAligned>
 __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_rows, uint8_t *mine, const QuadLayout<kTable> &at, const uint32_t *skips,
-                                         uint32_t odd, uint32_t inv, uint32_t x0, uint32_t n, int8_t *recv, int8_t *send)
+                                         uint32_t odd, uint32_t inv, uint32_t x0, uint32_t n, uint32_t lead, uint32_t shift,
+                                         int8_t *recv, int8_t *send)
 {
     const uint32_t lane = threadIdx.x & 31u;
     Segment *segments = reinterpret_cast<Segment *>(mine);
-    uint8_t *entries = mine + at.entries, *columns = mine + at.columns, *stage = mine + at.stage;
-    uint8_t *own = stage + lane * (4u * Q);
+    uint8_t *entries = mine + at.entries, *columns = mine + at.columns, *staged = mine + at.stage;
+    uint8_t *own = staged + lane * (4u * Q), *stage = staged + (kAligned ? 0u : shift);       // the lane's words, the first row
     const uint8_t *table = reinterpret_cast<const uint8_t *>(t.rows);
     const int starts = locate_run<Q, kTable>(t, segments, entries, odd, inv, x0, n, at.segments);
 
@@ -399,13 +513,24 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
             fence_before_bulk();
             if (b == 0u) grid_dependency_wait();                 // (the kernel before: not until the first store)
             __syncwarp();
-            int8_t *dst = out + b * Q;
-            if (elect_one() && bytes >= 16u) bulk_store(dst, stage, bytes & ~15u);
-            if (ranks != kPass && lane < (bytes & 15u)) dst[(bytes & ~15u) + lane] = (int8_t)stage[(bytes & ~15u) + lane];
+            if constexpr (kAligned) {
+                int8_t *dst = out + b * Q;
+                if (elect_one() && bytes >= 16u) bulk_store(dst, stage, bytes & ~15u);
+                if (ranks != kPass && lane < (bytes & 15u)) dst[(bytes & ~15u) + lane] = (int8_t)stage[(bytes & ~15u) + lane];
+            } else {                                             // bytes [begin, end) from a 16-byte boundary on, the ragged ends one by one
+                int8_t *dst = out + (int64_t)b * Q - shift;
+                const uint32_t begin = shift + (b == 0u ? lead * Q : 0u), end = shift + bytes;
+                const uint32_t head = (begin + 15u) & ~15u, tail = end & ~15u;
+                if (elect_one() && tail > head) bulk_store(dst + head, staged + head, tail - head);
+                const uint32_t stop = head < end ? head : end, rest = tail > head ? tail : stop;
+                if (begin + lane < stop) dst[begin + lane] = (int8_t)staged[begin + lane];
+                if (rest + lane < end) dst[rest + lane] = (int8_t)staged[rest + lane];
+            }
         };
 
         QuadState states[kTurns];
         int2 keys[kTurns];
+        Shifted<Q> shifted = {kAligned ? 0u : shift, {}};
         stage_free();
 #pragma unroll
         for (int j = 0; j < kTurns; ++j) {
@@ -415,7 +540,7 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
             if (kTable && recv == nullptr) continue;
             look_up(table, states[j], keys[j], lo, hi);
             if (!kTable && send != nullptr) put_columns(j * kQuads, 32u, states[j], lo, hi);
-            if (recv != nullptr) stage_quad<Q, false>(own + j * (int)(kQuads * Q), lo, hi, entries, states[j]);
+            if (recv != nullptr) stage_quad<Q, false, kAligned>(own + j * (int)(kQuads * Q), lo, hi, entries, states[j], shifted);
         }
         if (!kTable && send != nullptr) {                        // and the ranks behind
             QuadState s;
@@ -425,6 +550,7 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
             look_up(table, s, k, lo, hi);
             put_columns(turns * kQuads, (kHalo + 8u) / 4u, s, lo, hi);
         }
+        if (!kAligned && recv != nullptr) stage_rest<Q>(staged + turns * (kQuads * Q), shifted);
         __syncwarp();
         if (recv != nullptr) {
             for (uint32_t j = slot; j < slots; j += 8u) {
@@ -444,6 +570,7 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
         }
         if (send == nullptr) continue;
         if (recv != nullptr) stage_free();
+        if (!kAligned) shifted = {shift, {}};
 #pragma unroll
         for (int j = 0; j < kTurns; ++j) {
             if (j != 0 && turns == 1u) break;
@@ -461,8 +588,9 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
                 transpose(c[0], c[1], c[2], c[3], lo[0], lo[1], lo[2], lo[3]);
                 transpose(c[4], c[5], c[6], states[j].bases, hi[0], hi[1], hi[2], hi[3]);
             }
-            stage_quad<Q, true>(own + j * (int)(kQuads * Q), lo, hi, entries, states[j]);
+            stage_quad<Q, true, kAligned>(own + j * (int)(kQuads * Q), lo, hi, entries, states[j], shifted);
         }
+        if (!kAligned) stage_rest<Q>(staged + turns * (kQuads * Q), shifted);
         __syncwarp();
         for (uint32_t j = slot; j < slots; j += 8u) {
             const Segment seg = segments[j];

@@ -102,7 +102,7 @@ quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
             uint32_t x0 = first + (uint32_t)b;
             if (x0 >= rc.p) x0 -= rc.p;
             const uint64_t byte = b * Q;
-            quad_run<Q, kTable>(t, sm + at.table, mine, at, rc.s, rc.odd, rc.inv, x0, n, recv ? recv + byte : nullptr, send ? send + byte : nullptr);
+            quad_run<Q, kTable, true>(t, sm + at.table, mine, at, rc.s, rc.odd, rc.inv, x0, n, 0u, 0u, recv ? recv + byte : nullptr, send ? send + byte : nullptr);
         }
         if (once) break;
         if (!barrier_wait(&answered, parity)) {

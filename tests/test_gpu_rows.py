@@ -175,6 +175,14 @@ def test_batch_splits(bcs, plist):
     _batch(bcs, list(plist))
 
 
+# Four ranks per lane for lists of small p: tables that begin at any byte of a 16-byte group (rows of q = 8 at any of its bytes, of q = 10 one byte off, of q = 9
+# always on one with some rank), runs of a warp that begin in front of rank 0, in CTAs of 256 threads and of 128
+@pytest.mark.parametrize("first", [1, 2, 3, 5, 7, 9, 17, 33])
+@pytest.mark.parametrize("times", [3, 40])
+def test_batches_of_small_p_at_any_byte(bcs, first, times):
+    _batch(bcs, [first] + [1024, 1023, 513, 512, 511, 700, 129, 257, 256, 255, 1000, 130, 641] * times)
+
+
 # The plan of a batch as the work of the kernel before it on the stream, one that lets its successors start early: the list of p
 # is a stretch of a row of allgather tables, block numbers of about `row` each.  Nothing of what its memory held before may
 # reach the tables, be it another p of the kernel's range or none.
