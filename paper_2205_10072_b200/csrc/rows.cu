@@ -11,6 +11,7 @@
 #include "batch.cuh"     // (in this unit, too: the constants of rows.cuh are in the module once)
 #include "rows.cuh"
 #include "quad.cuh"
+#include "wide.cuh"
 
 namespace bcs {
 namespace {
@@ -59,6 +60,51 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
                                 send ? send + byte : nullptr);
     }
     stage_free();
+}
+
+// Send rows alone of 1.9 to 6 million ranks, 16 output bytes per lane (wide.cuh): a run per warp, one CTA per SM.  Its table of send rows holds those of all the
+// CTA's segments, and nothing is looked up twice.  us, this / quad_kernel: 2 million ranks of q = 21 11.3/11.4, of q = 28 12.1/12.8, 3.1 million of q = 23
+// 16.0/18.9, 4.8 million 22.4/23.5; 1.5 million of q = 21 10.2/9.1, 6.5 million of q = 24 31.7/29.9, of q = 28 34.7/30.9.
+constexpr unsigned kWideThreads = 640;
+constexpr uint32_t kWideFrom = 1900000, kWideTo = 6000000;
+
+template <bool kAnyStep>
+__global__ void __launch_bounds__(kWideThreads, 1)
+wide_send_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t run, int8_t *send)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    grid_launch_dependents();
+    const WideLayout at(rc.q);
+    const RowTable t(sm, at.base);
+    if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
+    const uint32_t warps = kWideThreads / 32u, warp = threadIdx.x >> 5, begin = blockIdx.x * warps * run;
+    if (begin >= count) {                                        // (stays until the kernel before is done, or CTAs of the next calls pile up here)
+        grid_dependency_wait();
+        return;
+    }
+    auto rank = [&](uint32_t b) {
+        const uint32_t x = first + b;
+        return x >= rc.p ? x - rc.p : x;
+    };
+    want_rows(t, rc.q, rc.inv, rank(begin), warps * run + 1u);   // (the last vectors look at the rank behind)
+    build_row_table(t, rc.q, rc.odd);
+    build_send_table_wide(t, reinterpret_cast<uint2 *>(sm + at.send), rc.q, rc.odd);
+    const uint32_t b = begin + warp * run;
+    if (b >= count) return;
+    const uint32_t n = count - b < run ? count - b : run;
+    WideLane mine;
+    mine.template init<kAnyStep>(rc.q, 0u);
+    wide_rows<true, kAnyStep, true>(t, sm, at.send, sm + at.ends + warp * 32u, rc.p, rc.q, rc.odd, rc.inv, mine, rank(b), n, b == 0u, b + n == count,
+                                    send + (uint64_t)b * (uint64_t)rc.q);
+}
+
+template <bool kAnyStep>
+bcs_status launch_wide_send(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *send, cudaStream_t stream)
+{
+    if (!allow_shared<wide_send_kernel<kAnyStep>>()) return BCS_ERR_CUDA;
+    const uint32_t all = kSms * kWideThreads / 32u * kStep, run = (count + all - 1u) / all * kStep;
+    launch_dependent(true, wide_send_kernel<kAnyStep>, kSms, kWideThreads, WideLayout(rc.q).bytes, stream, rc, first, count, run, send);
+    return launch_status();
 }
 
 constexpr unsigned kQuadThreads = 320;
@@ -162,6 +208,8 @@ bcs_status launch_quads(const RowConsts &rc, uint32_t first, uint32_t count, int
     if constexpr (Q > BCS_MAX_Q) return BCS_ERR_UNSUPPORTED;
     else {
         if (rc.q != Q) return launch_quads<Q + 1>(rc, first, count, recv, send, stream);
+        if (recv == nullptr && count >= kWideFrom && count < kWideTo)
+            return step_ranks(Q) == 16u ? launch_wide_send<false>(rc, first, count, send, stream) : launch_wide_send<true>(rc, first, count, send, stream);
         if (send != nullptr && count >= (1u << 22)) return launch_quad<Q, true>(rc, first, count, recv, send, stream);
         return launch_quad<Q, false>(rc, first, count, recv, send, stream);
     }

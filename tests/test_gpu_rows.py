@@ -279,6 +279,14 @@ def test_four_ranks_per_lane(bcs, q):
     assert bcs.bcs_wait_expired() == 0
 
 
+# Send rows alone of some million ranks take another kernel: around its lines, runs that end inside the last CTA, steps of 16, 20 and 24 ranks
+@pytest.mark.parametrize("n", [1899999, 1900000, 2500001, 5999999, 6000000])
+@pytest.mark.parametrize("p", [6000001, (1 << 24) - 5, (1 << 28) - 1, (1 << 31) - 1])
+def test_send_rows_alone_of_some_million_ranks(bcs, p, n):
+    _check(bcs, p, 0, n, recv=False)
+    _check(bcs, p, p - n, p, recv=False)
+
+
 # A call into tables that the kernel in front of it still reads: the row kernels are launched while that one runs, and wait for it in
 # front of their first store, warp by warp; warps and CTAs without ranks need not.  `between`: with a call of one CTA into other
 # tables in the middle, which must not be done before the one in front of it is.
