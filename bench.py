@@ -354,8 +354,8 @@ def _bench_single(torch, bcs, workloads, flush, steps, hbm_gbs, sm_max_mhz, coun
            "l2": "flushed before every timed step (256 MiB write)",
            "back_to_back_ms": e0.elapsed_time(e1) / 2000,
            "kernel_ms": {"receive rows alone": recv_ms},
-           "roofline": _alu_roofline(["wide_kernel@q21"], p, step_ms, 2 * nb, hbm_gbs, sm_max_mhz, counts, measured)}
-    res["roofline"]["traffic"] = counts["wide_kernel@q21"]["dram_bytes"]
+           "roofline": _alu_roofline(["quad_kernel@q21"], p, step_ms, 2 * nb, hbm_gbs, sm_max_mhz, counts, measured)}
+    res["roofline"]["traffic"] = counts["quad_kernel@q21"]["dram_bytes"]
     # property check and brute-force broadcast of the tables just built
     viol = torch.zeros(3, dtype=torch.int64, device="cuda")
     v_ms = statistics.mean(_event_ms(torch, lambda: bcs.bcs_validate(p, 0, p, recv, send, viol), flush, 10, 2))
@@ -591,12 +591,12 @@ def run_ours(args) -> None:
         measured = Probe(torch).all()
         rows_ms, send_ms = large.parts_ms()
         gbs = 2 * p * q / ms_per_step / 1e6
-        roof = {"bound": "hbm", "kernel": "wide_kernel (8 launches for the receive rows, 8 for the send rows: the whole step)",
+        roof = {"bound": "hbm", "kernel": "quad_kernel (8 launches for the receive rows, 8 for the send rows: the whole step)",
                 "achieved": gbs, "peak": hbm_gbs, "unit": "GB/s", "frac": gbs / hbm_gbs, "peak_source": peak_src,
                 "traffic": None,
                 "traffic_note": "not captured at this size (4 GB per launch); the DRAM bytes of a 2^24-rank range of the "
                                 "same p are in profiles/"}
-        step_roof = _alu_roofline(["wide_kernel@q30"], p, ms_per_step, 2 * p * q, hbm_gbs, sm_max_mhz, counts, measured)
+        step_roof = _alu_roofline(["quad_kernel@q30"], p, ms_per_step, 2 * p * q, hbm_gbs, sm_max_mhz, counts, measured)
         checked_ms, violations = large.checked_step()
         out = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

@@ -1,4 +1,4 @@
-// Large tables of a p with q >= 16: rows put together 16 output bytes at a time.
+// Rows of a p with q >= 16 put together 16 output bytes at a time: for the larger p of a list (batch.cuh), and for send rows alone of some million ranks (rows.cu).
 //
 // The per-rank form (warp_rows) pays for every rank: shifting a row to its place among the words of its neighbours, an
 // exchange with the next lane, stores q bytes apart, a copy out of shared memory.  Here a lane makes aligned
