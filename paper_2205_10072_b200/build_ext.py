@@ -15,7 +15,7 @@ HEADERS = sorted(glob.glob(os.path.join(_ROOT, "include", "*.h")) +
 # The unit with the kernels that read the constants below: all of them, so that these are in the library once (loaded by the first
 # call), and without line information, with which nvcc adds the unit's PTX, 7 MB of it the constants as text.  (First calls of a
 # process, one p and a batch: 5.5 + 0.2 ms, of which some 2 MB of quad_kernel for each q take 1; before that kernel 4.4 + 0.2, with line information 7.7 + 0.2,
-# in two such units 7.2 + 4.3, the file 5.8, 13.8, 23 MB.)
+# in two such units 7.2 + 4.3, the file 8.2 (before that kernel 5.8), 13.8, 23 MB.)
 ROWS_UNIT = os.path.join(_PKG, "csrc", "rows.cu")
 # The packed rows of all shapes of segments, written by a small program at build time.
 ROW_TABLE = os.path.join(_PKG, "csrc", "row_table.inc")

@@ -210,7 +210,8 @@ bcs_status launch_quads(const RowConsts &rc, uint32_t first, uint32_t count, int
         if (rc.q != Q) return launch_quads<Q + 1>(rc, first, count, recv, send, stream);
         if (recv == nullptr && count >= kWideFrom && count < kWideTo)
             return step_ranks(Q) == 16u ? launch_wide_send<false>(rc, first, count, send, stream) : launch_wide_send<true>(rc, first, count, send, stream);
-        if (send != nullptr && count >= (1u << 22)) return launch_quad<Q, true>(rc, first, count, recv, send, stream);
+        if constexpr (Q >= 22)                                   // (2^22 ranks are more than a smaller p has)
+            if (send != nullptr && count >= (1u << 22)) return launch_quad<Q, true>(rc, first, count, recv, send, stream);
         return launch_quad<Q, false>(rc, first, count, recv, send, stream);
     }
 }
