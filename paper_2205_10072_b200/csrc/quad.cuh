@@ -369,7 +369,7 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
                                            Shifted<Q> &shifted)
 {
     constexpr int kWords = (Q + 3) / 4;
-    uint32_t R[4][kWords], S[8], T[8];
+    uint32_t R[4][kWords], S[8];
     auto load = [&](uint32_t (&X)[8], const uint8_t *from) {
         const uint4 a = *reinterpret_cast<const uint4 *>(from);
         X[0] = a.x;
@@ -391,25 +391,41 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
         }
     };
     const uint8_t *from = entries + s.slot * 64u + (kSend ? 32u : 0u);
-    load(S, from);
+    uint32_t picks_of[4];
+    if constexpr (Q % 8 != 0) {
+        // (loaded once more for each rank rather than selected, word by word, from those of two segments: the integer pipe has more to do than shared
+        // memory, 1.06 million ranks of q = 21 10.1 -> 9.9 us; but q = 24, whose rows meet in banks, 12 million ranks 88.4 -> 91.4)
 #pragma unroll
-    for (int w = 0; w < 8; ++w) T[w] = S[w];
-    if (s.room < 4) load(T, from + 64);
+        for (int i = 0; i < 4; ++i) {
+            load(S, i == 0 || i < s.room ? from : from + 64);
+            picks_of[i] = S[0];
+            R[i][0] = lo[i];
+            R[i][1] = (hi[i] & 0xffffffu) | S[1];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const bool mine = i == 0 || i < s.room;
-        R[i][0] = lo[i];
-        R[i][1] = (hi[i] & 0xffffffu) | (mine ? S[1] : T[1]);
+            for (int w = 2; w < kWords; ++w) R[i][w] = S[w];
+        }
+    } else {
+        uint32_t T[8];
+        load(S, from);
 #pragma unroll
-        for (int w = 2; w < kWords; ++w) R[i][w] = mine ? S[w] : T[w];
+        for (int w = 0; w < 8; ++w) T[w] = S[w];
+        if (s.room < 4) load(T, from + 64);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool mine = i == 0 || i < s.room;
+            R[i][0] = lo[i];
+            picks_of[i] = mine ? S[0] : T[0];
+            R[i][1] = (hi[i] & 0xffffffu) | (mine ? S[1] : T[1]);
+#pragma unroll
+            for (int w = 2; w < kWords; ++w) R[i][w] = mine ? S[w] : T[w];
+        }
     }
     // The baseblock's bytes: of nearly all ranks in the last two words, of those below some 2^(q - 5) anywhere.
     if (!__any_sync(0xffffffffu, ((s.here | (s.room < 4 ? s.next : 0u)) >> 15) & 1u)) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const uint32_t picks = i == 0 || i < s.room ? S[0] : T[0];
-            R[i][kWords - 2] = __byte_perm(R[i][kWords - 2], hi[i], picks);
-            R[i][kWords - 1] = __byte_perm(R[i][kWords - 1], hi[i], picks >> 16);
+            R[i][kWords - 2] = __byte_perm(R[i][kWords - 2], hi[i], picks_of[i]);
+            R[i][kWords - 1] = __byte_perm(R[i][kWords - 1], hi[i], picks_of[i] >> 16);
         }
     } else {
         auto picks = [](uint32_t seg, int w) {

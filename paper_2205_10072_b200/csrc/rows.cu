@@ -5,7 +5,7 @@
 //     back, all ranks of 1152 3.3, 65 553 ranks 3.2 (2.7 on the device).  The table holds what the
 //     CTA's segments need where these are few, and a CTA has no more warps than items.
 //   * quad_kernel, four ranks per lane (quad.cuh).  Up to some 2^21 ranks bound by instruction issue, the integer pipe with it, above by
-//     memory writes.  All ranks of 100 003 2.4 us, of 1.06 million 10.2, 2^24 ranks of q = 28 132, 2^25 receive rows 134 (7.0 TB/s).  With vectors
+//     memory writes.  All ranks of 100 003 2.4 us, of 1.06 million 9.9, 2^24 ranks of q = 28 132, 2^25 receive rows 134 (7.0 TB/s).  With vectors
 //     of 16 output bytes per lane in its place, some 40 warp instructions for every 32 of them where a segment ends: 4.9, 13.6, 146 and 149.
 // Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
 #include "batch.cuh"     // (in this unit, too: the constants of rows.cuh are in the module once)
