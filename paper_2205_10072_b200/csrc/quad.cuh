@@ -11,7 +11,7 @@
 //     of column k from skips[k] further on are the entries of a lane's four ranks.  Transposed back they are their rows.  Long ranges look
 //     them up in a table of send rows (kTable).
 //
-// Some 730 warp instructions for both rows of 128 ranks of q = 21 (1000 with 128 ranks a pass and the exceptions segment after segment; 1230 by vectors of
+// Some 700 warp instructions for both rows of 128 ranks of q = 21 (1000 with 128 ranks a pass and the exceptions segment after segment; 1230 by vectors of
 // 16 output bytes), of which the integer pipe takes half at half rate: that and the issue slots bound the kernel until memory does.  The exceptions take
 // 85, the transpositions and the ranks behind 120, the packing and staging of rows 150, a bulk copy some 20.
 #pragma once
