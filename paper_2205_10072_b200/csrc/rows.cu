@@ -151,15 +151,17 @@ quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
             quad_run<Q, kTable, true>(t, sm + at.table, mine, at, rc.s, rc.odd, rc.inv, x0, n, 0u, 0u, recv ? recv + byte : nullptr, send ? send + byte : nullptr);
         }
         if (once) break;
-        if (!barrier_wait(&answered, parity)) {
+        const bool came = barrier_wait(&answered, parity);
+        uint32_t next = 0;
+        const bool more = came && work_given(&answer, &next);
+        fence_before_bulk();                                     // (the answer is written by the asynchronous proxy: it has been read)
+        if (!__syncthreads_and(came)) {                          // (all threads go on, or none)
             if (threadIdx.x == 0) atomicAdd(&expired_waits, 1ull);       // (bcs_wait_expired)
             break;
         }
-        parity ^= 1u;
-        const bool more = work_given(&answer, &turn);
         if (!more) break;
-        fence_before_bulk();                                     // (the answer is written by the asynchronous proxy: it has been read)
-        __syncthreads();
+        turn = next;
+        parity ^= 1u;
     }
     stage_free();
 }
