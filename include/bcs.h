@@ -25,6 +25,10 @@
  *     was enqueued and no output byte was written.  BCS_ERR_CUDA means that the runtime
  *     refused a launch or a copy in the middle of a call: kernels enqueued before that point
  *     still run, and the outputs of that call are to be discarded.
+ *   - One thing is found out behind the return code: long ranges (bcs_build and the calls like it, some two
+ *     million ranks and more) are cut into turns that the hardware hands out, and a turn whose answer never comes
+ *     (after two seconds of polling, where a microsecond is usual) is not written.  It has not been observed;
+ *     bcs_wait_expired tells.
  *   - Supported: 1 <= p <= 2^31 - 1 (block sets are 32-bit masks).  p == 1 has
  *     q == 0: every call succeeds and writes nothing.
  *   - An entry that the construction could not determine (Algorithm 4 finding no
@@ -272,7 +276,8 @@ bcs_status bcs_simulate(uint32_t p, uint32_t n, const int8_t *recv, const int8_t
 
 /* Waits for all work of the current device (cudaDeviceSynchronize) and stores in *count_host (host) how
  * many waits of the library's kernels on it ran out since the process began (tables of ranges that are
- * handed out turn by turn: a turn that was asked for, but not answered in two seconds).  Other than 0: rows are missing. */
+ * handed out turn by turn: a turn that was asked for, but not answered within two seconds of polling; time in which
+ * the context was not running does not count).  Other than 0: rows are missing. */
 bcs_status bcs_wait_expired(uint64_t *count_host);
 
 /* Position-weighted 64-bit checksum of a stretch of schedule entries, additive

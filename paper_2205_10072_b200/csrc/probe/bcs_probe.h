@@ -1,7 +1,8 @@
 /*
  * bcs_probe.h -- measurement helper of the benchmark, not part of the schedule construction
  * (the paper has no counterpart): the integer instruction rate of the GPU, which is the
- * denominator of the roofline of the schedule kernels.
+ * denominator of the roofline of the schedule kernels; and, for the tests, the turns that CTAs of
+ * long calls take from one another.
  */
 #ifndef BCS_PROBE_H_
 #define BCS_PROBE_H_
@@ -27,6 +28,14 @@ extern "C" {
  * value depending on all results (so that nothing can be optimised away), may not be NULL. */
 bcs_status bcs_probe_int_rate(int mix, uint32_t iters, uint32_t *sink_dev, double *ops_out,
                               float *ms_out, void *cuda_stream);
+
+/* A grid of `ctas` CTAs of 96 threads that take one another's turns as the row kernels do; each thread adds 1 to
+ * taken_dev[turn] (device, `ctas` words) for every turn that its CTA has. */
+bcs_status bcs_probe_turns(uint32_t ctas, uint32_t *taken_dev, void *cuda_stream);
+
+/* One CTA that waits for an answer without having asked, limit_ns (at most a second) long.  results_dev (device, 96
+ * words): 1 for each thread that was told that the wait has run out, 2 for others. */
+bcs_status bcs_probe_unanswered(uint64_t limit_ns, uint32_t *results_dev, void *cuda_stream);
 
 #ifdef __cplusplus
 }

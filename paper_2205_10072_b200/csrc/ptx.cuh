@@ -75,21 +75,44 @@ __device__ __forceinline__ void ask_for_work(uint4 *answer, uint64_t *bar)
                  :: "r"((uint32_t)__cvta_generic_to_shared(answer)), "r"(b) : "memory");
 }
 
-// Waits for the phase of the given parity, two seconds at most; false: it has not come.
-__device__ __forceinline__ bool barrier_wait(uint64_t *bar, uint32_t parity)
+// Polls came() until it is true or until the time spent waiting, by clock() in nanoseconds, reaches `limit`.  What passes between two looks at the clock
+// counts as a millisecond at most, and the last thing before giving up is a poll: a context that was switched out for seconds (a debugger, a suspended
+// process) finds what has come meanwhile, and goes on waiting for what has not.
+template <class Came, class Clock>
+__host__ __device__ __forceinline__ bool wait_with_limit(Came came, Clock clock, uint64_t limit)
 {
-    const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
-    uint64_t begin = 0, now = 0;
-    for (;;) {
+    constexpr uint64_t most = 1000000;
+    uint64_t waited = 0, last = 0;
+    for (bool timed = false; !came(); timed = true) {
+        if (waited >= limit) return false;
+        const uint64_t now = clock(), passed = timed ? now - last : 0;
+        waited += passed < most ? passed : most;
+        last = now;
+    }
+    return true;
+}
+
+struct NanosecondClock {
+    __device__ __forceinline__ uint64_t operator()() const
+    {
+        uint64_t now;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now) :: "memory");
+        return now;
+    }
+};
+
+// Whether the phase of the given parity has come (a poll: it may suspend the thread for a while).
+struct PhaseCame {
+    uint32_t bar, parity;
+    __device__ __forceinline__ PhaseCame(uint64_t *at, uint32_t of) : bar((uint32_t)__cvta_generic_to_shared(at)), parity(of) {}
+    __device__ __forceinline__ bool operator()() const
+    {
         uint32_t done;
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(b), "r"(parity) : "memory");
-        if (done) return true;
-        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now) :: "memory");
-        if (begin == 0) begin = now;
-        if (now - begin > 2000000000ull) return false;
+                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        return done != 0u;
     }
-}
+};
 
 // Whether an answer names a CTA, and which.
 __device__ __forceinline__ bool work_given(const uint4 *answer, uint32_t *cta)
@@ -102,6 +125,33 @@ __device__ __forceinline__ bool work_given(const uint4 *answer, uint32_t *cta)
                  : "=r"(given), "=r"(x) : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w) : "memory");
     *cta = x;
     return given != 0u;
+}
+
+// What a CTA learns from the answer to ask_for_work().
+enum class Work { given, none, expired };
+
+// For some thread of the CTA the time was up: whether the phase has come for any of them by now.  (Out of line: the kernels have few registers left.)
+static __device__ __noinline__ bool came_for_any(uint64_t *bar, uint32_t parity, bool came)
+{
+    if (!came) came = PhaseCame(bar, parity)();
+    return __syncthreads_or(came);
+}
+
+// Waits for the answer, `limit` nanoseconds at most; by all threads of the CTA, behind a barrier behind which nobody else reads an answer.  Ends with a barrier:
+// the next one may be asked for.  All threads return the same.
+__device__ __forceinline__ Work await_work(uint4 *answer, uint64_t *bar, uint32_t parity, uint64_t limit, uint32_t *cta)
+{
+    bool came = wait_with_limit(PhaseCame(bar, parity), NanosecondClock(), limit);
+    bool given = came && work_given(answer, cta);
+    fence_before_bulk();                                         // (the answer is written by the asynchronous proxy: it has been read)
+    if (!__syncthreads_and(came)) {
+        // If it has come for any, the answer is there for all; a turn that it names is nobody else's.
+        if (!came_for_any(bar, parity, came)) return Work::expired;
+        given = work_given(answer, cta);
+        fence_before_bulk();
+        __syncthreads();
+    }
+    return given ? Work::given : Work::none;
 }
 
 }  // namespace bcs

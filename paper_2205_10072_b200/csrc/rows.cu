@@ -110,6 +110,7 @@ bcs_status launch_wide_send(const RowConsts &rc, uint32_t first, uint32_t count,
 constexpr unsigned kQuadThreads = 320;
 
 __device__ unsigned long long expired_waits;      // waits with a limit that ran out
+constexpr uint64_t kWaitLimit = 2000000000;       // two seconds (an answer takes a microsecond)
 
 // Two CTAs per SM.  A turn of a CTA is a run per warp.  once: a CTA for each turn, all of them run at once.  Otherwise the CTAs that run take the turns of
 // those that have not started yet: SMs do not write equally fast (a fill by CTAs of equal shares reaches 6.3 TB/s, by CTAs of 16 KB in
@@ -151,16 +152,9 @@ quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
             quad_run<Q, kTable, true>(t, sm + at.table, mine, at, rc.s, rc.odd, rc.inv, x0, n, 0u, 0u, recv ? recv + byte : nullptr, send ? send + byte : nullptr);
         }
         if (once) break;
-        const bool came = barrier_wait(&answered, parity);
-        uint32_t next = 0;
-        const bool more = came && work_given(&answer, &next);
-        fence_before_bulk();                                     // (the answer is written by the asynchronous proxy: it has been read)
-        if (!__syncthreads_and(came)) {                          // (all threads go on, or none)
-            if (threadIdx.x == 0) atomicAdd(&expired_waits, 1ull);       // (bcs_wait_expired)
-            break;
-        }
-        if (!more) break;
-        turn = next;
+        const Work more = await_work(&answer, &answered, parity, kWaitLimit, &turn);
+        if (more == Work::expired && threadIdx.x == 0) atomicAdd(&expired_waits, 1ull);          // (bcs_wait_expired)
+        if (more != Work::given) break;
         parity ^= 1u;
     }
     stage_free();

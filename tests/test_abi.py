@@ -191,6 +191,70 @@ def test_calls_with_tensors_are_those_with_numbers(lib):
         lib.bcs_build(10, 0, 10, good, good, stream=3)
 
 
+WAITS = r"""
+#include <stdint.h>
+#include <stdio.h>
+#include "ptx.cuh"
+// A clock and an event on a time line: polls take `poll` each, between poll number `away` and the look at the clock behind it the context is away for `gone`.
+struct Line {
+    uint64_t now = 5000000000ull, comes, poll, gone;
+    int polls = 0, away;
+};
+struct Came {
+    Line *line;
+    bool operator()() const
+    {
+        const bool there = line->now >= line->comes;
+        line->now += line->poll;
+        if (++line->polls == line->away) line->now += line->gone;
+        return there;
+    }
+};
+struct Clock {
+    Line *line;
+    uint64_t operator()() const { return line->now; }
+};
+int main()
+{
+    unsigned long long comes, poll, gone, limit;
+    int away;
+    while (scanf("%llu %llu %d %llu %llu", &comes, &poll, &away, &gone, &limit) == 5) {
+        Line line;
+        const uint64_t begin = line.now;
+        line.comes = begin + comes, line.poll = poll, line.away = away, line.gone = gone;
+        const bool came = bcs::wait_with_limit(Came{&line}, Clock{&line}, limit);
+        printf("%d %llu %d\n", (int)came, (unsigned long long)(line.now - begin), line.polls);
+    }
+}
+"""
+
+
+def test_a_wait_does_not_give_up_on_what_has_come(tmp_path):
+    """The wait of the row kernels for an answer, on a time line (no GPU): time in which the context is away is not time spent waiting, what has come meanwhile
+    is found, and what never comes ends the wait within its limit and a few polls."""
+    import subprocess
+    from paper_2205_10072_b200 import build_ext
+    source = tmp_path / "waits.cu"
+    source.write_text(WAITS)
+    flags = [f for f in build_ext.NVCC_FLAGS if f != "--shared"]
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + flags +
+                          ["-I", os.path.join(os.path.dirname(build_ext.LIB_PATH), "csrc"), "-o", str(tmp_path / "waits"), str(source)])
+    s, never = 10**9, 10**15
+    cases = [(0, 100, 0, 0, 2 * s), (800, 100, 0, 0, 2 * s),             # there, or soon
+             (800, 100, 1, 3 * s, 2 * s), (800, 100, 3, 3 * s, 2 * s),   # comes while the context is away, for longer than the limit
+             (s, 1000, 5, 100 * s, 2 * s),
+             (100 * s + 500000, 1000, 5, 100 * s, 2 * s),                # comes a while after it is back
+             (never, 1000, 0, 0, s // 1000), (never, 5 * 10**6, 0, 0, s // 10), (never, 1000, 7, 50 * s, s // 1000)]
+    out = subprocess.run([str(tmp_path / "waits")], input="".join("%d %d %d %d %d\n" % c for c in cases), text=True, check=True, capture_output=True)
+    got = [tuple(map(int, line.split())) for line in out.stdout.splitlines()]
+    assert [came for came, _, _ in got] == [1] * 6 + [0] * 3
+    assert all(polls <= 2 for _, _, polls in got[:1])
+    for (_, poll, _, gone, limit), (_, took, polls) in list(zip(cases, got))[6:]:
+        counted = min(poll, 10**6)                                       # what a poll counts as
+        assert limit <= polls * counted + (10**6 if gone else 0)
+        assert polls <= limit // counted + 3 and took <= polls * poll + gone
+
+
 FAKE_RUNTIME = r"""
 #include <cuda_runtime.h>
 #include <stdio.h>

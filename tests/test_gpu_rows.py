@@ -332,3 +332,32 @@ def test_tables_are_not_written_before_they_are_read(bcs, reader, n, between):
         torch.cuda.synchronize()
         assert torch.equal(out, want)
         assert all(torch.equal(m[at:at + written], r) for m, r in zip(memory, rows))
+
+
+def _probe():
+    import ctypes
+    from paper_2205_10072_b200 import build_ext
+    probe = ctypes.CDLL(build_ext.build_probe())
+    probe.bcs_probe_turns.argtypes = [ctypes.c_uint32, ctypes.c_void_p, ctypes.c_void_p]
+    probe.bcs_probe_unanswered.argtypes = [ctypes.c_uint64, ctypes.c_void_p, ctypes.c_void_p]
+    return probe
+
+
+# Turns that CTAs take from one another: each is taken once, by all threads of one CTA, whether all CTAs run at once or some thousand wait.
+@pytest.mark.parametrize("ctas", [1, 2, 148, 3000, 100003])
+def test_turns_are_taken_once(bcs, ctas):
+    taken = torch.zeros(ctas, dtype=torch.int32, device="cuda")
+    assert _probe().bcs_probe_turns(ctas, taken.data_ptr(), torch.cuda.current_stream().cuda_stream or None) == 0
+    torch.cuda.synchronize()
+    assert bool((taken == 96).all())
+
+
+# An answer that never comes (none was asked for): all threads of the CTA are told so, not before the limit, and the context goes on.
+def test_a_wait_that_runs_out_ends(bcs):
+    results = torch.zeros(96, dtype=torch.int32, device="cuda")
+    begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    begin.record()
+    assert _probe().bcs_probe_unanswered(3000000, results.data_ptr(), torch.cuda.current_stream().cuda_stream or None) == 0
+    end.record()
+    torch.cuda.synchronize()
+    assert bool((results == 1).all()) and 3.0 <= begin.elapsed_time(end) < 1000.0
