@@ -12,7 +12,11 @@ namespace {
 // By the number of records, us with 512 records and 256 threads / 512, 128 / 1024, 128: 1.0 million (p = 40 000, n = 10) 7.6/8.0/12.3, 0.9 million (3000, 300)
 // 4.2/4.3/6.1; 1.9 million (30 000, 50) 8.5/7.3/8.7, 2.0 million (1000, 2000) 7.2/6.3/6.8; 5.4 million (200 000, 10) 32.5/27.8/27.6, 11.6 million
 // (100 003, 100) 40.6/32.2/28.0.
-constexpr uint32_t kExpandRecords = 1024, kExpandFewer = 512;
+// More than one CTA per SM, but fewer than run at once (eight per SM of 256 threads): as few records each as let them, a record or two per thread.
+// us with 512 / 256 or 384: 0.19 million (6000, 20) 4.0/2.4, 0.15 million (300, 500) 2.6/2.1, 0.32 million (20 000, 2) 5.7/4.6, 0.33 million (3000, 100) 3.2/2.7,
+// 0.36 million (1152, 300) 2.9/2.6, 0.40 million (12 000, 20) 4.3/3.5; but rows of more than 512 rounds, 0.30 million (300, 1000) 2.3/2.7, (100, 3000) 2.3/2.6.
+constexpr uint32_t kExpandRecords = 1024, kExpandFewer = 512, kExpandStep = 128, kExpandFewest = 256;
+constexpr uint32_t kExpandSms = 148, kExpandAtOnce = 148 * 8;
 constexpr uint64_t kExpandMany = 4000000, kExpandFew = 1200000;
 constexpr int kExpandThreads = 128, kExpandThreadsFew = 256;
 constexpr uint32_t kExpandBuilt = 8192;        // where the CTA builds the rows of its ranks, whole ranks then
@@ -46,9 +50,8 @@ expand_kernel(const __grid_constant__ PTable tab, const __grid_constant__ Walk w
     // Algorithm 6 adds q to an entry after each use and starts entries k < x at +q because
     // their first use is in the second phase; both are covered by adding q * floor(i / q).
     grid_launch_dependents();
-    extern __shared__ int4 base[];             // (kBuildRows) the skips, then [ranks][q]
-    uint32_t *skips_sh = reinterpret_cast<uint32_t *>(base);
-    int4 *entries = base + (kBuildRows ? kRow / 4 : 0);
+    extern __shared__ int4 entries[];          // [ranks][q], then (kBuildRows) the skips: in front of the entries all took 4 % longer
+    uint32_t *skips_sh = reinterpret_cast<uint32_t *>(entries + (kBuildRows ? (size_t)(records / walk.rounds) * tab.q : 0));
     if (kBuildRows) {
         if (threadIdx.x < kRow) skips_sh[threadIdx.x] = tab.s[threadIdx.x];
         __syncthreads();
@@ -178,6 +181,10 @@ bcs_status bcs_expand(uint32_t p, uint32_t n, uint64_t r_begin, uint64_t r_end,
     const uint64_t total = count * rounds;
     const bool few = recv == nullptr || total < kExpandFew;
     uint32_t records = total < kExpandMany ? kExpandFewer : kExpandRecords;
+    if (rounds <= kExpandFewer && total > kExpandFewer * kExpandSms) {
+        for (uint32_t r = kExpandFewest; r < kExpandFewer && records == kExpandFewer; r += kExpandStep)
+            if (total <= (uint64_t)r * kExpandAtOnce) records = r;
+    }
     uint64_t ranks = (records + rounds - 2u) / rounds + 1u;          // that a CTA's records can belong to
     uint32_t extra = 0;
     if (recv == nullptr) {                                           // no tables: whole ranks, as far as their entries fit in shared memory
