@@ -17,7 +17,10 @@ constexpr uint32_t kAgFewest = 4;               // while all CTAs run at once li
 constexpr uint32_t kAgFitBoth = 148 * 6;
 constexpr uint32_t kAgFitOne = 148 * 7;
 constexpr uint32_t kAgOneTurn = 1000;           // CTAs that a call aims for while they have fewer than
-constexpr uint32_t kAgRounds = 32, kAgRoundsEven = 48;             // (with one table: 64, 96; even q: the copy takes longer)
+constexpr uint32_t kAgMany = 1350;              // CTAs that are more than those that run at once,
+constexpr uint32_t kAgMost = 1000;              // and that nearly fill the card: where the longer ones of the following leave so many
+constexpr uint32_t kAgRounds = 32, kAgRoundsEven = 48;                         // both tables (even q: the copy takes longer)
+constexpr uint32_t kAgRoundsOne = 48, kAgRoundsTwice = 96, kAgRoundsLong = 128;         // one table (the last: twice as many)
 
 // A CTA's copy of a schedule table: rows of consecutive ranks as they lie there, that of rank number i (from the lowest of the CTA's on, going on at 0 behind
 // p - 1) from byte at(i) on.  A thread reads one byte of each of four rows, its neighbours of the next four: the lanes are an odd number of words apart
@@ -134,9 +137,10 @@ struct QuadStream {
 };
 
 // x: rounds before the first one; by_q: 2^32 / q, rounded up.
-// kMany: eight CTAs per SM, in 32 registers a thread, instead of six.
+// kMany: with both tables eight CTAs per SM, in 32 registers a thread, instead of six; with one table (six are as fast) two rows at a time, which pays
+// for long calls (even q, which has the more instructions: p = 150 000, n = 768 73.8 -> 72.2 us, 9000, 12 000 70.8 -> 69.3).  q >= 4.
 template <bool kPack, bool kUnpack, bool kPad, bool kMany>
-__global__ void __launch_bounds__(kAgThreads, kMany ? 8 : 6)
+__global__ void __launch_bounds__(kAgThreads, kMany && kPack && kUnpack ? 8 : 6)
 allgather_kernel(uint32_t p, uint32_t q, uint32_t by_q, uint32_t n, uint32_t x, uint32_t r, uint32_t rounds_per_cta, const int8_t *__restrict__ recv,
                  const int8_t *__restrict__ send, int32_t *__restrict__ pack_out, int32_t *__restrict__ unpack_out)
 {
@@ -169,6 +173,7 @@ allgather_kernel(uint32_t p, uint32_t q, uint32_t by_q, uint32_t n, uint32_t x, 
     uint32_t k = i0 - phase * q;
     int add = (int)(phase * q) - (int)x;                           // q * floor(i / q) - x
     __syncthreads();
+#pragma unroll(kMany && !(kPack && kUnpack) ? 2 : 1)
     for (; jr < jr1; jr += 4) {
         // entries are in [-q, q-1]: only rows of the first two and of the last phases can
         // leave 0..n-1 (the same test for all threads of a warp)
@@ -176,10 +181,29 @@ allgather_kernel(uint32_t p, uint32_t q, uint32_t by_q, uint32_t n, uint32_t x, 
         if (kPack) ps.store(slot, k, add, clamp, last, p, avail, top, head, edge);
         if (kUnpack) us.store(slot, k, add, clamp, last, p, avail, top, head, edge);
         k += 4u;
-        while (k >= q) {
+        while (k >= q) {                                           // (once at most; written as an `if` both tables took 5 to 7 % longer)
             k -= q;
             add += (int)q;
         }
+    }
+}
+
+// Up to eight buffers (q < 4): a row per thread.  (By the kernel above, five buffers and 50 000 rounds took 14.2 us.)
+__global__ void __launch_bounds__(kAgThreads)
+allgather_few_kernel(uint32_t p, uint32_t q, uint32_t n, uint32_t x, uint32_t r, const int8_t *__restrict__ recv, const int8_t *__restrict__ send,
+                     int32_t *__restrict__ pack_out, int32_t *__restrict__ unpack_out)
+{
+    grid_launch_dependents();
+    const uint32_t rounds = n - 1u + q, jr = blockIdx.x * kAgThreads + threadIdx.x;
+    grid_dependency_wait();                                        // (the rows may be the work of the kernel before this one)
+    if (jr >= rounds) return;
+    const uint32_t phase = (jr + x) / q, k = jr + x - phase * q;
+    const int add = (int)(phase * q) - (int)x;
+    for (uint32_t j = 0; j < p; ++j) {
+        const uint32_t entry = (r >= j ? r - j : r + p - j) * q + k;
+        const uint64_t at = (uint64_t)jr * p + j;
+        if (pack_out != nullptr) pack_out[at] = clamp_block((int)send[entry] + add, (int)n - 1);
+        if (unpack_out != nullptr) unpack_out[at] = clamp_block((int)recv[entry] + add, (int)n - 1);
     }
 }
 
@@ -187,7 +211,7 @@ template <bool kPack, bool kUnpack, bool kPad, bool kMany>
 void launch_tables(dim3 grid, uint32_t p, uint32_t q, uint32_t n, uint32_t r, uint32_t per_cta, const int8_t *recv, const int8_t *send, int32_t *pack_out,
                    int32_t *unpack_out, cudaStream_t stream)
 {
-    const uint32_t by_q = q > 1u ? 0xffffffffu / q + 1u : 0u, x = (q - (n - 1u + q) % q) % q;        // (q = 1 is odd: not used)
+    const uint32_t by_q = 0xffffffffu / q + 1u, x = (q - (n - 1u + q) % q) % q;
     const size_t shared = (size_t)staged_bytes(q) * ((kPack ? 1u : 0u) + (kUnpack ? 1u : 0u));
     launch_dependent(true, allgather_kernel<kPack, kUnpack, kPad, kMany>, grid, kAgThreads, shared, stream, p, q, by_q, n, x, r, per_cta, recv, send, pack_out,
                      unpack_out);
@@ -224,24 +248,36 @@ bcs_status bcs_allgather_tables(uint32_t p, uint32_t n, uint32_t r, const int8_t
         !aligned16(recv) || !aligned16(send))
         return BCS_ERR_ALIGN;
     // Four rounds per CTA while all of them run at once; then some thousand CTAs; from 30 000 pairs of 256 buffers and a round on (both tables) CTAs of 32
-    // or 48 rounds, eight per SM.  us, six per SM and about 1000 CTAs / eight per SM and 32 rounds / 48 rounds (before, with the rows copied and
+    // or 48 rounds, eight per SM.  us, six per SM and about 1000 CTAs / eight per SM and 32 rounds / 48 rounds (with the rows copied and
     // transposed: some 80 rounds): p = 20 262, n = 116 (10 000 pairs) 7.6/8.3/8.3 (13.0), 20 000, 300 (25 000) 11.6/12.8/12.7 (16.6), 3000, 3000 (36 000)
     // 18.4/15.7/18.4 (24.7), 5000, 5000 (100 000) 35.8/32.3/34.3 (42.2), 100 003, 1000 (397 000) 120/114.8/119 (130); even q: 50 000, 300 (62 000)
-    // 23.3/22.0/21.3 (28.8), 150 000, 400 (244 000) 79.9/79.5/74.3 (82.2).  One table of 100 003, 1000: 68.3 with 32 rounds, 64.9 with 48, 63.5 with
-    // 64 (63.6).
+    // 23.3/22.0/21.3 (28.8), 150 000, 400 (244 000) 79.9/79.5/74.3 (82.2); but where 48 rounds leave less than kAgMost CTAs, 9000, 1000
+    // (792) -/15.0/20.4 (24.7).  One table, six per SM, 48 / 96 / 128 rounds (the rows
+    // transposed): 12 000, 1500 (71 000 pairs) 14.3/16.1/20.6 (15.0), 9000, 3000 (108 000) 20.9/21.3/22.1 (22.1), 12 000, 3000 26.4/24.9/26.2 (25.6), 35 000, 1000
+    // 25.8/24.7/25.4 (27.1), 9000, 12 000 (432 000) 74.3/69.3/68.2 (66.7), 150 000, 768 79.7/72.2/71.0 (70.5), 262 144, 300 56.9/51.9/50.6 (52.3).
+    // Chunks are about equally long with one table, and with both where they all run at once: 150 000, 40, 57 rounds as 48 and 9 20.2, as 32 and 25 14.6 (18.9).
     const uint32_t rounds = n - 1u + (uint32_t)tab.q;
     const uint32_t col_blocks = (p + kAgThreads - 1) / kAgThreads;
     const uint32_t q = (uint32_t)tab.q, tables = pack_out && unpack_out ? 2u : 1u;
     const uint64_t pairs = (uint64_t)col_blocks * rounds;
     const bool many = pairs * tables >= 2u * 30000u;
     uint32_t per_cta = kAgFewest;
-    if (many) per_cta = (q % 2u ? kAgRounds : kAgRoundsEven) * (3u - tables);
-    else if ((uint64_t)col_blocks * ((rounds + kAgFewest - 1) / kAgFewest) > (tables == 2u ? kAgFitBoth : kAgFitOne))
+    if (many) {
+        auto leaves = [&](uint32_t per, uint32_t ctas) { return (uint64_t)col_blocks * ((rounds + per - 1) / per) >= ctas; };
+        if (tables == 2u) per_cta = q % 2u == 0u && leaves(kAgRoundsEven, kAgMost) ? kAgRoundsEven : kAgRounds;
+        else per_cta = leaves(kAgRoundsLong, 2u * kAgMany) ? kAgRoundsLong : (leaves(kAgRoundsTwice, kAgMany) ? kAgRoundsTwice : kAgRoundsOne);
+        const uint32_t chunks = (rounds + per_cta - 1) / per_cta;
+        if (tables == 1u || !leaves(per_cta, kAgMany)) per_cta = ((rounds + chunks - 1) / chunks + 3u) & ~3u;
+    } else if ((uint64_t)col_blocks * ((rounds + kAgFewest - 1) / kAgFewest) > (tables == 2u ? kAgFitBoth : kAgFitOne)) {
         per_cta = ((uint32_t)pairs / kAgOneTurn + 4u) & ~3u;
+    }
     while ((rounds + per_cta - 1) / per_cta > 65535u) per_cta *= 2u;         // (as many as a grid has in y)
     const dim3 grid(col_blocks, (rounds + per_cta - 1) / per_cta);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    if (pack_out && unpack_out)
+    if (q < 4u)
+        launch_dependent(true, allgather_few_kernel, (rounds + kAgThreads - 1) / kAgThreads, kAgThreads, 0, stream, p, q, n, (q - rounds % q) % q, r, recv, send,
+                         pack_out, unpack_out);
+    else if (pack_out && unpack_out)
         launch_allgather<true, true>(many, q, grid, p, q, n, r, per_cta, recv, send, pack_out, unpack_out, stream);
     else if (pack_out)
         launch_allgather<true, false>(many, q, grid, p, q, n, r, per_cta, recv, send, pack_out, unpack_out, stream);

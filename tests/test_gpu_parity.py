@@ -694,6 +694,21 @@ def test_allgather_rows_as_they_lie(bcs, p, n):
                 assert bool((raw[i] == -77).all()) if out is None else torch.equal(out, want[i]), (r, off, i)
 
 
+# up to eight buffers, and nine; chunks of 32 and 48 rounds (both tables, even q), of 48, 96 and 128 (one table) and what evening out makes of them
+@pytest.mark.parametrize("p,n", [(4, 700), (5, 255), (7, 256), (8, 1000), (9, 1000), (9001, 1000), (9001, 3000), (40001, 45), (40001, 401), (70001, 240)])
+def test_allgather_chunks(bcs, p, n):
+    test_allgather_rows_as_they_lie(bcs, p, n)
+
+
+# A quarter more rounds do not take 1.7 times as long: one table of 12 000 buffers, 1200 and 1500 blocks, whose rounds were cut into fewer CTAs than run at once.
+def test_more_rounds_do_not_leave_the_card_idle(bcs):
+    p = 12000
+    recv, send = (torch.from_numpy(t).cuda().view(-1) for t in oracle.full_table(p))
+    out = torch.empty((1500 - 1 + 14) * p, dtype=torch.int32, device="cuda")
+    fewer, more = (_us(lambda: bcs.bcs_allgather_tables(p, n, 7, recv, send, out, None), 100) for n in (1200, 1500))
+    assert more < 1.45 * fewer
+
+
 def test_allgather_tables_match_oracle(bcs):
     """Algorithm 9's pack / unpack block numbers: every entry against the oracle's literal loops
     for small p, the library's own tables simulated (all p processors) for tiny p, and the
