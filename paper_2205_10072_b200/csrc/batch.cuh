@@ -130,7 +130,7 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         if (threadIdx.x < 32u) load_p(p, t, job);
         __syncthreads();
         if (kQuad && q > kLow) build_row_table<true>(t, q, job.odd);
-        else build_row_table(t, q, job.odd);
+        else build_row_table<false, 1>(t, q, job.odd);
     };
     auto fits = [](uint32_t p) { return p > 1u && p <= kSmallP; };
     if (threadIdx.x == 0) guess = load_relaxed(ba.p_list + j);
@@ -149,6 +149,7 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         if (q == 8) quad_small<8>(t, sm, job, entry0, recv, send);
         else if (q == 9) quad_small<9>(t, sm, job, entry0, recv, send);
         else quad_small<10>(t, sm, job, entry0, recv, send);
+        stage_free<true>();
     } else {
         uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
         constexpr uint32_t warps = kThreads / 32;
@@ -157,8 +158,8 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         if (q <= 4) narrow_piece<1>(t, mine, job, entry0, q, 0u, p, item, recv, send);
         else if (q <= 8) narrow_piece<2>(t, mine, job, entry0, q, 0u, p, item, recv, send);
         else if constexpr (!kQuad) narrow_piece<3>(t, mine, job, entry0, q, 0u, p, item, recv, send);
+        stage_free<false>();
     }
-    stage_free();
 }
 
 // 1024 < p <= 2^21: the CTA's share is `share` (a multiple of 16) flattened ranks.
@@ -238,7 +239,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
         if (p != built) {
             built = 0u;
             if (p != 0u && r0 < r1) {
-                build_row_table(t, q, job.odd);
+                build_row_table<false, 1>(t, q, job.odd);
                 if (!narrow && send != nullptr) build_send_table_wide(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
                 built = p;
             }
@@ -253,7 +254,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
             uint8_t *mine = sm + at_narrow.warps + (threadIdx.x >> 5) * at_narrow.warp_bytes;
             if (q <= 12) narrow_piece<3>(t, mine, job, job.entry0, q, r0, r1, kItemRanks, recv, send);
             else narrow_piece<4>(t, mine, job, job.entry0, q, r0, r1, kItemRanks, recv, send);
-            stage_free();
+            stage_free<false>();
         } else {
             wide_piece(t, sm, at, sm + at.ends + (threadIdx.x >> 5) * 32u, job, q, r0, r1, recv, send);
         }
@@ -290,7 +291,7 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
         if (threadIdx.x < 32u) load_p(p, t, job);
         const uint64_t entry0 = ba.entry_off[j];
         __syncthreads();
-        build_row_table(t, q, job.odd);
+        build_row_table<false, 1>(t, q, job.odd);
         if (send != nullptr) build_send_table_wide(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
         const uint32_t warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
         auto all = [&](auto is_send, int8_t *out) {

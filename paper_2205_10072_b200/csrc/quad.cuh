@@ -547,7 +547,7 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
         QuadState states[kTurns];
         int2 keys[kTurns];
         Shifted<Q> shifted = {kAligned ? 0u : shift, {}};
-        stage_free();
+        stage_free<true>();
 #pragma unroll
         for (int j = 0; j < kTurns; ++j) {
             if (j != 0 && turns == 1u) break;
@@ -585,7 +585,7 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
             flush(recv);
         }
         if (send == nullptr) continue;
-        if (recv != nullptr) stage_free();
+        if (recv != nullptr) stage_free<true>();
         if (!kAligned) shifted = {shift, {}};
 #pragma unroll
         for (int j = 0; j < kTurns; ++j) {

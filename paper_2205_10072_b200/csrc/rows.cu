@@ -59,7 +59,7 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
         warp_rows<kWords, true>(t, mine, rc.q, rc.odd, rc.inv, rank(b), n, recv ? recv + byte : nullptr,
                                 send ? send + byte : nullptr);
     }
-    stage_free();
+    stage_free<true>();
 }
 
 // Send rows alone of 1.9 to 6 million ranks, 16 output bytes per lane (wide.cuh): a run per warp, one CTA per SM.  Its table of send rows holds those of all the
@@ -157,7 +157,7 @@ quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
         if (more != Work::given) break;
         parity ^= 1u;
     }
-    stage_free();
+    stage_free<true>();
 }
 
 // Turns and CTAs.  Runs are whole look-ups (128 ranks): partly filled ones cost as much.  The shortest run with which at most 296 CTAs of up to ten warps

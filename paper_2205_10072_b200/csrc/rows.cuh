@@ -124,7 +124,10 @@ __device__ __forceinline__ uint2 unpack_row(unsigned long long v, int q, int K)
 // (Two loads and some twenty instructions for two rows.  Computed by Algorithm 4 in every CTA it took 5000 cycles before the first row:
 // 65 553 ranks 4.2 -> 3.5 us, all ranks of 100 003 5.5 -> 4.8, of about 2^20 15.6 -> 13.6, every p up to 1024 in any order 18.3 -> 16.7, back
 // to back; a call alone 2 us less.)
-template <bool kPermuted = false>
+// kJobs: loads in flight per thread.  Their latency is most of the time of a table that a kernel begins with (four: all ranks of 100 003 2.6 -> 2.4 us); the kernels
+// for lists, which build one table beside the rows of another or spill, take longer with more than one (one p of 200 2.8 -> 3.0 us, of 2000 6.3 -> 6.6, receive rows
+// of 8 of 2^20 45.6 -> 48.6).
+template <bool kPermuted = false, int kJobs = 4>
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {
     auto place = [](uint32_t low) { return kPermuted ? permuted_row(low) : low; };
@@ -146,8 +149,6 @@ __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32
     const uint32_t six = t.s[6];
     const unsigned long long *shapes = row_shapes + (lows - 65u) * (52u * 64u), *sixes = row_six + (lows - 65u) * 64u;
     const int n = __popc(wanted) * 64;
-    // (the loads of up to four jobs at once: their latency is most of the time)
-    constexpr int kJobs = 4;
     for (int job0 = (int)threadIdx.x; job0 < n; job0 += kJobs * (int)blockDim.x) {
         unsigned long long v[kJobs], w[kJobs];
 #pragma unroll
@@ -291,6 +292,14 @@ __device__ __forceinline__ void join_row(uint32_t lo, uint32_t hi, const uint8_t
     }
 }
 
+// The lane that starts a warp's bulk copies and waits for them.  (An elected one is known to be one to the compiler, 32 ranks 1.73 -> 1.69 us; where rows begin at
+// any byte the same cost more than lane 0: one p of 200 2.8 -> 2.9 us.)
+template <bool kAligned>
+__device__ __forceinline__ bool copying_lane()
+{
+    return kAligned ? elect_one() : (threadIdx.x & 31u) == 0u;
+}
+
 // Sends the staged rows out: len bytes for `dst`, staged at the same offset in their 16-byte group.  All but
 // the ragged ends go as one bulk copy of the TMA unit.
 template <bool kAligned>
@@ -304,7 +313,7 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
     const uint32_t begin = (shift + 15u) & ~15u, end = shift + len;
     uint8_t *base = reinterpret_cast<uint8_t *>(dst) - shift;
     const uint32_t stop = end & ~15u;
-    if (elect_one() && stop > begin) bulk_store(base + begin, stage + begin, stop - begin);
+    if (copying_lane<kAligned>() && stop > begin) bulk_store(base + begin, stage + begin, stop - begin);
     if (!kAligned || (end & 15u) != 0u) {                        // bytes [shift, head) and [tail, end) one by one
         const uint32_t head = begin < end ? begin : end;
         if (shift + lane < head) base[shift + lane] = stage[shift + lane];
@@ -313,10 +322,11 @@ __device__ __forceinline__ void flush_item(uint8_t *stage, int8_t *dst, uint32_t
     }
 }
 
-// The staging buffer may be written again.
+// The staging buffer may be written again.  (kAligned: as for the copies.)
+template <bool kAligned>
 __device__ __forceinline__ void stage_free()
 {
-    if (elect_one()) bulk_stores_read();
+    if (copying_lane<kAligned>()) bulk_stores_read();
     __syncwarp();
 }
 
@@ -424,7 +434,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
         const uint32_t shift = kAligned ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(recv) & 15u);
         const RowPlace place(shift, q);
         uint8_t *at = stage + shift + lane * (uint32_t)q;
-        stage_free();
+        stage_free<kAligned>();
         for (uint32_t b = 0; b < n; b += 32u, at += 32 * q) {
             const uint2 row = looked[b + lane];
             const uint32_t note = notes[b + lane];
@@ -454,7 +464,7 @@ __device__ __forceinline__ void warp_rows(const RowTable &t, uint8_t *mine, int 
         const uint8_t *theirs[kLow];                             // entry k of the rank skips[k] further on
 #pragma unroll
         for (int k = 0; k < kLow; ++k) theirs[k] = mine_row + (k < L ? t.s[k] * 8u + k : 0u);
-        stage_free();
+        stage_free<kAligned>();
         for (uint32_t b = 0; b < n; b += 32u, at += 32 * q) {
             const uint32_t note = notes[b + lane];
             uint32_t e[kLow];
