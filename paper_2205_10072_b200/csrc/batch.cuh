@@ -92,12 +92,16 @@ __device__ __forceinline__ void wide_piece(const RowTable &t, const uint8_t *sm,
 }
 
 constexpr uint32_t kSmallRun = 256;               // ranks of a warp's run
+// With room for more segments than it can have, an eighth CTA of 128 threads did not fit an SM: 5000 p of 777 42.0 us and not 40.5, 1100 of 300..1024 12.3, 11.8.
+// (CTAs of 256 threads fit; one p of 500 3.48 us, with less room 3.56.)
+__host__ __device__ constexpr uint32_t small_segments(uint32_t threads) { return threads == 128u ? run_segments(kSmallRun) : roomy_segments(kSmallRun); }
 
 // All ranks of a p of 129..1024 by the warps of the CTA, four ranks per lane.  Runs begin where rows begin (nearly) on a 16-byte boundary.
-template <int Q>
+// kSegments: how many the warps have room for.
+template <int Q, uint32_t kSegments>
 __device__ __forceinline__ void quad_small(const RowTable &t, uint8_t *sm, const BatchJob &job, uint64_t entry0, int8_t *recv, int8_t *send)
 {
-    const QuadLayout<false> at(Q, kSmallRun);
+    const QuadLayout<false> at(Q, kSegments);
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     uint8_t *mine = sm + at.warps + warp * at.warp_bytes;
     const uint32_t best = quad_shift(entry0, Q), up = best & 15u, shift = best >> 4;
@@ -146,9 +150,10 @@ batch_small_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
     const RowLayout at(q);
     const RowTable t(sm, at);
     if (kQuad && q > kLow) {
-        if (q == 8) quad_small<8>(t, sm, job, entry0, recv, send);
-        else if (q == 9) quad_small<9>(t, sm, job, entry0, recv, send);
-        else quad_small<10>(t, sm, job, entry0, recv, send);
+        constexpr uint32_t segments = small_segments(kThreads);
+        if (q == 8) quad_small<8, segments>(t, sm, job, entry0, recv, send);
+        else if (q == 9) quad_small<9, segments>(t, sm, job, entry0, recv, send);
+        else quad_small<10, segments>(t, sm, job, entry0, recv, send);
         stage_free<true>();
     } else {
         uint8_t *mine = sm + at.warps + (threadIdx.x >> 5) * at.warp_bytes;
@@ -239,7 +244,7 @@ batch_middle_kernel(const __grid_constant__ BatchArgs ba, uint32_t share, int8_t
         if (p != built) {
             built = 0u;
             if (p != 0u && r0 < r1) {
-                build_row_table<false, 1>(t, q, job.odd);
+                build_row_table<false, 2>(t, q, job.odd);
                 if (!narrow && send != nullptr) build_send_table_wide(t, reinterpret_cast<uint2 *>(sm + at.send), q, job.odd);
                 built = p;
             }
@@ -315,10 +320,16 @@ batch_large_kernel(const __grid_constant__ BatchArgs ba, int8_t *recv, int8_t *s
 template <unsigned kThreads, int kCtas, bool kQuad>
 bcs_status launch_small(const BatchArgs &ba, bool alone, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
-    uint32_t shared = kQuad ? QuadLayout<false>(kSmallQ, kSmallRun).total(kThreads / 32) : RowLayout(kSmallQ).total(kThreads / 32);
+    constexpr uint32_t fits = 228u * 1024u / kCtas - 1024u - (uint32_t)sizeof(BatchJob) - 16u;       // (1 KB of each CTA is the system's)
+    uint32_t shared = RowLayout(kSmallQ).total(kThreads / 32);
+    if constexpr (kQuad) {
+        constexpr QuadLayout<false> at(kSmallQ, small_segments(kThreads));
+        static_assert(at.total(kThreads / 32) <= fits, "shared memory for kCtas CTAs per SM");
+        shared = at.total(kThreads / 32);
+    }
     const uint32_t per_sm = (ba.num_p + kSms - 1) / kSms;
     if (alone && per_sm < (uint32_t)kCtas) {
-        const uint32_t spread = (226u * 1024u / per_sm - 1280u) & ~127u;     // (1 KB of each CTA is the system's)
+        const uint32_t spread = (226u * 1024u / per_sm - 1280u) & ~127u;
         if (shared < spread) shared = spread;
     }
     if (!allow_shared<batch_small_kernel<kThreads, kCtas, kQuad>>()) return BCS_ERR_CUDA;

@@ -1,8 +1,8 @@
-// Larger tables of a p with q >= 17: four consecutive ranks per lane.
+// Larger tables of a p with q >= 17, and lists of p up to 1024 (q = 8..10): four consecutive ranks per lane.
 //
 // Four rows of q bytes are q words, so what a lane writes begins and ends on words, for every q: the four rows are joined in registers by
-// funnel shifts and byte permutations that are constants of q, without a word that two lanes share.  A warp makes the rows of 128
-// ranks (a pass) in shared memory and sends them out as one bulk copy of the TMA unit; the few exceptions (rows.cuh) are written as bytes
+// funnel shifts and byte permutations that are constants of q, without a word that two lanes share.  A warp makes the rows of 256
+// ranks (a pass: two look-ups of 128) in shared memory and sends them out as one bulk copy of the TMA unit; the few exceptions (rows.cuh) are written as bytes
 // in between.
 //
 //   * Receive rows: a lane looks its four table rows up and joins them with the entries of their segment.
@@ -60,25 +60,27 @@ __device__ __forceinline__ void build_send_table(const RowTable &t, uint2 *send,
 
 constexpr uint32_t kQuads = 128;                       // ranks that a warp looks up at a time, four a lane
 
-// A warp's segments lie in shared memory, all that `ranks` consecutive ones and those looked up behind them can touch, and one more (a
-// segment has 41 ranks or more).
-__host__ __device__ constexpr uint32_t run_segments(uint32_t ranks) { return (ranks + kQuads) / 41u + 4u; }
-constexpr uint32_t kMostRun = 896;                     // ranks of a run
-static_assert(run_segments(kMostRun) <= 29, "located by one warp, the first of them up to two behind the first lane's");
-
 constexpr int kTurns = 2;                              // look-ups of a pass: its rows are staged and sent out together
 constexpr uint32_t kPass = kTurns * kQuads;
+constexpr uint32_t kMostRun = 896;                     // ranks of a run
+
+// A warp's segments lie in shared memory: all that the look-ups of a run can touch, and one more.  Looked up are the ranks of whole passes (of a last one
+// that is half full, fewer) and 128 behind.  c segments in a row have more than 64 c - 25 ranks, so r ranks touch (r + 22) / 64 + 2 segments at most.
+__host__ __device__ constexpr uint32_t run_segments(uint32_t run) { return ((run + kPass - 1u) / kPass * kPass + kQuads + 22u) / 64u + 3u; }
+static_assert(run_segments(kMostRun) <= 30u, "located by one warp, the first of them up to two lanes behind the first");
+// Room for them in the kernel for one p, which takes 1 to 5 % longer with less (q = 30: 83 000 receive rows 1.98 us, with what they need 2.05).
+__host__ __device__ constexpr uint32_t roomy_segments(uint32_t run) { return ((run + kPass - 1u) / kPass * kPass + kQuads) / 41u + 4u; }
+static_assert(roomy_segments(kQuads) >= run_segments(kQuads) && roomy_segments(kMostRun) >= run_segments(kMostRun), "the steps between are larger, too");
 constexpr uint32_t kColumn = kPass + kHalo + 8u;       // bytes of a column
 
 // Byte offsets in the CTA's shared memory: the row table, with kTable that of send rows, and a warp's part (with columns otherwise).
 template <bool kTable>
 struct QuadLayout {
     RowLayout base;                                    // (its warps' part is not used)
-    uint32_t segments;                                 // of a run, whole passes of which are looked up
-    uint32_t table, warps, entries, columns, stage, warp_bytes;
-    __host__ __device__ QuadLayout(int q, uint32_t run) : base(q)
+    uint32_t segments;                                 // of a run
+    uint32_t table = 0, warps = 0, entries = 0, columns = 0, stage = 0, warp_bytes = 0;
+    __host__ __device__ constexpr QuadLayout(int q, uint32_t segments_of_run) : base(q), segments(segments_of_run)
     {
-        segments = run_segments((run + kPass - 1u) / kPass * kPass);
         table = base.warps;
         warps = table + (kTable ? 2u * (uint32_t)send_groups(q) * kLowRanks * 8u : 0u);
         entries = segments * 16u;
@@ -86,7 +88,7 @@ struct QuadLayout {
         stage = (columns + (kTable ? 0u : kLow * kColumn) + 15u) & ~15u;
         warp_bytes = stage + kPass * (uint32_t)q + 16u;      // (rows that are shifted end in the last 16 bytes)
     }
-    __host__ __device__ uint32_t total(uint32_t n_warps) const { return warps + n_warps * warp_bytes; }
+    __host__ __device__ constexpr uint32_t total(uint32_t n_warps) const { return warps + n_warps * warp_bytes; }
 };
 
 // What the run's look-up knows of a segment.
@@ -471,7 +473,8 @@ __device__ __forceinline__ void quad_run(const RowTable &t, const uint8_t *send_
         // Segments of the 128 ranks from rank `from` on.
         auto find = [&](uint32_t from, QuadState &s, int2 &keys) {
             const uint32_t first = __popc(__ballot_sync(0xffffffffu, starts <= (int)from)) - 1u;
-            const int quad = (starts - (int)from + 3) >> 2;      // the first lane whose first rank is in that segment
+            // the first lane whose first rank is in that segment (unsigned: the sum may wrap, to something negative, where there is none)
+            const int quad = (int)((uint32_t)starts - from + 3u) >> 2;
             const uint32_t begin = __reduce_or_sync(0xffffffffu, quad > 0 && quad < 32 ? 1u << quad : 0u);
             s.slot = first + __popc(begin & ((2u << lane) - 1u));
             const Segment here = segments[s.slot], next = segments[s.slot + 1u];

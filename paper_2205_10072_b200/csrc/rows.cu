@@ -123,7 +123,7 @@ quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     __shared__ __align__(16) uint4 answer;
     grid_launch_dependents();
     __shared__ uint64_t answered;
-    const QuadLayout<kTable> at(Q, run);
+    const QuadLayout<kTable> at(Q, roomy_segments(run));
     const uint32_t warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const RowTable t(sm, at.base);
     if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
@@ -172,7 +172,7 @@ bcs_status launch_quad(const RowConsts &rc, uint32_t first, uint32_t count, int8
 {
     if (!allow_shared<quad_kernel<Q, kTable>>()) return BCS_ERR_CUDA;
     constexpr uint32_t half = (228u * 512u - 1024u - 128u) & ~127u, most = kQuadThreads / 32u;
-    auto bytes = [](uint32_t warps, uint32_t run) { return QuadLayout<kTable>(Q, run).total(warps); };
+    auto bytes = [](uint32_t warps, uint32_t run) { return QuadLayout<kTable>(Q, roomy_segments(run)).total(warps); };
     auto fit = [&](uint32_t run) {
         uint32_t w = most;
         while (w > 4u && bytes(w, run) > half) --w;

@@ -56,7 +56,7 @@ struct RowConsts {
     uint32_t inv;                  // floor(2^(q - L + 32) / p)
 };
 
-__host__ __device__ inline int low_levels(int q) { return q < kLow ? q : kLow; }
+__host__ __device__ constexpr int low_levels(int q) { return q < kLow ? q : kLow; }
 
 // Number of e_t set, a < t <= b.
 __device__ __forceinline__ uint32_t count_odd(uint32_t odd, int a, int b)
@@ -75,8 +75,8 @@ static_assert(kItemSegments * 8u <= 48u && kWarpStage % 16u == 0, "layout of a w
 
 // Byte offsets in the CTA's dynamic shared memory.
 struct RowLayout {
-    uint32_t miss, s, flags, warps, warp_bytes;
-    __host__ __device__ explicit RowLayout(int q)
+    uint32_t miss = 0, s = 0, flags = 0, warps = 0, warp_bytes = 0;
+    __host__ __device__ constexpr explicit RowLayout(int q)
     {
         const uint32_t rows = (uint32_t)(q - low_levels(q) + 1);
         miss = rows * kLowRanks * 8u;
@@ -86,7 +86,7 @@ struct RowLayout {
         warps = (warps + 127u) & ~127u;
         warp_bytes = kWarpStage + ((kItemRanks * (uint32_t)q + 31u) & ~15u);
     }
-    __host__ __device__ uint32_t total(uint32_t n_warps) const { return warps + n_warps * warp_bytes; }
+    __host__ __device__ constexpr uint32_t total(uint32_t n_warps) const { return warps + n_warps * warp_bytes; }
 };
 
 struct RowTable {
@@ -125,8 +125,8 @@ __device__ __forceinline__ uint2 unpack_row(unsigned long long v, int q, int K)
 // 65 553 ranks 4.2 -> 3.5 us, all ranks of 100 003 5.5 -> 4.8, of about 2^20 15.6 -> 13.6, every p up to 1024 in any order 18.3 -> 16.7, back
 // to back; a call alone 2 us less.)
 // kJobs: loads in flight per thread.  Their latency is most of the time of a table that a kernel begins with (four: all ranks of 100 003 2.6 -> 2.4 us); the kernels
-// for lists, which build one table beside the rows of another or spill, take longer with more than one (one p of 200 2.8 -> 3.0 us, of 2000 6.3 -> 6.6, receive rows
-// of 8 of 2^20 45.6 -> 48.6).
+// for lists, which build one table beside the rows of another or spill, take longer with so many (one p of 200 2.8 -> 3.0 us with four and not one, of 2000 6.45 -> 6.7 with
+// four and not two, receive rows of 8 of 2^20 45.6 -> 48.4; 40 of 2^10..2^20 with one, two, four 68.6, 67.1, 67.3).
 template <bool kPermuted = false, int kJobs = 4>
 __device__ __forceinline__ void build_row_table(const RowTable &t, int q, uint32_t odd)
 {

@@ -51,6 +51,29 @@ def test_bounds_of_the_layout():
         assert np.all(low < length) and np.all(length >= 41), p
 
 
+def test_segments_that_a_run_touches():
+    """r consecutive ranks, also those that go on at 0 behind p - 1, touch (r + 22) / 64 + 2 segments at most: what the warps' shared memory is laid out for."""
+    rng = np.random.default_rng(9)
+    most = {}
+    for p in [129, 130, 255, 256, 257, 511, 513, 1023, 1024, (1 << 16) + 1, (1 << 17) - 1, (1 << 20) + 1, 65 << 9] + [int(2 ** e) for e in rng.uniform(7.1, 20, 120)]:
+        form = Form(p)
+        x = np.arange(p)
+        starts = x[form.locate(x)[1] == 0]
+        starts = np.concatenate([starts + turn * p for turn in range(20 if p < 1100 else 2)])
+        for r in (128, 192, 384, 512, 640, 1024):
+            begin = starts[1:len(starts) // 2] - 1                   # (the last rank of a segment: as many as can be)
+            touched = np.searchsorted(starts, begin + r) - np.arange(len(begin))
+            most[r] = max(most.get(r, 0), int(touched.max()))
+    for p in [(1 << 31) - 1, (1 << 30) + 1, (1 << 25) - 1] + [int(2 ** e) for e in rng.uniform(20, 31, 60)]:
+        form = Form(p)
+        for head in form.s[8:form.q + 1]:
+            for r in (384, 1024):
+                x = (np.arange(int(head) - r, int(head) + r)) % p
+                new = np.concatenate([[0], np.cumsum(form.locate(x)[1][1:] == 0)])
+                most[r] = max(most[r], int((new[r - 1:] - new[:len(new) - r + 1]).max()) + 1)
+    assert all(n <= (r + 22) // 64 + 2 for r, n in most.items()), most
+
+
 def test_rows_wanted_for_a_stretch():
     """The kernels that build table rows for a stretch of ranks only name all that these need: the segments' own lowest bits, those of
     the segments behind them, and where the send exceptions carry to."""
