@@ -59,6 +59,15 @@ __device__ __forceinline__ bool elect_one()
 // The copies that this thread has started have read their shared memory.
 __device__ __forceinline__ void bulk_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
+// Bytes of a (0..3) and b (4..7) by the nibbles of kPick, one for each byte of the result; with 8 added the sign of that byte eight times.
+template <uint32_t kPick>
+__device__ __forceinline__ uint32_t sign_bytes(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "n"(kPick));
+    return r;
+}
+
 // ---------------------------------------------------------------- work that CTAs take from one another
 // A CTA that asks for the work of one that has not started yet gets its index, and that one is not launched (cluster launch control).  The answer
 // (16 bytes) arrives in shared memory and completes a phase of the barrier.

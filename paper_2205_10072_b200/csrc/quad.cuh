@@ -371,6 +371,8 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
                                            Shifted<Q> &shifted)
 {
     constexpr int kWords = (Q + 3) / 4;
+    // The baseblock's bytes: of nearly all ranks in the last two words, of those below some 2^(q - 5) anywhere.  (Small q have no other words.)
+    constexpr bool kAnywhere = 4 * (kWords - 2) > kLow;
     uint32_t R[4][kWords], S[8];
     auto load = [&](uint32_t (&X)[8], const uint8_t *from) {
         const uint4 a = *reinterpret_cast<const uint4 *>(from);
@@ -394,6 +396,10 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
     };
     const uint8_t *from = entries + s.slot * 64u + (kSend ? 32u : 0u);
     uint32_t picks_of[4];
+    auto pick = [&](int i) {
+        R[i][kWords - 2] = __byte_perm(R[i][kWords - 2], hi[i], picks_of[i]);
+        R[i][kWords - 1] = __byte_perm(R[i][kWords - 1], hi[i], picks_of[i] >> 16);
+    };
     if constexpr (Q % 8 != 0) {
         // (loaded once more for each rank rather than selected, word by word, from those of two segments: the integer pipe has more to do than shared
         // memory, 1.06 million ranks of q = 21 10.1 -> 9.9 us; but q = 24, whose rows meet in banks, 12 million ranks 88.4 -> 91.4)
@@ -405,6 +411,7 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
             R[i][1] = (hi[i] & 0xffffffu) | S[1];
 #pragma unroll
             for (int w = 2; w < kWords; ++w) R[i][w] = S[w];
+            if constexpr (!kAnywhere) pick(i);                   // (here, or the kernel of eight CTAs per SM spills)
         }
     } else {
         uint32_t T[8];
@@ -420,27 +427,34 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
             R[i][1] = (hi[i] & 0xffffffu) | (mine ? S[1] : T[1]);
 #pragma unroll
             for (int w = 2; w < kWords; ++w) R[i][w] = mine ? S[w] : T[w];
+            if constexpr (!kAnywhere) pick(i);
         }
     }
-    // The baseblock's bytes: of nearly all ranks in the last two words, of those below some 2^(q - 5) anywhere.
-    if (!__any_sync(0xffffffffu, ((s.here | (s.room < 4 ? s.next : 0u)) >> 15) & 1u)) {
+    if constexpr (!kAnywhere) {
+    } else if (!__any_sync(0xffffffffu, ((s.here | (s.room < 4 ? s.next : 0u)) >> 15) & 1u)) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            R[i][kWords - 2] = __byte_perm(R[i][kWords - 2], hi[i], picks_of[i]);
-            R[i][kWords - 1] = __byte_perm(R[i][kWords - 1], hi[i], picks_of[i] >> 16);
-        }
+        for (int i = 0; i < 4; ++i) pick(i);
     } else {
-        auto picks = [](uint32_t seg, int w) {
-            const int home = (int)((seg >> 10) & 31u);
-            if (!kSend) return home >> 2 == w ? 0x3210u | 7u << (4 * (home & 3)) : 0x3210u;
-            const int from = (home ? home + 1 : kLow) - 4 * w;   // the first of the word's bytes
-            return from >= 4 ? 0x3210u : 0x3210u | 0x7777u << (from > 0 ? 4 * from : 0);
+        // They are the zero bytes of the entries (all others are negative): look at those of the last four words, and of the words before where a home round
+        // is among them (or none there, the root's segment).  Two instructions a word and rank; a selector for each word from the home rounds of both segments
+        // took five: a million ranks from 0 on, q = 27, 29, 31: 12.2, 12.8, 12.8 -> 10.8, 11.4, 11.0 us.
+        constexpr int kFirst = kWords > 5 ? kWords - 4 : 1;
+        auto fill = [&](int i, int w) {                          // (word 1: round L, the others are from the table)
+            const uint32_t others = w == 1 ? sign_bytes<0xb444>(R[i][w], 0xffffffffu) : sign_bytes<0xba98>(R[i][w], 0u);
+            R[i][w] |= __byte_perm(hi[i], 0u, 0x3333) & ~others;
         };
 #pragma unroll
-        for (int w = 1; w < kWords; ++w) {
-            const uint32_t here = picks(s.here, w), next = picks(s.next, w);
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) R[i][w] = __byte_perm(R[i][w], hi[i], i == 0 || i < s.room ? here : next);
+            for (int w = kFirst; w < kWords; ++w) fill(i, w);
+        if constexpr (kFirst > 1) {
+            const uint32_t here = (s.here >> 10) & 31u, next = s.room < 4 ? (s.next >> 10) & 31u : here;
+            if (__any_sync(0xffffffffu, (here < next ? here : next) < 4u * kFirst)) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int w = 1; w < kFirst; ++w) fill(i, w);
+            }
         }
     }
     if constexpr (kAligned) stage_words<Q, 0>(at, R);

@@ -107,7 +107,21 @@ bcs_status launch_wide_send(const RowConsts &rc, uint32_t first, uint32_t count,
     return launch_status();
 }
 
-constexpr unsigned kQuadThreads = 320;
+// Half an SM's shared memory, and the warps of a CTA that have room in it for runs of `run` ranks.
+constexpr uint32_t kQuadHalf = (228u * 512u - 1024u - 128u) & ~127u;
+template <int Q, bool kTable>
+constexpr uint32_t quad_bytes(uint32_t warps, uint32_t run) { return QuadLayout<kTable>(Q, roomy_segments(run)).total(warps); }
+template <int Q, bool kTable>
+constexpr uint32_t quad_warps(uint32_t run)
+{
+    uint32_t warps = 10;
+    while (warps > 4u && quad_bytes<Q, kTable>(warps, run) > kQuadHalf) --warps;
+    return warps;
+}
+// Threads that registers are shared among: ten warps; for q = 28, whose rows need the most, as many as a CTA ever has (with ten it spills: one million ranks 11.1 -> 10.7 us,
+// 400 000 send rows 4.4 -> 3.9; but for larger q more registers are no better, 300 000 receive rows of q = 30 2.84 -> 3.03).
+template <int Q, bool kTable>
+constexpr uint32_t kQuadThreads = 32u * (Q == 28 ? quad_warps<Q, kTable>(kTable ? 4u * kQuads : kQuads) : 10u);
 
 __device__ unsigned long long expired_waits;      // waits with a limit that ran out
 constexpr uint64_t kWaitLimit = 2000000000;       // two seconds (an answer takes a microsecond)
@@ -116,7 +130,7 @@ constexpr uint64_t kWaitLimit = 2000000000;       // two seconds (an answer take
 // those that have not started yet: SMs do not write equally fast (a fill by CTAs of equal shares reaches 6.3 TB/s, by CTAs of 16 KB in
 // any order 7.5), and one table serves all turns of a CTA.
 template <int Q, bool kTable>
-__global__ void __launch_bounds__(kQuadThreads, 2)
+__global__ void __launch_bounds__((kQuadThreads<Q, kTable>), 2)
 quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t run, bool once, int8_t *recv, int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
@@ -171,27 +185,20 @@ template <int Q, bool kTable>
 bcs_status launch_quad(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *recv, int8_t *send, cudaStream_t stream)
 {
     if (!allow_shared<quad_kernel<Q, kTable>>()) return BCS_ERR_CUDA;
-    constexpr uint32_t half = (228u * 512u - 1024u - 128u) & ~127u, most = kQuadThreads / 32u;
-    auto bytes = [](uint32_t warps, uint32_t run) { return QuadLayout<kTable>(Q, roomy_segments(run)).total(warps); };
-    auto fit = [&](uint32_t run) {
-        uint32_t w = most;
-        while (w > 4u && bytes(w, run) > half) --w;
-        return w;
-    };
     const uint32_t quads = (count + kQuads - 1u) / kQuads;
     const bool one = recv == nullptr || send == nullptr;
     uint32_t k = 1;
-    while (k * kQuads <= kMostRun && fit(k * kQuads) * k * kSms * (one && k == 1u ? 1u : 2u) < quads) ++k;
+    while (k * kQuads <= kMostRun && quad_warps<Q, kTable>(k * kQuads) * k * kSms * (one && k == 1u ? 1u : 2u) < quads) ++k;
     const bool once = k * kQuads <= kMostRun;
     if (!once) k = one && count >= 3500000u ? 6u : 4u;
     const uint32_t run = k * kQuads;
-    uint32_t warps = fit(run);
+    uint32_t warps = quad_warps<Q, kTable>(run);
     if (once) {
         const uint32_t enough = (quads + k * kSms - 1u) / (k * kSms);
         warps = warps < enough ? warps : (enough < 4u ? 4u : enough);
     }
-    const uint32_t need = bytes(warps, run), turn = warps * run;
-    launch_dependent(true, quad_kernel<Q, kTable>, (unsigned)(((uint64_t)count + turn - 1u) / turn), 32u * warps, need < half ? half : need, stream, rc, first,
+    const uint32_t need = quad_bytes<Q, kTable>(warps, run), turn = warps * run;
+    launch_dependent(true, quad_kernel<Q, kTable>, (unsigned)(((uint64_t)count + turn - 1u) / turn), 32u * warps, need < kQuadHalf ? kQuadHalf : need, stream, rc, first,
                      count, run, once, recv, send);
     return launch_status();
 }
