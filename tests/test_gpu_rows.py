@@ -425,3 +425,101 @@ def test_send_rows_alone_where_the_form_changes(bcs, q):
         _check(bcs, p, 0, n, recv=False)
         _check(bcs, p, (p - n) // 2 | 1 if n < p else 0, ((p - n) // 2 | 1 if n < p else 0) + n, recv=False)
         _check(bcs, p, p - n, p, recv=False)
+
+
+# Larger p of a list, each q whose tables fit: the steps of 16, 20 and 24 ranks for receive and send rows, in tables that begin off a 16-byte boundary
+@pytest.mark.parametrize("p", [(1 << 23) + 1, (1 << 24) - 3, (1 << 24) + 1, (3 << 24) + 7, (1 << 26) - 1, (1 << 26) + 1, (1 << 27) + 1, (1 << 28) + 1])
+def test_batches_of_large_p(bcs, p):
+    _batch(bcs, [7, p, 129])
+
+
+def _check_rooted(bcs, p, root, r0, r1, recv, send):
+    q, n = bcs.bcs_q(p), r1 - r0
+    buffers = [_buffer(n * q) for _ in range(2)]
+    ws = torch.empty(bcs.bcs_build_rooted_workspace_bytes(p, root, r0, r1), dtype=torch.int8, device="cuda")
+    bcs.bcs_build_rooted(p, root, r0, r1, *(out if asked else None for (_, out), asked in zip(buffers, (recv, send))), ws)
+    torch.cuda.synchronize()
+    passed = root - r0                                           # the row of rank 0, behind that of p - 1
+    at = np.unique(np.concatenate([np.arange(300), n - 1 - np.arange(300), np.arange(passed - 600, passed + 600), np.random.default_rng(p).integers(0, n, 1000)]))
+    want = oracle.build_ranks(p, ((at + r0 - root) % p).astype(np.uint32))
+    rows = torch.from_numpy(at).cuda()
+    for (raw, out), asked, expect in zip(buffers, (recv, send), want):
+        assert np.array_equal(out.view(n, q)[rows].cpu().numpy(), expect) if asked else bool((raw == 99).all())
+        assert bool((raw[:32] == 99).all()) and bool((raw[32 + n * q:] == 99).all())
+
+
+# Ranges that pass p - 1 in the middle of a run, with one run per warp: even and odd q, multiples of 4 and of 8
+@pytest.mark.parametrize("q", [17, 18, 19, 20, 21, 22, 24, 26, 28, 31])
+def test_one_run_per_warp_rooted(bcs, q):
+    p = min((3 << q - 2) + 12345, (1 << 31) - 1)
+    for n in (80003, 300001):
+        n = min(n, p)
+        r0 = (p - n) // 2
+        for root in (r0 + n // 2, r0 + n - 700):
+            _check_rooted(bcs, p, root, r0, r0 + n, True, True)
+    _check_rooted(bcs, p, root, r0, r0 + n, True, False)
+    _check_rooted(bcs, p, root, r0, r0 + n, False, True)
+
+
+# The same for send rows alone by vectors of 16 bytes, CTAs of half an SM and of a whole one, and for ranges that take turns
+@pytest.mark.parametrize("p,n", [(1000003, 1000003), ((1 << 24) - 5, 700001), ((1 << 24) + 1, 1 << 20), (2000003, 2000003), (5000011, 5000011), (3 << 28, 1900001)])
+def test_send_rows_alone_rooted(bcs, p, n):
+    r0 = (p - n) // 2
+    for root in (r0 + n // 2, r0 + 601, r0 + n - 601):
+        _check_rooted(bcs, p, root, r0, r0 + n, False, True)
+
+
+@pytest.mark.parametrize("p,n", [(3000017, 3000017), ((1 << 28) + 1, 5000001)])
+def test_turns_rooted(bcs, p, n):
+    r0 = (p - n) // 2
+    for recv, send in ((True, True), (True, False)):
+        _check_rooted(bcs, p, r0 + n // 2, r0, r0 + n, recv, send)
+
+
+# Lines of the kernel of four ranks per lane, both sides: runs of one to seven look-ups in 148 or 296 CTAs of ten warps (q = 28: eight), the longest that have one run per
+# warp, turns of 768 ranks, the table of send rows; `tables`: both, receive rows, send rows.
+@pytest.mark.parametrize("p,n,tables", [(2000003, 148 * 10 * 128, "brs"), (2000003, 296 * 10 * 128, "brs"), (2000003, 296 * 10 * 256, "br"), (2000003, 296 * 10 * 384, "brs"),
+                                        (2000003, 296 * 10 * 640, "brs"), ((1 << 22) - 3, 296 * 9 * 896, "br"), (1 << 28, 296 * 8 * 128, "brs"),
+                                        (1 << 28, 296 * 8 * 512, "br"), (1 << 28, 296 * 7 * 896, "br"), ((1 << 24) - 1, 3500000, "r"), ((1 << 23) + 1, 1 << 22, "b")])
+def test_four_ranks_per_lane_on_both_sides_of_its_lines(bcs, p, n, tables):
+    for count in (n, n + 1):
+        for r0 in (0, (p - count) // 2 | 1):
+            for which in tables:
+                _check(bcs, p, r0, r0 + count, recv=which != "s", send=which != "r")
+    assert bcs.bcs_wait_expired() == 0
+
+
+# As test_tables_are_not_written_before_they_are_read, with turns that CTAs take from one another (the wait is in each of them), and with send rows by vectors,
+# some CTAs of which have no ranks.
+@pytest.mark.parametrize("n,which", [(2700001, "both"), (4300001, "both"), (3000001, "recv"), (1000003, "send"), (1900001, "send")])
+@pytest.mark.parametrize("between", [False, True])
+def test_long_tables_are_not_written_before_they_are_read(bcs, n, which, between):
+    p, blocks, next_p = 100003, 150, 6000011
+    q, next_q = bcs.bcs_q(p), bcs.bcs_q(next_p)
+    tables = [torch.from_numpy(t).cuda().view(-1) for t in oracle.full_table(p)]
+    size, written = p * q, n * next_q
+    memory = [torch.empty(written, dtype=torch.int8, device="cuda") for _ in range(2)]         # (longer than the tables: turns in front of, over and behind them)
+    other = [torch.empty(32 * next_q, dtype=torch.int8, device="cuda") for _ in range(2)]
+    out = torch.empty((p, blocks - 1 + q, 4), dtype=torch.int32, device="cuda")
+    busy = torch.empty(1 << 29, dtype=torch.int8, device="cuda")
+    asked = [which != "send", which != "recv"]
+    rows = [torch.empty(written, dtype=torch.int8, device="cuda") if a else None for a in asked]
+    bcs.bcs_build(next_p, 77, 77 + n, *rows)
+    bcs.bcs_expand(p, blocks, 0, p, *tables, out)
+    want = out.clone()
+    for at in (0, (written - size) // 32 * 16, (written - size) // 16 * 16):
+        lie = [m[at:at + size] for m in memory]
+        for m, t in zip(lie, tables):
+            m.copy_(t)
+        out.fill_(-9)
+        torch.cuda.synchronize()
+        for _ in range(4):
+            busy.zero_()                                         # (all that follows is enqueued while this lasts)
+        bcs.bcs_expand(p, blocks, 0, p, *lie, out)
+        if between:
+            bcs.bcs_build(next_p, 0, 32, *other)
+        bcs.bcs_build(next_p, 77, 77 + n, *(m if a else None for m, a in zip(memory, asked)))
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        assert all(torch.equal(m, r) for m, r, a in zip(memory, rows, asked) if a)
+    assert bcs.bcs_wait_expired() == 0
