@@ -123,7 +123,9 @@ class _Calls:
 
     def __getattr__(self, name):
         library = lib()
-        plain = _PLAIN[name[3:]] if name.startswith("on_") else getattr(library, "bcs_" + name)
+        plain = _PLAIN.get(name[3:]) if name.startswith("on_") else getattr(library, "bcs_" + name)
+        if plain is None:
+            raise AttributeError(name)
         call = getattr(_extension(library), name, None) or plain
         setattr(self, name, call)
         return call

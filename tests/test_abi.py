@@ -191,6 +191,16 @@ def test_calls_with_tensors_are_those_with_numbers(lib):
         lib.bcs_build(10, 0, 10, good, good, stream=3)
 
 
+def test_unknown_calls_are_attribute_errors(lib):
+    """Names that are no calls, with tensors or without, are missing attributes."""
+    from paper_2205_10072_b200 import binding
+    for name in ("nothing", "on_nothing", "on_", "on_prepare"):
+        assert not hasattr(binding._call, name)
+        with pytest.raises(AttributeError):
+            getattr(binding._call, name)
+    assert callable(binding._call.on_build)
+
+
 WAITS = r"""
 #include <stdint.h>
 #include <stdio.h>
