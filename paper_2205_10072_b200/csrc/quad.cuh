@@ -271,20 +271,20 @@ __device__ __forceinline__ void stage_words_shifted(uint8_t *at, const uint32_t 
     }
 }
 
-// How the rows of a run lie in memory, and the words that a lane hands on.  Where q is a multiple of 8 the rows of all ranks begin at the same or at two places
-// of a 16-byte group, so up to 15 bytes of shift are left, else 3 (quad_shift()).
+// How the rows of a run lie in memory, and the words that a lane hands on.  Where q is 8 (mod 16) rows begin at one of two places of a 16-byte group, so up to 7 bytes of
+// shift are left, else 3 (quad_shift()).
 template <int Q>
 struct Shifted {
-    static constexpr int kCarry = Q % 8 == 0 ? 4 : 1;
+    static constexpr int kCarry = Q % 8 == 0 ? 2 : 1;
     uint32_t bytes;                                    // by which the run's first row is off a 16-byte group
     uint32_t carry[kCarry];                            // the last words of the 128 ranks before, the last one first
 };
 
 template <int Q, int o, int kWords>
-__device__ __forceinline__ void join_words(const uint32_t (&R)[4][kWords], uint32_t (&V)[Q + 4])
+__device__ __forceinline__ void join_words(const uint32_t (&R)[4][kWords], uint32_t (&V)[Q + 2])
 {
     if constexpr (o < Q) {
-        V[o + 4] = joined<Q, o>(R);
+        V[o + 2] = joined<Q, o>(R);
         join_words<Q, o + 1>(R, V);
     }
 }
@@ -294,28 +294,25 @@ __device__ __forceinline__ void stage_shifted(uint8_t *at, const uint32_t (&R)[4
 {
     const uint32_t lane = threadIdx.x & 31u;
     if constexpr (Q % 8 == 0) {
-        uint32_t V[Q + 4];                             // V[w + 4]: word w
+        static_assert(Q % 16 != 0, "7 bytes of shift at most");
+        uint32_t V[Q + 2];                             // V[w + 2]: word w
         join_words<Q, 0>(R, V);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t before = __shfl_up_sync(0xffffffffu, V[Q + 3 - j], 1);
-            V[3 - j] = lane ? before : sh.carry[j];
+        for (int j = 0; j < 2; ++j) {
+            const uint32_t before = __shfl_up_sync(0xffffffffu, V[Q + 1 - j], 1);
+            V[1 - j] = lane ? before : sh.carry[j];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) sh.carry[j] = __shfl_sync(0xffffffffu, V[Q + 3 - j], 31);
+        for (int j = 0; j < 2; ++j) sh.carry[j] = __shfl_sync(0xffffffffu, V[Q + 1 - j], 31);
         const uint32_t bits = 8u * (sh.bytes & 3u);
 #pragma unroll
-        for (int w = Q + 3; w > 0; --w) V[w] = __funnelshift_l(V[w - 1], V[w], bits);
+        for (int w = Q + 1; w > 0; --w) V[w] = __funnelshift_l(V[w - 1], V[w], bits);
         if (sh.bytes & 4u) {
 #pragma unroll
-            for (int w = Q + 3; w > 1; --w) V[w] = V[w - 1];
-        }
-        if (sh.bytes & 8u) {
-#pragma unroll
-            for (int w = Q + 3; w > 3; --w) V[w] = V[w - 2];
+            for (int w = Q + 1; w > 1; --w) V[w] = V[w - 1];
         }
 #pragma unroll
-        for (int w = 0; w < Q; w += 4) *reinterpret_cast<uint4 *>(at + 4 * w) = make_uint4(V[w + 4], V[w + 5], V[w + 6], V[w + 7]);
+        for (int w = 0; w < Q; w += 4) *reinterpret_cast<uint4 *>(at + 4 * w) = make_uint4(V[w + 2], V[w + 3], V[w + 4], V[w + 5]);
     } else {
         const uint32_t last = joined<Q, Q - 1>(R), before = __shfl_up_sync(0xffffffffu, last, 1);
         stage_words_shifted<Q, 0>(at, R, lane ? before : sh.carry[0], 8u * sh.bytes);
@@ -329,27 +326,16 @@ __device__ __forceinline__ void stage_rest(uint8_t *at, const Shifted<Q> &sh)
 {
     if ((threadIdx.x & 31u) != 0u || sh.bytes == 0u) return;
     if constexpr (Q % 8 == 0) {
-        const uint32_t bits = 8u * (sh.bytes & 3u), s = sh.bytes >> 2;
-        uint32_t F[5];                                 // words -4 .. 0 behind the end, shifted by `bits`
-        F[0] = 0u;
-#pragma unroll
-        for (int j = 1; j < 4; ++j) F[j] = __funnelshift_l(sh.carry[4 - j], sh.carry[3 - j], bits);
-        F[4] = __funnelshift_l(sh.carry[0], 0u, bits);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {                  // word w: word w - s of these
-            uint32_t v = 0u;
-#pragma unroll
-            for (int j = 0; j < 5; ++j)
-                if (w - (int)s == j - 4) v = F[j];
-            reinterpret_cast<uint32_t *>(at)[w] = v;
-        }
+        const uint32_t bits = 8u * (sh.bytes & 3u);
+        const uint32_t one = __funnelshift_l(sh.carry[1], sh.carry[0], bits), two = __funnelshift_l(sh.carry[0], 0u, bits);
+        *reinterpret_cast<uint2 *>(at) = sh.bytes & 4u ? make_uint2(one, two) : make_uint2(two, 0u);
     } else {
         *reinterpret_cast<uint32_t *>(at) = __funnelshift_l(sh.carry[0], 0u, 8u * sh.bytes);
     }
 }
 
 // Of 16 consecutive ranks of a p whose rows begin at byte `entry`, one whose row begins the least behind a 16-byte boundary: 0 bytes for odd q, 1 at most
-// for q = 2 (mod 4), 3 for 4 (mod 8).  Returns rank + 16 bytes.  By a warp.
+// for q = 2 (mod 4), 3 for 4 (mod 8), 7 for 8 (mod 16).  Returns rank + 16 bytes.  By a warp.
 __device__ __forceinline__ uint32_t quad_shift(uint64_t entry, int q)
 {
     const uint32_t rank = threadIdx.x & 15u;
