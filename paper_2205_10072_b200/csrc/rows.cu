@@ -62,18 +62,14 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     stage_free<true>();
 }
 
-// Send rows alone, 16 output bytes per lane (wide.cuh): a run per warp, a CTA for every SM.  Its table of send rows holds those of all the CTA's segments, and
-// nothing is looked up twice.  Two sizes:
-//   * From 13.3 million bytes up to 2^20 ranks, where quad_kernel needs three look-ups a warp and more: CTAs of half an SM, so that the next call's tables are built beside
-//     the rows.  us, this / quad_kernel: 600 000 ranks of q = 21 4.8/4.8, 800 000 5.4/6.1, a million of q = 24 6.0/7.1, of q = 28 6.2/7.2, 500 000 of q = 31
-//     4.5/5.0; 500 000 of q = 21 4.5/4.2, 400 000 of q = 28 4.2/3.8; 1.1 million of q = 21 8.5/7.1.
-//   * From 1.9 million ranks, or where quad_kernel takes turns, to 6 million: 640 threads.  us: 2 million ranks of q = 21 11.3/11.4, of q = 28 12.1/12.8, 3.1 million of q = 23
-//     16.0/18.9, 4.8 million 22.4/23.5, 1.6 million of q = 31 11.6/12.6; 1.5 million of q = 21 10.2/9.1, 6.5 million of q = 24 31.7/29.9, of q = 28 34.7/30.9.
-constexpr uint32_t kWideFrom = 1900000, kWideTo = 6000000, kWideHalf = 1u << 20;
-constexpr uint64_t kWideBytes = 13300000;
+// Send rows alone of 1.9 to 6 million ranks, 16 output bytes per lane (wide.cuh): a run per warp, one CTA per SM.  Its table of send rows holds those of all the
+// CTA's segments, and nothing is looked up twice.  us, this / quad_kernel: 2 million ranks of q = 21 11.3/11.4, of q = 28 12.1/12.8, 3.1 million of q = 23
+// 16.0/18.9, 4.8 million 22.4/23.5; 1.5 million of q = 21 10.2/9.1, 6.5 million of q = 24 31.7/29.9, of q = 28 34.7/30.9.
+constexpr unsigned kWideThreads = 640;
+constexpr uint32_t kWideFrom = 1900000, kWideTo = 6000000;
 
-template <unsigned kThreads, int kCtas, bool kAnyStep>
-__global__ void __launch_bounds__(kThreads, kCtas)
+template <bool kAnyStep>
+__global__ void __launch_bounds__(kWideThreads, 1)
 wide_send_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count, uint32_t run, int8_t *send)
 {
     extern __shared__ __align__(128) uint8_t sm[];
@@ -81,7 +77,7 @@ wide_send_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t 
     const WideLayout at(rc.q);
     const RowTable t(sm, at.base);
     if (threadIdx.x < kRow + kLow + 1) t.s[threadIdx.x] = rc.s[threadIdx.x];
-    const uint32_t warps = kThreads / 32u, warp = threadIdx.x >> 5, begin = blockIdx.x * warps * run;
+    const uint32_t warps = kWideThreads / 32u, warp = threadIdx.x >> 5, begin = blockIdx.x * warps * run;
     if (begin >= count) {                                        // (stays until the kernel before is done, or CTAs of the next calls pile up here)
         grid_dependency_wait();
         return;
@@ -102,12 +98,12 @@ wide_send_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t 
                                     send + (uint64_t)b * (uint64_t)rc.q);
 }
 
-template <unsigned kThreads, int kCtas, bool kAnyStep>
+template <bool kAnyStep>
 bcs_status launch_wide_send(const RowConsts &rc, uint32_t first, uint32_t count, int8_t *send, cudaStream_t stream)
 {
-    if (!allow_shared<wide_send_kernel<kThreads, kCtas, kAnyStep>>()) return BCS_ERR_CUDA;
-    const uint32_t all = kSms * kThreads / 32u * kStep, run = (count + all - 1u) / all * kStep;
-    launch_dependent(true, wide_send_kernel<kThreads, kCtas, kAnyStep>, kSms, kThreads, WideLayout(rc.q).bytes, stream, rc, first, count, run, send);
+    if (!allow_shared<wide_send_kernel<kAnyStep>>()) return BCS_ERR_CUDA;
+    const uint32_t all = kSms * kWideThreads / 32u * kStep, run = (count + all - 1u) / all * kStep;
+    launch_dependent(true, wide_send_kernel<kAnyStep>, kSms, kWideThreads, WideLayout(rc.q).bytes, stream, rc, first, count, run, send);
     return launch_status();
 }
 
@@ -215,10 +211,8 @@ bcs_status launch_quads(const RowConsts &rc, uint32_t first, uint32_t count, int
     if constexpr (Q > BCS_MAX_Q) return BCS_ERR_UNSUPPORTED;
     else {
         if (rc.q != Q) return launch_quads<Q + 1>(rc, first, count, recv, send, stream);
-        constexpr bool any = step_ranks(Q) != 16u;
-        constexpr uint32_t at_once = quad_warps<Q, false>(kMostRun) * (kMostRun / kQuads) * 2u * kSms * kQuads;
-        if (recv == nullptr && count <= kWideHalf && (uint64_t)count * Q >= kWideBytes) return launch_wide_send<384, 2, any>(rc, first, count, send, stream);
-        if (recv == nullptr && count < kWideTo && (count >= kWideFrom || count > at_once)) return launch_wide_send<640, 1, any>(rc, first, count, send, stream);
+        if (recv == nullptr && count >= kWideFrom && count < kWideTo)
+            return step_ranks(Q) == 16u ? launch_wide_send<false>(rc, first, count, send, stream) : launch_wide_send<true>(rc, first, count, send, stream);
         if constexpr (Q >= 22)                                   // (2^22 ranks are more than a smaller p has)
             if (send != nullptr && count >= (1u << 22)) return launch_quad<Q, true>(rc, first, count, recv, send, stream);
         return launch_quad<Q, false>(rc, first, count, recv, send, stream);
