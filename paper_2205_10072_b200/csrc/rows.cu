@@ -62,9 +62,9 @@ rows_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
     stage_free<true>();
 }
 
-// Send rows alone of 1.9 to 6 million ranks, 16 output bytes per lane (wide.cuh): a run per warp, one CTA per SM.  Its table of send rows holds those of all the
+// Send rows alone of 1.9 to 6 million ranks, or from where quad_kernel takes turns (q >= 27), 16 output bytes per lane (wide.cuh): a run per warp, one CTA per SM.  Its table of send rows holds those of all the
 // CTA's segments, and nothing is looked up twice.  us, this / quad_kernel: 2 million ranks of q = 21 11.3/11.4, of q = 28 12.1/12.8, 3.1 million of q = 23
-// 16.0/18.9, 4.8 million 22.4/23.5; 1.5 million of q = 21 10.2/9.1, 6.5 million of q = 24 31.7/29.9, of q = 28 34.7/30.9.
+// 16.0/18.9, 4.8 million 22.4/23.5, 1.7 million of q = 31 12.0/12.9, 1.86 million of q = 28 11.2/12.8; 1.5 million of q = 21 10.2/9.1, 6.5 million of q = 24 31.7/29.9, of q = 28 34.7/30.9.
 constexpr unsigned kWideThreads = 640;
 constexpr uint32_t kWideFrom = 1900000, kWideTo = 6000000;
 
@@ -211,7 +211,8 @@ bcs_status launch_quads(const RowConsts &rc, uint32_t first, uint32_t count, int
     if constexpr (Q > BCS_MAX_Q) return BCS_ERR_UNSUPPORTED;
     else {
         if (rc.q != Q) return launch_quads<Q + 1>(rc, first, count, recv, send, stream);
-        if (recv == nullptr && count >= kWideFrom && count < kWideTo)
+        constexpr uint32_t at_once = quad_warps<Q, false>(kMostRun) * (kMostRun / kQuads) * 2u * kSms * kQuads;
+        if (recv == nullptr && (count >= kWideFrom || count > at_once) && count < kWideTo)
             return step_ranks(Q) == 16u ? launch_wide_send<false>(rc, first, count, send, stream) : launch_wide_send<true>(rc, first, count, send, stream);
         if constexpr (Q >= 22)                                   // (2^22 ranks are more than a smaller p has)
             if (send != nullptr && count >= (1u << 22)) return launch_quad<Q, true>(rc, first, count, recv, send, stream);

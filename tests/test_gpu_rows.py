@@ -499,3 +499,20 @@ def test_long_tables_are_not_written_before_they_are_read(bcs, n, which, between
         assert torch.equal(out, want)
         assert all(torch.equal(m, r) for m, r, a in zip(memory, rows, asked) if a)
     assert bcs.bcs_wait_expired() == 0
+
+
+# Send rows alone that the kernel of four ranks per lane would make in turns are made by vectors from there on, both sides of the line: 1.6 million of q = 31 took 1.22 times as
+# long as 1.58 million (12.6 us), 1.7 million 1.25 times (12.9); 1.10 and 1.16 now.
+@pytest.mark.parametrize("q", [27, 28, 29, 30, 31])
+def test_send_rows_alone_where_turns_begin(bcs, q):
+    p = min((3 << q - 2) + 12345, (1 << 31) - 1)
+    line = (6 if q == 31 else 7) * 7 * 296 * 128
+    for n in (line, line + 1):
+        for r0 in (0, (p - n) // 2 | 1, p - n):
+            _check(bcs, p, r0, r0 + n, recv=False)
+
+
+def test_send_rows_alone_keep_the_faster_form(bcs):
+    p, r0 = (1 << 31) - 1, 306783378
+    fewer, more = (_us_of_range(bcs, p, r0, r0 + n, recv=False) for n in (1580000, 1600000))
+    assert more < 1.17 * fewer
