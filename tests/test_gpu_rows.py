@@ -71,7 +71,7 @@ def test_rows_where_the_split_changes(bcs, p, n):
     _check(bcs, p, r0, r0 + n)
 
 
-# one table alone changes kernels earlier
+# one table alone, at the line between a rank and four ranks per lane
 @pytest.mark.parametrize("n", [148 * 16 * 32, 148 * 16 * 32 + 1, 90001])
 @pytest.mark.parametrize("p", [148 * 16 * 32 + 15000, (1 << 20) + 1, (1 << 23) - 1, 40000003])
 def test_rows_of_one_table_where_the_split_changes(bcs, p, n):
@@ -80,15 +80,15 @@ def test_rows_of_one_table_where_the_split_changes(bcs, p, n):
     _check(bcs, p, r0, r0 + n, recv=False)
 
 
-# steps of 24, 16 and 20 ranks (32 for q = 16: the batches below), runs and items that end inside one
+# four ranks per lane for multiples of 2, 4 and 8 and odd q, runs that end inside a look-up (steps of 16 to 32 ranks, by vectors: the batches below)
 @pytest.mark.parametrize("p,r0,n", [(140001, 0, 140001), (262144, 100000, 98311), (600011, 0, 600011), (1 << 20, 777, 98304 + 24),
                                     ((1 << 23) + 1, (1 << 22) + 12345, 100001), (1 << 24, (1 << 23) - 200000, 400009)])
 def test_rows_of_other_steps(bcs, p, r0, n):
     _check(bcs, p, r0, r0 + n)
 
 
-# the wide form places bytes by q: each q that the tests above leave out, skips that are all odd but the first ones or all even
-# or neither, from an odd rank on, in the launches of up to 2^20 ranks (the per-rank form ends at 151 552) and above it
+# each q that the tests above leave out, skips that are all odd but the first ones or all even or neither, from an odd rank on, with runs of one or two look-ups per
+# warp and of more
 @pytest.mark.parametrize("p", [(1 << q - 1) + 1 for q in (23, 24, 25, 26, 27, 28, 29)] + [(1 << q) - 1 for q in (23, 25, 26, 27, 28, 29)] +
                               [(3 << q - 2) + 12345 for q in (23, 24, 25, 26, 27, 28, 29)])
 def test_wide_rows_of_every_q(bcs, p):
@@ -97,7 +97,7 @@ def test_wide_rows_of_every_q(bcs, p):
             _check(bcs, p, r0, r0 + n)
 
 
-# the kernel for 2^23 ranks and more: its lanes' places repeat every 16 ranks, 30 segments are located at a time
+# turns that CTAs take from one another, send rows by their table
 @pytest.mark.parametrize("p,r0,n", [((1 << 23) + 1, 0, (1 << 23) + 1), (100 << 17, 4000003, (1 << 23) + 385),
                                     ((1 << 24) - 1, 0, (1 << 24) - 1), ((1 << 30) + 20, (1 << 29) - 777777, (1 << 23) + 1),
                                     ((1 << 31) - 1, (1 << 31) - 1 - (1 << 23) - 15, (1 << 23) + 15)])
@@ -238,16 +238,17 @@ def _back_to_back(bcs, p, n, recv=True, send=True, calls=200):
     return min(times)
 
 
-# Fewer ranks do not take longer because some CTAs of the launch have none: 1 000 003 ranks (147 of 148 CTAs have some) took 1.34 times
-# as long as 2^20 (all have), receive rows alone 1.33 and send rows 1.21 times, when those CTAs left at once; 0.97 and 1.01 since they wait.
+# Fewer ranks do not take longer because some CTAs of the launch have none: by vectors, 1 000 003 ranks (147 of 148 CTAs had some) took 1.34 times
+# as long as 2^20 (all had), receive rows alone 1.33 and send rows 1.21 times, when those CTAs left at once; 0.97 and 1.01 since they waited.  (Four ranks per lane: no CTA is without
+# ranks.  Send rows alone of 1.9 million ranks have such CTAs.)
 @pytest.mark.parametrize("recv,send", [(True, True), (True, False), (False, True)])
 def test_ctas_without_ranks_do_not_hold_up_a_row_of_calls(bcs, recv, send):
     p = 1398101
     assert _back_to_back(bcs, p, 1000003, recv, send) < 1.1 * _back_to_back(bcs, p, 1 << 20, recv, send)
 
 
-# One table alone stays with the per-rank form while two of its CTAs fit an SM: 80 000 ranks of q = 21 take 2.4 us (send rows 2.8), a
-# twentieth more than 75 776, and took 3.5 (3.4) in the wide form.
+# One table alone does not take much longer where the form changes: 80 000 ranks of q = 21 took 3.5 us (send rows 3.4) by vectors, 75 776 a rank per lane 2.3 (2.7); four ranks per
+# lane 1.8 (1.9).
 @pytest.mark.parametrize("recv", [True, False])
 def test_one_table_keeps_the_faster_form(bcs, recv):
     assert _back_to_back(bcs, 1398101, 80000, recv, not recv) < 1.15 * _back_to_back(bcs, 1398101, 75776, recv, not recv)
@@ -516,3 +517,10 @@ def test_send_rows_alone_keep_the_faster_form(bcs):
     p, r0 = (1 << 31) - 1, 306783378
     fewer, more = (_us_of_range(bcs, p, r0, r0 + n, recv=False) for n in (1580000, 1600000))
     assert more < 1.17 * fewer
+
+
+# Send rows alone of 1.9 million ranks (145 of 148 CTAs have some), made by vectors, take no longer than 1 894 400 and 1 941 760 (148 have, runs of 640 and 656 ranks)
+def test_send_rows_with_ctas_without_ranks_take_no_longer(bcs):
+    p = (1 << 24) - 5
+    some, all_ = (_us_of_range(bcs, p, 12345, 12345 + n, recv=False) for n in (1900001, 148 * 20 * 656))
+    assert some < 1.1 * all_
