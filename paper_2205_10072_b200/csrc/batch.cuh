@@ -15,8 +15,8 @@
 // this, 25.4 with the first load behind the wait, 22.5 with an ordinary launch; one p of 2000: 6.7, 7.2, 10.5, 10.3; 16 p of 2^10..2^13: 16.8,
 // 18.7.)
 //
-// Up to 1024 ranks: instruction issue, and a CTA's chain from its p to its last row.  Every p up to 1024, four ranks per lane, 11.7 us in any order, 10.9
-// ascending, 11.1 descending (a rank per lane 13.9, 15.4, 12.4).
+// Up to 1024 ranks: instruction issue, and a CTA's chain from its p to its last row.  Every p up to 1024, four ranks per lane, 10.2 us in any order
+// (a rank per lane 13.9).
 // Above, instruction issue and the integer pipe: 1024 p of 2^10..2^20 1250 us (both tables 4.7 TB/s).  That kernel holds two narrow and two wide
 // forms in 80 registers and spills a few bytes at its three CTAs per SM; two per SM take 1368 us, four 1490.
 #pragma once
@@ -398,7 +398,7 @@ bcs_status bcs_build_batch(const uint32_t *p_list_dev, const uint64_t *rank_off_
         }
     }
     // Four ranks per lane for lists without a larger p whose p are 400 on average or more; us with it / the per-rank form: every p up to 1024 in any order
-    // 11.7/13.9, ascending 10.8/15.4, 5000 of 777 43.6/60.8, 800 of 1000 8.1/12.9, 740 of 280..1019 8.8/9.8.  A CTA takes one p, and CTAs whose p
+    // 10.2/13.9, and with seven CTAs per SM 11.7, ascending 10.8/15.4, 5000 of 777 43.6/60.8, 800 of 1000 8.1/12.9, 740 of 280..1019 8.8/9.8.  A CTA takes one p, and CTAs whose p
     // have other q run other code, which counts where there is little to do for each: 900 of 64..256 6.3/5.9, 300 of 64..1000 7.5/6.7, 700 of 2^6..2^12
     // (beside the kernel for larger p) 33.3/29.8.  CTAs of 256 threads while three of them per SM take the list (140 of 900 4.6, with 128 threads 5.1).
     if (small_only && total_ranks >= 400ull * num_p) {

@@ -11,7 +11,7 @@
 //     of column k from skips[k] further on are the entries of a lane's four ranks.  Transposed back they are their rows.  Long ranges look
 //     them up in a table of send rows (kTable).
 //
-// Some 700 warp instructions for both rows of 128 ranks of q = 21 (1000 with 128 ranks a pass and the exceptions segment after segment; 1230 by vectors of
+// Some 700 warp instructions for both rows of 128 ranks of q = 21, 520 where send rows come from their table (1000 with 128 ranks a pass and the exceptions segment after segment; 1230 by vectors of
 // 16 output bytes), of which the integer pipe takes half at half rate: that and the issue slots bound the kernel until memory does.  The exceptions take
 // 85, the transpositions and the ranks behind 120, the packing and staging of rows 150, a bulk copy some 20.
 #pragma once
@@ -388,7 +388,7 @@ __device__ __forceinline__ void stage_quad(uint8_t *at, const uint32_t (&lo)[4],
     };
     if constexpr (Q % 8 != 0) {
         // (loaded once more for each rank rather than selected, word by word, from those of two segments: the integer pipe has more to do than shared
-        // memory, 1.06 million ranks of q = 21 10.1 -> 9.9 us; but q = 24, whose rows meet in banks, 12 million ranks 88.4 -> 91.4)
+        // memory, 1.06 million ranks of q = 21 0.2 us less, of about 10; but q = 24, whose rows meet in banks, 12 million ranks 88.4 -> 91.4)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             load(S, i == 0 || i < s.room ? from : from + 64);

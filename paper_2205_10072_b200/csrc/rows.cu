@@ -1,13 +1,14 @@
 // Receive and send rows of a stretch of ranks of one p: the kernels behind bcs_build and its relatives.
 //
-// One launch, nothing read from memory but constants, no table of all ranks (rows.cuh).  Two forms, by size (launch_rows):
+// One launch, nothing read from memory but constants, no table of all ranks (rows.cuh).  By size (launch_rows):
 //   * rows_kernel, a rank per lane.  Bound by latency: launch, table, one or two items per warp.  From Python 32 ranks 3.2 us back to
 //     back, all ranks of 1152 3.3, 65 553 ranks 3.2 (2.7 on the device).  The table holds what the
 //     CTA's segments need where these are few, and a CTA has no more warps than items.
 //   * quad_kernel, four ranks per lane (quad.cuh).  Up to some 2^21 ranks bound by instruction issue, the integer pipe with it, above by
-//     memory writes.  All ranks of 100 003 2.4 us, of 1.06 million 9.9, 2^24 ranks of q = 28 132, 2^25 receive rows 134 (7.0 TB/s).  With vectors
-//     of 16 output bytes per lane in its place, some 40 warp instructions for every 32 of them where a segment ends: 4.9, 13.6, 146 and 149.
-// Both are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
+//     memory writes.  All ranks of 100 003 2.4 us, of 1.06 million 9.6, 2^24 ranks of q = 28 133, 2^25 receive rows 140 (6.7 TB/s).  With vectors
+//     of 16 output bytes per lane in its place, some 40 warp instructions for every 32 of them where a segment ends: 4.9, 13.3, 148 and 148.
+//   * wide_send_kernel, 16 output bytes per lane (wide.cuh): send rows alone of some million ranks.
+// All are launched as dependents of whatever runs before them on the stream and wait for it before their first store.
 #include "batch.cuh"     // (in this unit, too: the constants of rows.cuh are in the module once)
 #include "rows.cuh"
 #include "quad.cuh"
@@ -119,7 +120,7 @@ constexpr uint32_t quad_warps(uint32_t run)
     return warps;
 }
 // Threads that registers are shared among: ten warps; for q = 28, whose rows need the most, as many as a CTA ever has (with ten it spills: one million ranks 11.1 -> 10.7 us,
-// 400 000 send rows 4.4 -> 3.9; but for larger q more registers are no better, 300 000 receive rows of q = 30 2.84 -> 3.03).
+// 400 000 send rows 4.4 -> 3.9; q = 25 to 27 spill a word; for larger q more registers are no better, 300 000 receive rows of q = 30 2.84 -> 3.03).
 template <int Q, bool kTable>
 constexpr uint32_t kQuadThreads = 32u * (Q == 28 ? quad_warps<Q, kTable>(kTable ? 4u * kQuads : kQuads) : 10u);
 
@@ -176,7 +177,7 @@ quad_kernel(const __grid_constant__ RowConsts rc, uint32_t first, uint32_t count
 
 // Turns and CTAs.  Runs are whole look-ups (128 ranks): partly filled ones cost as much.  The shortest run with which at most 296 CTAs of up to ten warps
 // (as many as two CTAs per SM have shared memory for) have all ranks at once; and no more warps than make 148 CTAs, which leave room for the
-// next call's (back to back, us: all ranks of 100 003 2.4, with the ranks spread over 296 CTAs 4.5; 200 000 ranks of q = 21 4.2 and 4.9, 524 288 6.6
+// next call's (back to back, us, the kernel as it was when this was chosen: all ranks of 100 003 2.4, with the ranks spread over 296 CTAs 4.5; 200 000 ranks of q = 21 4.2 and 4.9, 524 288 6.6
 // and 6.5, 1.06 million 10.2 and 10.3).  One table: two look-ups as soon as 148 CTAs do not do with one (200 000 receive rows 2.6 us, with runs of 128 3.0).
 // The shared memory is filled up to half an SM, lest three CTAs of one call meet on an SM while another one has one.
 // Longer ranges: turns of 512 ranks per warp, of 768 for one table from 3.5 million on (2^24 send rows of q = 28 71 us, with 512 74; receive rows of 3
@@ -268,8 +269,9 @@ bcs_status launch_rows(uint32_t p, uint64_t first, uint64_t count, int8_t *recv,
     //     ranks          q = 20                 q = 24                 q = 28                 q = 31
     //     32 768    2.0/2.2 (14.3/16.0)    2.1/2.5 (14.3/15.0)    2.1/2.6 (14.3/15.2)    2.1/2.9 (14.6/15.5)
     //     65 553    2.7/2.4 (14.6/15.4)    2.7/2.6 (14.6/15.1)    2.8/2.7 (14.6/15.0)    2.8/2.9 (14.9/15.5)
-    //     75 777    2.9/2.4 (14.6/14.9)    3.0/2.6 (14.5/15.2)    4.6/2.8 (14.6/15.3)    4.7/3.1 (14.7/15.4)
-    //     98 304    5.2/2.5 (17.6/15.1)    4.9/2.8 (15.1/15.0)    4.8/3.2 (14.8/15.2)    5.0/3.5 (15.4/14.9)
+    //     75 777    2.7/2.2 (15.5/15.1)    2.8/2.3 (15.7/15.5)    4.4/2.3 (15.9/15.7)    4.5/2.6 (16.0/15.9)
+    //     98 304    4.9/2.4 (17.5/15.0)    4.6/2.7 (16.1/15.4)    4.5/2.7 (16.3/15.6)    4.7/3.0 (16.4/15.7)
+    // (The first two lines with the kernel as it was before low ranks were put together by their entries' zero bytes, on another box.)
     if (rc.q >= kQuadMinQ && count > kSms * 16u * 32u) return launch_quads<kQuadMinQ>(rc, x0, ranks, recv, send, stream);
     return launch<1>(rc, x0, ranks, recv, send, stream);
 }
